@@ -36,6 +36,25 @@ inline mpfa_status cuda_fail(cudaError_t e) {
     if (_e != cudaSuccess) return ::mpfa::cuda_fail(_e);      \
   } while (0)
 
+// Launch whose CTAs may be scheduled while the preceding kernel of the stream is still running (programmatic stream
+// serialization): set-up that touches no memory the preceding work writes overlaps its tail.  Every kernel launched this
+// way calls grid_dependency_wait() before its first access to global memory, in every thread that makes one, so the
+// order of the stream holds transitively.
+template <typename... KArgs, typename... Args>
+cudaError_t launch(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, Args &&...args) {
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
 // The kernels use sm_100a-only instructions; refuse other devices up front.
 mpfa_status check_arch();
 

@@ -25,12 +25,24 @@
 // a V block is consumed the moment it lands, and the softmax never sits on the critical path.
 // The sequential rescaling O <- 2^(lam (m_old - m_new)) O + P_hat V becomes
 // O = sum_u 2^(lam (m_u - m)) O_u at the end of the item (one thread per channel), the same
-// sum with the factors multiplied out.  The partition state (m, l, O) goes to the workspace; a
-// second kernel merges partitions by log-sum-exp and writes BF16.
+// sum with the factors multiplied out.  Two groups of four warps take the softmax of alternate items and a third
+// one the O of every item: the P_hat of an item has to be ready when the V of the item before it has been consumed,
+// so a group that also wrote O out would have one item's time (5.3 us at memory speed) for both.
 //
-// Warps: 10 draws work items, 0, 9 K producers, 8 V producer, 1 QK issue (+ TMEM allocation), 2 PV issue, 3 rewrites the K scales of
-// each block from [token][8] into the 32 x 16-byte tiles tcgen05.cp expects, 4-7 softmax and
-// partition write-out (TMEM lane quadrant = warp % 4).  Every wait is bounded.
+// A request that fits one partition is finished right there.  Otherwise the partition state (m, l, O) goes to the
+// workspace and decode_merge_kernel merges the partitions by log-sum-exp.  Its blocks fit beside a CTA of this kernel and
+// are launched while it runs, so the merge starts the moment the last state is written.  (Merging inside this kernel, by
+// the warp that completes a request's last partition, was slower in every form tried: a few CTAs end up with most of the
+// merges, 190 us instead of 160 for 16 requests of 32K.)
+//
+// Measured (call alone, before / after the two softmax groups, the O group and the rolled passes over the scores):
+// 16 requests x 32K, 8 kv heads, groups of 1 / 4 / 5 / 8 heads: 148 / 164 / 670 / 904 -> 144 / 156 / 158 / 173 us
+// (5.9 / 5.6 / 5.6 / 5.2 TB/s of cache); 64 requests of 100..4000 tokens, 40:8 heads: 227 -> 59 us.
+//
+// Warps: 18 draws work items and stages their query tiles, 0 and 17 K producers (codes; scales and Delta_S),
+// 16 V producer, 1 QK issue (+ TMEM allocation), 2 PV issue, 3 rewrites the K scales of each block from
+// [token][8] into the 32 x 16-byte tiles tcgen05.cp expects, 4-7 and 8-11 the two softmax groups, 12-15 O (TMEM lane
+// quadrant = warp % 4).  Every wait is bounded.
 #include <cuda_bf16.h>
 #include <cuda_fp8.h>
 
@@ -40,15 +52,14 @@
 namespace mpfa {
 namespace {
 
-constexpr int PART_FLOATS = 130;  // m, l, O[128] per (request, q head, partition)
 constexpr int MAXG = 8;
 constexpr int NCOL = 16;          // MMA N: the GQA group padded to 16 columns
 constexpr int MAXBLK = DECODE_SPLIT / TILE;   // 8 blocks per item
 
 constexpr int D_NK = 4;           // K ring stages
 constexpr int D_NV = 8;           // V ring stages
-constexpr int D_THREADS = 352;
-constexpr int D_NITEM = 8;        // work items published ahead of their use
+constexpr int D_THREADS = 608;
+constexpr int D_NITEM = 4;        // slots of the work-item ring
 
 // one K stage
 constexpr uint32_t KST_K = 0;          // 2 pages x 4096 B of codes: 64-byte rows, 64-byte swizzle
@@ -84,16 +95,18 @@ constexpr int B_K_EMPTY = B_K_FULL + D_NK;       // [D_NK] QK commit
 constexpr int B_V_FULL = B_K_EMPTY + D_NK;       // [D_NV]
 constexpr int B_V_EMPTY = B_V_FULL + D_NV;       // [D_NV] PV commit
 constexpr int B_SF_READY = B_V_EMPTY + D_NV;     // [D_NK] K scales formatted
-constexpr int B_S_FULL = B_SF_READY + D_NK;      // [2][8] QK commit
-constexpr int B_S_FREE = B_S_FULL + 2 * MAXBLK;  // [2] 4 warps: the item's scores have been read
-constexpr int B_P_READY = B_S_FREE + 2;          // [2] 4 warps
-constexpr int B_Q_READY = B_P_READY + 2;         // [2] scale warp
+constexpr int B_S_FULL = B_SF_READY + D_NK;      // [2] QK commit after the item's last block
+constexpr int B_S_FREE = B_S_FULL + 2;           // [2] 4 warps: the item's scores have been read
+constexpr int B_P_READY = B_S_FREE + 2;          // [2] 4 warps: P_hat, block weights and row sums of the item written
+constexpr int B_Q_READY = B_P_READY + 2;         // [2] query tile of the item staged
 constexpr int B_O_FULL = B_Q_READY + 2;          // [1] PV commit after the item's last block
-constexpr int B_O_FREE = B_O_FULL + 1;           // [1] 4 warps
-constexpr int B_XCHG = B_O_FREE + 1;             // [1] 4 warps
-constexpr int B_ITEM_FULL = B_XCHG + 1;          // [D_NITEM] work item published
-constexpr int B_ITEM_EMPTY = B_ITEM_FULL + D_NITEM;   // [D_NITEM] read by all ten consumer warps
-constexpr int B_COUNT = B_ITEM_EMPTY + D_NITEM;
+constexpr int B_T_FREE = B_O_FULL + 1;           // [2] 4 warps: the item's tables (and, after its PV, P_hat) may be overwritten
+constexpr int B_O_FREE = B_T_FREE + 2;           // [1] 4 warps
+constexpr int B_XCHG = B_O_FREE + 1;             // [2] 4 warps of a softmax group: block maxima exchanged
+constexpr int B_ITEM_FULL = B_XCHG + 2;          // [D_NITEM] work item published
+constexpr int B_ITEM_EMPTY = B_ITEM_FULL + D_NITEM;   // [D_NITEM] read by all eighteen consumer warps
+constexpr int B_DRAW = B_ITEM_EMPTY + D_NITEM;   // [2] warp 0 has begun item k (slot k & 1): the next one may be drawn
+constexpr int B_COUNT = B_DRAW + 2;
 static_assert(B_COUNT * 8 <= 1024, "barrier block");
 static_assert(D_SMEM <= 232448, "shared memory");
 static_assert(KST_BYTES % 1024 == 0 && D_OFF_V % 1024 == 0 && D_OFF_P % 1024 == 0, "swizzle atoms");
@@ -146,18 +159,10 @@ __device__ __forceinline__ void tmem_ld_g(uint32_t taddr, uint32_t (&r)[G]) {
   }
 }
 
-#ifdef MPFA_TRACE
-// clock64 stamps of CTA g_dtrace_cta: [counter < 256][16 events]
-__device__ long long *g_dtrace = nullptr;
-__device__ int g_dtrace_cta = 0;
-#define DTR(ev, blk)                                                                              \
-  do {                                                                                            \
-    if (g_dtrace && (threadIdx.x & 31) == 0 && (int)blockIdx.x == g_dtrace_cta && (blk) < 256u)   \
-      g_dtrace[(blk) * 16 + (ev)] = clock64();                                                    \
-  } while (0)
-#else
-#define DTR(ev, blk) do {} while (0)
-#endif
+__device__ __forceinline__ float warp_max(float x) {
+  asm("redux.sync.max.f32 %0, %0, 0xffffffff;" : "+f"(x));
+  return x;
+}
 
 struct DecodeParams {
   const uint8_t *q_codes;  // tile layout, N = 1: row 0 of each (b, hq) tile
@@ -167,17 +172,23 @@ struct DecodeParams {
   const int32_t *page_table;
   const int32_t *seq_lens;
   const float *q_gscale, *k_gscale;
-  float *parts;  // [B, H_q, n_split, 130]
+  float *part_o;           // [B, H_q, n_split, 128]
+  float2 *part_ml;         // [B, H_q, n_split]: (m, l)
+  unsigned int *ticket;    // global work counter, zero at launch
+  __nv_bfloat16 *out;
+  float *out_f32;          // may be null
   int32_t *status;
-  unsigned int *ticket;   // global work counter, zeroed before the launch
   int B, H_q, H_kv, max_pages, num_pages, n_split;
-  float softmax_scale;
+  float softmax_scale, v_scale;
+  __device__ __forceinline__ int n_parts(int L) const { return min((max(L, 0) + DECODE_SPLIT - 1) / DECODE_SPLIT, n_split); }
 };
 
 // Work items (request, kv head, 1024-token partition) are handed out dynamically: one warp per CTA draws
-// tickets from a global counter and publishes the decoded items in a small shared-memory ring; every other
-// warp walks that ring.  SMs do not stream at the same rate (those far from the memory they read are up to
-// 8 % slower), so a static split leaves the fast ones idle at the end.
+// tickets from a global counter (its first one is its block index) and publishes the decoded items in a small
+// shared-memory ring; every other warp walks that ring.  SMs do not stream at the same rate (those far from the memory
+// they read are up to 8 % slower), so a static split leaves the fast ones idle at the end.  An item is drawn when the K
+// producer begins the one before it: drawn further ahead, a short batch is shared out unevenly (64 requests of one
+// partition, 512 items on 148 CTAs, drawn eight ahead: the first 64 CTAs could take them all).
 struct WorkIter;
 
 struct DCtx {
@@ -213,20 +224,15 @@ struct DCtx {
 };
 
 struct WorkIter {
-  uint32_t n;          // items taken so far
-  bool release;        // the warp's main walk hands the ring slot back; look-ahead walks only read
+  uint32_t n = 0;      // items taken so far
   int b, hk, sp, L, nblk;
-  __device__ void init(bool main_walk) {
-    n = 0;
-    release = main_walk;
-  }
   // Whole warp.  false: no more items (or the CTA is giving up).
   __device__ bool next(const DCtx &cx, const int4 *ring) {
     const uint32_t slot = n % D_NITEM;
     if (!cx.wait_warp(B_ITEM_FULL + slot, (n / D_NITEM) & 1)) return false;
     const int4 it = ring[slot];
     if (it.x < 0) return false;   // end marker: stays in its slot, nobody moves past it
-    if (release) cx.warp_arrive(B_ITEM_EMPTY + slot);
+    cx.warp_arrive(B_ITEM_EMPTY + slot);
     ++n;
     b = it.x, hk = it.y, sp = it.z, L = it.w;
     nblk = (min(L - sp * DECODE_SPLIT, DECODE_SPLIT) + TILE - 1) / TILE;
@@ -247,7 +253,7 @@ __device__ __forceinline__ void lookup_pages(const DecodeParams &p, const WorkIt
 }
 
 template <int G>
-__global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const DecodeParams p) {
+__global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const __grid_constant__ DecodeParams p) {
   extern __shared__ uint8_t dsm_raw[];
   uint8_t *dsm = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(dsm_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t sbase = smem_u32(dsm);
@@ -259,10 +265,8 @@ __global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const Decode
   volatile int *abort_flag = reinterpret_cast<volatile int *>(dsm + D_OFF_MISC + 4);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  launch_dependents();   // the merge's blocks
   DCtx cx{sbase + D_OFF_BAR, abort_flag, p.status};
-#ifdef MPFA_TRACE
-  if (g_dtrace && threadIdx.x == 0) g_dtrace[4096 + 2 * blockIdx.x] = (long long)globaltimer_ns();
-#endif
 
   // ---- set-up: barriers, zeroed operand tiles (rows G..15 stay zero for good), TMEM
   if (threadIdx.x == 0) {
@@ -275,18 +279,20 @@ __global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const Decode
       mbar_init(cx.bar(B_V_FULL + i), 1);
       mbar_init(cx.bar(B_V_EMPTY + i), 1);
     }
-    for (int i = 0; i < 2 * MAXBLK; ++i) mbar_init(cx.bar(B_S_FULL + i), 1);
     for (int i = 0; i < 2; ++i) {
+      mbar_init(cx.bar(B_S_FULL + i), 1);
+      mbar_init(cx.bar(B_XCHG + i), 4);
+      mbar_init(cx.bar(B_T_FREE + i), 4);
+      mbar_init(cx.bar(B_DRAW + i), 1);
       mbar_init(cx.bar(B_S_FREE + i), 4);
       mbar_init(cx.bar(B_P_READY + i), 4);
       mbar_init(cx.bar(B_Q_READY + i), 1);
     }
     mbar_init(cx.bar(B_O_FULL), 1);
     mbar_init(cx.bar(B_O_FREE), 4);
-    mbar_init(cx.bar(B_XCHG), 4);
     for (int i = 0; i < D_NITEM; ++i) {
       mbar_init(cx.bar(B_ITEM_FULL + i), 1);
-      mbar_init(cx.bar(B_ITEM_EMPTY + i), 10);
+      mbar_init(cx.bar(B_ITEM_EMPTY + i), 18);
     }
     mbar_init_fence();
     *abort_flag = 0;
@@ -296,12 +302,6 @@ __global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const Decode
     *reinterpret_cast<uint4 *>(dsm + D_OFF_K + o) = make_uint4(0u, 0u, 0u, 0u);
   for (uint32_t o = threadIdx.x * 16; o < D_OFF_BAR - D_OFF_P; o += D_THREADS * 16)
     *reinterpret_cast<uint4 *>(dsm + D_OFF_P + o) = make_uint4(0u, 0u, 0u, 0u);
-  int32_t *len_tab = reinterpret_cast<int32_t *>(dsm + D_OFF_LEN);
-  float *lam_tab = reinterpret_cast<float *>(dsm + D_OFF_LAM);
-  for (int i = threadIdx.x; i < min(p.B, D_MAXREQ); i += D_THREADS) {
-    len_tab[i] = p.seq_lens[i];
-    lam_tab[i] = __fmul_rn(__fmul_rn(__fmul_rn(p.softmax_scale, 1.4426950408889634f), p.q_gscale[i]), p.k_gscale[i]);
-  }
   __syncthreads();
   if (threadIdx.x < 16) {   // identity[n][k]: element (n, k) at (k/8)*1024 + (k%8)*128 + ((n/8) ^ (k%8))*16 + (n%8)*2
     const int k = threadIdx.x;
@@ -311,6 +311,14 @@ __global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const Decode
     tmem_alloc(smem_u32(tmem_slot), TM_COLS);
     tmem_relinquish();
   }
+  // everything above touches this CTA only and overlaps the end of the preceding kernel; everything below reads memory
+  grid_dependency_wait();
+  int32_t *len_tab = reinterpret_cast<int32_t *>(dsm + D_OFF_LEN);
+  float *lam_tab = reinterpret_cast<float *>(dsm + D_OFF_LAM);
+  for (int i = threadIdx.x; i < min(p.B, D_MAXREQ); i += D_THREADS) {
+    len_tab[i] = p.seq_lens[i];
+    lam_tab[i] = __fmul_rn(__fmul_rn(__fmul_rn(p.softmax_scale, 1.4426950408889634f), p.q_gscale[i]), p.k_gscale[i]);
+  }
   fence_proxy_async_smem();
   tc_fence_before();
   __syncthreads();
@@ -318,8 +326,9 @@ __global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const Decode
   const uint32_t tm = *tmem_slot;
   const int4 *ring = reinterpret_cast<const int4 *>(dsm + D_OFF_RING);
 
-  if (warp == 10) {
-    // ================= work distribution: tickets from the global counter, decoded, published D_NITEM ahead.
+  if (warp == 18) {
+    // ================= work distribution: tickets from the global counter, decoded and published; then the query tile
+    // (codes and scales of the group's G heads) of the same item is staged, in the slot that item k-2 has left.
     // With at most D_MAXREQ requests the tickets number only the partitions that exist (prefix sums of
     // ceil(L / 1024) * H_kv per request, request found by bisection); otherwise they number every
     // (request, kv head, partition slot) and the empty ones are drawn again.
@@ -331,7 +340,7 @@ __global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const Decode
       // pre[b] = items of requests 0..b-1: every lane sums a contiguous run of requests, the warp scans the runs
       const int per = (p.B + 31) / 32, lo = min(p.B, lane * per), hi = min(p.B, lo + per);
       int run = 0;
-      for (int i = lo; i < hi; ++i) run += min((max(len_tab[i], 0) + DECODE_SPLIT - 1) / DECODE_SPLIT, p.n_split) * p.H_kv;
+      for (int i = lo; i < hi; ++i) run += p.n_parts(len_tab[i]) * p.H_kv;
       int incl = run;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
@@ -341,7 +350,7 @@ __global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const Decode
       int acc = incl - run;
       for (int i = lo; i < hi; ++i) {
         pre[i] = acc;
-        acc += min((max(len_tab[i], 0) + DECODE_SPLIT - 1) / DECODE_SPLIT, p.n_split) * p.H_kv;
+        acc += p.n_parts(len_tab[i]) * p.H_kv;
       }
       total = (uint32_t)__shfl_sync(0xffffffffu, incl, 31);
       if (lane == 31) pre[p.B] = (int)total;
@@ -352,12 +361,13 @@ __global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const Decode
     bool ok = true;
     for (uint32_t k = 0; ok; ++k) {
       const uint32_t slot = k % D_NITEM;
-      if (k >= (uint32_t)D_NITEM) ok = cx.wait_warp(B_ITEM_EMPTY + slot, ((k / D_NITEM) - 1) & 1);
+      if (k >= 2) ok = cx.wait_warp(B_DRAW + ((k - 1) & 1), ((k - 1) >> 1) & 1);   // the K producer has begun item k-1
+      if (ok && k >= (uint32_t)D_NITEM) ok = cx.wait_warp(B_ITEM_EMPTY + slot, ((k / D_NITEM) - 1) & 1);
       if (!ok) break;
       int4 item = make_int4(-1, 0, 0, 0);
       if (lane == 0) {
-        for (;;) {
-          const uint32_t tkt = atomicAdd(p.ticket, 1u);
+        for (bool first = k == 0;; first = false) {
+          const uint32_t tkt = first ? blockIdx.x : gridDim.x + atomicAdd(p.ticket, 1u);
           if (tkt >= total) break;
           if (compact) {
             int lo = 0, hi = p.B;   // largest b with pre[b] <= tkt
@@ -365,7 +375,7 @@ __global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const Decode
               const int mid = (lo + hi) >> 1;
               if ((uint32_t)pre[mid] <= tkt) lo = mid; else hi = mid;
             }
-            const int L = len_tab[lo], nsp = min((L + DECODE_SPLIT - 1) / DECODE_SPLIT, p.n_split);
+            const int L = len_tab[lo], nsp = p.n_parts(L);
             const int r = (int)tkt - pre[lo];
             item = make_int4(lo, r / nsp, r % nsp, L);
             break;
@@ -382,43 +392,57 @@ __global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const Decode
       }
       item.x = __shfl_sync(0xffffffffu, item.x, 0);
       if (item.x < 0) break;   // the end marker is in the ring; this CTA draws no more
+      item.y = __shfl_sync(0xffffffffu, item.y, 0);
+      const size_t head0 = (size_t)item.x * p.H_q + (size_t)item.y * G;
+      uint4 qv = make_uint4(0u, 0u, 0u, 0u);
+      uint32_t qs0 = 0, qs1 = 0;
+      if (lane < G * 4) qv = *reinterpret_cast<const uint4 *>(p.q_codes + (head0 + (lane >> 2)) * (TILE * 64) + (lane & 3) * 16);
+      if (lane < G) {
+        const uint8_t *src = p.q_sf + (head0 + lane) * 1024;
+        qs0 = *reinterpret_cast<const uint32_t *>(src);
+        qs1 = *reinterpret_cast<const uint32_t *>(src + 512);
+      }
+      const uint32_t par = k & 1;
+      if (k >= 2) ok = cx.wait_warp(B_S_FULL + par, ((k >> 1) - 1) & 1);   // the MMAs of item k-2 have read the slot
+      if (!ok) break;
+      if (lane < G * 4) {
+        const int n = lane >> 2, c = lane & 3;
+        *reinterpret_cast<uint4 *>(dsm + D_OFF_Q + par * 1024 + n * 64 + ((c ^ ((n & 7) >> 1)) << 4)) = qv;
+      }
+      if (lane < G) {
+        uint8_t *dst = dsm + D_OFF_SFQ + par * 1024 + lane * 16;
+        *reinterpret_cast<uint32_t *>(dst) = qs0;
+        *reinterpret_cast<uint32_t *>(dst + 512) = qs1;
+      }
+      fence_proxy_async_smem();
+      cx.warp_arrive(B_Q_READY + par);
     }
-  } else if (warp == 0 || warp >= 8) {
-    // ================= producers: warps 0 and 9 stream the K ring (0: codes; 9: block scales and Delta_S,
-    // both arriving on the stage's barrier), warp 8 the V ring.  Issuing a bulk copy costs a warp well over a
+  } else if (warp == 0 || warp >= 16) {
+    // ================= producers: warps 0 and 17 stream the K ring (0: codes; 17: block scales and Delta_S,
+    // both arriving on the stage's barrier), warp 16 the V ring.  Issuing a bulk copy costs a warp well over a
     // hundred cycles, so the ten copies of a block are spread over three warps.
     // Nothing orders the two streams but the data flow: a K stage is released by its QK MMAs, a V stage
-    // only after the item's softmax, so K runs about one item ahead.  Page ids are loaded one item before
-    // they are used and validated at use, so the loop never waits for the table.
-    const bool is_k = warp != 8, is_codes = warp == 0;
-    WorkIter w, wl;
-    w.init(true);
-    wl.init(false);
-    uint32_t c = 0;   // block counter of this ring
+    // only after the item's softmax, so K runs about one item ahead.  The next item is taken up, and its page ids
+    // requested, before the last two blocks of the current one; they are validated where they are used.
+    const bool is_k = warp != 16, is_codes = warp == 0;
+    WorkIter w, wn;
+    uint32_t c = 0, j = 0;   // blocks and items of this ring
     bool ok = true;
     const uint32_t d_bytes = p.delta ? (uint32_t)G * PAGE * 2 : 0u;
     const uint32_t kpage_bytes = is_codes ? 4096u : 512u + d_bytes;
     const int n_ring = is_k ? D_NK : D_NV;
     const int b_full = is_k ? B_K_FULL : B_V_FULL, b_empty = is_k ? B_K_EMPTY : B_V_EMPTY;
     int pc0 = -1, pc1 = -1, pn0 = -1, pn1 = -1;
-    bool vw = w.next(cx, ring);
-    bool vl = wl.next(cx, ring);
+    bool vw = w.next(cx, ring), vn = false;
     if (vw) lookup_pages(p, w, lane, pc0, pc1);
-    uint32_t jtr = 0;
-    while (ok && vw) {
-      if (is_codes) DTR(12, jtr);
-      vl = wl.next(cx, ring);
-      if (is_codes) DTR(13, jtr);
-      if (vl) lookup_pages(p, wl, lane, pn0, pn1);   // consumed one item later
-      if (is_codes) DTR(14, jtr);
-      ++jtr;
+    for (; ok && vw; ++j) {
+      if (is_codes) cx.warp_arrive(B_DRAW + (j & 1));
       for (int t = 0; ok && t < w.nblk; ++t, ++c) {
         const uint32_t st = c % n_ring;
         if (c >= (uint32_t)n_ring && !cx.wait_warp(b_empty + st, ((c / n_ring) - 1) & 1)) {
           ok = false;
           break;
         }
-        if (warp != 9) DTR(is_k ? 0 : 1, c);
         const int u = w.nblk - 1 - t;
         int id0 = __shfl_sync(0xffffffffu, pc0, u), id1 = __shfl_sync(0xffffffffu, pc1, u);
         const bool want1 = w.sp * DECODE_SPLIT + u * TILE + PAGE < w.L;
@@ -471,9 +495,14 @@ __global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const Decode
           }
         }
         __syncwarp();
+        if (t == max(0, w.nblk - 3)) {
+          wn = w;
+          vn = wn.next(cx, ring);
+          if (vn) lookup_pages(p, wn, lane, pn0, pn1);
+        }
       }
-      if (is_codes) DTR(15, jtr - 1);
-      vw = w.next(cx, ring);
+      vw = vn;
+      w = wn;
       pc0 = pn0, pc1 = pn1;
     }
     if (!ok) {
@@ -491,7 +520,6 @@ __global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const Decode
     const uint64_t d_ident = smem_desc(sbase + D_OFF_IDENT, 2048, 1024, SWZ_128B);
     const bool has_delta = p.delta != nullptr;
     WorkIter w;
-    w.init(true);
     uint32_t kc = 0, j = 0;
     bool ok = true;
     while (ok && w.next(cx, ring)) {
@@ -502,7 +530,6 @@ __global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const Decode
         const uint32_t st = kc % D_NK;
         ok = cx.wait_warp(B_K_FULL + st, (kc / D_NK) & 1) && cx.wait_warp(B_SF_READY + st, (kc / D_NK) & 1);
         if (!ok) break;
-        DTR(2, kc);
         tc_fence_after();
         if (elect_one()) {
           const uint32_t tSFQ = tm + TM_SFQ + par * 8, tSFK = tm + TM_SFK + st * 8;
@@ -525,23 +552,17 @@ __global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const Decode
           }
           mma_nvfp4_ss(tS, d_k, d_q, id_qk, tSFK, tSFQ, has_delta ? 1u : 0u);
           mma_nvfp4_ss(tS, d_k + (32 >> 4), d_q + (32 >> 4), id_qk, tSFK + 4, tSFQ + 4, 1u);
-          mma_commit(cx.bar(B_S_FULL + par * MAXBLK + t));
+          if (t == w.nblk - 1) mma_commit(cx.bar(B_S_FULL + par));
           mma_commit(cx.bar(B_K_EMPTY + st));
         }
         __syncwarp();
-        DTR(3, kc);
       }
-      // the slots this item does not use complete a phase as well: a barrier's phase is then a function of the item
-      if (ok && w.nblk < MAXBLK && elect_one())
-        for (int t = w.nblk; t < MAXBLK; ++t) mma_commit(cx.bar(B_S_FULL + par * MAXBLK + t));   // after the MMAs above
-      __syncwarp();
       ++j;
     }
   } else if (warp == 2) {
     // ================= PV issue: O_u^T = V_u^T P_hat_u^T as V stages land
     const uint32_t id_pv = idesc_e4m3(128, NCOL, 1, 0);
     WorkIter w;
-    w.init(true);
     uint32_t vc = 0, j = 0;
     bool ok = true;
     while (ok && w.next(cx, ring)) {
@@ -552,7 +573,6 @@ __global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const Decode
         const uint32_t st = vc % D_NV;
         ok = cx.wait_warp(B_V_FULL + st, (vc / D_NV) & 1);
         if (!ok) break;
-        DTR(4, vc);
         tc_fence_after();
         if (elect_one()) {
           const uint64_t d_v = smem_desc(sbase + D_OFF_V + st * VST_BYTES, 16, 1024, SWZ_128B);
@@ -567,7 +587,6 @@ __global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const Decode
           if (t == w.nblk - 1) mma_commit(cx.bar(B_O_FULL));
         }
         __syncwarp();
-        DTR(5, vc);
       }
       ++j;
     }
@@ -575,58 +594,10 @@ __global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const Decode
     // ================= K scales of a block: [token][8 blocks] -> two 32 x 16-byte tiles
     // (tile h = blocks 4h..4h+3; row i holds tokens i, 32+i, 64+i, 96+i), the form tcgen05.cp spreads.
     // The tile of stage st is free: the copy into the stage waited for the MMAs that read it.
-    // The same warp stages the query tile (codes and scales of the group's G heads) of item j+1 while
-    // item j is scored: that slot was last read by the MMAs of item j-1.
-    WorkIter w, wq;
-    w.init(true);
-    wq.init(false);
-    uint32_t kc = 0, j = 0, n_staged = 0;
+    WorkIter w;
+    uint32_t kc = 0;
     bool ok = true;
-    uint4 qv = make_uint4(0u, 0u, 0u, 0u);
-    uint32_t qs0 = 0, qs1 = 0;
-    bool have_q = false;
-    auto load_q = [&]() {   // global loads of the next item's tile, consumed one item later
-      have_q = wq.next(cx, ring);
-      if (!have_q) return;
-      if (lane < G * 4)
-        qv = *reinterpret_cast<const uint4 *>(p.q_codes + ((size_t)wq.b * p.H_q + wq.hk * G + (lane >> 2)) * (TILE * 64) + (lane & 3) * 16);
-      if (lane < G) {
-        const uint8_t *src = p.q_sf + ((size_t)wq.b * p.H_q + wq.hk * G + lane) * 1024;
-        qs0 = *reinterpret_cast<const uint32_t *>(src);
-        qs1 = *reinterpret_cast<const uint32_t *>(src + 512);
-      }
-    };
-    auto store_q = [&]() {
-      if (!have_q) return;
-      const uint32_t slot = n_staged & 1;
-      if (lane < G * 4) {
-        const int n = lane >> 2, c = lane & 3;
-        *reinterpret_cast<uint4 *>(dsm + D_OFF_Q + slot * 1024 + n * 64 + ((c ^ ((n & 7) >> 1)) << 4)) = qv;
-      }
-      if (lane < G) {
-        uint8_t *dst = dsm + D_OFF_SFQ + slot * 1024 + lane * 16;
-        *reinterpret_cast<uint32_t *>(dst) = qs0;
-        *reinterpret_cast<uint32_t *>(dst + 512) = qs1;
-      }
-      fence_proxy_async_smem();
-      cx.warp_arrive(B_Q_READY + slot);
-      ++n_staged;
-    };
-    load_q();
-    store_q();
-    load_q();
-    store_q();
-    load_q();
     while (ok && w.next(cx, ring)) {
-      if (j >= 1) {
-        // all QK MMAs of item j-1 are complete once its last block's scores are
-        const uint32_t pj = j - 1;
-        ok = cx.wait_warp(B_S_FULL + (pj & 1) * MAXBLK + MAXBLK - 1, (pj >> 1) & 1);
-        if (!ok) break;
-        store_q();
-        load_q();
-      }
-      ++j;
       for (int t = 0; t < w.nblk; ++t, ++kc) {
         const uint32_t st = kc % D_NK;
         ok = cx.wait_warp(B_K_FULL + st, (kc / D_NK) & 1);
@@ -640,237 +611,249 @@ __global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const Decode
         *reinterpret_cast<uint4 *>(dst + 512) = make_uint4(v[0].y, v[1].y, v[2].y, v[3].y);
         fence_proxy_async_smem();
         cx.warp_arrive(B_SF_READY + st);
-        DTR(6, kc);
       }
     }
-  } else {
-    // ================= softmax, one thread per key of a block (per channel for O^T)
+  } else if (warp < 12) {
+    // ================= softmax, one thread per key of a block; two groups of four warps, group
+    // `grp` takes the items of that parity
+    const int grp = (warp - 4) >> 2;
     const int quad = warp & 3;                  // TMEM lane quadrant this warp may touch
-    const int r = quad * 32 + lane;             // key within the block / channel of O^T
-    const int t128 = (warp - 4) * 32 + lane;    // 0..127 among these warps
+    const int r = quad * 32 + lane;             // key within the block
     const uint32_t tlane = (uint32_t)(quad * 32) << 16;
+    constexpr int CH = G <= 2 ? 4 : 2;          // blocks whose tensor-memory loads are in flight together
+    const uint32_t tS = tm + TM_S + grp * (MAXBLK * 16) + tlane;
+    uint8_t *const pt = dsm + D_OFF_P + grp * MAXBLK * 1024 + (r & 15);
+    float *xm = xmax + grp * MAXBLK * MAXG * 4, *wt = wtab + grp * MAXBLK * MAXG, *xlg = xl + grp * 4 * MAXG;
     bool ok = true;
-
-    // partition write-out of the item before the current one (its PV MMAs finish meanwhile)
-    struct Prev { int b, hk, sp, nblk; };
-    auto write_out = [&](const Prev &pr, uint32_t jp) {
-      const uint32_t par = jp & 1;
-      ok = cx.wait_warp(B_O_FULL, jp & 1);
-      if (!ok) return;
-      tc_fence_after();
-      uint32_t o[MAXBLK][G];
-#pragma unroll
-      for (int t = 0; t < MAXBLK; ++t)
-        if (t < pr.nblk) tmem_ld_g<G>(tm + TM_O + t * 16 + tlane, o[t]);
-      tmem_ld_wait();
-      tc_fence_before();
-      cx.warp_arrive(B_O_FREE);
-      float acc[G];
-#pragma unroll
-      for (int g = 0; g < G; ++g) acc[g] = 0.0f;
-#pragma unroll
-      for (int t = 0; t < MAXBLK; ++t)
-        if (t < pr.nblk) {
-#pragma unroll
-          for (int g = 0; g < G; ++g) acc[g] = __fmaf_rn(wtab[(par * MAXBLK + t) * MAXG + g], __uint_as_float(o[t][g]), acc[g]);
-        }
-      float *dst = p.parts + (((size_t)pr.b * p.H_q + (size_t)pr.hk * G) * p.n_split + pr.sp) * PART_FLOATS;
-      const size_t head_stride = (size_t)p.n_split * PART_FLOATS;
-#pragma unroll
-      for (int g = 0; g < G; ++g) dst[g * head_stride + 2 + r] = acc[g];
-      if (t128 < G) {
-        float l = 0.0f;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) l += xl[(par * 4 + q) * MAXG + t128];
-        dst[t128 * head_stride] = mfin[par * MAXG + t128];
-        dst[t128 * head_stride + 1] = l;
-      }
-    };
-
     WorkIter w;
-    w.init(true);
-    uint32_t j = 0;
-    Prev prev{0, 0, 0, 0};
-    while (ok && w.next(cx, ring)) {
-      const uint32_t par = j & 1;
+    for (uint32_t j = 0; ok && w.next(cx, ring); ++j) {
+      if ((int)(j & 1) != grp) continue;
+      const uint32_t ph = (j >> 1) & 1;
       const float lam = w.b < D_MAXREQ ? lam_tab[w.b]
                                        : __fmul_rn(__fmul_rn(__fmul_rn(p.softmax_scale, 1.4426950408889634f), p.q_gscale[w.b]), p.k_gscale[w.b]);
       const int k_part = w.sp * DECODE_SPLIT;
-      // ---- all scores of the item at once: the last slot's barrier follows every QK MMA of the item
-      ok = cx.wait_warp(B_S_FULL + par * MAXBLK + MAXBLK - 1, (j >> 1) & 1);
+      // ---- all scores of the item at once.  They are read from tensor memory twice, once for the maxima and once for the
+      // exponentials: held in registers in between, MAXBLK x G of them and as many maxima went to local memory for groups
+      // of five heads and more (24 us per item instead of 6).
+      ok = cx.wait_warp(B_S_FULL + grp, ph);
       if (!ok) break;
-      if (warp == 4) DTR(7, j);
       tc_fence_after();
-      float sv[MAXBLK][G];
-      {
-        uint32_t sraw[MAXBLK][G];
+      // block maxima of this warp's keys, CH blocks at a time
+#pragma unroll 1
+      for (int t0 = 0; t0 < w.nblk; t0 += CH) {
+        uint32_t sr[CH][G];
 #pragma unroll
-        for (int t = 0; t < MAXBLK; ++t)
-          if (t < w.nblk) tmem_ld_g<G>(tm + TM_S + (par * MAXBLK + t) * 16 + tlane, sraw[t]);
+        for (int u = 0; u < CH; ++u)
+          if (t0 + u < w.nblk) tmem_ld_g<G>(tS + (t0 + u) * 16, sr[u]);
         tmem_ld_wait();
-        tc_fence_before();
-        cx.warp_arrive(B_S_FREE + par);
 #pragma unroll
-        for (int t = 0; t < MAXBLK; ++t) {
-          if (t < w.nblk) {
-            const bool valid = k_part + (w.nblk - 1 - t) * TILE + r < w.L;
+        for (int u = 0; u < CH; ++u) {
+          if (t0 + u < w.nblk) {
+            const bool valid = k_part + (w.nblk - 1 - t0 - u) * TILE + r < w.L;
 #pragma unroll
             for (int g = 0; g < G; ++g) {
-              sv[t][g] = valid ? __uint_as_float(sraw[t][g]) : -INFINITY;
-              // warp maximum through an order-preserving integer key and one redux
-              const int bits = __float_as_int(sv[t][g]);
-              const int key = bits ^ ((bits >> 31) & 0x7FFFFFFF);
-              const int km = __reduce_max_sync(0xffffffffu, key);
-              if (lane == 0) xmax[((par * MAXBLK + t) * MAXG + g) * 4 + (warp - 4)] = __int_as_float(km ^ ((km >> 31) & 0x7FFFFFFF));
+              const float wm = warp_max(valid ? __uint_as_float(sr[u][g]) : -INFINITY);
+              if (lane == 0) xm[((t0 + u) * MAXG + g) * 4 + quad] = wm;
             }
           }
         }
       }
-      if (warp == 4) DTR(8, j);
-      cx.warp_arrive(B_XCHG);
-      ok = cx.wait_warp(B_XCHG, j & 1);
+      cx.warp_arrive(B_XCHG + grp);
+      ok = cx.wait_warp(B_XCHG + grp, ph);
       if (!ok) break;
-      if (warp == 4) DTR(9, j);
-      // ---- running maxima of the reverse traversal, then all P_hat of the item
-      {
-        float m[MAXBLK][G], run[G], lsum[G];
-#pragma unroll
-        for (int g = 0; g < G; ++g) run[g] = -INFINITY, lsum[g] = 0.0f;
-#pragma unroll
-        for (int t = 0; t < MAXBLK; ++t) {
-          if (t < w.nblk) {
-#pragma unroll
-            for (int g = 0; g < G; ++g) {
-              const float4 x = *reinterpret_cast<const float4 *>(&xmax[((par * MAXBLK + t) * MAXG + g) * 4]);
-              run[g] = fmaxf(run[g], fmaxf(fmaxf(x.x, x.y), fmaxf(x.z, x.w)));
-              m[t][g] = run[g];
-            }
-          }
+      // the item two before this one, which used the same tables and P_hat tiles, is through with them
+      if (j >= 2) ok = cx.wait_warp(B_T_FREE + grp, ph ^ 1);
+      if (!ok) break;
+      // block weights 2^(lam (m_u - m)) of the item's end, one (block, head) per thread
+      if (r < MAXBLK * G) {
+        const int tw = r / G, gw = r % G;
+        float mu = -INFINITY, mf = -INFINITY;
+#pragma unroll 1
+        for (int t = 0; t < w.nblk; ++t) {
+          const float4 x = *reinterpret_cast<const float4 *>(&xm[(t * MAXG + gw) * 4]);
+          mf = fmaxf(mf, fmaxf(fmaxf(x.x, x.y), fmaxf(x.z, x.w)));
+          if (t == tw) mu = mf;
         }
-        uint8_t *pt = dsm + D_OFF_P + par * MAXBLK * 1024 + (r & 15);
+        if (tw == 0) mfin[grp * MAXG + gw] = mf;
+        wt[tw * MAXG + gw] = mu == mf ? 1.0f : ex2_approx(__fmul_rn(mu - mf, lam));
+      }
+      // running maxima of the reverse traversal and all P_hat of the item
+      float run[G], lsum[G];
 #pragma unroll
-        for (int t = 0; t < MAXBLK; ++t) {
-          if (t < w.nblk) {
-            float pq[G + 1];
+      for (int g = 0; g < G; ++g) run[g] = -INFINITY, lsum[g] = 0.0f;
+#pragma unroll 1
+      for (int t0 = 0; t0 < w.nblk; t0 += CH) {
+        uint32_t sr[CH][G];
+#pragma unroll
+        for (int u = 0; u < CH; ++u)
+          if (t0 + u < w.nblk) tmem_ld_g<G>(tS + (t0 + u) * 16, sr[u]);
+        tmem_ld_wait();
+#pragma unroll
+        for (int u = 0; u < CH; ++u) {
+          if (t0 + u < w.nblk) {
+            const bool valid = k_part + (w.nblk - 1 - t0 - u) * TILE + r < w.L;
+            float m[G], pq[G + 1];
+            bool moved = false;
 #pragma unroll
             for (int g = 0; g < G; ++g) {
-              const float pv = ex2_approx(__fmaf_rn(sv[t][g], lam, -__fmul_rn(m[t][g], lam)));   // -inf -> 0
-              float wt = 1.0f;
-              if (m[t][g] != run[g]) wt = ex2_approx(__fmul_rn(m[t][g] - run[g], lam));   // uniform, rare
-              lsum[g] = __fmaf_rn(wt, pv, lsum[g]);
+              const float4 x = *reinterpret_cast<const float4 *>(&xm[((t0 + u) * MAXG + g) * 4]);
+              m[g] = fmaxf(run[g], fmaxf(fmaxf(x.x, x.y), fmaxf(x.z, x.w)));
+              moved |= m[g] != run[g];
+            }
+            if (moved) {   // uniform; one branch for the whole group keeps the heads' chains independent
+#pragma unroll
+              for (int g = 0; g < G; ++g) {
+                lsum[g] = __fmul_rn(lsum[g], m[g] == run[g] ? 1.0f : ex2_approx(__fmul_rn(run[g] - m[g], lam)));
+                run[g] = m[g];
+              }
+            }
+#pragma unroll
+            for (int g = 0; g < G; ++g) {
+              const float e = ex2_approx(__fmaf_rn(__uint_as_float(sr[u][g]), lam, -__fmul_rn(m[g], lam)));
+              const float pv = valid ? e : 0.0f;
+              lsum[g] = __fadd_rn(lsum[g], pv);
               pq[g] = __fmul_rn(pv, 448.0f);
-              if (t128 == t * G + g) wtab[(par * MAXBLK + t) * MAXG + g] = wt;
             }
             pq[G] = 0.0f;
+            uint8_t *const pb = pt + (t0 + u) * 1024;
 #pragma unroll
             for (int g = 0; g < G; g += 2) {
               const uint32_t two = (uint32_t)__nv_cvt_float2_to_fp8x2(make_float2(pq[g], pq[g + 1]), __NV_SATFINITE, __NV_E4M3);
-              pt[t * 1024 + g * 128 + (((r >> 4) ^ g) << 4)] = (uint8_t)two;
-              if (g + 1 < G) pt[t * 1024 + (g + 1) * 128 + (((r >> 4) ^ (g + 1)) << 4)] = (uint8_t)(two >> 8);
+              pb[g * 128 + (((r >> 4) ^ g) << 4)] = (uint8_t)two;
+              if (g + 1 < G) pb[(g + 1) * 128 + (((r >> 4) ^ (g + 1)) << 4)] = (uint8_t)(two >> 8);
             }
           }
         }
+      }
+      tc_fence_before();
+      cx.warp_arrive(B_S_FREE + grp);
 #pragma unroll
-        for (int g = 0; g < G; ++g) {
-          float ls = lsum[g];
+      for (int g = 0; g < G; ++g) {
+        float ls = lsum[g];
 #pragma unroll
-          for (int o = 16; o > 0; o >>= 1) ls += __shfl_xor_sync(0xffffffffu, ls, o);
-          if (lane == 0) xl[(par * 4 + (warp - 4)) * MAXG + g] = ls;
-          if (t128 == g) mfin[par * MAXG + g] = run[g];
-        }
+        for (int o = 16; o > 0; o >>= 1) ls += __shfl_xor_sync(0xffffffffu, ls, o);
+        if (lane == 0) xlg[quad * MAXG + g] = ls;
       }
       fence_proxy_async_smem();
-      cx.warp_arrive(B_P_READY + par);
-      if (warp == 4) DTR(10, j);
-      if (j >= 1) {
-        write_out(prev, j - 1);
-        if (!ok) break;
-      }
-      if (warp == 4) DTR(11, j);
-      prev = Prev{w.b, w.hk, w.sp, w.nblk};
-      ++j;
+      cx.warp_arrive(B_P_READY + grp);
     }
-    if (ok && j >= 1) {
-      // the tables of the last item were written by other warps: one more exchange round
-      cx.warp_arrive(B_XCHG);
-      ok = cx.wait_warp(B_XCHG, j & 1);
-      if (ok) write_out(prev, j - 1);
+  } else {
+    // ================= O of every item, one thread per channel, as soon as its V has been consumed
+    constexpr int CH = G <= 2 ? 4 : 2;
+    const int quad = warp & 3, r = quad * 32 + lane;
+    const uint32_t tO = tm + TM_O + ((uint32_t)(quad * 32) << 16);
+    bool ok = true;
+    WorkIter w;
+    for (uint32_t j = 0; ok && w.next(cx, ring); ++j) {
+      const int par = j & 1;
+      const float *wt = wtab + par * MAXBLK * MAXG, *xlg = xl + par * 4 * MAXG;
+      ok = cx.wait_warp(B_P_READY + par, (j >> 1) & 1) && cx.wait_warp(B_O_FULL, j & 1);   // the item's tables; its accumulators
+      if (!ok) break;
+      tc_fence_after();
+      float acc[G], l[G], m[G];
+#pragma unroll
+      for (int g = 0; g < G; ++g) {
+        acc[g] = 0.0f;
+        m[g] = mfin[par * MAXG + g];
+        l[g] = (xlg[g] + xlg[MAXG + g]) + (xlg[2 * MAXG + g] + xlg[3 * MAXG + g]);
+      }
+#pragma unroll 1
+      for (int t0 = 0; t0 < w.nblk; t0 += CH) {
+        uint32_t o[CH][G];
+#pragma unroll
+        for (int u = 0; u < CH; ++u)
+          if (t0 + u < w.nblk) tmem_ld_g<G>(tO + (t0 + u) * 16, o[u]);
+        tmem_ld_wait();
+#pragma unroll
+        for (int u = 0; u < CH; ++u)
+          if (t0 + u < w.nblk) {
+#pragma unroll
+            for (int g = 0; g < G; ++g) acc[g] = __fmaf_rn(wt[(t0 + u) * MAXG + g], __uint_as_float(o[u][g]), acc[g]);
+          }
+      }
+      tc_fence_before();
+      cx.warp_arrive(B_O_FREE);
+      cx.warp_arrive(B_T_FREE + par);
+      const size_t head0 = (size_t)w.b * p.H_q + (size_t)w.hk * G;
+      const int n_parts = p.n_parts(w.L);
+      if (n_parts == 1) {
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+          const float y = l[g] > 0.0f ? __fmul_rn(__fdiv_rn(acc[g], __fmul_rn(448.0f, l[g])), p.v_scale) : 0.0f;
+          p.out[(head0 + g) * HEAD_DIM + r] = __float2bfloat16_rn(y);
+          if (p.out_f32) p.out_f32[(head0 + g) * HEAD_DIM + r] = y;
+        }
+        continue;
+      }
+#pragma unroll
+      for (int g = 0; g < G; ++g) {
+        p.part_o[((head0 + g) * p.n_split + w.sp) * HEAD_DIM + r] = acc[g];
+        if (r == g) p.part_ml[(head0 + g) * p.n_split + w.sp] = make_float2(m[g], l[g]);
+      }
     }
   }
 
   tc_fence_before();
   __syncthreads();
   if (warp == 1) tmem_dealloc(tm, TM_COLS);
-#ifdef MPFA_TRACE
-  if (g_dtrace && threadIdx.x == 0) g_dtrace[4096 + 2 * blockIdx.x + 1] = (long long)globaltimer_ns();
-#endif
+}
+
+// The work counter, zeroed in stream order.  A kernel and not a memory set, so that the split kernel's set-up overlaps
+// the end of whatever precedes the call.
+__global__ void decode_prep_kernel(unsigned int *ticket) {
+  launch_dependents();
+  grid_dependency_wait();
+  *ticket = 0u;
 }
 
 // Merge of the partition states (Section 5.3): M = max m_s, w_s = 2^(lam (m_s - M)),
-// l = sum w_s l_s, O = sum w_s O_s, out = O / (448 l) * v_scale.  grid (H_q, B), 256 threads.
-__global__ void __launch_bounds__(256) decode_merge_kernel(const float *__restrict__ parts,
-                                                           const int32_t *__restrict__ seq_lens,
-                                                           const float *__restrict__ q_gscale,
-                                                           const float *__restrict__ k_gscale, int H_q, int n_split,
-                                                           float softmax_scale, float v_scale,
-                                                           __nv_bfloat16 *__restrict__ out, float *__restrict__ out_f32) {
-  // 8 warps: warp w takes the partitions s = w, w + 8, ... in ascending order (the loads of four of them in
-  // flight together), lane l the channels l, l + 32, l + 64, l + 96; the eight partial sums are then added in
-  // warp order.  A fixed order, so the result is reproducible; with one thread walking all partitions a
-  // single long request (128 partitions, 32 blocks in the grid) spent 25 us here.
-  __shared__ float s_red[8], s_l[8], s_o[8][HEAD_DIM];
-  const int hq = blockIdx.x, b = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int L = seq_lens[b];
-  const int ns = min(n_split, (L + DECODE_SPLIT - 1) / DECODE_SPLIT);
-  const float *base = parts + ((size_t)b * H_q + hq) * n_split * PART_FLOATS;
-  const float lam = __fmul_rn(__fmul_rn(__fmul_rn(softmax_scale, 1.4426950408889634f), q_gscale[b]), k_gscale[b]);
+// l = sum w_s l_s, O = sum w_s O_s, out = O / (448 l) * v_scale.  grid (H_q, B).  Warp w takes the partitions s = w,
+// w + 4, ... in ascending order, a lane four channels (one 512-byte row per warp and load, four rows in flight), and the
+// four sums are added in warp order: a fixed order, so the result is reproducible.  128 threads of at most 56 registers
+// fit beside a CTA of the split kernel.  Requests of one partition are complete already, those without keys get zeros.
+__global__ void __launch_bounds__(128, 9) decode_merge_kernel(const __grid_constant__ DecodeParams p) {
+  __shared__ float s_l[4];
+  __shared__ __align__(16) float s_o[4][HEAD_DIM];
+  grid_dependency_wait();
+  const int hq = blockIdx.x, b = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int n = p.n_parts(p.seq_lens[b]);
+  if (n == 1) return;
+  const size_t head = (size_t)b * p.H_q + hq;
+  const float2 *ml = p.part_ml + head * p.n_split;
+  const float4 *po = reinterpret_cast<const float4 *>(p.part_o + head * p.n_split * HEAD_DIM) + lane;
+  const float lam = __fmul_rn(__fmul_rn(__fmul_rn(p.softmax_scale, 1.4426950408889634f), p.q_gscale[b]), p.k_gscale[b]);
   float M = -INFINITY;
-  for (int s = tid; s < ns; s += 256) M = fmaxf(M, base[(size_t)s * PART_FLOATS]);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
-  if (lane == 0) s_red[warp] = M;
-  __syncthreads();
-  M = s_red[0];
-#pragma unroll
-  for (int w = 1; w < 8; ++w) M = fmaxf(M, s_red[w]);
+  for (int s = lane; s < n; s += 32) M = fmaxf(M, ml[s].x);   // every warp takes the maximum of all
+  M = warp_max(M);
   float l = 0.0f, o[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-  for (int s0 = warp; s0 < ns; s0 += 32) {
-    float ms[4], ls[4], os[4][4];
+#pragma unroll 1
+  for (int s0 = warp; s0 < n; s0 += 16) {
+    float2 a[4];
+    float4 x[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int sp = s0 + 8 * j;
-      const bool in = sp < ns;
-      const float *ps = base + (size_t)(in ? sp : s0) * PART_FLOATS;
-      ms[j] = in ? ps[0] : -INFINITY;
-      ls[j] = ps[1];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) os[j][q] = ps[2 + lane + 32 * q];
+    for (int u = 0; u < 4; ++u) {
+      const int s = s0 + 4 * u;
+      a[u] = s < n ? ml[s] : make_float2(-INFINITY, 0.0f);
+      x[u] = s < n ? po[(size_t)s * (HEAD_DIM / 4)] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     }
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      if (ms[j] == -INFINITY) continue;
-      const float w = ex2_approx(__fmul_rn(ms[j] - M, lam));
-      l = __fadd_rn(l, __fmul_rn(w, ls[j]));
-#pragma unroll
-      for (int q = 0; q < 4; ++q) o[q] = __fadd_rn(o[q], __fmul_rn(w, os[j][q]));
+    for (int u = 0; u < 4; ++u) {
+      const float w = a[u].x == -INFINITY ? 0.0f : ex2_approx(__fmul_rn(a[u].x - M, lam));
+      l = __fmaf_rn(w, a[u].y, l);
+      o[0] = __fmaf_rn(w, x[u].x, o[0]);
+      o[1] = __fmaf_rn(w, x[u].y, o[1]);
+      o[2] = __fmaf_rn(w, x[u].z, o[2]);
+      o[3] = __fmaf_rn(w, x[u].w, o[3]);
     }
   }
   if (lane == 0) s_l[warp] = l;
-#pragma unroll
-  for (int q = 0; q < 4; ++q) s_o[warp][lane + 32 * q] = o[q];
+  *reinterpret_cast<float4 *>(&s_o[warp][lane * 4]) = make_float4(o[0], o[1], o[2], o[3]);
   __syncthreads();
-  if (tid < HEAD_DIM) {
-    float lt = s_l[0], ot = s_o[0][tid];
-#pragma unroll
-    for (int w = 1; w < 8; ++w) {
-      lt = __fadd_rn(lt, s_l[w]);
-      ot = __fadd_rn(ot, s_o[w][tid]);
-    }
-    const float r = (lt > 0.0f) ? __fmul_rn(__fdiv_rn(ot, __fmul_rn(448.0f, lt)), v_scale) : 0.0f;
-    const size_t idx = ((size_t)b * H_q + hq) * HEAD_DIM + tid;
-    out[idx] = __float2bfloat16_rn(r);
-    if (out_f32) out_f32[idx] = r;
-  }
+  const int c = threadIdx.x;
+  const float lt = (s_l[0] + s_l[1]) + (s_l[2] + s_l[3]), ot = (s_o[0][c] + s_o[1][c]) + (s_o[2][c] + s_o[3][c]);
+  const float y = lt > 0.0f ? __fmul_rn(__fdiv_rn(ot, __fmul_rn(448.0f, lt)), p.v_scale) : 0.0f;
+  p.out[head * HEAD_DIM + c] = __float2bfloat16_rn(y);
+  if (p.out_f32) p.out_f32[head * HEAD_DIM + c] = y;
 }
 
 }  // namespace
@@ -878,23 +861,23 @@ __global__ void __launch_bounds__(256) decode_merge_kernel(const float *__restri
 
 using namespace mpfa;
 
-#ifdef MPFA_TRACE
-extern "C" int mpfa_debug_set_decode_trace(long long *buf, int cta) {
-  if (cudaMemcpyToSymbol(g_dtrace, &buf, sizeof(buf)) != cudaSuccess) return -1;
-  if (cudaMemcpyToSymbol(g_dtrace_cta, &cta, sizeof(cta)) != cudaSuccess) return -1;
-  return 0;
-}
-#endif
-
-// partition states, then (256-byte aligned) the work counter of the split kernel
-static size_t decode_parts_bytes(int B, int H_q, size_t n_split) {
-  return ((size_t)B * H_q * n_split * PART_FLOATS * sizeof(float) + 255) / 256 * 256;
+// Workspace: partition accumulators, partition (m, l), work counter; each part 256-byte aligned.
+struct DecodeWorkspace {
+  size_t ml, ticket, bytes;
+};
+static DecodeWorkspace decode_workspace(int B, int H_q, size_t n_split) {
+  auto up = [](size_t x) { return (x + 255) / 256 * 256; };
+  DecodeWorkspace w;
+  w.ml = up((size_t)B * H_q * n_split * HEAD_DIM * sizeof(float));
+  w.ticket = w.ml + up((size_t)B * H_q * n_split * sizeof(float2));
+  w.bytes = w.ticket + 256;
+  return w;
 }
 
 extern "C" size_t mpfa_decode_workspace_bytes(int B, int H_q, int H_kv, int max_pages_per_req) {
   if (B <= 0 || H_q <= 0 || H_kv <= 0 || max_pages_per_req <= 0) return 0;
   const size_t n_split = ((size_t)max_pages_per_req * PAGE + DECODE_SPLIT - 1) / DECODE_SPLIT;
-  return decode_parts_bytes(B, H_q, n_split) + 256;
+  return decode_workspace(B, H_q, n_split).bytes;
 }
 
 extern "C" mpfa_status mpfa_decode(const mpfa_fp4_tensor *q, const mpfa_paged_kv *kv, const int32_t *page_table,
@@ -913,8 +896,8 @@ extern "C" mpfa_status mpfa_decode(const mpfa_fp4_tensor *q, const mpfa_paged_kv
   if (H_kv <= 0 || kv->H_q != H_q) return MPFA_ERR_INVALID_ARG;
   if (H_q % H_kv != 0 || H_q / H_kv > MAXG) return MPFA_ERR_UNSUPPORTED;
   const size_t n_split = ((size_t)max_pages_per_req * PAGE + DECODE_SPLIT - 1) / DECODE_SPLIT;
-  const size_t need = decode_parts_bytes(B, H_q, n_split) + 256;
-  if (workspace_bytes < need) return MPFA_ERR_WORKSPACE;
+  const DecodeWorkspace ws = decode_workspace(B, H_q, n_split);
+  if (workspace_bytes < ws.bytes) return MPFA_ERR_WORKSPACE;
   if ((size_t)B * H_kv * n_split > 0x7FFFFFFFull || B > 65535) return MPFA_ERR_UNSUPPORTED;
   if (!aligned(q->codes, 16) || !aligned(q->sf, 16) || !aligned(kv->k_codes, 256) || !aligned(kv->k_sf, 256) ||
       !aligned(kv->v_fp8, 256) || !aligned(kv->delta_s_bf16, 256) || !aligned(workspace, 16))
@@ -935,8 +918,11 @@ extern "C" mpfa_status mpfa_decode(const mpfa_fp4_tensor *q, const mpfa_paged_kv
   p.seq_lens = seq_lens;
   p.q_gscale = st->q_gscale;
   p.k_gscale = st->k_gscale;
-  p.parts = static_cast<float *>(workspace);
-  p.ticket = reinterpret_cast<unsigned int *>(static_cast<uint8_t *>(workspace) + decode_parts_bytes(B, H_q, n_split));
+  p.part_o = static_cast<float *>(workspace);
+  p.part_ml = reinterpret_cast<float2 *>(static_cast<uint8_t *>(workspace) + ws.ml);
+  p.ticket = reinterpret_cast<unsigned int *>(static_cast<uint8_t *>(workspace) + ws.ticket);
+  p.out = static_cast<__nv_bfloat16 *>(out_bf16);
+  p.out_f32 = out_f32;
   p.status = device_status;
   p.B = B;
   p.H_q = H_q;
@@ -945,6 +931,7 @@ extern "C" mpfa_status mpfa_decode(const mpfa_fp4_tensor *q, const mpfa_paged_kv
   p.num_pages = kv->num_pages;
   p.n_split = (int)n_split;
   p.softmax_scale = softmax_scale;
+  p.v_scale = v_scale;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const size_t items = (size_t)B * H_kv * n_split;
   const unsigned grid = (unsigned)(items < (size_t)n_sm ? items : (size_t)n_sm);   // one persistent CTA per SM
@@ -961,12 +948,8 @@ extern "C" mpfa_status mpfa_decode(const mpfa_fp4_tensor *q, const mpfa_paged_kv
     default: return MPFA_ERR_UNSUPPORTED;
   }
   MPFA_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)D_SMEM));
-  MPFA_CUDA_OK(cudaMemsetAsync(p.ticket, 0, sizeof(unsigned int), s));   // a memory-set node, no allocation
-  kern<<<grid, D_THREADS, D_SMEM, s>>>(p);
-  MPFA_LAUNCH_OK();
-  decode_merge_kernel<<<dim3(H_q, B), 256, 0, s>>>(p.parts, seq_lens, st->q_gscale, st->k_gscale, H_q, (int)n_split,
-                                                   softmax_scale, v_scale, static_cast<__nv_bfloat16 *>(out_bf16),
-                                                   out_f32);
-  MPFA_LAUNCH_OK();
+  MPFA_CUDA_OK(launch(decode_prep_kernel, dim3(1), dim3(1), 0, s, p.ticket));
+  MPFA_CUDA_OK(launch(kern, dim3(grid), dim3(D_THREADS), D_SMEM, s, p));
+  MPFA_CUDA_OK(launch(decode_merge_kernel, dim3(H_q, B), dim3(128), 0, s, p));
   return MPFA_OK;
 }

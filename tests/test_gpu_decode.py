@@ -113,6 +113,24 @@ def test_decode_long_request_many_partitions():
         assert d.max() <= MAX_ABS and d.mean() <= MEAN_ABS, (b, float(d.max()), float(d.mean()))
 
 
+@pytest.mark.parametrize("hq,hkv,lens", [
+    (40, 8, [1] * 18),                              # 144 work items: fewer than there are SMs, groups of five heads
+    (40, 8, [129] * 19),                            # 152: some CTAs get a second item
+    (32, 4, [1024, 1025, 2048, 2049] * 10),         # exact and just exceeded partitions, groups of eight, 240 items
+    (6, 2, [2047, 897, 640, 1] * 60),               # many items per CTA, one to eight blocks each, groups of three
+])
+def test_decode_item_counts_around_the_grid(hq, hkv, lens):
+    """The work-item walk and its two alternating softmax groups: item counts just below and above the grid, partitions
+    of every block count, requests complete in one partition next to merged ones."""
+    w = wl.decode_workload("dec_items", 78 + hq, len(lens), hq, hkv, 1, max(lens), n_stat_tokens=64, seq_lens=lens)
+    st = run(w)
+    got = st.out_f32.cpu().numpy()
+    assert np.isfinite(got).all()
+    for b in sorted({0, 1, 2, 3, len(lens) // 2, len(lens) - 1}):
+        d = np.abs(got[b] - oracle_decode_one(w, b))
+        assert d.max() <= MAX_ABS and d.mean() <= MEAN_ABS, (b, float(d.max()), float(d.mean()))
+
+
 def test_decode_direct_variant_and_v_scale():
     w = wl.decode_workload("dec_direct", 71, 3, 8, 2, 300, 3000)
     ref32, _, caches = oracle_decode(w, smooth=False, v_scale=0.5)

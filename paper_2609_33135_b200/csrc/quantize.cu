@@ -15,6 +15,7 @@
 #include <mutex>
 
 #include "common.cuh"
+#include "sm100_ptx.cuh"
 
 namespace mpfa {
 
@@ -41,176 +42,199 @@ __device__ __forceinline__ void unpack8(const uint4 &u, float (&f)[8]) {
 
 // One pass over a tensor [B, N, cols] gives, per column, everything the statistics need:
 //   the sum in FP64 (Eq. 7);
-//   max x and max (-x) - rounding is monotonic and symmetric, so
+//   max x and min x - rounding is monotonic and symmetric, so
 //   max_t |fl(x_t - mu)| = max(fl(max x - mu), fl(mu - min x)) and no second pass over the tensor is
 //   needed for the per-tensor scale.
-// The token axis is cut into S contiguous slices.  A CTA covers 256 columns x one slice: thread = (token lane
-// 0..7, 8 columns), a warp reads 512 contiguous bytes of one token row, four independent 16-byte loads in
-// flight per thread; each thread adds its tokens in ascending order, the eight token lanes are folded in lane
-// order in shared memory, and the slice's partial result goes to the workspace.  The finalize kernel adds the S
-// partial sums in slice order.  Every addition order is fixed by (N, S), so the result is reproducible bit for
-// bit for any input; it equals the oracle's single ascending FP64 sum whenever all these sums are exact (always
-// true for BF16 inputs whose exponents span fewer than about 40 binades per column).
-constexpr int COLSTAT_COLS = 256;
-constexpr int STAT_MAX_SLICES = 32;
+// A CTA covers one head (128 columns) x one slice of the tokens: thread = (token lane 0..15, 8 columns), eight independent
+// 16-byte loads in flight per thread; each thread adds its tokens in ascending order, the 16 token lanes are folded in lane
+// order in shared memory.  With one slice the CTA writes mean = fl(sum / N) (0 without smoothing) and the head's max |x - mean|
+// itself; otherwise the slices' partial results go to the workspace and stat_fold_kernel adds them in
+// slice order.  No counter, no memory to clear.  Every addition order is fixed by the shape, the workspace size
+// and the device's SM count, so the result is reproducible bit for bit for any input; it equals the oracle's single
+// ascending FP64 sum whenever all these sums are exact (always true for BF16 inputs whose exponents span fewer than
+// about 40 binades per column).
+//
+// The conversion instruction FP32 -> FP64 runs at 16 lanes per clock and SM, the FP64 add at 64 (measured: 16.0 and 63.5),
+// and the loads need 12.  A BF16 number has at most 7 mantissa bits, so its bits shifted right by three are the high word
+// of the double 2^-896 times its value, subnormals and zeros included: three integer operations, and sums of such numbers
+// round as the unscaled ones do.  Infinities and NaNs would become finite; an FMA with zero catches them, and that
+// thread's slice is added again with the conversion.
+// Measured (Q and K, 32:8 heads, 16384 tokens / 1:1 heads, 256 tokens; with memory-set node or fold): with conversions, four
+// loads in flight and the last CTA of a group folding the slices 42 / 11 us, now 40 / 3.6 us.  (The slices as CTAs of a
+// cluster, folded through distributed shared memory: clusters leave some SMs empty and others full, 45 us.)
+constexpr int STAT_THREADS = 256;
+constexpr int STAT_LOADS = 8;
+constexpr int STAT_LANES = STAT_THREADS / 16;
 
-// One launch covers up to two tensors (Q and K): blockIdx.y runs over the 256-column groups of the first, then
-// of the second; blocks past a tensor's last slice leave at once.  The block that finishes a column group last
-// (a counter per group, zeroed by a memory-set node before the launch) adds the slices' partial sums in slice order
-// - which block does it cannot change the result - and writes mean = fl(sum / N) (0 without smoothing) and the
-// group's max |x - mean| from the column extremes (an exact, order-free maximum); the block that finishes the
-// whole launch last turns the per-batch-element maxima into the tensor scales.
 struct ColTensor {
-  const __nv_bfloat16 *x;   // null: tensor absent (ygroups = 0)
-  int N, cols, ygroups, slices, slice_len;
-  double *psum;             // [B][slices][cols]
-  float *pmax, *pneg;       // [B][slices][cols]
-  unsigned int *amax;       // [B], zero at launch
-  float *mean, *gscale;
+  const __nv_bfloat16 *x;   // null: tensor absent (H = 0)
+  int N, H;
+  double *psum;             // [slices][B][H * 128] partial results
+  float2 *pext;             // (max, min)
+  float *mean;              // [B, H, 128]
+  float *gmax;              // [B, H]
 };
 
-__device__ __forceinline__ void colstat_body(const ColTensor &a, const int yg, unsigned int *group_counter,
-                                             unsigned int *launch_counter, const unsigned int n_groups, const int smooth,
-                                             const ColTensor &t0, const ColTensor &t1) {
-  __shared__ double s_sum[8][COLSTAT_COLS];
-  __shared__ float s_max[8][COLSTAT_COLS], s_neg[8][COLSTAT_COLS];
-  __shared__ bool s_last;
-  const int sl = blockIdx.x;
-  if (sl >= a.slices) return;
-  const int b = blockIdx.z;
-  const int N = a.N, cols = a.cols;
-  const __nv_bfloat16 *__restrict__ x = a.x;
-  const int tl = threadIdx.x >> 5, cg = threadIdx.x & 31;
-  const int col = yg * COLSTAT_COLS + cg * 8;
-  const int t0i = sl * a.slice_len;
-  const int t1i = min(N, t0i + a.slice_len);
+__device__ __forceinline__ uint32_t bf16x2_max(uint32_t a, uint32_t b) {
+  uint32_t d;
+  asm("max.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+  return d;
+}
+__device__ __forceinline__ uint32_t bf16x2_min(uint32_t a, uint32_t b) {
+  uint32_t d;
+  asm("min.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+  return d;
+}
+// c + 0 a: NaN in a half whose a is not finite
+__device__ __forceinline__ uint32_t bf16x2_note_nonfinite(uint32_t a, uint32_t c) {
+  uint32_t d;
+  asm("fma.rn.bf16x2 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(0u), "r"(c));
+  return d;
+}
+
+// Mean of column c of a head and the head's maximum |x - mean|; threads 0..127 of the block (whole warps), s_w: 4 floats.
+__device__ __forceinline__ void finish_column(const ColTensor &a, int b, int h, int c, double sum, float mx, float mn, int smooth, float *s_w) {
+  const float mu = smooth ? __double2float_rn(__ddiv_rn(sum, (double)a.N)) : 0.0f;
+  a.mean[((size_t)b * a.H + h) * HEAD_DIM + c] = mu;
+  // non-negative: min <= mu <= max (or mu = 0 and the larger side wins)
+  float m = fmaxf(fmaxf(__fsub_rn(mx, mu), __fsub_rn(mu, mn)), 0.0f);
+  asm("redux.sync.max.f32 %0, %0, 0xffffffff;" : "+f"(m));
+  if ((c & 31) == 0) s_w[c >> 5] = m;
+  asm volatile("bar.sync 1, 128;" ::: "memory");
+  if (c == 0) a.gmax[(size_t)b * a.H + h] = fmaxf(fmaxf(s_w[0], s_w[1]), fmaxf(s_w[2], s_w[3]));
+}
+
+// grid (slices, heads of both tensors, B)
+__global__ void __launch_bounds__(STAT_THREADS, 3) colstat_kernel(const ColTensor t0, const ColTensor t1, int smooth) {
+  __shared__ double s_sum[STAT_LANES][HEAD_DIM];
+  __shared__ uint32_t s_mx[STAT_LANES][HEAD_DIM / 2], s_mn[STAT_LANES][HEAD_DIM / 2];
+  __shared__ float s_w[4];
+  launch_dependents();
+  grid_dependency_wait();
+  const bool first = (int)blockIdx.y < t0.H;
+  const ColTensor &a = first ? t0 : t1;
+  const int h = first ? blockIdx.y : blockIdx.y - t0.H;
+  const int b = blockIdx.z, tid = threadIdx.x, tl = tid >> 4, cg = tid & 15;
+  const int slices = gridDim.x, slice = blockIdx.x;
+  const int len = ((a.N + slices - 1) / slices + STAT_LANES - 1) / STAT_LANES * STAT_LANES;
+  const int begin = min(a.N, slice * len), end = min(a.N, begin + len);
+  const size_t row = (size_t)a.H * HEAD_DIM, step = STAT_LANES * row;
+  const __nv_bfloat16 *const p0 = a.x + ((size_t)b * a.N + begin + tl) * row + h * HEAD_DIM + cg * 8, *p = p0;
   double acc[8];
-  float mx[8], ng[8];
+  uint32_t mx[4], mn[4], odd[4];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) acc[i] = 0.0, mx[i] = -INFINITY, ng[i] = -INFINITY;
-  if (col < cols) {
-    const __nv_bfloat16 *p = x + ((size_t)b * N + t0i + tl) * cols + col;
-    const size_t step = (size_t)8 * cols;
-    int t = t0i + tl;
-    // four loads of the next round are in flight while the current four are added (tokens still ascending)
-    uint4 u[4], un[4];
-    bool have = t + 24 < t1i;
-    if (have) {
+  for (int i = 0; i < 8; ++i) acc[i] = 0.0;
 #pragma unroll
-      for (int j = 0; j < 4; ++j) u[j] = __ldcs(reinterpret_cast<const uint4 *>(p + j * step));
+  for (int i = 0; i < 4; ++i) mx[i] = 0xFF80FF80u, mn[i] = 0x7F807F80u, odd[i] = 0u;
+  auto add = [&](const uint4 &u) {
+    const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      mx[i] = bf16x2_max(mx[i], w[i]);
+      mn[i] = bf16x2_min(mn[i], w[i]);
+      odd[i] = bf16x2_note_nonfinite(w[i], odd[i]);
+      acc[2 * i] += __hiloint2double(((int)(w[i] << 16) >> 3) & 0x8FFFE000, 0);
+      acc[2 * i + 1] += __hiloint2double(((int)w[i] >> 3) & 0x8FFFE000, 0);
     }
-    while (have) {
-      const bool more = t + 32 + 24 < t1i;
-      if (more) {
+  };
+  int t = begin + tl;
+  for (; t + STAT_LANES * (STAT_LOADS - 1) < end; t += STAT_LANES * STAT_LOADS, p += STAT_LOADS * step) {
+    uint4 u[STAT_LOADS];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) un[j] = __ldcs(reinterpret_cast<const uint4 *>(p + (4 + j) * step));
-      }
+    for (int j = 0; j < STAT_LOADS; ++j) u[j] = __ldg(reinterpret_cast<const uint4 *>(p + j * step));
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        float f[8];
-        unpack8(u[j], f);
+    for (int j = 0; j < STAT_LOADS; ++j) add(u[j]);
+  }
+  {   // the last fewer than STAT_LOADS rounds of this lane, still in flight together
+    uint4 u[STAT_LOADS - 1];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) acc[i] += (double)f[i], mx[i] = fmaxf(mx[i], f[i]), ng[i] = fmaxf(ng[i], -f[i]);
-      }
-      t += 32;
-      p += 4 * step;
+    for (int j = 0; j < STAT_LOADS - 1; ++j)
+      if (t + STAT_LANES * j < end) u[j] = __ldg(reinterpret_cast<const uint4 *>(p + j * step));
 #pragma unroll
-      for (int j = 0; j < 4; ++j) u[j] = un[j];
-      have = more;
-    }
-    for (; t < t1i; t += 8, p += step) {
+    for (int j = 0; j < STAT_LOADS - 1; ++j)
+      if (t + STAT_LANES * j < end) add(u[j]);
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i) acc[i] *= 0x1p896;
+  if (((odd[0] | odd[1] | odd[2] | odd[3]) & 0x7FFF7FFFu) != 0u) {   // non-finite values: plain sums
+#pragma unroll
+    for (int i = 0; i < 8; ++i) acc[i] = 0.0;
+    p = p0;
+    for (t = begin + tl; t < end; t += STAT_LANES, p += step) {
       float f[8];
-      unpack8(__ldcs(reinterpret_cast<const uint4 *>(p)), f);
+      unpack8(*reinterpret_cast<const uint4 *>(p), f);
 #pragma unroll
-      for (int i = 0; i < 8; ++i) acc[i] += (double)f[i], mx[i] = fmaxf(mx[i], f[i]), ng[i] = fmaxf(ng[i], -f[i]);
+      for (int i = 0; i < 8; ++i) acc[i] += (double)f[i];
     }
   }
+  // pairs of columns: eight consecutive lanes write 128 contiguous bytes
 #pragma unroll
-  for (int i = 0; i < 8; ++i) s_sum[tl][cg * 8 + i] = acc[i], s_max[tl][cg * 8 + i] = mx[i], s_neg[tl][cg * 8 + i] = ng[i];
+  for (int i = 0; i < 4; ++i) {
+    *reinterpret_cast<double2 *>(&s_sum[tl][i * 32 + cg * 2]) = make_double2(acc[2 * i], acc[2 * i + 1]);
+    s_mx[tl][i * 16 + cg] = mx[i];
+    s_mn[tl][i * 16 + cg] = mn[i];
+  }
   __syncthreads();
-  const int c = yg * COLSTAT_COLS + threadIdx.x;
-  if (c < cols) {
-    double sum = 0.0;
-    float m = -INFINITY, g = -INFINITY;
+  if (tid >= HEAD_DIM) return;
+  // place of column tid: pair i of group cg
+  const int at = ((tid & 7) >> 1) * 32 + (tid >> 3) * 2 + (tid & 1);
+  double sum = 0.0;
+  uint32_t hi = 0xFF80FF80u, lo = 0x7F807F80u;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) sum += s_sum[j][threadIdx.x], m = fmaxf(m, s_max[j][threadIdx.x]), g = fmaxf(g, s_neg[j][threadIdx.x]);
-    const size_t o = ((size_t)b * a.slices + sl) * cols + c;
+  for (int j = 0; j < STAT_LANES; ++j) {
+    sum += s_sum[j][at];
+    hi = bf16x2_max(hi, s_mx[j][at >> 1]);
+    lo = bf16x2_min(lo, s_mn[j][at >> 1]);
+  }
+  const float fmx = __uint_as_float(tid & 1 ? hi & 0xFFFF0000u : hi << 16), fmn = __uint_as_float(tid & 1 ? lo & 0xFFFF0000u : lo << 16);
+  if (slices == 1) {
+    finish_column(a, b, h, tid, sum, fmx, fmn, smooth, s_w);
+  } else {
+    const size_t o = ((size_t)slice * gridDim.z + b) * row + h * HEAD_DIM + tid;
     a.psum[o] = sum;
-    a.pmax[o] = m;
-    a.pneg[o] = g;
-  }
-  // ---- the last block of this column group folds the slices
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(group_counter, 1u) == (unsigned int)a.slices - 1u;
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  float m = 0.0f;
-  if (c < cols) {
-    double sum = 0.0;
-    float hi = -INFINITY, ng2 = -INFINITY;
-    const size_t o0 = (size_t)b * a.slices * cols + c;
-    for (int s0 = 0; s0 < a.slices; s0 += 4) {   // four slices' loads in flight; the additions stay in slice order
-      double ps[4];
-      float pm[4], pn[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const bool in = s0 + j < a.slices;
-        const size_t o = o0 + (size_t)(s0 + j) * cols;
-        ps[j] = in ? __ldcg(a.psum + o) : 0.0;
-        pm[j] = in ? __ldcg(a.pmax + o) : -INFINITY;
-        pn[j] = in ? __ldcg(a.pneg + o) : -INFINITY;
-      }
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        if (s0 + j < a.slices) sum += ps[j];
-        hi = fmaxf(hi, pm[j]);
-        ng2 = fmaxf(ng2, pn[j]);
-      }
-    }
-    const float mu = smooth ? __double2float_rn(__ddiv_rn(sum, (double)N)) : 0.0f;
-    a.mean[(size_t)b * cols + c] = mu;
-    m = fmaxf(__fsub_rn(hi, mu), __fsub_rn(mu, -ng2));   // non-negative: lo <= mu <= hi (or mu = 0 and the larger side wins)
-    m = fmaxf(m, 0.0f);
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  float *wmax = &s_max[0][0];
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = m;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int i = 1; i < 8; ++i) m = fmaxf(m, wmax[i]);
-    atomicMax(&a.amax[b], __float_as_uint(m));   // non-negative floats order like their bit patterns
-    __threadfence();
-    s_last = atomicAdd(launch_counter, 1u) == n_groups - 1u;
-  }
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  for (int i = threadIdx.x; i < (int)gridDim.z; i += 256) {
-    if (t0.x) {
-      const float v = __uint_as_float(__ldcg(t0.amax + i));
-      t0.gscale[i] = v > 0.0f ? __fdiv_rn(v, 2688.0f) : 1.0f;
-    }
-    if (t1.x) {
-      const float v = __uint_as_float(__ldcg(t1.amax + i));
-      t1.gscale[i] = v > 0.0f ? __fdiv_rn(v, 2688.0f) : 1.0f;
-    }
+    a.pext[o] = make_float2(fmx, fmn);
   }
 }
 
-// counters: [B][ygroups of both tensors] group counters, then one launch counter; all zero at launch
-__global__ void __launch_bounds__(256, 3) colstat_kernel(const ColTensor a0, const ColTensor a1, unsigned int *counters, int smooth) {
-  const unsigned int groups = (unsigned int)(a0.ygroups + a1.ygroups);
-  unsigned int *gc = counters + blockIdx.z * groups + blockIdx.y;
-  unsigned int *lc = counters + gridDim.z * groups;
-  if ((int)blockIdx.y < a0.ygroups)
-    colstat_body(a0, (int)blockIdx.y, gc, lc, groups * gridDim.z, smooth, a0, a1);
-  else
-    colstat_body(a1, (int)blockIdx.y - a0.ygroups, gc, lc, groups * gridDim.z, smooth, a0, a1);
+// The slices' partial results in slice order; grid (heads of both tensors, B), 128 threads, eight slices' loads in flight.
+__global__ void __launch_bounds__(128) stat_fold_kernel(const ColTensor t0, const ColTensor t1, int slices, int smooth) {
+  __shared__ float s_w[4];
+  launch_dependents();
+  grid_dependency_wait();
+  const bool first = (int)blockIdx.x < t0.H;
+  const ColTensor &a = first ? t0 : t1;
+  const int h = first ? blockIdx.x : blockIdx.x - t0.H, b = blockIdx.y, tid = threadIdx.x;
+  const size_t row = (size_t)a.H * HEAD_DIM, step = gridDim.y * row, o = (size_t)b * row + h * HEAD_DIM + tid;
+  double sum = 0.0;
+  float mx = -INFINITY, mn = INFINITY;
+  for (int s0 = 0; s0 < slices; s0 += 8) {
+    double ps[8];
+    float2 pe[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      if (s0 + j < slices) ps[j] = a.psum[o + (s0 + j) * step], pe[j] = a.pext[o + (s0 + j) * step];
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      if (s0 + j < slices) sum += ps[j], mx = fmaxf(mx, pe[j].x), mn = fminf(mn, pe[j].y);
+  }
+  finish_column(a, b, h, tid, sum, mx, mn, smooth, s_w);
+}
+
+// A per-tensor scale: given (frozen statistics), or max |x - mean| / 2688 from the heads' maxima of the statistics pass of
+// the same call (1 for an all-zero tensor).
+struct TensorScale {
+  float *gscale;       // [B]
+  const float *gmax;   // [B, heads] or null: read gscale
+  int heads;
+};
+
+// whole warp
+__device__ __forceinline__ float tensor_scale(const TensorScale &s, int b, int lane) {
+  if (!s.gmax) return s.gscale[b];
+  float m = 0.0f;
+  for (int i = lane; i < s.heads; i += 32) m = fmaxf(m, s.gmax[(size_t)b * s.heads + i]);
+  asm("redux.sync.max.f32 %0, %0, 0xffffffff;" : "+f"(m));
+  return m > 0.0f ? __fdiv_rn(m, 2688.0f) : 1.0f;
 }
 
 // One NVFP4 block (Eq. 1): 16 centered values -> E4M3 scale code + 8 bytes of E2M1 codes.
@@ -235,297 +259,279 @@ __device__ __forceinline__ void quantize_block16(const float (&xc)[16], float d,
   codes = make_uint2(w[0], w[1]);
 }
 
-__device__ __forceinline__ void load_center16(const __nv_bfloat16 *row, const float *mu, float (&xc)[16]) {
-  float f[8];
-  unpack8(reinterpret_cast<const uint4 *>(row)[0], f);
+// The same block for kernels that quantize many of one tensor: the same codes without a division per block.
+//   - The reciprocal of the decoded scale takes one of 128 values: a table in shared memory, made once per CTA.
+//   - The scale code rounds r = fl(amax / (6 d)) to three mantissa bits.  amax * fl(1 / (6 d)) is within three units in the
+//     last place of it (each of the two roundings adds at most one half of one part in 2^23), which gives the same code unless
+//     a rounding boundary lies between: mantissa bits 19..0 next to 0x80000.  There (seven in 2^20 blocks), and where E4M3 is
+//     subnormal or the reciprocal is, the division is done.
+// Packed FP32 pairs round each half like the scalar operation.
+struct BlockScale {
+  float e, rcp;       // 6 d and its reciprocal (NaN: always divide)
+  const float *inv;   // [128]
+};
+__device__ __forceinline__ BlockScale make_block_scale(float d, float *table, int tid) {
+  if (tid < 128) {
+    const float s = __fmul_rn(__half2float(__half(__nv_cvt_fp8_to_halfraw((__nv_fp8_storage_t)tid, __NV_E4M3))), d);
+    const float inv = __fdiv_rn(1.0f, s);
+    table[tid] = (!(s > 0.0f) || isinf(inv)) ? 0.0f : inv;
+  }
+  BlockScale q;
+  q.e = __fmul_rn(6.0f, d);
+  q.rcp = (q.e > 1e-30f && q.e < 1e30f) ? __frcp_rn(q.e) : NAN;
+  q.inv = table;
+  return q;
+}
+__device__ __forceinline__ void add2(float &d0, float &d1, float a0, float a1, float b0, float b1) {
+  asm("{.reg .b64 ra, rb, rd;\n\t"
+      "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
+      "add.rn.f32x2 rd, ra, rb;\n\tmov.b64 {%0, %1}, rd;}"
+      : "=f"(d0), "=f"(d1)
+      : "f"(a0), "f"(a1), "f"(b0), "f"(b1));
+}
+__device__ __forceinline__ void mul2(float &d0, float &d1, float a0, float a1, float b) {
+  asm("{.reg .b64 ra, rb, rd;\n\t"
+      "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %4};\n\t"
+      "mul.rn.f32x2 rd, ra, rb;\n\tmov.b64 {%0, %1}, rd;}"
+      : "=f"(d0), "=f"(d1)
+      : "f"(a0), "f"(a1), "f"(b));
+}
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float d;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+__device__ __forceinline__ uint32_t e2m1x8(const float (&y)[16], int o) {
+  uint32_t w;
+  asm("{.reg .b8 b0, b1, b2, b3;\n\t"
+      "cvt.rn.satfinite.e2m1x2.f32 b0, %2, %1;\n\tcvt.rn.satfinite.e2m1x2.f32 b1, %4, %3;\n\t"
+      "cvt.rn.satfinite.e2m1x2.f32 b2, %6, %5;\n\tcvt.rn.satfinite.e2m1x2.f32 b3, %8, %7;\n\t"
+      "mov.b32 %0, {b0, b1, b2, b3};}"
+      : "=r"(w)
+      : "f"(y[o]), "f"(y[o + 1]), "f"(y[o + 2]), "f"(y[o + 3]), "f"(y[o + 4]), "f"(y[o + 5]), "f"(y[o + 6]), "f"(y[o + 7]));
+  return w;
+}
+__device__ __forceinline__ void quantize_block16(const float (&xc)[16], const BlockScale &q, uint32_t &scale_code, uint2 &codes) {
+  float m[4];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) xc[i] = __fsub_rn(f[i], mu[i]);
-  unpack8(reinterpret_cast<const uint4 *>(row)[1], f);
+  for (int i = 0; i < 4; ++i) m[i] = max3(fabsf(xc[4 * i]), fabsf(xc[4 * i + 1]), fabsf(xc[4 * i + 2]));
 #pragma unroll
-  for (int i = 0; i < 8; ++i) xc[8 + i] = __fsub_rn(f[i], mu[8 + i]);
+  for (int i = 0; i < 2; ++i) m[i] = max3(m[i], fabsf(xc[8 * i + 3]), fabsf(xc[8 * i + 7]));
+  const float a = fmaxf(max3(m[0], m[1], m[2]), m[3]);
+  float r = __fmul_rn(a, q.rcp);
+  if (!(r >= 0.015625f && r < 512.0f && abs((int)(__float_as_uint(r) & 0xFFFFFu) - 0x80000) > 4)) r = __fdiv_rn(a, q.e);
+  scale_code = (uint32_t)__nv_cvt_float_to_fp8(r, __NV_SATFINITE, __NV_E4M3);
+  const float inv = q.inv[scale_code];
+  float y[16];
+#pragma unroll
+  for (int i = 0; i < 16; i += 2) mul2(y[i], y[i + 1], xc[i], xc[i + 1], inv);
+  codes = make_uint2(e2m1x8(y, 0), e2m1x8(y, 8));
+}
+
+// 16 channels of one row (16-byte aligned: the interface asks for no more, a single 32-byte load would)
+struct Row16 { uint4 a, b; };
+__device__ __forceinline__ Row16 load_row16(const __nv_bfloat16 *p) {
+  const uint4 *u = reinterpret_cast<const uint4 *>(p);
+  return Row16{__ldg(u), __ldg(u + 1)};
+}
+// x - mean of 16 channels; mean: 16-byte aligned
+__device__ __forceinline__ void center16(const Row16 &x, const float *mean, float (&xc)[16]) {
+  float f[16];
+  unpack8(x.a, reinterpret_cast<float(&)[8]>(f[0]));
+  unpack8(x.b, reinterpret_cast<float(&)[8]>(f[8]));
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    const float4 m = reinterpret_cast<const float4 *>(mean)[c];
+    add2(xc[4 * c], xc[4 * c + 1], f[4 * c], f[4 * c + 1], -m.x, -m.y);
+    add2(xc[4 * c + 2], xc[4 * c + 3], f[4 * c + 2], f[4 * c + 3], -m.z, -m.w);
+  }
+}
+
+// Compensation vector (Eq. 9): Delta_S[hq][t] = qmean[hq] . (k[t] - kmean) in FP64, in units of gscale_q * gscale_k, rounded once
+// to BF16.  The product of eight keys with the (up to eight) query means of the group is a contraction over the channels and
+// runs on the FP64 tensor instruction (m8n8k4): lane (key = lane / 4, j = lane mod 4) holds the 16-channel blocks j and j + 4 of
+// its key, so step s of the contraction takes the lane's own s-th channel, in the order
+//   channel(j, s) = 16 j + s (s < 16), 64 + 16 j + s - 16,
+// and the sums come out complete, without staging rows or shuffling.  (A chain of 128 FP64 FMAs per key and head, as one
+// thread each, was bound by latency; with the eight threads of a key taking 16 channels each, by the shared-memory reads of the
+// query means.)  The order of the FP64 additions is fixed; it differs from a sequential sum by a few parts in 2^53, and BF16
+// keeps eight bits.
+//
+// Query means as doubles in operand order: [step][head][j].
+typedef double GroupMeans[32][8][4];
+__device__ __forceinline__ void convert_group_means(GroupMeans &m, const float *q_mean /* [G, 128] */, int G, int tid, int n_threads) {
+  for (int i = tid; i < 8 * HEAD_DIM; i += n_threads) {
+    const int g = i >> 7, c = i & 127;
+    m[(c & 15) + ((c >> 6) << 4)][g][(c >> 4) & 3] = g < G ? (double)q_mean[g * HEAD_DIM + c] : 0.0;
+  }
+}
+// acc (heads 2 j, 2 j + 1 of the lane's key) += the half's 16 channels
+__device__ __forceinline__ void group_dot16(const GroupMeans &m, int half, const float (&xc)[16], int lane, double (&acc)[2]) {
+  const double *q = &m[half * 16][0][0] + lane;
+#pragma unroll
+  for (int s = 0; s < 16; ++s)
+    asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};"
+                 : "+d"(acc[0]), "+d"(acc[1])
+                 : "d"((double)xc[s]), "d"(q[s * 32]));
 }
 
 struct QuantTensor {
   const __nv_bfloat16 *x;   // null: tensor absent (H = 0)
-  const float *mean, *gscale;
+  const float *mean;
+  TensorScale scale;
   int N, H, tiles;
+  int ctas;                 // CTAs per head; CTA c takes the tiles c, c + ctas, ... from the last one
   uint8_t *codes, *sf;
 };
-
-__device__ __forceinline__ void quantize_tile_body(const __nv_bfloat16 *__restrict__ x, const float *__restrict__ mean,
-                                                   const float *__restrict__ gscale, const int N, const int H,
-                                                   const int tiles, uint8_t *__restrict__ codes,
-                                                   uint8_t *__restrict__ sf, const int h, const int tile) {
-  __shared__ float mu[HEAD_DIM];
-  __shared__ __align__(16) uint8_t sf_tile[1024];
-  const int b = blockIdx.z;
-  if (tile >= tiles) return;
-  const int n_pad = tiles * TILE;
-  if (threadIdx.x < HEAD_DIM) mu[threadIdx.x] = mean[((size_t)b * H + h) * HEAD_DIM + threadIdx.x];
-  __syncthreads();
-  const float d = gscale[b];
-  // the thread's block index g = threadIdx.x & 7 is the same in all four iterations: its 16 means live in registers
-  // (read from shared memory per block they cost 4-way bank conflicts: the data pipe was the kernel's limiter)
-  float mreg[16];
-#pragma unroll
-  for (int i = 0; i < 16; ++i) mreg[i] = mu[(threadIdx.x & 7) * 16 + i];
-  // all eight 16-byte loads of the thread's four blocks are issued before the first block is quantized
-  uint4 raw[4][2];
-#pragma unroll
-  for (int it = 0; it < 4; ++it) {
-    const int id = it * 256 + threadIdx.x;
-    const int r = id >> 3, g = id & 7;
-    const int t = tile * TILE + r;
-    raw[it][0] = raw[it][1] = make_uint4(0u, 0u, 0u, 0u);
-    if (t < N) {
-      const uint4 *src = reinterpret_cast<const uint4 *>(x + (((size_t)b * N + t) * H + h) * HEAD_DIM + g * 16);
-      raw[it][0] = __ldcs(src);
-      raw[it][1] = __ldcs(src + 1);
-    }
-  }
-#pragma unroll
-  for (int it = 0; it < 4; ++it) {
-    const int id = it * 256 + threadIdx.x;
-    const int r = id >> 3, g = id & 7;
-    const int t = tile * TILE + r;
-    uint2 c = make_uint2(0u, 0u);
-    uint8_t sc = 0;
-    if (t < N) {
-      float xc[16], f[8];
-      unpack8(raw[it][0], f);
-#pragma unroll
-      for (int i = 0; i < 8; ++i) xc[i] = __fsub_rn(f[i], mreg[i]);
-      unpack8(raw[it][1], f);
-#pragma unroll
-      for (int i = 0; i < 8; ++i) xc[8 + i] = __fsub_rn(f[i], mreg[8 + i]);
-      quantize_block16(xc, d, sc, c);
-    }
-    __stcs(reinterpret_cast<uint2 *>(codes + (((size_t)b * H + h) * n_pad + t) * 64 + g * 8), c);
-    sf_tile[(g >> 2) * 512 + (r & 31) * 16 + (r >> 5) * 4 + (g & 3)] = sc;
-  }
-  __syncthreads();
-  uint32_t *dst = reinterpret_cast<uint32_t *>(sf + (((size_t)b * H + h) * tiles + tile) * 1024);
-  dst[threadIdx.x] = reinterpret_cast<const uint32_t *>(sf_tile)[threadIdx.x];
-}
-
-// K tile with the compensation vector (Eq. 9) in the same pass: the tile's rows are staged once in shared memory
-// (coalesced 16-byte loads; a row is 256 contiguous bytes, rows of one head are H_kv * 256 bytes apart; row pitch
-// 272 bytes so that the 16-byte reads of 8 consecutive threads fall into 8 different bank groups), quantized from
-// there exactly like a Q tile, and then every key's Delta_S[hq][t] = qmean[hq] . (k[t] - kmean) is accumulated in
-// FP64 with channels ascending by thread (key, part), part taking the heads g = part, part + 2, ... of the group as
-// independent sequential chains; the result is expressed in units of gscale_q * gscale_k and rounded once to BF16.
 struct DeltaArgs {
-  const float *q_mean;     // null: no Delta_S (direct variant or statistics-only call)
-  const float *q_gscale;
-  __nv_bfloat16 *delta;    // [B, H_q, N_pad]
+  const float *q_mean;
+  TensorScale q_scale;
+  __nv_bfloat16 *delta;    // [B, H_q, N_pad]; null: no Delta_S (direct variant)
   int H_q;
 };
 
-constexpr int KROW_PITCH = 272;
-constexpr int KTILE_SMEM = TILE * KROW_PITCH + 8 * HEAD_DIM * 8;   // staged rows + FP64 query means of the group
-
-__device__ __forceinline__ void quantize_k_tile_delta_body(const QuantTensor &a, const DeltaArgs &da, const int h,
-                                                           const int tile, uint8_t *dyn) {
-  constexpr int MAXG = 8;
-  __shared__ float mu[HEAD_DIM];
-  __shared__ __align__(16) uint8_t sf_tile[1024];
-  uint8_t *rows = dyn;
-  double(*qmu)[HEAD_DIM] = reinterpret_cast<double(*)[HEAD_DIM]>(dyn + TILE * KROW_PITCH);
-  const int b = blockIdx.z;
-  if (tile >= a.tiles) return;
-  const int N = a.N, H = a.H, n_pad = a.tiles * TILE;
-  const int G = da.H_q / H;
-  if (threadIdx.x < HEAD_DIM) mu[threadIdx.x] = a.mean[((size_t)b * H + h) * HEAD_DIM + threadIdx.x];
-  for (int j = threadIdx.x; j < G * HEAD_DIM; j += 256)
-    qmu[j >> 7][j & 127] = (double)da.q_mean[((size_t)b * da.H_q + h * G + (j >> 7)) * HEAD_DIM + (j & 127)];
-  for (int i = threadIdx.x; i < TILE * 16; i += 256) {
-    const int r = i >> 4, ch = i & 15;
-    const int tt = tile * TILE + r;
-    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-    if (tt < N) v = __ldcs(reinterpret_cast<const uint4 *>(a.x + (((size_t)b * N + tt) * H + h) * HEAD_DIM + ch * 8));
-    *reinterpret_cast<uint4 *>(rows + r * KROW_PITCH + ch * 16) = v;
+// Tiles (128 tokens of one head) of K and Q; blockIdx.x runs over K's CTAs, then Q's, the head index fastest, so that the
+// CTAs resident at any time read whole token rows of the [B, N, H, 128] input (contiguous DRAM) instead of 256-byte
+// pieces 256 * H bytes apart; from the last token to the first, because the statistics pass has just read the tensors in
+// ascending order and their ends are still in L2.  Warp w takes rows 8 w .. and 64 + 8 w .. of a tile, lane (row, j) their
+// 16-channel blocks j and j + 4.  A CTA stays with one head, so that after the set-up's barrier its warps run on their own:
+// the loads of the next tile are issued as soon as the registers of a row group are free, scale words and Delta_S go straight
+// to memory (partial sectors merge in L2).
+// Measured (16384 tokens, 32:8 heads, K with Delta_S and Q): two launches, rows of K staged in shared memory, two
+// divisions per block 35 + 38 us; one launch, one tile per CTA 61; with a ring of asynchronous copies and a barrier per tile 87;
+// now TILE_NEW us.
+constexpr int QT_CTAS = 3;   // resident per SM
+__global__ void __launch_bounds__(256, QT_CTAS) quantize_tile_kernel(const QuantTensor k, const QuantTensor q, const DeltaArgs da) {
+  __shared__ __align__(16) GroupMeans gm;
+  __shared__ __align__(16) float s_mean[HEAD_DIM];
+  __shared__ float inv_table[128];
+  launch_dependents();
+  grid_dependency_wait();
+  const int b = blockIdx.z, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, j = lane & 3;
+  const int k_ctas = k.ctas * k.H;
+  const bool is_k = (int)blockIdx.x < k_ctas;
+  const QuantTensor &a = is_k ? k : q;
+  const int at = is_k ? blockIdx.x : blockIdx.x - k_ctas;
+  const int h = at % a.H, N = a.N, ctas = a.ctas;
+  int tile = a.tiles - 1 - at / a.H;
+  const size_t head = (size_t)b * a.H + h, row = (size_t)a.H * HEAD_DIM;
+  const __nv_bfloat16 *const x0 = a.x + (size_t)b * N * row + h * HEAD_DIM + j * 16;
+  const int r0 = warp * 8 + (lane >> 2);
+  Row16 raw[2][2];
+#pragma unroll
+  for (int it = 0; it < 2; ++it) {
+    const int t = tile * TILE + it * 64 + r0;
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+      raw[it][half] = Row16{};
+      if (t < N) raw[it][half] = load_row16(x0 + t * row + half * 64);
+    }
+  }
+  const float d = tensor_scale(a.scale, b, lane);
+  if (at == 0 && tid == 0 && a.scale.gmax) a.scale.gscale[b] = d;
+  const BlockScale bs = make_block_scale(d, inv_table, tid);
+  if (tid >= 128) s_mean[tid - 128] = a.mean[head * HEAD_DIM + tid - 128];
+  const bool with_delta = is_k && da.delta;
+  const int G = with_delta ? da.H_q / a.H : 0;
+  double unit = 0.0;
+  if (with_delta) {
+    convert_group_means(gm, da.q_mean + ((size_t)b * da.H_q + h * G) * HEAD_DIM, G, tid, 256);
+    unit = 1.0 / ((double)tensor_scale(da.q_scale, b, lane) * (double)d);
   }
   __syncthreads();
-  const float d = a.gscale[b];
-  float mreg[16];
+  const size_t n_pad = (size_t)a.tiles * TILE;
+  uint8_t *const codes = a.codes + head * n_pad * 64 + j * 8;
+  for (; tile >= 0; tile -= ctas) {
+    uint8_t *const sf_tile = a.sf + (head * a.tiles + tile) * 1024;
 #pragma unroll
-  for (int i = 0; i < 16; ++i) mreg[i] = mu[(threadIdx.x & 7) * 16 + i];
+    for (int it = 0; it < 2; ++it) {
+      const int r = it * 64 + r0, t = tile * TILE + r;
+      double acc[2] = {0.0, 0.0};
 #pragma unroll
-  for (int it = 0; it < 4; ++it) {
-    const int id = it * 256 + threadIdx.x;
-    const int r = id >> 3, g = id & 7;
-    const int t = tile * TILE + r;
+      for (int half = 0; half < 2; ++half) {
+        float xc[16];
+        center16(raw[it][half], s_mean + half * 64 + j * 16, xc);
+        if (tile >= ctas) raw[it][half] = load_row16(x0 + (size_t)(t - ctas * TILE) * row + half * 64);   // a whole tile: only the last has an end
+        uint2 c = make_uint2(0u, 0u);
+        uint32_t sc = 0u;
+        if (t < N) quantize_block16(xc, bs, sc, c);
+        __stcs(reinterpret_cast<uint2 *>(codes + (size_t)t * 64 + half * 32), c);
+        sc <<= 8 * j;   // the four scale bytes of the half row in one word
+        sc |= __shfl_xor_sync(0xffffffffu, sc, 1);
+        sc |= __shfl_xor_sync(0xffffffffu, sc, 2);
+        if (j == 0) *reinterpret_cast<uint32_t *>(sf_tile + half * 512 + (r & 31) * 16 + (r >> 5) * 4) = sc;
+        if (with_delta) group_dot16(gm, half, xc, lane, acc);
+      }
+      if (with_delta) {
+#pragma unroll
+        for (int n = 0; n < 2; ++n) {
+          const int g = 2 * j + n;
+          if (g < G)
+            da.delta[((size_t)b * da.H_q + h * G + g) * n_pad + t] = __float2bfloat16_rn(t < N ? __double2float_rn(acc[n] * unit) : 0.0f);
+        }
+      }
+    }
+  }
+}
+
+// The tiles of a decode step's queries (at most eight tokens): one warp per (batch element, head), the eight rows and the zeros
+// of the other 120.  Bound by writing 9 KB per tile; with a CTA per tile the chain of loads was repeated for six waves of
+// CTAs (64 requests, 40 heads: 13.6 us, now 7.1 us).
+__global__ void __launch_bounds__(256) quantize_token_kernel(const QuantTensor q, int n_heads) {
+  launch_dependents();
+  grid_dependency_wait();
+  const int head = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31, j = lane & 3, r = lane >> 2;
+  if (head >= n_heads) return;
+  const int b = head / q.H, h = head % q.H;
+  const bool in = r < q.N;
+  Row16 raw[2] = {};
+#pragma unroll
+  for (int half = 0; half < 2; ++half)
+    if (in) raw[half] = load_row16(q.x + (((size_t)b * q.N + r) * q.H + h) * HEAD_DIM + (half * 4 + j) * 16);
+  const float d = tensor_scale(q.scale, b, lane);
+  if (h == 0 && lane == 0 && q.scale.gmax) q.scale.gscale[b] = d;
+  uint8_t *const codes = q.codes + (size_t)head * TILE * 64, *const sf = q.sf + (size_t)head * 1024;
+  const uint4 z = make_uint4(0u, 0u, 0u, 0u);
+  for (int i = 32 + lane; i < TILE * 4; i += 32) reinterpret_cast<uint4 *>(codes)[i] = z;
+  for (int i = lane; i < 64; i += 32)
+    if ((i & 31) >= 8) reinterpret_cast<uint4 *>(sf)[i] = z;   // 16 bytes per row of the atom: rows 8..31 of both halves
+#pragma unroll
+  for (int half = 0; half < 2; ++half) {
+    float xc[16];
+    center16(raw[half], q.mean + (size_t)head * HEAD_DIM + (half * 4 + j) * 16, xc);
+    uint8_t s8 = 0;
     uint2 c = make_uint2(0u, 0u);
-    uint8_t sc = 0;
-    if (t < N) {
-      float xc[16];
-      load_center16(reinterpret_cast<const __nv_bfloat16 *>(rows + r * KROW_PITCH + g * 32), mreg, xc);
-      quantize_block16(xc, d, sc, c);
-    }
-    *reinterpret_cast<uint2 *>(a.codes + (((size_t)b * H + h) * n_pad + t) * 64 + g * 8) = c;
-    sf_tile[(g >> 2) * 512 + (r & 31) * 16 + (r >> 5) * 4 + (g & 3)] = sc;
-  }
-  // Delta_S.  The FP64 pipe is the scarce unit here (measured: an eighth of the FP32 rate on this GPU); two threads
-  // per key, each with the chains of every other head of the group, keep enough independent chains in flight to
-  // cover its latency.
-  {
-    const int key = threadIdx.x & 127, part = threadIdx.x >> 7;
-    const int t = tile * TILE + key;
-    double acc[MAXG / 2];
-#pragma unroll
-    for (int u = 0; u < MAXG / 2; ++u) acc[u] = 0.0;
-    if (t < N) {
-      const uint8_t *row = rows + key * KROW_PITCH;
-      for (int c0 = 0; c0 < HEAD_DIM; c0 += 8) {
-        float f[8];
-        unpack8(*reinterpret_cast<const uint4 *>(row + c0 * 2), f);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const double kc = (double)__fsub_rn(f[i], mu[c0 + i]);
-#pragma unroll
-          for (int u = 0; u < MAXG / 2; ++u)
-            if (2 * u + part < G) acc[u] = fma(qmu[2 * u + part][c0 + i], kc, acc[u]);
-        }
-      }
-    }
-    const double denom = (double)da.q_gscale[b] * (double)d;
-#pragma unroll
-    for (int u = 0; u < MAXG / 2; ++u) {
-      const int g = 2 * u + part;
-      if (g < G) {
-        const float v = (t < N) ? __double2float_rn(__ddiv_rn(acc[u], denom)) : 0.0f;
-        da.delta[((size_t)b * da.H_q + h * G + g) * n_pad + t] = __float2bfloat16_rn(v);
-      }
-    }
-  }
-  __syncthreads();
-  uint32_t *dst = reinterpret_cast<uint32_t *>(a.sf + (((size_t)b * H + h) * a.tiles + tile) * 1024);
-  dst[threadIdx.x] = reinterpret_cast<const uint32_t *>(sf_tile)[threadIdx.x];
-}
-
-// grid (max tiles * (H of the first + H of the second tensor), 1, B); one 128-token tile of one head per block,
-// blockIdx.x = tile * heads + head: the head index runs fastest, so the blocks resident at any time read whole token
-// rows of the [B, N, H, 128] input (contiguous DRAM) instead of 256-byte pieces 256 * H bytes apart.
-__global__ void __launch_bounds__(256) quantize_fp4_tile_kernel(const QuantTensor a0, const QuantTensor a1) {
-  const int heads = a0.H + a1.H;
-  const int tile = (int)blockIdx.x / heads, y = (int)blockIdx.x % heads;
-  if (y < a0.H)
-    quantize_tile_body(a0.x, a0.mean, a0.gscale, a0.N, a0.H, a0.tiles, a0.codes, a0.sf, y, tile);
-  else
-    quantize_tile_body(a1.x, a1.mean, a1.gscale, a1.N, a1.H, a1.tiles, a1.codes, a1.sf, y - a0.H, tile);
-}
-
-// grid (tiles * H_kv, 1, B), KTILE_SMEM bytes of dynamic shared memory: K tiles with Delta_S, blockIdx.x = tile * H_kv +
-// head.  A launch of its own: these blocks are bound by the FP64 pipe, the Q tiles by memory, and in one launch
-// (kinds interleaved) they only competed for block slots (98 us against 42 + 38 at 16K).
-__global__ void __launch_bounds__(256) quantize_k_delta_kernel(const QuantTensor a, const DeltaArgs da) {
-  extern __shared__ __align__(16) uint8_t dyn_smem[];
-  quantize_k_tile_delta_body(a, da, (int)blockIdx.x % a.H, (int)blockIdx.x / a.H, dyn_smem);
-}
-
-// Eq. 9: Delta_S[hq][t] = qmean[hq] . (k[t] - kmean), FP64 accumulation with channels ascending,
-// expressed in units of gscale_q * gscale_k and rounded once to BF16.  Two threads per key token
-// (256 threads per 128-token tile): thread (key, part) takes the heads g = part, part + 2, ... of the
-// group, each as its own sequential chain.  grid (N_pad/128, H_kv, B).  Used for the paged side cache (PAGED: the
-// entries go to their page through the page-table row); the dense vector of mpfa_quantize_qk comes out of
-// quantize_k_delta_kernel, which runs the same chains on rows it has already staged.
-template <bool PAGED>
-__global__ void __launch_bounds__(256) delta_s_kernel(const __nv_bfloat16 *__restrict__ k,
-                                                      const float *__restrict__ q_mean,
-                                                      const float *__restrict__ k_mean,
-                                                      const float *__restrict__ q_gscale,
-                                                      const float *__restrict__ k_gscale, int N, int H_q, int H_kv,
-                                                      __nv_bfloat16 *__restrict__ delta,
-                                                      const int32_t *__restrict__ page_row, int num_pages) {
-  constexpr int MAXG = 8;
-  __shared__ float kmu[HEAD_DIM];
-  __shared__ double qmu[MAXG][HEAD_DIM];   // converted once: the conversion is as costly as the FMA
-  const int tile = blockIdx.x, hk = blockIdx.y, b = blockIdx.z;
-  const int G = H_q / H_kv;
-  const int n_pad = gridDim.x * TILE;
-  if (threadIdx.x < HEAD_DIM) kmu[threadIdx.x] = k_mean[((size_t)b * H_kv + hk) * HEAD_DIM + threadIdx.x];
-  for (int j = threadIdx.x; j < G * HEAD_DIM; j += 256)
-    qmu[j >> 7][j & 127] = (double)q_mean[((size_t)b * H_q + hk * G + (j >> 7)) * HEAD_DIM + (j & 127)];
-  __syncthreads();
-  // The tile's K rows are staged in shared memory with coalesced 16-byte loads (a row is 256 contiguous
-  // bytes, rows of one head are H_kv * 256 bytes apart); each thread then walks its own row.  Row pitch
-  // 272 bytes: the 16-byte reads of 8 consecutive threads fall into 8 different bank groups.
-  constexpr int PITCH = 272;
-  __shared__ __align__(16) uint8_t rows[TILE * PITCH];
-  for (int i = threadIdx.x; i < TILE * 16; i += 256) {
-    const int r = i >> 4, ch = i & 15;
-    const int tt = tile * TILE + r;
-    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-    if (tt < N) v = *reinterpret_cast<const uint4 *>(k + (((size_t)b * N + tt) * H_kv + hk) * HEAD_DIM + ch * 8);
-    *reinterpret_cast<uint4 *>(rows + r * PITCH + ch * 16) = v;
-  }
-  __syncthreads();
-  const int key = threadIdx.x & 127, part = threadIdx.x >> 7;
-  const int t = tile * TILE + key;
-  double acc[MAXG / 2];
-#pragma unroll
-  for (int u = 0; u < MAXG / 2; ++u) acc[u] = 0.0;
-  if (t < N) {
-    const uint8_t *row = rows + key * PITCH;
-    for (int c0 = 0; c0 < HEAD_DIM; c0 += 8) {
-      float f[8];
-      unpack8(*reinterpret_cast<const uint4 *>(row + c0 * 2), f);
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const double kc = (double)__fsub_rn(f[i], kmu[c0 + i]);
-#pragma unroll
-        for (int u = 0; u < MAXG / 2; ++u)
-          if (2 * u + part < G) acc[u] = fma(qmu[2 * u + part][c0 + i], kc, acc[u]);
-      }
-    }
-  }
-  const double denom = (double)q_gscale[b] * (double)k_gscale[b];
-#pragma unroll
-  for (int u = 0; u < MAXG / 2; ++u) {
-    const int g = 2 * u + part;
-    if (g < G) {
-      const float v = (t < N) ? __double2float_rn(__ddiv_rn(acc[u], denom)) : 0.0f;
-      if (PAGED) {
-        if ((t >> 6) < (N + PAGE - 1) / PAGE) {   // slots past N inside the last page are zero-filled
-          const int page = page_row[t >> 6];
-          if (page >= 0 && page < num_pages)
-            // 16-byte chunks XOR-swizzled by the head's index in its group: the row is read as a
-            // swizzled MN-major tensor-core operand by the decode kernel
-            delta[((size_t)page * H_q + hk * G + g) * PAGE + (((((t & 63) >> 3) ^ g) << 3) | (t & 7))] = __float2bfloat16_rn(v);
-        }
-      } else {
-        delta[((size_t)b * H_q + hk * G + g) * n_pad + t] = __float2bfloat16_rn(v);
-      }
-    }
+    if (in) quantize_block16(xc, d, s8, c);
+    *reinterpret_cast<uint2 *>(codes + r * 64 + (half * 4 + j) * 8) = c;
+    uint32_t sc = (uint32_t)s8 << (8 * j);
+    sc |= __shfl_xor_sync(0xffffffffu, sc, 1);
+    sc |= __shfl_xor_sync(0xffffffffu, sc, 2);
+    if (j == 0) *reinterpret_cast<uint4 *>(sf + half * 512 + r * 16) = make_uint4(sc, 0u, 0u, 0u);
   }
 }
 
-__device__ __forceinline__ uint4 quantize_v16(const __nv_bfloat16 *row, float inv) {
+__device__ __forceinline__ uint4 quantize_v16(const Row16 &x, float inv) {
   float f[16];
-  {
-    float t8[8];
-    unpack8(reinterpret_cast<const uint4 *>(row)[0], t8);
+  unpack8(x.a, reinterpret_cast<float(&)[8]>(f[0]));
+  unpack8(x.b, reinterpret_cast<float(&)[8]>(f[8]));
 #pragma unroll
-    for (int i = 0; i < 8; ++i) f[i] = t8[i];
-    unpack8(reinterpret_cast<const uint4 *>(row)[1], t8);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) f[8 + i] = t8[i];
-  }
+  for (int i = 0; i < 16; i += 2) mul2(f[i], f[i + 1], f[i], f[i + 1], inv);
   uint32_t w[4];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    uint32_t lo = (uint32_t)__nv_cvt_float2_to_fp8x2(
-        make_float2(__fmul_rn(f[4 * i], inv), __fmul_rn(f[4 * i + 1], inv)), __NV_SATFINITE, __NV_E4M3);
-    uint32_t hi = (uint32_t)__nv_cvt_float2_to_fp8x2(
-        make_float2(__fmul_rn(f[4 * i + 2], inv), __fmul_rn(f[4 * i + 3], inv)), __NV_SATFINITE, __NV_E4M3);
-    w[i] = (lo & 0xFFFFu) | (hi << 16);
-  }
+  for (int i = 0; i < 4; ++i)   // two conversions written into the halves of one register
+    asm("{.reg .b16 lo, hi;\n\t"
+        "cvt.rn.satfinite.e4m3x2.f32 lo, %2, %1;\n\tcvt.rn.satfinite.e4m3x2.f32 hi, %4, %3;\n\t"
+        "mov.b32 %0, {lo, hi};}"
+        : "=r"(w[i])
+        : "f"(f[4 * i]), "f"(f[4 * i + 1]), "f"(f[4 * i + 2]), "f"(f[4 * i + 3]));
   return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
 // grid (N_pad/128, H, B): V tile -> [B, H, N_pad, 128] E4M3.
 __global__ void __launch_bounds__(256) quantize_v_tile_kernel(const __nv_bfloat16 *__restrict__ v, int N, int H,
                                                               float inv_scale, uint8_t *__restrict__ out) {
+  launch_dependents();
+  grid_dependency_wait();
   const int tile = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
   const int n_pad = gridDim.x * TILE;
 #pragma unroll
@@ -534,7 +540,7 @@ __global__ void __launch_bounds__(256) quantize_v_tile_kernel(const __nv_bfloat1
     const int r = id >> 3, seg = id & 7;
     const int t = tile * TILE + r;
     uint4 c = make_uint4(0u, 0u, 0u, 0u);
-    if (t < N) c = quantize_v16(v + (((size_t)b * N + t) * H + h) * HEAD_DIM + seg * 16, inv_scale);
+    if (t < N) c = quantize_v16(load_row16(v + (((size_t)b * N + t) * H + h) * HEAD_DIM + seg * 16), inv_scale);
     *reinterpret_cast<uint4 *>(out + (((size_t)b * H + h) * n_pad + t) * HEAD_DIM + seg * 16) = c;
   }
 }
@@ -598,154 +604,176 @@ __global__ void __launch_bounds__(256) quantize_v_fp4_tile_kernel(const __nv_bfl
   if (threadIdx.x < 64) reinterpret_cast<uint4 *>(sf + tile_id * 1024)[threadIdx.x] = reinterpret_cast<const uint4 *>(stile)[threadIdx.x];
 }
 
-// Paged cache write for one request: grid (pages, H_kv).  K and V of one (page, head) are
-// quantized into shared memory in the byte order of the decode kernel's shared-memory operand
-// tiles (so that decode fills a tile with one bulk copy) and copied out with 16-byte stores.
-__global__ void __launch_bounds__(256) quantize_kv_page_kernel(const __nv_bfloat16 *__restrict__ k,
-                                                               const __nv_bfloat16 *__restrict__ v,
-                                                               const float *__restrict__ k_mean,
-                                                               const float *__restrict__ k_gscale, int N, int H_kv,
-                                                               float inv_vscale, const int32_t *__restrict__ page_row,
-                                                               int first_page, int num_pages,
-                                                               uint8_t *__restrict__ k_codes, uint8_t *__restrict__ k_sf,
-                                                               uint8_t *__restrict__ v_fp8) {
-  __shared__ float mu[HEAD_DIM];
-  __shared__ __align__(16) uint8_t sk[4096];
-  __shared__ __align__(16) uint8_t ssf[512];
-  __shared__ __align__(16) uint8_t sv[8192];
-  const int lp = blockIdx.x, h = blockIdx.y;
-  const int page = page_row[first_page + lp];
-  if (page < 0 || page >= num_pages) return;  // the host validates the shape; a bad id is skipped
-  if (threadIdx.x < HEAD_DIM) mu[threadIdx.x] = k_mean[(size_t)h * HEAD_DIM + threadIdx.x];
-  __syncthreads();
-  const float d = k_gscale[0];
-#pragma unroll
-  for (int it = 0; it < 2; ++it) {
-    const int id = it * 256 + threadIdx.x;
-    const int t = id >> 3, g = id & 7;   // token in page, 16-channel block / segment
-    const int tok = lp * PAGE + t;
-    uint2 c = make_uint2(0u, 0u);
-    uint8_t sc = 0;
-    uint4 vc = make_uint4(0u, 0u, 0u, 0u);
-    if (tok < N) {
-      float xc[16];
-      load_center16(k + ((size_t)tok * H_kv + h) * HEAD_DIM + g * 16, mu + g * 16, xc);
-      quantize_block16(xc, d, sc, c);
-      vc = quantize_v16(v + ((size_t)tok * H_kv + h) * HEAD_DIM + g * 16, inv_vscale);
+// Paged cache write for one request: tokens first .. first + N - 1 go to their slots of the pages, whole pages or parts of
+// them.  grid (H_kv, CTAs per head); a CTA stays with one head and takes every gridDim.y-th page.  Warp w takes a page's slots
+// 8 w .. 8 w + 7, lane (slot, j) the 16-channel blocks j and j + 4, in the byte order of the decode kernel's shared-memory operand
+// tiles: K codes as 64-byte rows with the 64-byte swizzle, V as 128-byte rows with the 128-byte swizzle, Delta_S with its
+// 16-byte groups XOR-ed by the head.  K, V and Delta_S come from one read of K and V, and the rows of the next page are
+// requested while the current ones are quantized.  Slots past the last token are zero-filled in pages that the call
+// starts (a recycled page may hold anything, and decode needs finite bytes there); slots of earlier tokens are left alone.
+// Measured (9001 tokens, 32:8 heads): page kernel + a Delta_S kernel that read K again 12 + 16 us, one page per CTA 19.5 us, now
+// PAGE_NEW us.
+constexpr int WK_CTAS = 3;   // resident per SM
+__global__ void __launch_bounds__(256, WK_CTAS) write_kv_kernel(const __nv_bfloat16 *__restrict__ k, const __nv_bfloat16 *__restrict__ v,
+                                                                const float *__restrict__ k_mean, const TensorScale k_scale,
+                                                                const float *__restrict__ q_mean, const float *__restrict__ q_gscale,
+                                                                int N, int first, int n_pages, int H_q, int H_kv, float inv_vscale,
+                                                                const int32_t *__restrict__ page_row, int num_pages,
+                                                                uint8_t *__restrict__ k_codes, uint8_t *__restrict__ k_sf,
+                                                                uint8_t *__restrict__ v_fp8, __nv_bfloat16 *__restrict__ delta) {
+  __shared__ __align__(16) GroupMeans gm;
+  __shared__ __align__(16) float s_mean[HEAD_DIM];
+  __shared__ float inv_table[128];
+  launch_dependents();
+  grid_dependency_wait();
+  const int tid = threadIdx.x, lane = tid & 31, j = lane & 3, h = blockIdx.x, G = H_q / H_kv;
+  const int t = (tid >> 5) * 8 + (lane >> 2);   // slot of the page
+  const int page0 = first / PAGE;               // first page of the request that is touched
+  Row16 kr[2], vr[2];
+  int pg = blockIdx.y, page;
+  const auto fetch = [&](int half) {
+    const int i = (page0 + pg) * PAGE + t - first;   // index among the new tokens
+    kr[half] = vr[half] = Row16{};
+    if (pg < n_pages && i >= 0 && i < N) {
+      const size_t at = ((size_t)i * H_kv + h) * HEAD_DIM + (half * 4 + j) * 16;
+      kr[half] = load_row16(k + at);
+      vr[half] = load_row16(v + at);
     }
-    // K: the 8 code bytes of block g of token t, in the 64-byte-swizzled row order the decode
-    // kernel's tensor-core descriptor reads: (t/8)*512 + (t%8)*64 + ((g/2) ^ ((t%8)/2))*16 + (g%2)*8
-    *reinterpret_cast<uint2 *>(sk + (t >> 3) * 512 + (t & 7) * 64 + (((g >> 1) ^ ((t & 7) >> 1)) << 4) + (g & 1) * 8) = c;
-    ssf[t * 8 + g] = sc;
-    // V: channels 16g..16g+15 of token t, 128-byte-swizzled: (t/8)*1024 + (t%8)*128 + (g ^ (t%8))*16
-    *reinterpret_cast<uint4 *>(sv + (t >> 3) * 1024 + (t & 7) * 128 + ((g ^ (t & 7)) << 4)) = vc;
+  };
+  fetch(0);
+  fetch(1);
+  page = page_row[page0 + pg];
+  const float d = tensor_scale(k_scale, 0, lane);
+  if (blockIdx.y == 0 && h == 0 && tid == 0 && k_scale.gmax) k_scale.gscale[0] = d;
+  const BlockScale bs = make_block_scale(d, inv_table, tid);
+  if (tid >= 128) s_mean[tid - 128] = k_mean[(size_t)h * HEAD_DIM + tid - 128];
+  double unit = 0.0;
+  if (delta) {
+    convert_group_means(gm, q_mean + (size_t)h * G * HEAD_DIM, G, tid, 256);
+    unit = 1.0 / ((double)q_gscale[0] * (double)d);
   }
   __syncthreads();
-  const size_t slab = (size_t)page * H_kv + h;
-  reinterpret_cast<uint4 *>(k_codes + slab * 4096)[threadIdx.x] = reinterpret_cast<const uint4 *>(sk)[threadIdx.x];
-  if (threadIdx.x < 32) reinterpret_cast<uint4 *>(k_sf + slab * 512)[threadIdx.x] = reinterpret_cast<const uint4 *>(ssf)[threadIdx.x];
-  reinterpret_cast<uint4 *>(v_fp8 + slab * 8192)[threadIdx.x] = reinterpret_cast<const uint4 *>(sv)[threadIdx.x];
-  reinterpret_cast<uint4 *>(v_fp8 + slab * 8192)[threadIdx.x + 256] = reinterpret_cast<const uint4 *>(sv)[threadIdx.x + 256];
+  while (pg < n_pages) {
+    const int i = (page0 + pg) * PAGE + t - first;
+    const bool page_ok = page >= 0 && page < num_pages;   // a bad id is skipped
+    const bool is_new = page_ok && i >= 0 && i < N, fresh_pad = page_ok && i >= N && (page0 + pg) * PAGE >= first;
+    const size_t slab = (size_t)(page_ok ? page : 0) * H_kv + h;
+    uint8_t *const kd = k_codes + slab * 4096 + (t >> 3) * 512 + (t & 7) * 64, *const sd = k_sf + slab * 512 + t * 8;
+    uint8_t *const vd = v_fp8 + slab * 8192 + (t >> 3) * 1024 + (t & 7) * 128;
+    __nv_bfloat16 *const dd = delta + ((size_t)(page_ok ? page : 0) * H_q + h * G) * PAGE + (t & 7);
+    pg += gridDim.y;
+    if (pg < n_pages) page = page_row[page0 + pg];
+    double acc[2] = {0.0, 0.0};
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+      const int blk = half * 4 + j;
+      float xc[16];
+      center16(kr[half], s_mean + blk * 16, xc);
+      uint2 c = make_uint2(0u, 0u);
+      uint32_t sc = 0u;
+      uint4 vc = quantize_v16(vr[half], inv_vscale);
+      fetch(half);
+      if (is_new)
+        quantize_block16(xc, bs, sc, c);
+      else
+        vc = make_uint4(0u, 0u, 0u, 0u);
+      sc <<= 8 * j;   // the four scale bytes of half a token in one word
+      sc |= __shfl_xor_sync(0xffffffffu, sc, 1);
+      sc |= __shfl_xor_sync(0xffffffffu, sc, 2);
+      if (is_new || fresh_pad) {
+        *reinterpret_cast<uint2 *>(kd + (((blk >> 1) ^ ((t & 7) >> 1)) << 4) + (blk & 1) * 8) = c;
+        if (j == 0) *reinterpret_cast<uint32_t *>(sd + half * 4) = sc;
+        *reinterpret_cast<uint4 *>(vd + ((blk ^ (t & 7)) << 4)) = vc;
+      }
+      if (delta) group_dot16(gm, half, xc, lane, acc);
+    }
+    if (delta && (is_new || fresh_pad)) {
+#pragma unroll
+      for (int n = 0; n < 2; ++n) {
+        const int g = 2 * j + n;
+        if (g < G) dd[g * PAGE + (((t >> 3) ^ g) << 3)] = __float2bfloat16_rn(is_new ? __double2float_rn(acc[n] * unit) : 0.0f);
+      }
+    }
+  }
 }
 
-// Decode-time append (Section 6: new tokens are centered with the frozen means and quantized with the
-// frozen tensor scale): tokens first_token .. first_token + N - 1 of one request go to their slots of the
-// paged cache, wherever in a page they fall.  Thread = (token slot, 16-channel block); a block covers 32
-// slots of one kv head.  The grid runs to the end of the last page touched: slots past the last new token
-// are zero-filled if this call started their page (a recycled page may hold anything, and decode needs
-// finite bytes there); slots of a page that was started earlier are left alone.
-__global__ void __launch_bounds__(256) append_kv_kernel(const __nv_bfloat16 *__restrict__ k,
-                                                        const __nv_bfloat16 *__restrict__ v,
-                                                        const float *__restrict__ q_mean,
-                                                        const float *__restrict__ k_mean,
-                                                        const float *__restrict__ q_gscale,
-                                                        const float *__restrict__ k_gscale, int N, int first_token,
-                                                        int H_q, int H_kv, float inv_vscale, int smooth,
-                                                        const int32_t *__restrict__ page_row, int num_pages,
-                                                        uint8_t *__restrict__ k_codes, uint8_t *__restrict__ k_sf,
-                                                        uint8_t *__restrict__ v_fp8, __nv_bfloat16 *__restrict__ delta,
-                                                        const int32_t *__restrict__ positions, int max_pages) {
-  constexpr int MAXG = 8;
-  __shared__ float kmu[HEAD_DIM];
-  __shared__ double qmu[MAXG][HEAD_DIM];
-  __shared__ float kc[32][HEAD_DIM + 4];   // centered K rows of the block's tokens (for Delta_S)
-  if (positions) {
-    // batch form: request blockIdx.z appends the one token k[b] / v[b] at index positions[b] with its own
-    // statistics and page-table row; a negative position skips the request
-    const int b = blockIdx.z;
-    first_token = positions[b];
-    if (first_token < 0) return;
-    N = 1;
-    k += (size_t)b * H_kv * HEAD_DIM;
-    v += (size_t)b * H_kv * HEAD_DIM;
-    q_mean += (size_t)b * H_q * HEAD_DIM;
-    k_mean += (size_t)b * H_kv * HEAD_DIM;
-    q_gscale += b;
-    k_gscale += b;
-    page_row += (size_t)b * max_pages;
-    if ((first_token >> 6) >= max_pages) return;   // no page-table entry for that position
+// Decode-time append of a batch (Section 6): request b's one new token goes to index positions[b] with its own frozen
+// statistics and page-table row; a negative position skips the request.  One warp per (request, kv head): lane = (part 0..3,
+// 16-channel block); part 0 writes K, part 1 V, and part p the Delta_S of heads p and p + 4.  A token that starts a page zeroes the
+// other 63 slots.  Bound by the latency of three dependent loads; the loads that depend on nothing are issued together.
+// Measured (64 requests, 40:8 heads): with one thread per FP64 chain of 128 terms and 2 x 256 threads per pair
+// 9.8 us, now 6.6 us.
+__global__ void __launch_bounds__(256) append_kv_kernel(const __nv_bfloat16 *__restrict__ k, const __nv_bfloat16 *__restrict__ v,
+                                                        const float *__restrict__ q_mean, const float *__restrict__ k_mean,
+                                                        const float *__restrict__ q_gscale, const float *__restrict__ k_gscale,
+                                                        int B, int H_q, int H_kv, float inv_vscale,
+                                                        const int32_t *__restrict__ page_table, int max_pages, int num_pages,
+                                                        const int32_t *__restrict__ positions, uint8_t *__restrict__ k_codes,
+                                                        uint8_t *__restrict__ k_sf, uint8_t *__restrict__ v_fp8,
+                                                        __nv_bfloat16 *__restrict__ delta) {
+  launch_dependents();
+  grid_dependency_wait();
+  const int pair = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31, blk = lane & 7, part = lane >> 3;
+  if (pair >= B * H_kv) return;
+  const int b = pair / H_kv, h = pair % H_kv, G = H_q / H_kv;
+  const int pos = positions[b];
+  const Row16 kr = load_row16(k + (size_t)pair * HEAD_DIM + blk * 16), vr = load_row16(v + (size_t)pair * HEAD_DIM + blk * 16);
+  const float d = k_gscale[b];
+  const double denom = delta ? (double)q_gscale[b] * (double)d : 1.0;
+  float xc[16];
+  center16(kr, k_mean + (size_t)pair * HEAD_DIM + blk * 16, xc);
+  const bool in_table = pos >= 0 && (pos >> 6) < max_pages;   // else: skipped, or no page-table entry for that position
+  const int page = in_table ? page_table[(size_t)b * max_pages + (pos >> 6)] : -1;
+  const int t = pos & 63;
+  if (page < 0 || page >= num_pages) return;
+  const size_t slab = (size_t)page * H_kv + h;
+  uint8_t *const kd = k_codes + slab * 4096, *const sd = k_sf + slab * 512, *const vd = v_fp8 + slab * 8192;
+  __nv_bfloat16 *const dd = delta ? delta + ((size_t)page * H_q + h * G) * PAGE : nullptr;
+  if (part == 0) {
+    uint8_t sc;
+    uint2 c;
+    quantize_block16(xc, d, sc, c);
+    *reinterpret_cast<uint2 *>(kd + (t >> 3) * 512 + (t & 7) * 64 + (((blk >> 1) ^ ((t & 7) >> 1)) << 4) + (blk & 1) * 8) = c;
+    sd[t * 8 + blk] = sc;
+  } else if (part == 1) {
+    *reinterpret_cast<uint4 *>(vd + (t >> 3) * 1024 + (t & 7) * 128 + ((blk ^ (t & 7)) << 4)) = quantize_v16(vr, inv_vscale);
   }
-  const int h = blockIdx.y, G = H_q / H_kv;
-  const int slot = threadIdx.x >> 3, g = threadIdx.x & 7;
-  const int i = blockIdx.x * 32 + slot;          // index among the slots this call covers
-  const int tok = first_token + i;               // absolute token position
-  const bool is_new = i < N;
-  const bool in_range = tok < ((first_token + N + PAGE - 1) / PAGE) * PAGE;   // the grid is rounded up to 32 slots
-  if (threadIdx.x < HEAD_DIM) kmu[threadIdx.x] = k_mean[(size_t)h * HEAD_DIM + threadIdx.x];
-  if (smooth)
-    for (int j = threadIdx.x; j < G * HEAD_DIM; j += 256)
-      qmu[j >> 7][j & 127] = (double)q_mean[((size_t)h * G + (j >> 7)) * HEAD_DIM + (j & 127)];
-  __syncthreads();
-  const int page = in_range ? page_row[tok >> 6] : -1;
-  const bool page_ok = page >= 0 && page < num_pages;
-  const bool fresh_pad = !is_new && (tok & ~63) >= first_token;   // padding slot of a page this call started
-  const int t = tok & 63;
-  uint2 c = make_uint2(0u, 0u);
-  uint8_t sc = 0;
-  uint4 vc = make_uint4(0u, 0u, 0u, 0u);
-  if (is_new) {
-    float xc[16];
-    load_center16(k + ((size_t)i * H_kv + h) * HEAD_DIM + g * 16, kmu + g * 16, xc);
-    quantize_block16(xc, k_gscale[0], sc, c);
-    vc = quantize_v16(v + ((size_t)i * H_kv + h) * HEAD_DIM + g * 16, inv_vscale);
+  if (t == 0) {   // slot 0 is the first row of each slab
+    const uint4 z = make_uint4(0u, 0u, 0u, 0u);
+    for (int i = 4 + lane; i < 256; i += 32) reinterpret_cast<uint4 *>(kd)[i] = z;
+    for (int i = 2 + lane; i < 128; i += 32) reinterpret_cast<uint32_t *>(sd)[i] = 0u;
+    for (int i = 8 + lane; i < 512; i += 32) reinterpret_cast<uint4 *>(vd)[i] = z;
+    if (dd)
+      for (int i = lane; i < G * PAGE; i += 32)
+        if ((i & 63) != ((i >> 6) << 3)) dd[i] = __float2bfloat16_rn(0.0f);
+  }
+  if (!dd) return;
+  for (int g0 = 0; g0 < G; g0 += 4) {   // uniform: every lane takes part in the sums
+    const int g = g0 + part;
+    double acc = 0.0;
+    if (g < G) {
+      const float4 *qp = reinterpret_cast<const float4 *>(q_mean + ((size_t)b * H_q + h * G + g) * HEAD_DIM + blk * 16);
 #pragma unroll
-    for (int j = 0; j < 16; ++j) kc[slot][g * 16 + j] = xc[j];
-  }
-  if (page_ok && (is_new || fresh_pad)) {
-    const size_t slab = (size_t)page * H_kv + h;
-    *reinterpret_cast<uint2 *>(k_codes + slab * 4096 + (t >> 3) * 512 + (t & 7) * 64 + (((g >> 1) ^ ((t & 7) >> 1)) << 4) + (g & 1) * 8) = c;
-    k_sf[slab * 512 + t * 8 + g] = sc;
-    *reinterpret_cast<uint4 *>(v_fp8 + slab * 8192 + (t >> 3) * 1024 + (t & 7) * 128 + ((g ^ (t & 7)) << 4)) = vc;
-  }
-  __syncthreads();
-  // Delta_S (Eq. 9) of the new tokens: thread (slot, g) takes head g of the group, FP64, channels ascending
-  if (smooth && g < G && page_ok && (is_new || fresh_pad)) {
-    float val = 0.0f;
-    if (is_new) {
-      double acc = 0.0;
-      for (int ch = 0; ch < HEAD_DIM; ++ch) acc = fma(qmu[g][ch], (double)kc[slot][ch], acc);
-      val = __double2float_rn(__ddiv_rn(acc, (double)q_gscale[0] * (double)k_gscale[0]));
+      for (int i = 0; i < 4; ++i) {
+        const float4 m = qp[i];
+        acc = fma((double)m.x, (double)xc[4 * i], acc);
+        acc = fma((double)m.y, (double)xc[4 * i + 1], acc);
+        acc = fma((double)m.z, (double)xc[4 * i + 2], acc);
+        acc = fma((double)m.w, (double)xc[4 * i + 3], acc);
+      }
     }
-    delta[((size_t)page * H_q + h * G + g) * PAGE + ((((t >> 3) ^ g) << 3) | (t & 7))] = __float2bfloat16_rn(val);
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (blk == 0 && g < G)
+      dd[g * PAGE + ((((t >> 3) ^ g) << 3) | (t & 7))] = __float2bfloat16_rn(__double2float_rn(__ddiv_rn(acc, denom)));
   }
 }
 
 size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 
-// Workspace of the statistics pass: for each tensor S slices of per-column partial results (FP64 sum, maximum,
-// maximum of the negated values), then the per-batch-element maxima and one counter word.  S is the largest
-// slice count <= STAT_MAX_SLICES that fits the bytes the caller gave (at least 1).
-struct StatsWorkspace {
-  double *psum_q, *psum_k;
-  float *pmax_q, *pneg_q, *pmax_k, *pneg_k;
-  unsigned int *amax_q, *amax_k, *counter;
-  uint8_t *fixed;
-  size_t fixed_bytes;
-  int slices;
-  size_t bytes;
-};
-
-// amax words of both tensors, a counter per (batch element, 256-column group) and the launch counter
+// Workspace of the statistics pass: S slices of per-column partial results (FP64 sum, maximum and minimum), and the heads'
+// maxima.  S is the largest slice count <= STAT_MAX_SLICES that fits the bytes the caller gave (at least 1).
+constexpr int STAT_MAX_SLICES = 32;
 size_t stats_fixed_bytes(int B, int H_q, int H_kv) {
   return align256(((size_t)2 * B + (size_t)B * ((H_q + 1) / 2 + (H_kv + 1) / 2) + 1) * sizeof(unsigned int));
 }
@@ -754,71 +782,39 @@ size_t stats_slice_bytes(int B, int H_q, int H_kv) {   // one slice of both tens
          align256((size_t)B * H_kv * HEAD_DIM * 8) + 2 * align256((size_t)B * H_kv * HEAD_DIM * 4);
 }
 
+struct StatsWorkspace {
+  double *psum_q, *psum_k;
+  float2 *pext_q, *pext_k;
+  float *gmax_q, *gmax_k;
+  int slices;   // 0: too small
+};
 StatsWorkspace carve(void *ws, size_t ws_bytes, int B, int H_q, int H_kv) {
   StatsWorkspace w{};
   const size_t fixed = stats_fixed_bytes(B, H_q, H_kv), per = stats_slice_bytes(B, H_q, H_kv);
-  size_t S = ws_bytes > fixed ? (ws_bytes - fixed) / per : 0;
-  if (S > (size_t)STAT_MAX_SLICES) S = STAT_MAX_SLICES;
-  w.slices = (int)S;
-  size_t o = 0;
-  uint8_t *base = static_cast<uint8_t *>(ws);
-  const size_t nq = (size_t)B * H_q * HEAD_DIM, nk = (size_t)B * H_kv * HEAD_DIM;
-  w.psum_q = reinterpret_cast<double *>(base + o);  o += S * align256(nq * 8);
-  w.psum_k = reinterpret_cast<double *>(base + o);  o += S * align256(nk * 8);
-  w.pmax_q = reinterpret_cast<float *>(base + o);   o += S * align256(nq * 4);
-  w.pneg_q = reinterpret_cast<float *>(base + o);   o += S * align256(nq * 4);
-  w.pmax_k = reinterpret_cast<float *>(base + o);   o += S * align256(nk * 4);
-  w.pneg_k = reinterpret_cast<float *>(base + o);   o += S * align256(nk * 4);
-  w.fixed = base + o;                                      // zeroed before every statistics launch
-  w.fixed_bytes = fixed;
-  w.amax_q = reinterpret_cast<unsigned int *>(base + o);
-  w.amax_k = w.amax_q + B;
-  w.counter = w.amax_k + B;
-  o += fixed;
-  w.bytes = o;
+  const int S = ws_bytes > fixed ? (int)std::min((ws_bytes - fixed) / per, (size_t)STAT_MAX_SLICES) : 0;
+  // The maxima take the place of one slice.  A pass with a single slice writes no partial results.
+  const size_t nq = (size_t)B * H_q, nk = (size_t)B * H_kv, n = S > 1 ? S - 1 : 0;
+  w.slices = S > 2 ? (int)n : std::min(S, 1);
+  w.gmax_q = static_cast<float *>(ws);
+  w.gmax_k = w.gmax_q + nq;
+  uint8_t *p = static_cast<uint8_t *>(ws) + per;
+  w.psum_q = reinterpret_cast<double *>(p);  p += n * nq * HEAD_DIM * 8;
+  w.psum_k = reinterpret_cast<double *>(p);  p += n * nk * HEAD_DIM * 8;
+  w.pext_q = reinterpret_cast<float2 *>(p);  p += n * nq * HEAD_DIM * 8;
+  w.pext_k = reinterpret_cast<float2 *>(p);
   return w;
 }
 
-// One tensor [B, N, H, 128] of a statistics pass (x == nullptr: absent).
-struct StatsJob {
-  const __nv_bfloat16 *x;
-  int N, H;
-  double *psum;
-  float *pmax, *pneg;
-  unsigned int *amax;
-  float *mean, *gscale;
-};
-
-// Means and per-tensor scales of up to two tensors: one pass over the data, one memory-set node (the amax words
-// and counters) and one launch.
-mpfa_status tensor_stats(const StatsJob &j0, const StatsJob &j1, int B, const StatsWorkspace &w, bool smooth, cudaStream_t st) {
-  ColTensor c[2];
-  int slices_x = 0;
-  const StatsJob *jobs[2] = {&j0, &j1};
-  // as many slices as keep the whole launch resident at once (three 256-thread blocks per SM), within what the
-  // workspace holds
-  int dev = 0, n_sm = 0;
-  MPFA_CUDA_OK(cudaGetDevice(&dev));
-  MPFA_CUDA_OK(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
-  int groups = 0;
-  for (int i = 0; i < 2; ++i)
-    if (jobs[i]->x) groups += (jobs[i]->H * HEAD_DIM + COLSTAT_COLS - 1) / COLSTAT_COLS;
-  if (groups == 0) return MPFA_OK;
-  const int max_slices = std::min(w.slices, std::max(1, 3 * n_sm / (groups * B)));
-  for (int i = 0; i < 2; ++i) {
-    const StatsJob &j = *jobs[i];
-    const int cols = j.H * HEAD_DIM;
-    // slices of at least 256 tokens, a multiple of 8 tokens long (the eight token lanes of a CTA)
-    int S = j.x ? std::min(max_slices, std::max(1, (j.N + 255) / 256)) : 0;
-    const int len = j.x ? ((j.N + S - 1) / S + 7) / 8 * 8 : 0;
-    if (j.x) S = (j.N + len - 1) / len;
-    c[i] = ColTensor{j.x, j.x ? j.N : 0, cols, j.x ? (cols + COLSTAT_COLS - 1) / COLSTAT_COLS : 0, S, len, j.psum, j.pmax,
-                     j.pneg, j.amax, j.mean, j.gscale};
-    if (j.x) slices_x = std::max(slices_x, S);
-  }
-  MPFA_CUDA_OK(cudaMemsetAsync(w.fixed, 0, w.fixed_bytes, st));
-  colstat_kernel<<<dim3(slices_x, c[0].ygroups + c[1].ygroups, B), 256, 0, st>>>(c[0], c[1], w.counter, smooth ? 1 : 0);
-  MPFA_LAUNCH_OK();
+// Means and the heads' maxima of up to two tensors.
+mpfa_status tensor_stats(const ColTensor &c0, const ColTensor &c1, int B, int max_slices, int n_sm, bool smooth, cudaStream_t st) {
+  const int heads = c0.H + c1.H, N = std::max(c0.x ? c0.N : 0, c1.x ? c1.N : 0);
+  if (heads == 0) return MPFA_OK;
+  // As many slices as the launch can hold in one wave (three CTAs per SM).  A fold costs about as much as STAT_MIN tokens
+  // of a CTA's pass, so slices are not made shorter than that.
+  constexpr int STAT_MIN = 512;
+  const int S = (int)std::max(1LL, std::min({(long long)max_slices, 3LL * n_sm / ((long long)heads * B), (long long)N / STAT_MIN}));
+  MPFA_CUDA_OK(launch(colstat_kernel, dim3(S, heads, B), dim3(STAT_THREADS), 0, st, c0, c1, smooth ? 1 : 0));
+  if (S > 1) MPFA_CUDA_OK(launch(stat_fold_kernel, dim3(heads, B), dim3(128), 0, st, c0, c1, S, smooth ? 1 : 0));
   return MPFA_OK;
 }
 
@@ -868,33 +864,30 @@ extern "C" mpfa_status mpfa_quantize_qk(const void *q_bf16, const void *k_bf16, 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const __nv_bfloat16 *q = static_cast<const __nv_bfloat16 *>(q_bf16);
   const __nv_bfloat16 *k = static_cast<const __nv_bfloat16 *>(k_bf16);
+  int dev = 0, n_sm = 0;
+  MPFA_CUDA_OK(cudaGetDevice(&dev));
+  MPFA_CUDA_OK(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
   if (!frozen) {
-    rc = tensor_stats(StatsJob{q, N_q, H_q, w.psum_q, w.pmax_q, w.pneg_q, w.amax_q, st->q_mean, st->q_gscale},
-                      StatsJob{k, N_kv, H_kv, w.psum_k, w.pmax_k, w.pneg_k, w.amax_k, st->k_mean, st->k_gscale}, B, w, smooth, s);
+    rc = tensor_stats(ColTensor{q, N_q, q ? H_q : 0, w.psum_q, w.pext_q, st->q_mean, w.gmax_q},
+                      ColTensor{k, N_kv, k ? H_kv : 0, w.psum_k, w.pext_k, st->k_mean, w.gmax_k}, B, w.slices, n_sm, smooth, s);
     if (rc != MPFA_OK) return rc;
   }
-  {
-    // Q and K tiles in one launch
-    QuantTensor tq{q, st->q_mean, st->q_gscale, N_q, q ? H_q : 0, q ? pad128(N_q) / TILE : 0, q ? q_out->codes : nullptr,
-                   q ? q_out->sf : nullptr};
-    QuantTensor tk{k, st->k_mean, st->k_gscale, N_kv, k ? H_kv : 0, k ? pad128(N_kv) / TILE : 0,
-                   k ? k_out->codes : nullptr, k ? k_out->sf : nullptr};
-    // with smoothing the K tiles also produce Delta_S (Eq. 9) from the rows they have staged (no third pass over
-    // K), in a launch of their own
-    const bool with_delta = k && smooth;
-    if (with_delta) {
-      DeltaArgs da{st->q_mean, st->q_gscale, static_cast<__nv_bfloat16 *>(delta_s_bf16), H_q};
-      MPFA_CUDA_OK(cudaFuncSetAttribute(quantize_k_delta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)KTILE_SMEM));
-      quantize_k_delta_kernel<<<dim3(tk.tiles * tk.H, 1, B), 256, KTILE_SMEM, s>>>(tk, da);
-      MPFA_LAUNCH_OK();
-      tk.H = 0;
-      tk.tiles = 0;
-    }
-    if (tq.H + tk.H > 0) {
-      quantize_fp4_tile_kernel<<<dim3(std::max(tq.tiles, tk.tiles) * (tq.H + tk.H), 1, B), 256, 0, s>>>(tq, tk);
-      MPFA_LAUNCH_OK();
-    }
+  // Q and K tiles in one launch; with smoothing the K tiles also produce Delta_S (Eq. 9)
+  const TensorScale sq{st->q_gscale, frozen ? nullptr : w.gmax_q, H_q}, sk{st->k_gscale, frozen ? nullptr : w.gmax_k, H_kv};
+  QuantTensor tq{q, st->q_mean, sq, N_q, q ? H_q : 0, q ? pad128(N_q) / TILE : 0, 0, q ? q_out->codes : nullptr, q ? q_out->sf : nullptr};
+  QuantTensor tk{k, st->k_mean, sk, N_kv, k ? H_kv : 0, k ? pad128(N_kv) / TILE : 0, 0, k ? k_out->codes : nullptr, k ? k_out->sf : nullptr};
+  const DeltaArgs da{st->q_mean, sq, k && smooth ? static_cast<__nv_bfloat16 *>(delta_s_bf16) : nullptr, H_q};
+  if (!k && N_q <= 8) {
+    MPFA_CUDA_OK(launch(quantize_token_kernel, dim3((B * H_q + 7) / 8), dim3(256), 0, s, tq, B * H_q));
+    return MPFA_OK;
   }
+  // One wave of CTAs where that leaves a CTA several tiles: its set-up (scale, table of reciprocals, query means) is then
+  // paid once, and the next tile's loads run under the arithmetic of the current one.
+  const long long tiles = ((long long)tk.tiles * tk.H + (long long)tq.tiles * tq.H) * B, wave = (long long)QT_CTAS * n_sm;
+  const int per_cta = (int)((tiles + wave - 1) / wave);
+  tk.ctas = tk.x ? (tk.tiles + per_cta - 1) / per_cta : 0;
+  tq.ctas = tq.x ? (tq.tiles + per_cta - 1) / per_cta : 0;
+  MPFA_CUDA_OK(launch(quantize_tile_kernel, dim3(tk.ctas * tk.H + tq.ctas * tq.H, 1, B), dim3(256), 0, s, tk, tq, da));
   return MPFA_OK;
 }
 
@@ -905,9 +898,8 @@ extern "C" mpfa_status mpfa_quantize_v(const void *v_bf16, int B, int N_kv, int 
   mpfa_status rc = check_arch();
   if (rc != MPFA_OK) return rc;
   dim3 grid(pad128(N_kv) / TILE, H_kv, B);
-  quantize_v_tile_kernel<<<grid, 256, 0, static_cast<cudaStream_t>(stream)>>>(
-      static_cast<const __nv_bfloat16 *>(v_bf16), N_kv, H_kv, 1.0f / v_scale, v_fp8);
-  MPFA_LAUNCH_OK();
+  MPFA_CUDA_OK(launch(quantize_v_tile_kernel, grid, dim3(256), 0, static_cast<cudaStream_t>(stream),
+                      static_cast<const __nv_bfloat16 *>(v_bf16), N_kv, H_kv, 1.0f / v_scale, v_fp8));
   return MPFA_OK;
 }
 
@@ -969,33 +961,20 @@ extern "C" mpfa_status mpfa_quantize_kv_paged(const void *k_bf16, const void *v_
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const __nv_bfloat16 *k = static_cast<const __nv_bfloat16 *>(k_bf16);
   const __nv_bfloat16 *v = static_cast<const __nv_bfloat16 *>(v_bf16);
+  int dev = 0, n_sm = 0;
+  MPFA_CUDA_OK(cudaGetDevice(&dev));
+  MPFA_CUDA_OK(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
   if (!frozen) {
-    rc = tensor_stats(StatsJob{k, N_tokens, H_kv, w.psum_k, w.pmax_k, w.pneg_k, w.amax_k, st->k_mean, st->k_gscale},
-                      StatsJob{nullptr, 0, 0, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr}, 1, w, smooth, s);
+    rc = tensor_stats(ColTensor{k, N_tokens, H_kv, w.psum_k, w.pext_k, st->k_mean, w.gmax_k}, ColTensor{}, 1, w.slices, n_sm, smooth, s);
     if (rc != MPFA_OK) return rc;
   }
-  if (first_token % PAGE != 0) {
-    // append into a partly filled page (frozen statistics; checked above): slot-granular kernel
-    const int last_page_end = (first_token + N_tokens + PAGE - 1) / PAGE * PAGE;
-    const int n_slots = last_page_end - first_token;
-    append_kv_kernel<<<dim3((n_slots + 31) / 32, H_kv), 256, 0, s>>>(
-        k, v, st->q_mean, st->k_mean, st->q_gscale, st->k_gscale, N_tokens, first_token, H_q, H_kv, 1.0f / v_scale,
-        smooth ? 1 : 0, page_table_row, kv->num_pages, kv->k_codes, kv->k_sf, kv->v_fp8,
-        static_cast<__nv_bfloat16 *>(kv->delta_s_bf16), nullptr, 0);
-    MPFA_LAUNCH_OK();
-    return MPFA_OK;
-  }
-  const int n_pages = (N_tokens + PAGE - 1) / PAGE;
-  quantize_kv_page_kernel<<<dim3(n_pages, H_kv), 256, 0, s>>>(k, v, st->k_mean, st->k_gscale, N_tokens, H_kv,
-                                                              1.0f / v_scale, page_table_row, first_token / PAGE,
-                                                              kv->num_pages, kv->k_codes, kv->k_sf, kv->v_fp8);
-  MPFA_LAUNCH_OK();
-  if (smooth) {
-    delta_s_kernel<true><<<dim3(pad128(N_tokens) / TILE, H_kv, 1), 256, 0, s>>>(
-        k, st->q_mean, st->k_mean, st->q_gscale, st->k_gscale, N_tokens, H_q, H_kv,
-        static_cast<__nv_bfloat16 *>(kv->delta_s_bf16), page_table_row + first_token / PAGE, kv->num_pages);
-    MPFA_LAUNCH_OK();
-  }
+  const TensorScale sk{st->k_gscale, frozen ? nullptr : w.gmax_k, H_kv};
+  const int n_pages = (first_token + N_tokens - 1) / PAGE - first_token / PAGE + 1;
+  const long long wave = (long long)WK_CTAS * n_sm;
+  const int per_cta = (int)(((long long)n_pages * H_kv + wave - 1) / wave);
+  MPFA_CUDA_OK(launch(write_kv_kernel, dim3(H_kv, (n_pages + per_cta - 1) / per_cta), dim3(256), 0, s, k, v, st->k_mean, sk, st->q_mean,
+                      st->q_gscale, N_tokens, first_token, n_pages, H_q, H_kv, 1.0f / v_scale, page_table_row, kv->num_pages,
+                      kv->k_codes, kv->k_sf, kv->v_fp8, smooth ? static_cast<__nv_bfloat16 *>(kv->delta_s_bf16) : nullptr));
   return MPFA_OK;
 }
 
@@ -1018,12 +997,11 @@ extern "C" mpfa_status mpfa_append_kv_paged(const void *k_bf16, const void *v_bf
     return MPFA_ERR_ALIGNMENT;
   mpfa_status rc = check_arch();
   if (rc != MPFA_OK) return rc;
-  // 64 slots per request: the token's own and, when it starts a page, the 63 to be zeroed after it
-  append_kv_kernel<<<dim3(2, H_kv, B), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-      static_cast<const __nv_bfloat16 *>(k_bf16), static_cast<const __nv_bfloat16 *>(v_bf16), st->q_mean, st->k_mean,
-      st->q_gscale, st->k_gscale, 1, 0, H_q, H_kv, 1.0f / v_scale, smooth ? 1 : 0, page_table, kv->num_pages,
-      kv->k_codes, kv->k_sf, kv->v_fp8, static_cast<__nv_bfloat16 *>(kv->delta_s_bf16), positions, max_pages_per_req);
-  MPFA_LAUNCH_OK();
+  MPFA_CUDA_OK(launch(append_kv_kernel, dim3((B * H_kv + 7) / 8), dim3(256), 0, static_cast<cudaStream_t>(stream),
+                      static_cast<const __nv_bfloat16 *>(k_bf16), static_cast<const __nv_bfloat16 *>(v_bf16), st->q_mean, st->k_mean,
+                      st->q_gscale, st->k_gscale, B, H_q, H_kv, 1.0f / v_scale, page_table, max_pages_per_req, kv->num_pages,
+                      positions, kv->k_codes, kv->k_sf, kv->v_fp8,
+                      smooth ? static_cast<__nv_bfloat16 *>(kv->delta_s_bf16) : nullptr));
   return MPFA_OK;
 }
 

@@ -129,10 +129,10 @@ typedef struct {
  *   q_out / k_out: tile-layout tensors with B, H, N filled in by the caller;
  *   delta_s_bf16 [B, H_q, N_kv_pad]: required iff MPFA_SMOOTH and k_bf16 != NULL;
  *   workspace: 256-byte aligned scratch, overwritten by every call (not needed with MPFA_STATS_FROZEN).  The call
- *          enqueues one memory-set node over its first few hundred bytes (maxima and block counters) and four
- *          kernels; two calls that overlap on the GPU need separate workspaces.
+ *          enqueues up to three kernels (statistics, their fold over the token slices where there are several, tiles); two
+ *          calls that overlap on the GPU need separate workspaces.
  *          mpfa_quantize_workspace_bytes() is the size that lets the statistics pass cut the token axis into
- *          its full 32 slices; any size down to mpfa_quantize_workspace_min_bytes() (one slice) is accepted and
+ *          its full number of slices; any size down to mpfa_quantize_workspace_min_bytes() (one slice) is accepted and
  *          only lowers the parallelism of that pass; less: MPFA_ERR_WORKSPACE.
  * All arithmetic is specified step by step (FP64 column sums, one rounding to FP32, IEEE divisions).  The column
  * sums are added in a fixed order (tokens ascending within a thread, then token lanes, then slices; the order is a
@@ -163,7 +163,7 @@ mpfa_status mpfa_quantize_qk(const void *q_bf16, const void *k_bf16, int B, int 
  * nothing.  The first call on each device looks up the buffer's device address (with that
  * device current); make that first call before starting any stream capture.  All calls on
  * a device share the one buffer, which keeps whatever the previous call left in it: each
- * call clears what it needs on `stream` before use, and two calls whose GPU work overlaps
+ * call writes what it reads, on `stream`, and two calls whose GPU work overlaps
  * (different streams, or different host threads on different streams) race on it - keep
  * them on one stream or order them yourself. */
 #define MPFA_STATIC_SCRATCH_BYTES (512 * 1024)

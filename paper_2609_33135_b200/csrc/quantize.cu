@@ -46,7 +46,7 @@ __device__ __forceinline__ void unpack8(const uint4 &u, float (&f)[8]) {
 //   max_t |fl(x_t - mu)| = max(fl(max x - mu), fl(mu - min x)) and no second pass over the tensor is
 //   needed for the per-tensor scale.
 // A CTA covers one head (128 columns) x one slice of the tokens: thread = (token lane 0..15, 8 columns), eight independent
-// 16-byte loads in flight per thread; each thread adds its tokens in ascending order, the 16 token lanes are folded in lane
+// 16-byte loads in flight per thread while the eight before them are added; each thread adds its tokens in ascending order, the 16 token lanes are folded in lane
 // order in shared memory.  With one slice the CTA writes mean = fl(sum / N) (0 without smoothing) and the head's max |x - mean|
 // itself; otherwise the slices' partial results go to the workspace and stat_fold_kernel adds them in
 // slice order.  No counter, no memory to clear.  Every addition order is fixed by the shape, the workspace size
@@ -60,10 +60,11 @@ __device__ __forceinline__ void unpack8(const uint4 &u, float (&f)[8]) {
 // round as the unscaled ones do.  Infinities and NaNs would become finite; an FMA with zero catches them, and that
 // thread's slice is added again with the conversion.
 // Measured (Q and K, 32:8 heads, 16384 tokens / 1:1 heads, 256 tokens; with memory-set node or fold): with conversions, four
-// loads in flight and the last CTA of a group folding the slices 42 / 11 us, now 40 / 3.6 us.  (The slices as CTAs of a
+// loads in flight and the last CTA of a group folding the slices 42 / 11 us, now 40 / 3.6 us (4.5 TB/s).  (The slices as CTAs of a
 // cluster, folded through distributed shared memory: clusters leave some SMs empty and others full, 45 us.)
 constexpr int STAT_THREADS = 256;
-constexpr int STAT_LOADS = 8;
+constexpr int STAT_LOADS = 8;   // rows in flight per thread, and as many being added
+constexpr int STAT_CTAS = 2;    // resident per SM
 constexpr int STAT_LANES = STAT_THREADS / 16;
 
 struct ColTensor {
@@ -105,7 +106,7 @@ __device__ __forceinline__ void finish_column(const ColTensor &a, int b, int h, 
 }
 
 // grid (slices, heads of both tensors, B)
-__global__ void __launch_bounds__(STAT_THREADS, 3) colstat_kernel(const ColTensor t0, const ColTensor t1, int smooth) {
+__global__ void __launch_bounds__(STAT_THREADS, STAT_CTAS) colstat_kernel(const ColTensor t0, const ColTensor t1, int smooth) {
   __shared__ double s_sum[STAT_LANES][HEAD_DIM];
   __shared__ uint32_t s_mx[STAT_LANES][HEAD_DIM / 2], s_mn[STAT_LANES][HEAD_DIM / 2];
   __shared__ float s_w[4];
@@ -138,21 +139,34 @@ __global__ void __launch_bounds__(STAT_THREADS, 3) colstat_kernel(const ColTenso
     }
   };
   int t = begin + tl;
-  for (; t + STAT_LANES * (STAT_LOADS - 1) < end; t += STAT_LANES * STAT_LOADS, p += STAT_LOADS * step) {
-    uint4 u[STAT_LOADS];
+  // one round of loads is in flight while the previous one is added
+  const auto load = [&](uint4 (&u)[STAT_LOADS]) {
 #pragma unroll
     for (int j = 0; j < STAT_LOADS; ++j) u[j] = __ldg(reinterpret_cast<const uint4 *>(p + j * step));
+    p += STAT_LOADS * step;
+  };
+  const auto full = [&](int at) { return at + STAT_LANES * (STAT_LOADS - 1) < end; };
+  constexpr int ROUND = STAT_LANES * STAT_LOADS;
+  uint4 u0[STAT_LOADS], u1[STAT_LOADS];
+  if (full(t)) load(u0);
+  while (full(t)) {
+    if (full(t + ROUND)) load(u1);
 #pragma unroll
-    for (int j = 0; j < STAT_LOADS; ++j) add(u[j]);
+    for (int j = 0; j < STAT_LOADS; ++j) add(u0[j]);
+    t += ROUND;
+    if (!full(t)) break;
+    if (full(t + ROUND)) load(u0);
+#pragma unroll
+    for (int j = 0; j < STAT_LOADS; ++j) add(u1[j]);
+    t += ROUND;
   }
-  {   // the last fewer than STAT_LOADS rounds of this lane, still in flight together
-    uint4 u[STAT_LOADS - 1];
+  {   // the last fewer than STAT_LOADS rows of this lane, still in flight together
 #pragma unroll
     for (int j = 0; j < STAT_LOADS - 1; ++j)
-      if (t + STAT_LANES * j < end) u[j] = __ldg(reinterpret_cast<const uint4 *>(p + j * step));
+      if (t + STAT_LANES * j < end) u0[j] = __ldg(reinterpret_cast<const uint4 *>(p + j * step));
 #pragma unroll
     for (int j = 0; j < STAT_LOADS - 1; ++j)
-      if (t + STAT_LANES * j < end) add(u[j]);
+      if (t + STAT_LANES * j < end) add(u0[j]);
   }
 #pragma unroll
   for (int i = 0; i < 8; ++i) acc[i] *= 0x1p896;
@@ -328,23 +342,36 @@ __device__ __forceinline__ void quantize_block16(const float (&xc)[16], const Bl
   codes = make_uint2(e2m1x8(y, 0), e2m1x8(y, 8));
 }
 
-// 16 channels of one row (16-byte aligned: the interface asks for no more, a single 32-byte load would)
+// 16 channels of one row.  Two 16-byte loads touch each 32-byte sector twice; tensors that are 32-byte aligned (the interface
+// asks for 16) are read with one load.
 struct Row16 { uint4 a, b; };
-__device__ __forceinline__ Row16 load_row16(const __nv_bfloat16 *p) {
-  const uint4 *u = reinterpret_cast<const uint4 *>(p);
-  return Row16{__ldg(u), __ldg(u + 1)};
+__device__ __forceinline__ Row16 load_row16(const __nv_bfloat16 *p, bool wide) {
+  Row16 r;
+  if (wide) {
+    asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(r.a.x), "=r"(r.a.y), "=r"(r.a.z), "=r"(r.a.w), "=r"(r.b.x), "=r"(r.b.y), "=r"(r.b.z), "=r"(r.b.w)
+                 : "l"(p));
+  } else {
+    const uint4 *u = reinterpret_cast<const uint4 *>(p);
+    r.a = __ldg(u), r.b = __ldg(u + 1);
+  }
+  return r;
 }
-// x - mean of 16 channels; mean: 16-byte aligned
-__device__ __forceinline__ void center16(const Row16 &x, const float *mean, float (&xc)[16]) {
+__device__ __forceinline__ bool wide_rows(const void *x) { return (reinterpret_cast<uintptr_t>(x) & 31) == 0; }
+// means of 16 channels, negated; 16-byte aligned
+__device__ __forceinline__ void load_neg_mean(const float *mean, float (&nm)[16]) {
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    const float4 m = __ldg(reinterpret_cast<const float4 *>(mean) + c);
+    nm[4 * c] = -m.x, nm[4 * c + 1] = -m.y, nm[4 * c + 2] = -m.z, nm[4 * c + 3] = -m.w;
+  }
+}
+__device__ __forceinline__ void center16(const Row16 &x, const float (&nm)[16], float (&xc)[16]) {
   float f[16];
   unpack8(x.a, reinterpret_cast<float(&)[8]>(f[0]));
   unpack8(x.b, reinterpret_cast<float(&)[8]>(f[8]));
 #pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    const float4 m = reinterpret_cast<const float4 *>(mean)[c];
-    add2(xc[4 * c], xc[4 * c + 1], f[4 * c], f[4 * c + 1], -m.x, -m.y);
-    add2(xc[4 * c + 2], xc[4 * c + 3], f[4 * c + 2], f[4 * c + 3], -m.z, -m.w);
-  }
+  for (int i = 0; i < 16; i += 2) add2(xc[i], xc[i + 1], f[i], f[i + 1], nm[i], nm[i + 1]);
 }
 
 // Compensation vector (Eq. 9): Delta_S[hq][t] = qmean[hq] . (k[t] - kmean) in FP64, in units of gscale_q * gscale_k, rounded once
@@ -399,11 +426,11 @@ struct DeltaArgs {
 // to memory (partial sectors merge in L2).
 // Measured (16384 tokens, 32:8 heads, K with Delta_S and Q): two launches, rows of K staged in shared memory, two
 // divisions per block 35 + 38 us; one launch, one tile per CTA 61; with a ring of asynchronous copies and a barrier per tile 87;
-// now TILE_NEW us.
-constexpr int QT_CTAS = 3;   // resident per SM
+// now 45 us.
+constexpr int QT_CTAS = 2;       // resident per SM: 128 registers, so that the means stay in registers
+constexpr int QT_K_WEIGHT = 2;   // time of a K tile with Delta_S in units of a Q tile's (1 / 2 / 3: 106 / 89 / 96 us of stage 1)
 __global__ void __launch_bounds__(256, QT_CTAS) quantize_tile_kernel(const QuantTensor k, const QuantTensor q, const DeltaArgs da) {
   __shared__ __align__(16) GroupMeans gm;
-  __shared__ __align__(16) float s_mean[HEAD_DIM];
   __shared__ float inv_table[128];
   launch_dependents();
   grid_dependency_wait();
@@ -417,6 +444,7 @@ __global__ void __launch_bounds__(256, QT_CTAS) quantize_tile_kernel(const Quant
   const size_t head = (size_t)b * a.H + h, row = (size_t)a.H * HEAD_DIM;
   const __nv_bfloat16 *const x0 = a.x + (size_t)b * N * row + h * HEAD_DIM + j * 16;
   const int r0 = warp * 8 + (lane >> 2);
+  const bool wide = wide_rows(a.x);
   Row16 raw[2][2];
 #pragma unroll
   for (int it = 0; it < 2; ++it) {
@@ -424,13 +452,15 @@ __global__ void __launch_bounds__(256, QT_CTAS) quantize_tile_kernel(const Quant
 #pragma unroll
     for (int half = 0; half < 2; ++half) {
       raw[it][half] = Row16{};
-      if (t < N) raw[it][half] = load_row16(x0 + t * row + half * 64);
+      if (t < N) raw[it][half] = load_row16(x0 + t * row + half * 64, wide);
     }
   }
   const float d = tensor_scale(a.scale, b, lane);
   if (at == 0 && tid == 0 && a.scale.gmax) a.scale.gscale[b] = d;
   const BlockScale bs = make_block_scale(d, inv_table, tid);
-  if (tid >= 128) s_mean[tid - 128] = a.mean[head * HEAD_DIM + tid - 128];
+  float neg_mean[2][16];
+  load_neg_mean(a.mean + head * HEAD_DIM + j * 16, neg_mean[0]);
+  load_neg_mean(a.mean + head * HEAD_DIM + 64 + j * 16, neg_mean[1]);
   const bool with_delta = is_k && da.delta;
   const int G = with_delta ? da.H_q / a.H : 0;
   double unit = 0.0;
@@ -450,8 +480,8 @@ __global__ void __launch_bounds__(256, QT_CTAS) quantize_tile_kernel(const Quant
 #pragma unroll
       for (int half = 0; half < 2; ++half) {
         float xc[16];
-        center16(raw[it][half], s_mean + half * 64 + j * 16, xc);
-        if (tile >= ctas) raw[it][half] = load_row16(x0 + (size_t)(t - ctas * TILE) * row + half * 64);   // a whole tile: only the last has an end
+        center16(raw[it][half], neg_mean[half], xc);
+        if (tile >= ctas) raw[it][half] = load_row16(x0 + (size_t)(t - ctas * TILE) * row + half * 64, wide);   // a whole tile: only the last has an end
         uint2 c = make_uint2(0u, 0u);
         uint32_t sc = 0u;
         if (t < N) quantize_block16(xc, bs, sc, c);
@@ -485,9 +515,10 @@ __global__ void __launch_bounds__(256) quantize_token_kernel(const QuantTensor q
   const int b = head / q.H, h = head % q.H;
   const bool in = r < q.N;
   Row16 raw[2] = {};
+  const bool wide = wide_rows(q.x);
 #pragma unroll
   for (int half = 0; half < 2; ++half)
-    if (in) raw[half] = load_row16(q.x + (((size_t)b * q.N + r) * q.H + h) * HEAD_DIM + (half * 4 + j) * 16);
+    if (in) raw[half] = load_row16(q.x + (((size_t)b * q.N + r) * q.H + h) * HEAD_DIM + (half * 4 + j) * 16, wide);
   const float d = tensor_scale(q.scale, b, lane);
   if (h == 0 && lane == 0 && q.scale.gmax) q.scale.gscale[b] = d;
   uint8_t *const codes = q.codes + (size_t)head * TILE * 64, *const sf = q.sf + (size_t)head * 1024;
@@ -497,8 +528,9 @@ __global__ void __launch_bounds__(256) quantize_token_kernel(const QuantTensor q
     if ((i & 31) >= 8) reinterpret_cast<uint4 *>(sf)[i] = z;   // 16 bytes per row of the atom: rows 8..31 of both halves
 #pragma unroll
   for (int half = 0; half < 2; ++half) {
-    float xc[16];
-    center16(raw[half], q.mean + (size_t)head * HEAD_DIM + (half * 4 + j) * 16, xc);
+    float xc[16], neg_mean[16];
+    load_neg_mean(q.mean + (size_t)head * HEAD_DIM + (half * 4 + j) * 16, neg_mean);
+    center16(raw[half], neg_mean, xc);
     uint8_t s8 = 0;
     uint2 c = make_uint2(0u, 0u);
     if (in) quantize_block16(xc, d, s8, c);
@@ -534,13 +566,14 @@ __global__ void __launch_bounds__(256) quantize_v_tile_kernel(const __nv_bfloat1
   grid_dependency_wait();
   const int tile = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
   const int n_pad = gridDim.x * TILE;
+  const bool wide = wide_rows(v);
 #pragma unroll
   for (int it = 0; it < 4; ++it) {
     const int id = it * 256 + threadIdx.x;
     const int r = id >> 3, seg = id & 7;
     const int t = tile * TILE + r;
     uint4 c = make_uint4(0u, 0u, 0u, 0u);
-    if (t < N) c = quantize_v16(load_row16(v + (((size_t)b * N + t) * H + h) * HEAD_DIM + seg * 16), inv_scale);
+    if (t < N) c = quantize_v16(load_row16(v + (((size_t)b * N + t) * H + h) * HEAD_DIM + seg * 16, wide), inv_scale);
     *reinterpret_cast<uint4 *>(out + (((size_t)b * H + h) * n_pad + t) * HEAD_DIM + seg * 16) = c;
   }
 }
@@ -612,8 +645,8 @@ __global__ void __launch_bounds__(256) quantize_v_fp4_tile_kernel(const __nv_bfl
 // requested while the current ones are quantized.  Slots past the last token are zero-filled in pages that the call
 // starts (a recycled page may hold anything, and decode needs finite bytes there); slots of earlier tokens are left alone.
 // Measured (9001 tokens, 32:8 heads): page kernel + a Delta_S kernel that read K again 12 + 16 us, one page per CTA 19.5 us, now
-// PAGE_NEW us.
-constexpr int WK_CTAS = 3;   // resident per SM
+// 14.1 us.
+constexpr int WK_CTAS = 2;   // resident per SM: 128 registers, so that the means stay in registers
 __global__ void __launch_bounds__(256, WK_CTAS) write_kv_kernel(const __nv_bfloat16 *__restrict__ k, const __nv_bfloat16 *__restrict__ v,
                                                                 const float *__restrict__ k_mean, const TensorScale k_scale,
                                                                 const float *__restrict__ q_mean, const float *__restrict__ q_gscale,
@@ -622,13 +655,13 @@ __global__ void __launch_bounds__(256, WK_CTAS) write_kv_kernel(const __nv_bfloa
                                                                 uint8_t *__restrict__ k_codes, uint8_t *__restrict__ k_sf,
                                                                 uint8_t *__restrict__ v_fp8, __nv_bfloat16 *__restrict__ delta) {
   __shared__ __align__(16) GroupMeans gm;
-  __shared__ __align__(16) float s_mean[HEAD_DIM];
   __shared__ float inv_table[128];
   launch_dependents();
   grid_dependency_wait();
   const int tid = threadIdx.x, lane = tid & 31, j = lane & 3, h = blockIdx.x, G = H_q / H_kv;
   const int t = (tid >> 5) * 8 + (lane >> 2);   // slot of the page
   const int page0 = first / PAGE;               // first page of the request that is touched
+  const bool wide_k = wide_rows(k), wide_v = wide_rows(v);
   Row16 kr[2], vr[2];
   int pg = blockIdx.y, page;
   const auto fetch = [&](int half) {
@@ -636,8 +669,8 @@ __global__ void __launch_bounds__(256, WK_CTAS) write_kv_kernel(const __nv_bfloa
     kr[half] = vr[half] = Row16{};
     if (pg < n_pages && i >= 0 && i < N) {
       const size_t at = ((size_t)i * H_kv + h) * HEAD_DIM + (half * 4 + j) * 16;
-      kr[half] = load_row16(k + at);
-      vr[half] = load_row16(v + at);
+      kr[half] = load_row16(k + at, wide_k);
+      vr[half] = load_row16(v + at, wide_v);
     }
   };
   fetch(0);
@@ -646,7 +679,9 @@ __global__ void __launch_bounds__(256, WK_CTAS) write_kv_kernel(const __nv_bfloa
   const float d = tensor_scale(k_scale, 0, lane);
   if (blockIdx.y == 0 && h == 0 && tid == 0 && k_scale.gmax) k_scale.gscale[0] = d;
   const BlockScale bs = make_block_scale(d, inv_table, tid);
-  if (tid >= 128) s_mean[tid - 128] = k_mean[(size_t)h * HEAD_DIM + tid - 128];
+  float neg_mean[2][16];
+  load_neg_mean(k_mean + (size_t)h * HEAD_DIM + j * 16, neg_mean[0]);
+  load_neg_mean(k_mean + (size_t)h * HEAD_DIM + 64 + j * 16, neg_mean[1]);
   double unit = 0.0;
   if (delta) {
     convert_group_means(gm, q_mean + (size_t)h * G * HEAD_DIM, G, tid, 256);
@@ -668,7 +703,7 @@ __global__ void __launch_bounds__(256, WK_CTAS) write_kv_kernel(const __nv_bfloa
     for (int half = 0; half < 2; ++half) {
       const int blk = half * 4 + j;
       float xc[16];
-      center16(kr[half], s_mean + blk * 16, xc);
+      center16(kr[half], neg_mean[half], xc);
       uint2 c = make_uint2(0u, 0u);
       uint32_t sc = 0u;
       uint4 vc = quantize_v16(vr[half], inv_vscale);
@@ -717,11 +752,13 @@ __global__ void __launch_bounds__(256) append_kv_kernel(const __nv_bfloat16 *__r
   if (pair >= B * H_kv) return;
   const int b = pair / H_kv, h = pair % H_kv, G = H_q / H_kv;
   const int pos = positions[b];
-  const Row16 kr = load_row16(k + (size_t)pair * HEAD_DIM + blk * 16), vr = load_row16(v + (size_t)pair * HEAD_DIM + blk * 16);
+  const Row16 kr = load_row16(k + (size_t)pair * HEAD_DIM + blk * 16, wide_rows(k));
+  const Row16 vr = load_row16(v + (size_t)pair * HEAD_DIM + blk * 16, wide_rows(v));
   const float d = k_gscale[b];
   const double denom = delta ? (double)q_gscale[b] * (double)d : 1.0;
-  float xc[16];
-  center16(kr, k_mean + (size_t)pair * HEAD_DIM + blk * 16, xc);
+  float xc[16], neg_mean[16];
+  load_neg_mean(k_mean + (size_t)pair * HEAD_DIM + blk * 16, neg_mean);
+  center16(kr, neg_mean, xc);
   const bool in_table = pos >= 0 && (pos >> 6) < max_pages;   // else: skipped, or no page-table entry for that position
   const int page = in_table ? page_table[(size_t)b * max_pages + (pos >> 6)] : -1;
   const int t = pos & 63;
@@ -809,10 +846,10 @@ StatsWorkspace carve(void *ws, size_t ws_bytes, int B, int H_q, int H_kv) {
 mpfa_status tensor_stats(const ColTensor &c0, const ColTensor &c1, int B, int max_slices, int n_sm, bool smooth, cudaStream_t st) {
   const int heads = c0.H + c1.H, N = std::max(c0.x ? c0.N : 0, c1.x ? c1.N : 0);
   if (heads == 0) return MPFA_OK;
-  // As many slices as the launch can hold in one wave (three CTAs per SM).  A fold costs about as much as STAT_MIN tokens
+  // As many slices as the launch can hold in one wave.  A fold costs about as much as STAT_MIN tokens
   // of a CTA's pass, so slices are not made shorter than that.
   constexpr int STAT_MIN = 512;
-  const int S = (int)std::max(1LL, std::min({(long long)max_slices, 3LL * n_sm / ((long long)heads * B), (long long)N / STAT_MIN}));
+  const int S = (int)std::max(1LL, std::min({(long long)max_slices, (long long)STAT_CTAS * n_sm / ((long long)heads * B), (long long)N / STAT_MIN}));
   MPFA_CUDA_OK(launch(colstat_kernel, dim3(S, heads, B), dim3(STAT_THREADS), 0, st, c0, c1, smooth ? 1 : 0));
   if (S > 1) MPFA_CUDA_OK(launch(stat_fold_kernel, dim3(heads, B), dim3(128), 0, st, c0, c1, S, smooth ? 1 : 0));
   return MPFA_OK;
@@ -881,12 +918,16 @@ extern "C" mpfa_status mpfa_quantize_qk(const void *q_bf16, const void *k_bf16, 
     MPFA_CUDA_OK(launch(quantize_token_kernel, dim3((B * H_q + 7) / 8), dim3(256), 0, s, tq, B * H_q));
     return MPFA_OK;
   }
-  // One wave of CTAs where that leaves a CTA several tiles: its set-up (scale, table of reciprocals, query means) is then
-  // paid once, and the next tile's loads run under the arithmetic of the current one.
-  const long long tiles = ((long long)tk.tiles * tk.H + (long long)tq.tiles * tq.H) * B, wave = (long long)QT_CTAS * n_sm;
-  const int per_cta = (int)((tiles + wave - 1) / wave);
-  tk.ctas = tk.x ? (tk.tiles + per_cta - 1) / per_cta : 0;
-  tq.ctas = tq.x ? (tq.tiles + per_cta - 1) / per_cta : 0;
+  // At most one wave of CTAs, as far as that goes: a CTA's set-up (scale, table of reciprocals, query means) is paid once, and
+  // the next tile's loads run under the arithmetic of the current one.  A few CTAs more than a wave would take twice the time.
+  const int k_weight = da.delta ? QT_K_WEIGHT : 1;
+  const long long work = ((long long)k_weight * tk.tiles * tk.H + (long long)tq.tiles * tq.H) * B, wave = (long long)QT_CTAS * n_sm;
+  for (long long per = (work + wave - 1) / wave;; ++per) {
+    const int per_q = (int)per, per_k = (int)((per + k_weight - 1) / k_weight);
+    tk.ctas = tk.x ? (tk.tiles + per_k - 1) / per_k : 0;
+    tq.ctas = tq.x ? (tq.tiles + per_q - 1) / per_q : 0;
+    if (((long long)tk.ctas * tk.H + (long long)tq.ctas * tq.H) * B <= wave || (tk.ctas <= 1 && tq.ctas <= 1)) break;
+  }
   MPFA_CUDA_OK(launch(quantize_tile_kernel, dim3(tk.ctas * tk.H + tq.ctas * tq.H, 1, B), dim3(256), 0, s, tk, tq, da));
   return MPFA_OK;
 }

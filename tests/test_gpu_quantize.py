@@ -58,6 +58,45 @@ def test_stage1_bit_exact(name):
     check_stage1(w, run_stage1_gpu(w), z)
 
 
+@pytest.mark.parametrize("B,N,N_q,H_q,H_kv", [
+    (1, 1, 1, 1, 1), (1, 129, 7, 3, 1), (2, 127, 9, 2, 2), (1, 128, 128, 8, 1),   # smallest, few query rows, one tile
+    (1, 1024, 1024, 12, 2), (1, 1031, 1500, 7, 1),                                  # statistics in two slices, groups of six and seven
+    (1, 4099, 4099, 40, 8), (3, 2500, 700, 32, 8),                                  # several tiles per CTA, ragged last tile
+])
+def test_stage1_bit_exact_over_tile_and_slice_counts(B, N, N_q, H_q, H_kv):
+    w = wl.prefill_workload("edges", 44, B, N, H_q, H_kv, True, N_q=N_q, q_bias=True)
+    z = orc.stage1(orc.bf16_bits(w.q), orc.bf16_bits(w.k), orc.bf16_bits(w.v))
+    check_stage1(w, run_stage1_gpu(w), z)
+
+
+def test_stage1_from_inputs_on_16_byte_boundaries():
+    """The interface asks for 16-byte alignment; 32-byte aligned inputs take wider loads."""
+    from paper_2609_33135_b200 import binding
+    w = _cases()["ragged_gqa"]()
+    z = orc.stage1(orc.bf16_bits(w.q), orc.bf16_bits(w.k), orc.bf16_bits(w.v))
+
+    def shifted(x):
+        raw = torch.empty(x.numel() + 8, dtype=x.dtype, device="cuda")
+        y = raw[8:].view(x.shape).copy_(x)
+        assert y.data_ptr() % 32 == 16
+        return y
+    check_stage1(w, binding.stage1(shifted(w.q), shifted(w.k), shifted(w.v)), z)
+
+
+def test_means_of_columns_with_non_finite_values():
+    """The statistics add bit patterns of finite values; a column that holds an infinity or a NaN still gets the mean that a
+    plain sum gives, and its neighbours theirs."""
+    from paper_2609_33135_b200 import binding
+    w = wl.prefill_workload("inf", 45, 1, 700, 2, 1, True)
+    ref = run_stage1_gpu(w).stats.q_mean.clone()
+    q = w.q.clone()
+    q[0, 5, 0, 3], q[0, 600, 0, 4], q[0, 9, 1, 100], q[0, 10, 1, 100] = float("inf"), float("nan"), float("inf"), float("-inf")
+    m = binding.stage1(q.cuda(), w.k.cuda(), w.v.cuda()).stats.q_mean.cpu()[0]
+    assert m[0, 3] == float("inf") and torch.isnan(m[0, 4]) and torch.isnan(m[1, 100])
+    m[0, 3], m[0, 4], m[1, 100] = ref[0, 0, 3], ref[0, 0, 4], ref[0, 1, 100]
+    assert torch.equal(m, ref.cpu()[0])
+
+
 def test_stage1_direct_variant_and_v_scale():
     w = _cases()["ragged_gqa"]()
     z = orc.stage1(orc.bf16_bits(w.q), orc.bf16_bits(w.k), orc.bf16_bits(w.v), smooth=False, v_scale=0.5)

@@ -131,12 +131,17 @@ def _check(rc: int, what: str) -> None:
         raise MpfaError(f"{what}: {msg} (status {rc}, cuda error {L.mpfa_last_cuda_error()})")
 
 
-def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
+    return None if t is None else t.data_ptr()
 
 
-def _stream() -> ctypes.c_void_p:
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+# The raw handle of torch's current stream: the same as torch.cuda.current_stream().cuda_stream without building a Stream
+# object (3.4 us a call, as much as a launch).
+_raw_stream, _device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+
+
+def _stream() -> int:
+    return _raw_stream(_device())
 
 
 def _pad128(n: int) -> int:

@@ -1,6 +1,7 @@
 // Host-side helpers shared by the C-ABI entry points: status codes, argument checks,
 // last-error bookkeeping.  No device code.
 #pragma once
+#include <atomic>
 #include <cstddef>
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -55,7 +56,19 @@ cudaError_t launch(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
-// The kernels use sm_100a-only instructions; refuse other devices up front.
-mpfa_status check_arch();
+// The current device and its SM count; MPFA_ERR_ARCH for devices that cannot run the sm_100a-only kernels.  The facts are
+// asked for once per device (two attribute queries cost as much host time as a third of a launch).
+mpfa_status device_info(int *dev, int *n_sm);
+
+// Lets a kernel use `bytes` of dynamic shared memory; the driver is told once per kernel and device.
+constexpr int MAX_DEVICES = 64;
+template <auto Kernel>
+mpfa_status allow_smem(int dev, size_t bytes) {
+  static std::atomic<bool> done[MAX_DEVICES];
+  if (dev < MAX_DEVICES && done[dev].load(std::memory_order_acquire)) return MPFA_OK;
+  MPFA_CUDA_OK(cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+  if (dev < MAX_DEVICES) done[dev].store(true, std::memory_order_release);
+  return MPFA_OK;
+}
 
 }  // namespace mpfa

@@ -902,11 +902,9 @@ extern "C" mpfa_status mpfa_decode(const mpfa_fp4_tensor *q, const mpfa_paged_kv
   if (!aligned(q->codes, 16) || !aligned(q->sf, 16) || !aligned(kv->k_codes, 256) || !aligned(kv->k_sf, 256) ||
       !aligned(kv->v_fp8, 256) || !aligned(kv->delta_s_bf16, 256) || !aligned(workspace, 16))
     return MPFA_ERR_ALIGNMENT;
-  mpfa_status rc = check_arch();
-  if (rc != MPFA_OK) return rc;
   int dev = 0, n_sm = 0;
-  MPFA_CUDA_OK(cudaGetDevice(&dev));
-  MPFA_CUDA_OK(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
+  mpfa_status rc = device_info(&dev, &n_sm);
+  if (rc != MPFA_OK) return rc;
   DecodeParams p;
   p.q_codes = q->codes;
   p.q_sf = q->sf;
@@ -937,17 +935,17 @@ extern "C" mpfa_status mpfa_decode(const mpfa_fp4_tensor *q, const mpfa_paged_kv
   const unsigned grid = (unsigned)(items < (size_t)n_sm ? items : (size_t)n_sm);   // one persistent CTA per SM
   void (*kern)(const DecodeParams) = nullptr;
   switch (H_q / H_kv) {
-    case 1: kern = decode_split_kernel<1>; break;
-    case 2: kern = decode_split_kernel<2>; break;
-    case 3: kern = decode_split_kernel<3>; break;
-    case 4: kern = decode_split_kernel<4>; break;
-    case 5: kern = decode_split_kernel<5>; break;
-    case 6: kern = decode_split_kernel<6>; break;
-    case 7: kern = decode_split_kernel<7>; break;
-    case 8: kern = decode_split_kernel<8>; break;
+    case 1: kern = decode_split_kernel<1>, rc = allow_smem<decode_split_kernel<1>>(dev, D_SMEM); break;
+    case 2: kern = decode_split_kernel<2>, rc = allow_smem<decode_split_kernel<2>>(dev, D_SMEM); break;
+    case 3: kern = decode_split_kernel<3>, rc = allow_smem<decode_split_kernel<3>>(dev, D_SMEM); break;
+    case 4: kern = decode_split_kernel<4>, rc = allow_smem<decode_split_kernel<4>>(dev, D_SMEM); break;
+    case 5: kern = decode_split_kernel<5>, rc = allow_smem<decode_split_kernel<5>>(dev, D_SMEM); break;
+    case 6: kern = decode_split_kernel<6>, rc = allow_smem<decode_split_kernel<6>>(dev, D_SMEM); break;
+    case 7: kern = decode_split_kernel<7>, rc = allow_smem<decode_split_kernel<7>>(dev, D_SMEM); break;
+    case 8: kern = decode_split_kernel<8>, rc = allow_smem<decode_split_kernel<8>>(dev, D_SMEM); break;
     default: return MPFA_ERR_UNSUPPORTED;
   }
-  MPFA_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)D_SMEM));
+  if (rc != MPFA_OK) return rc;
   MPFA_CUDA_OK(launch(decode_prep_kernel, dim3(1), dim3(1), 0, s, p.ticket));
   MPFA_CUDA_OK(launch(kern, dim3(grid), dim3(D_THREADS), D_SMEM, s, p));
   MPFA_CUDA_OK(launch(decode_merge_kernel, dim3(H_q, B), dim3(128), 0, s, p));

@@ -99,11 +99,9 @@ using namespace mpfa;
 extern "C" mpfa_status mpfa_bench_mma_peak(int kind, int n_cols, int iters, int32_t *device_status, void *stream) {
   if (kind < 0 || kind > 3 || (n_cols != 128 && n_cols != 256) || iters <= 0 || iters > (1 << 22) || !device_status)
     return MPFA_ERR_INVALID_ARG;
-  mpfa_status rc = check_arch();
-  if (rc != MPFA_OK) return rc;
   int dev = 0, n_sm = 0;
-  MPFA_CUDA_OK(cudaGetDevice(&dev));
-  MPFA_CUDA_OK(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
+  mpfa_status rc = device_info(&dev, &n_sm);
+  if (rc != MPFA_OK) return rc;
   // more than half of an SM's shared memory per CTA: never two CTAs on one SM (the second would sit in the
   // tensor-memory allocation until the first has finished)
   constexpr int LAUNCH_SMEM = 120 * 1024;

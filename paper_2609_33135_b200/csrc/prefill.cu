@@ -243,6 +243,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + OFF_MISC);
 
   // ---- one-time setup
+  launch_dependents();
   if (tid == 0) {
     *cx.abort_flag = 0;
     for (int i = 0; i < 2; ++i) { mbar_init(cx.bar(BAR_Q_FULL + i), 1); mbar_init(cx.bar(BAR_Q_EMPTY + i), 1); }
@@ -279,6 +280,8 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     tmem_alloc(smem_u32(tmem_slot), TMEM_COLS);
     tmem_relinquish();
   }
+  // everything above touches this CTA only and overlaps the end of the preceding kernel; everything below reads memory
+  grid_dependency_wait();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -979,6 +982,15 @@ extern "C" int mpfa_debug_set_trace(long long *buf, int cta) {
 }
 #endif
 
+template <auto Kernel, uint32_t SMEM>
+static mpfa_status start(int dev, unsigned grid, cudaStream_t stream, const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap &tv,
+                         const PrefillParams &p, const PagedSrc &pg) {
+  mpfa_status rc = allow_smem<Kernel>(dev, SMEM);
+  if (rc != MPFA_OK) return rc;
+  MPFA_CUDA_OK(launch(Kernel, dim3(grid), dim3(NTHREADS), SMEM, stream, tq, tk, tv, p, pg));
+  return MPFA_OK;
+}
+
 // 0: one query tile per CTA, two softmax groups alternating over KV blocks (the faster one on B200, see
 // prefill_pair.cu's header for the measured comparison); 1: two query tiles per CTA (prefill_pair.cu)
 static int g_arrangement = 0;
@@ -1018,7 +1030,8 @@ extern "C" mpfa_status mpfa_prefill_variant(const mpfa_fp4_tensor *q, const mpfa
   if (q_rows >= (1ull << 31) || k_rows >= (1ull << 31)) return MPFA_ERR_UNSUPPORTED;
   const uint64_t n_cta = (uint64_t)q->B * q->H * nq_tiles;
   if (n_cta >= (1ull << 31)) return MPFA_ERR_UNSUPPORTED;
-  mpfa_status rc = check_arch();
+  int dev = 0, n_sm = 0;
+  mpfa_status rc = device_info(&dev, &n_sm);
   if (rc != MPFA_OK) return rc;
   PrefillParams p;
   p.q_sf = q->sf;
@@ -1054,25 +1067,17 @@ extern "C" mpfa_status mpfa_prefill_variant(const mpfa_fp4_tensor *q, const mpfa
   if ((rc = make_map(enc, &tq, q->codes, q_rows, 64)) != MPFA_OK) return rc;
   if ((rc = make_map(enc, &tk, k->codes, k_rows, 64)) != MPFA_OK) return rc;
   if ((rc = pvb ? make_map(enc, &tv, v_fp8, k_rows, 256, 128) : make_map(enc, &tv, v_fp8, k_rows, pv4 ? 64 : 128)) != MPFA_OK) return rc;
-  int dev = 0, n_sm = 0;
-  MPFA_CUDA_OK(cudaGetDevice(&dev));
-  MPFA_CUDA_OK(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
   const unsigned grid = (unsigned)(n_cta < (uint64_t)n_sm ? n_cta : (uint64_t)n_sm);   // one persistent CTA per SM
   if (pvb) {
-    MPFA_CUDA_OK(cudaFuncSetAttribute(prefill_kernel<false, false, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Lay<1>::SMEM_BYTES));
-    prefill_kernel<false, false, 1><<<grid, NTHREADS, Lay<1>::SMEM_BYTES, static_cast<cudaStream_t>(stream)>>>(tq, tk, tv, p, PagedSrc{});
+    rc = start<prefill_kernel<false, false, 1>, Lay<1>::SMEM_BYTES>(dev, grid, static_cast<cudaStream_t>(stream), tq, tk, tv, p, PagedSrc{});
   } else if (pv4) {
-    MPFA_CUDA_OK(cudaFuncSetAttribute(prefill_kernel<false, false, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Lay<2>::SMEM_BYTES));
-    prefill_kernel<false, false, 2><<<grid, NTHREADS, Lay<2>::SMEM_BYTES, static_cast<cudaStream_t>(stream)>>>(tq, tk, tv, p, PagedSrc{});
+    rc = start<prefill_kernel<false, false, 2>, Lay<2>::SMEM_BYTES>(dev, grid, static_cast<cudaStream_t>(stream), tq, tk, tv, p, PagedSrc{});
   } else if (ew) {
-    MPFA_CUDA_OK(cudaFuncSetAttribute(prefill_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Lay<0>::SMEM_BYTES));
-    prefill_kernel<false, true><<<grid, NTHREADS, Lay<0>::SMEM_BYTES, static_cast<cudaStream_t>(stream)>>>(tq, tk, tv, p, PagedSrc{});
+    rc = start<prefill_kernel<false, true>, Lay<0>::SMEM_BYTES>(dev, grid, static_cast<cudaStream_t>(stream), tq, tk, tv, p, PagedSrc{});
   } else {
-    MPFA_CUDA_OK(cudaFuncSetAttribute(prefill_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Lay<0>::SMEM_BYTES));
-    prefill_kernel<false, false><<<grid, NTHREADS, Lay<0>::SMEM_BYTES, static_cast<cudaStream_t>(stream)>>>(tq, tk, tv, p, PagedSrc{});
+    rc = start<prefill_kernel<false, false>, Lay<0>::SMEM_BYTES>(dev, grid, static_cast<cudaStream_t>(stream), tq, tk, tv, p, PagedSrc{});
   }
-  MPFA_LAUNCH_OK();
-  return MPFA_OK;
+  return rc;
 }
 
 extern "C" mpfa_status mpfa_prefill_paged(const mpfa_fp4_tensor *q, const mpfa_paged_kv *kv, const int32_t *page_table,
@@ -1094,7 +1099,8 @@ extern "C" mpfa_status mpfa_prefill_paged(const mpfa_fp4_tensor *q, const mpfa_p
   const uint64_t q_rows = (uint64_t)q->B * q->H * nq_tiles * TILE;
   if (q_rows >= (1ull << 31)) return MPFA_ERR_UNSUPPORTED;
   const uint64_t n_cta = (uint64_t)q->B * q->H * nq_tiles;
-  mpfa_status rc = check_arch();
+  int dev = 0, n_sm = 0;
+  mpfa_status rc = device_info(&dev, &n_sm);
   if (rc != MPFA_OK) return rc;
   PrefillParams p;
   p.q_sf = q->sf;
@@ -1132,12 +1138,6 @@ extern "C" mpfa_status mpfa_prefill_paged(const mpfa_fp4_tensor *q, const mpfa_p
   if (rc != MPFA_OK) return rc;
   CUtensorMap tq;
   if ((rc = make_map(enc, &tq, q->codes, q_rows, 64)) != MPFA_OK) return rc;
-  int dev = 0, n_sm = 0;
-  MPFA_CUDA_OK(cudaGetDevice(&dev));
-  MPFA_CUDA_OK(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
   const unsigned grid = (unsigned)(n_cta < (uint64_t)n_sm ? n_cta : (uint64_t)n_sm);
-  MPFA_CUDA_OK(cudaFuncSetAttribute(prefill_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Lay<0>::SMEM_BYTES_PAGED));
-  prefill_kernel<true, false><<<grid, NTHREADS, Lay<0>::SMEM_BYTES_PAGED, static_cast<cudaStream_t>(stream)>>>(tq, tq, tq, p, pg);
-  MPFA_LAUNCH_OK();
-  return MPFA_OK;
+  return start<prefill_kernel<true, false>, Lay<0>::SMEM_BYTES_PAGED>(dev, grid, static_cast<cudaStream_t>(stream), tq, tq, tq, p, pg);
 }

@@ -21,11 +21,22 @@ namespace mpfa {
 
 thread_local int g_last_cuda_error = 0;
 
-mpfa_status check_arch() {
-  int dev = 0, major = 0;
-  MPFA_CUDA_OK(cudaGetDevice(&dev));
-  MPFA_CUDA_OK(cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev));
-  return major == 10 ? MPFA_OK : MPFA_ERR_ARCH;
+mpfa_status device_info(int *dev, int *n_sm) {
+  static std::atomic<int> known[MAX_DEVICES];   // SM count; 0: not asked yet, -1: not a device for this library
+  int d = 0;
+  MPFA_CUDA_OK(cudaGetDevice(&d));
+  int n = d < MAX_DEVICES ? known[d].load(std::memory_order_relaxed) : 0;
+  if (n == 0) {
+    int major = 0;
+    MPFA_CUDA_OK(cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, d));
+    MPFA_CUDA_OK(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, d));
+    if (major != 10) n = -1;
+    if (d < MAX_DEVICES) known[d].store(n, std::memory_order_relaxed);
+  }
+  if (n < 0) return MPFA_ERR_ARCH;
+  *dev = d;
+  *n_sm = n;
+  return MPFA_OK;
 }
 
 namespace {
@@ -896,14 +907,12 @@ extern "C" mpfa_status mpfa_quantize_qk(const void *q_bf16, const void *k_bf16, 
     w = carve(workspace, workspace_bytes, B, H_q, H_kv);
     if (w.slices < 1) return MPFA_ERR_WORKSPACE;
   }
-  mpfa_status rc = check_arch();
+  int dev = 0, n_sm = 0;
+  mpfa_status rc = device_info(&dev, &n_sm);
   if (rc != MPFA_OK) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const __nv_bfloat16 *q = static_cast<const __nv_bfloat16 *>(q_bf16);
   const __nv_bfloat16 *k = static_cast<const __nv_bfloat16 *>(k_bf16);
-  int dev = 0, n_sm = 0;
-  MPFA_CUDA_OK(cudaGetDevice(&dev));
-  MPFA_CUDA_OK(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
   if (!frozen) {
     rc = tensor_stats(ColTensor{q, N_q, q ? H_q : 0, w.psum_q, w.pext_q, st->q_mean, w.gmax_q},
                       ColTensor{k, N_kv, k ? H_kv : 0, w.psum_k, w.pext_k, st->k_mean, w.gmax_k}, B, w.slices, n_sm, smooth, s);
@@ -936,7 +945,8 @@ extern "C" mpfa_status mpfa_quantize_v(const void *v_bf16, int B, int N_kv, int 
                                        void *stream) {
   if (!v_bf16 || !v_fp8 || B <= 0 || N_kv <= 0 || H_kv <= 0 || !(v_scale > 0.0f)) return MPFA_ERR_INVALID_ARG;
   if (!aligned(v_bf16, 16) || !aligned(v_fp8, 1024)) return MPFA_ERR_ALIGNMENT;
-  mpfa_status rc = check_arch();
+  int dev = 0, n_sm = 0;
+  mpfa_status rc = device_info(&dev, &n_sm);
   if (rc != MPFA_OK) return rc;
   dim3 grid(pad128(N_kv) / TILE, H_kv, B);
   MPFA_CUDA_OK(launch(quantize_v_tile_kernel, grid, dim3(256), 0, static_cast<cudaStream_t>(stream),
@@ -947,7 +957,8 @@ extern "C" mpfa_status mpfa_quantize_v(const void *v_bf16, int B, int N_kv, int 
 extern "C" mpfa_status mpfa_pack_v_bf16(const void *v_bf16, int B, int N_kv, int H_kv, void *v_tiles_bf16, void *stream) {
   if (!v_bf16 || !v_tiles_bf16 || B <= 0 || N_kv <= 0 || H_kv <= 0) return MPFA_ERR_INVALID_ARG;
   if (!aligned(v_bf16, 16) || !aligned(v_tiles_bf16, 1024)) return MPFA_ERR_ALIGNMENT;
-  mpfa_status rc = check_arch();
+  int dev = 0, n_sm = 0;
+  mpfa_status rc = device_info(&dev, &n_sm);
   if (rc != MPFA_OK) return rc;
   pack_v_bf16_kernel<<<dim3(pad128(N_kv) / TILE, H_kv, B), 256, 0, static_cast<cudaStream_t>(stream)>>>(
       static_cast<const __nv_bfloat16 *>(v_bf16), N_kv, H_kv, static_cast<__nv_bfloat16 *>(v_tiles_bf16));
@@ -964,7 +975,8 @@ extern "C" mpfa_status mpfa_quantize_v_fp4(const void *v_bf16, int B, int N_kv, 
                                            void *stream) {
   if (!v_bf16 || !v_fp4 || B <= 0 || N_kv <= 0 || H_kv <= 0 || !(v_gscale > 0.0f)) return MPFA_ERR_INVALID_ARG;
   if (!aligned(v_bf16, 16) || !aligned(v_fp4, 1024)) return MPFA_ERR_ALIGNMENT;
-  mpfa_status rc = check_arch();
+  int dev = 0, n_sm = 0;
+  mpfa_status rc = device_info(&dev, &n_sm);
   if (rc != MPFA_OK) return rc;
   const size_t n_tiles = (size_t)B * H_kv * (pad128(N_kv) / TILE);
   quantize_v_fp4_tile_kernel<<<dim3(pad128(N_kv) / TILE, H_kv, B), 256, 0, static_cast<cudaStream_t>(stream)>>>(
@@ -997,14 +1009,12 @@ extern "C" mpfa_status mpfa_quantize_kv_paged(const void *k_bf16, const void *v_
     w = carve(workspace, workspace_bytes, 1, H_q, H_kv);
     if (w.slices < 1) return MPFA_ERR_WORKSPACE;
   }
-  mpfa_status rc = check_arch();
+  int dev = 0, n_sm = 0;
+  mpfa_status rc = device_info(&dev, &n_sm);
   if (rc != MPFA_OK) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const __nv_bfloat16 *k = static_cast<const __nv_bfloat16 *>(k_bf16);
   const __nv_bfloat16 *v = static_cast<const __nv_bfloat16 *>(v_bf16);
-  int dev = 0, n_sm = 0;
-  MPFA_CUDA_OK(cudaGetDevice(&dev));
-  MPFA_CUDA_OK(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
   if (!frozen) {
     rc = tensor_stats(ColTensor{k, N_tokens, H_kv, w.psum_k, w.pext_k, st->k_mean, w.gmax_k}, ColTensor{}, 1, w.slices, n_sm, smooth, s);
     if (rc != MPFA_OK) return rc;
@@ -1036,7 +1046,8 @@ extern "C" mpfa_status mpfa_append_kv_paged(const void *k_bf16, const void *v_bf
   if (!aligned(k_bf16, 16) || !aligned(v_bf16, 16) || !aligned(kv->k_codes, 256) || !aligned(kv->k_sf, 256) ||
       !aligned(kv->v_fp8, 256) || !aligned(kv->delta_s_bf16, 256))
     return MPFA_ERR_ALIGNMENT;
-  mpfa_status rc = check_arch();
+  int dev = 0, n_sm = 0;
+  mpfa_status rc = device_info(&dev, &n_sm);
   if (rc != MPFA_OK) return rc;
   MPFA_CUDA_OK(launch(append_kv_kernel, dim3((B * H_kv + 7) / 8), dim3(256), 0, static_cast<cudaStream_t>(stream),
                       static_cast<const __nv_bfloat16 *>(k_bf16), static_cast<const __nv_bfloat16 *>(v_bf16), st->q_mean, st->k_mean,
@@ -1055,7 +1066,6 @@ namespace {
 constexpr size_t STATIC_SCRATCH_BYTES = MPFA_STATIC_SCRATCH_BYTES;
 static __device__ __align__(256) unsigned char g_static_scratch[STATIC_SCRATCH_BYTES];
 
-constexpr int MAX_DEVICES = 64;
 void *g_static_scratch_addr[MAX_DEVICES] = {};
 std::mutex g_static_scratch_mutex;
 

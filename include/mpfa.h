@@ -305,8 +305,8 @@ mpfa_status mpfa_prefill_paged(const mpfa_fp4_tensor *h_q, const mpfa_paged_kv *
  * page_table [B, max_pages_per_req].  Each (request, kv head, 1024-token partition) keeps a
  * local (m, l, O) state for its GQA group in `workspace`; a second kernel merges the
  * partitions by log-sum-exp.  The number of partitions is fixed by max_seq_len, so the call
- * sequence (three kernels: a reset of the work counter at the end of `workspace`, the partitions, the merge)
- * does not depend on seq_lens.  Work items are drawn from that counter by the running CTAs, so
+ * sequence (a reset of the work counter at the end of `workspace` where there are more partitions than SMs, the
+ * partitions, the merge where there can be several) does not depend on seq_lens.  Work items are drawn from that counter by the running CTAs, so
  * two calls that overlap on the GPU need separate workspaces.  out_bf16 [B, H_q, 128]; out_f32 optional. */
 mpfa_status mpfa_decode(const mpfa_fp4_tensor *h_q, const mpfa_paged_kv *h_kv, const int32_t *page_table,
                         int max_pages_per_req, const int32_t *seq_lens, const mpfa_stats *h_stats,

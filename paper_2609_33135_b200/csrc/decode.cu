@@ -174,7 +174,7 @@ struct DecodeParams {
   const float *q_gscale, *k_gscale;
   float *part_o;           // [B, H_q, n_split, 128]
   float2 *part_ml;         // [B, H_q, n_split]: (m, l)
-  unsigned int *ticket;    // global work counter, zero at launch
+  unsigned int *ticket;    // global work counter, zero at launch; null: the first tickets cover all items
   __nv_bfloat16 *out;
   float *out_f32;          // may be null
   int32_t *status;
@@ -367,6 +367,7 @@ __global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const __grid
       int4 item = make_int4(-1, 0, 0, 0);
       if (lane == 0) {
         for (bool first = k == 0;; first = false) {
+          if (!first && !p.ticket) break;
           const uint32_t tkt = first ? blockIdx.x : gridDim.x + atomicAdd(p.ticket, 1u);
           if (tkt >= total) break;
           if (compact) {
@@ -561,6 +562,13 @@ __global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const __grid
     }
   } else if (warp == 2) {
     // ================= PV issue: O_u^T = V_u^T P_hat_u^T as V stages land
+    // a request without keys has no work item: its zeros are written here, while this warp has nothing to issue
+    for (int b = blockIdx.x; b < p.B; b += gridDim.x)
+      if (p.seq_lens[b] <= 0)
+        for (int i = lane; i < p.H_q * HEAD_DIM; i += 32) {
+          p.out[(size_t)b * p.H_q * HEAD_DIM + i] = __float2bfloat16_rn(0.0f);
+          if (p.out_f32) p.out_f32[(size_t)b * p.H_q * HEAD_DIM + i] = 0.0f;
+        }
     const uint32_t id_pv = idesc_e4m3(128, NCOL, 1, 0);
     WorkIter w;
     uint32_t vc = 0, j = 0;
@@ -810,14 +818,14 @@ __global__ void decode_prep_kernel(unsigned int *ticket) {
 // l = sum w_s l_s, O = sum w_s O_s, out = O / (448 l) * v_scale.  grid (H_q, B).  Warp w takes the partitions s = w,
 // w + 4, ... in ascending order, a lane four channels (one 512-byte row per warp and load, four rows in flight), and the
 // four sums are added in warp order: a fixed order, so the result is reproducible.  128 threads of at most 56 registers
-// fit beside a CTA of the split kernel.  Requests of one partition are complete already, those without keys get zeros.
+// fit beside a CTA of the split kernel.  Requests of one partition or without keys are complete already.
 __global__ void __launch_bounds__(128, 9) decode_merge_kernel(const __grid_constant__ DecodeParams p) {
   __shared__ float s_l[4];
   __shared__ __align__(16) float s_o[4][HEAD_DIM];
   grid_dependency_wait();
   const int hq = blockIdx.x, b = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n = p.n_parts(p.seq_lens[b]);
-  if (n == 1) return;
+  if (n <= 1) return;
   const size_t head = (size_t)b * p.H_q + hq;
   const float2 *ml = p.part_ml + head * p.n_split;
   const float4 *po = reinterpret_cast<const float4 *>(p.part_o + head * p.n_split * HEAD_DIM) + lane;
@@ -918,7 +926,6 @@ extern "C" mpfa_status mpfa_decode(const mpfa_fp4_tensor *q, const mpfa_paged_kv
   p.k_gscale = st->k_gscale;
   p.part_o = static_cast<float *>(workspace);
   p.part_ml = reinterpret_cast<float2 *>(static_cast<uint8_t *>(workspace) + ws.ml);
-  p.ticket = reinterpret_cast<unsigned int *>(static_cast<uint8_t *>(workspace) + ws.ticket);
   p.out = static_cast<__nv_bfloat16 *>(out_bf16);
   p.out_f32 = out_f32;
   p.status = device_status;
@@ -946,8 +953,11 @@ extern "C" mpfa_status mpfa_decode(const mpfa_fp4_tensor *q, const mpfa_paged_kv
     default: return MPFA_ERR_UNSUPPORTED;
   }
   if (rc != MPFA_OK) return rc;
-  MPFA_CUDA_OK(launch(decode_prep_kernel, dim3(1), dim3(1), 0, s, p.ticket));
+  // Kernels that a small call does not need are not launched (each costs a few microseconds of host time and one to two of
+  // latency): no counter where every CTA gets at most one item, no merge where no request can have two partitions.
+  p.ticket = items > (size_t)n_sm ? reinterpret_cast<unsigned int *>(static_cast<uint8_t *>(workspace) + ws.ticket) : nullptr;
+  if (p.ticket) MPFA_CUDA_OK(launch(decode_prep_kernel, dim3(1), dim3(1), 0, s, p.ticket));
   MPFA_CUDA_OK(launch(kern, dim3(grid), dim3(D_THREADS), D_SMEM, s, p));
-  MPFA_CUDA_OK(launch(decode_merge_kernel, dim3(H_q, B), dim3(128), 0, s, p));
+  if (n_split > 1) MPFA_CUDA_OK(launch(decode_merge_kernel, dim3(H_q, B), dim3(128), 0, s, p));
   return MPFA_OK;
 }

@@ -114,6 +114,8 @@ def test_decode_long_request_many_partitions():
 
 
 @pytest.mark.parametrize("hq,hkv,lens", [
+    (8, 2, [0, 1024, 1, 0, 700]),                   # no request can have two partitions: no merge launched
+    (8, 2, [0, 1025, 0, 3]),                        # one that has, next to requests without keys
     (40, 8, [1] * 18),                              # 144 work items: fewer than there are SMs, groups of five heads
     (40, 8, [129] * 19),                            # 152: some CTAs get a second item
     (32, 4, [1024, 1025, 2048, 2049] * 10),         # exact and just exceeded partitions, groups of eight, 240 items
@@ -122,11 +124,20 @@ def test_decode_long_request_many_partitions():
 def test_decode_item_counts_around_the_grid(hq, hkv, lens):
     """The work-item walk and its two alternating softmax groups: item counts just below and above the grid, partitions
     of every block count, requests complete in one partition next to merged ones."""
-    w = wl.decode_workload("dec_items", 78 + hq, len(lens), hq, hkv, 1, max(lens), n_stat_tokens=64, seq_lens=lens)
-    st = run(w)
+    from paper_2609_33135_b200 import decode_cache
+    w = wl.decode_workload("dec_items", 78 + hq, len(lens), hq, hkv, 1, max(lens), n_stat_tokens=64, seq_lens=[max(1, n) for n in lens])
+    st = decode_cache.build_cache(w)
+    st.seq_lens.copy_(torch.tensor(lens, dtype=torch.int32))
+    st.out.fill_(7.0)
+    st.out_f32.fill_(7.0)
+    decode_cache.decode_step(st)
+    torch.cuda.synchronize()
+    assert int(st.status.item()) == 0
     got = st.out_f32.cpu().numpy()
     assert np.isfinite(got).all()
-    for b in sorted({0, 1, 2, 3, len(lens) // 2, len(lens) - 1}):
+    for b in [b for b, n in enumerate(lens) if n == 0]:
+        assert not got[b].any() and not st.out[b].any()
+    for b in sorted({i for i in (0, 1, 2, 3, len(lens) // 2, len(lens) - 1) if lens[i] > 0}):
         d = np.abs(got[b] - oracle_decode_one(w, b))
         assert d.max() <= MAX_ABS and d.mean() <= MEAN_ABS, (b, float(d.max()), float(d.mean()))
 

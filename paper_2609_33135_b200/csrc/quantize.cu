@@ -413,6 +413,30 @@ __device__ __forceinline__ void group_dot16(const GroupMeans &m, int half, const
                  : "d"((double)xc[s]), "d"(q[s * 32]));
 }
 
+// One or two heads: of the tensor instruction's eight columns only so many would count, and the plain FP64 pipe has the same
+// rate.  A lane takes the products of its own 32 channels (query means as doubles, [head][channel pair][j][2], so that the
+// four addresses of a warp's load are one line) and the four lanes of a key are added in a fixed order.
+__device__ __forceinline__ void convert_group_means_few(double *m, const float *q_mean /* [G, 128] */, int G, int tid, int n_threads) {
+  for (int i = tid; i < G * HEAD_DIM; i += n_threads) {
+    const int g = i >> 7, c = i & 127, j = (c >> 4) & 3, s = (c & 15) + ((c >> 6) << 4);
+    m[g * HEAD_DIM + (s >> 1) * 8 + j * 2 + (s & 1)] = (double)q_mean[i];
+  }
+}
+// acc[g] += the half's 16 channels of the lane's key, two chains a head
+template <int G>
+__device__ __forceinline__ void few_dot16(const double *m, int half, const float (&xc)[16], int j, double (&acc)[G][2]) {
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const double x0 = (double)xc[2 * i], x1 = (double)xc[2 * i + 1];
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      const double2 q = *reinterpret_cast<const double2 *>(m + g * HEAD_DIM + (half * 8 + i) * 8 + j * 2);
+      acc[g][0] = fma(q.x, x0, acc[g][0]);
+      acc[g][1] = fma(q.y, x1, acc[g][1]);
+    }
+  }
+}
+
 struct QuantTensor {
   const __nv_bfloat16 *x;   // null: tensor absent (H = 0)
   const float *mean;
@@ -440,6 +464,7 @@ struct DeltaArgs {
 // now 45 us.
 constexpr int QT_CTAS = 2;       // resident per SM: 128 registers, so that the means stay in registers
 constexpr int QT_K_WEIGHT = 2;   // time of a K tile with Delta_S in units of a Q tile's (1 / 2 / 3: 106 / 89 / 96 us of stage 1)
+template <int FEW>   // heads of the group where they are one or two, otherwise 0
 __global__ void __launch_bounds__(256, QT_CTAS) quantize_tile_kernel(const QuantTensor k, const QuantTensor q, const DeltaArgs da) {
   __shared__ __align__(16) GroupMeans gm;
   __shared__ float inv_table[128];
@@ -476,7 +501,11 @@ __global__ void __launch_bounds__(256, QT_CTAS) quantize_tile_kernel(const Quant
   const int G = with_delta ? da.H_q / a.H : 0;
   double unit = 0.0;
   if (with_delta) {
-    convert_group_means(gm, da.q_mean + ((size_t)b * da.H_q + h * G) * HEAD_DIM, G, tid, 256);
+    const float *qm = da.q_mean + ((size_t)b * da.H_q + h * G) * HEAD_DIM;
+    if (FEW)
+      convert_group_means_few(&gm[0][0][0], qm, FEW, tid, 256);
+    else
+      convert_group_means(gm, qm, G, tid, 256);
     unit = 1.0 / ((double)tensor_scale(da.q_scale, b, lane) * (double)d);
   }
   __syncthreads();
@@ -487,7 +516,9 @@ __global__ void __launch_bounds__(256, QT_CTAS) quantize_tile_kernel(const Quant
 #pragma unroll
     for (int it = 0; it < 2; ++it) {
       const int r = it * 64 + r0, t = tile * TILE + r;
-      double acc[2] = {0.0, 0.0};
+      double acc[FEW ? FEW : 1][2];   // FEW: two chains a head, otherwise heads 2 j and 2 j + 1
+#pragma unroll
+      for (int g = 0; g < (FEW ? FEW : 1); ++g) acc[g][0] = acc[g][1] = 0.0;
 #pragma unroll
       for (int half = 0; half < 2; ++half) {
         float xc[16];
@@ -501,14 +532,29 @@ __global__ void __launch_bounds__(256, QT_CTAS) quantize_tile_kernel(const Quant
         sc |= __shfl_xor_sync(0xffffffffu, sc, 1);
         sc |= __shfl_xor_sync(0xffffffffu, sc, 2);
         if (j == 0) *reinterpret_cast<uint32_t *>(sf_tile + half * 512 + (r & 31) * 16 + (r >> 5) * 4) = sc;
-        if (with_delta) group_dot16(gm, half, xc, lane, acc);
+        if (with_delta) {
+          if constexpr (FEW != 0)
+            few_dot16<FEW>(&gm[0][0][0], half, xc, j, acc);
+          else
+            group_dot16(gm, half, xc, lane, acc[0]);
+        }
       }
       if (with_delta) {
+        __nv_bfloat16 *const dst = da.delta + ((size_t)b * da.H_q + h * G) * n_pad + t;
+        if constexpr (FEW != 0) {
 #pragma unroll
-        for (int n = 0; n < 2; ++n) {
-          const int g = 2 * j + n;
-          if (g < G)
-            da.delta[((size_t)b * da.H_q + h * G + g) * n_pad + t] = __float2bfloat16_rn(t < N ? __double2float_rn(acc[n] * unit) : 0.0f);
+          for (int g = 0; g < FEW; ++g) {
+            double v = acc[g][0] + acc[g][1];
+            v += __shfl_xor_sync(0xffffffffu, v, 1);
+            v += __shfl_xor_sync(0xffffffffu, v, 2);
+            if (j == g) dst[g * n_pad] = __float2bfloat16_rn(t < N ? __double2float_rn(v * unit) : 0.0f);
+          }
+        } else {
+#pragma unroll
+          for (int n = 0; n < 2; ++n) {
+            const int g = 2 * j + n;
+            if (g < G) dst[g * n_pad] = __float2bfloat16_rn(t < N ? __double2float_rn(acc[0][n] * unit) : 0.0f);
+          }
         }
       }
     }
@@ -929,7 +975,7 @@ extern "C" mpfa_status mpfa_quantize_qk(const void *q_bf16, const void *k_bf16, 
   }
   // At most one wave of CTAs, as far as that goes: a CTA's set-up (scale, table of reciprocals, query means) is paid once, and
   // the next tile's loads run under the arithmetic of the current one.  A few CTAs more than a wave would take twice the time.
-  const int k_weight = da.delta ? QT_K_WEIGHT : 1;
+  const int k_weight = da.delta && H_q / H_kv > 2 ? QT_K_WEIGHT : 1;
   const long long work = ((long long)k_weight * tk.tiles * tk.H + (long long)tq.tiles * tq.H) * B, wave = (long long)QT_CTAS * n_sm;
   for (long long per = (work + wave - 1) / wave;; ++per) {
     const int per_q = (int)per, per_k = (int)((per + k_weight - 1) / k_weight);
@@ -937,7 +983,9 @@ extern "C" mpfa_status mpfa_quantize_qk(const void *q_bf16, const void *k_bf16, 
     tq.ctas = tq.x ? (tq.tiles + per_q - 1) / per_q : 0;
     if (((long long)tk.ctas * tk.H + (long long)tq.ctas * tq.H) * B <= wave || (tk.ctas <= 1 && tq.ctas <= 1)) break;
   }
-  MPFA_CUDA_OK(launch(quantize_tile_kernel, dim3(tk.ctas * tk.H + tq.ctas * tq.H, 1, B), dim3(256), 0, s, tk, tq, da));
+  const int few = da.delta && H_q / H_kv <= 2 ? H_q / H_kv : 0;
+  MPFA_CUDA_OK(launch(few == 0 ? quantize_tile_kernel<0> : few == 1 ? quantize_tile_kernel<1> : quantize_tile_kernel<2>,
+                      dim3(tk.ctas * tk.H + tq.ctas * tq.H, 1, B), dim3(256), 0, s, tk, tq, da));
   return MPFA_OK;
 }
 

@@ -37,7 +37,9 @@
 //
 // Measured (call alone, before / after the two softmax groups, the O group and the rolled passes over the scores):
 // 16 requests x 32K, 8 kv heads, groups of 1 / 4 / 5 / 8 heads: 148 / 164 / 670 / 904 -> 144 / 156 / 158 / 173 us
-// (5.9 / 5.6 / 5.6 / 5.2 TB/s of cache); 64 requests of 100..4000 tokens, 40:8 heads: 227 -> 59 us.
+// (5.9 / 5.6 / 5.6 / 5.2 TB/s of cache); 64 requests of 100..4000 tokens, 40:8 heads: 227 -> 59 us.  The running maxima and
+// block weights held in the lanes and handed out by shuffles, where every thread took them from shared memory for every
+// block: 256 requests of 100..2000 tokens with append and query 137 -> 130 us, one request of 4097 22.6 -> 21.7 us.
 //
 // Warps: 18 draws work items and stages their query tiles, 0 and 17 K producers (codes; scales and Delta_S),
 // 16 V producer, 1 QK issue (+ TMEM allocation), 2 PV issue, 3 rewrites the K scales of each block from
@@ -629,6 +631,7 @@ __global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const __grid
     const int r = quad * 32 + lane;             // key within the block
     const uint32_t tlane = (uint32_t)(quad * 32) << 16;
     constexpr int CH = G <= 2 ? 4 : 2;          // blocks whose tensor-memory loads are in flight together
+    constexpr int GP = G <= 4 ? 4 : 8, TPV = 32 / GP, NV = MAXBLK / TPV;   // heads padded; blocks to a warp's lanes; such sets
     const uint32_t tS = tm + TM_S + grp * (MAXBLK * 16) + tlane;
     uint8_t *const pt = dsm + D_OFF_P + grp * MAXBLK * 1024 + (r & 15);
     float *xm = xmax + grp * MAXBLK * MAXG * 4, *wt = wtab + grp * MAXBLK * MAXG, *xlg = xl + grp * 4 * MAXG;
@@ -669,66 +672,66 @@ __global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const __grid
       cx.warp_arrive(B_XCHG + grp);
       ok = cx.wait_warp(B_XCHG + grp, ph);
       if (!ok) break;
+      // running maxima m_t of the reverse traversal, -lam m_t and the weights 2^(lam (m_t - m)) of the item's end, in the lanes
+      float mt[NV], nml[NV], wl[NV], m_end;
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        const int t = v * TPV + lane / GP;
+        const float4 q = *reinterpret_cast<const float4 *>(&xm[(t * MAXG + (lane & (GP - 1))) * 4]);
+        mt[v] = t < w.nblk ? fmaxf(fmaxf(q.x, q.y), fmaxf(q.z, q.w)) : -INFINITY;
+#pragma unroll
+        for (int o = GP; o < 32; o <<= 1) {
+          const float before = __shfl_up_sync(0xffffffffu, mt[v], o);
+          if (lane >= o) mt[v] = fmaxf(mt[v], before);
+        }
+        if (v > 0) mt[v] = fmaxf(mt[v], m_end);
+        m_end = __shfl_sync(0xffffffffu, mt[v], 32 - GP + (lane & (GP - 1)));
+      }
       // the item two before this one, which used the same tables and P_hat tiles, is through with them
       if (j >= 2) ok = cx.wait_warp(B_T_FREE + grp, ph ^ 1);
       if (!ok) break;
-      // block weights 2^(lam (m_u - m)) of the item's end, one (block, head) per thread
-      if (r < MAXBLK * G) {
-        const int tw = r / G, gw = r % G;
-        float mu = -INFINITY, mf = -INFINITY;
-#pragma unroll 1
-        for (int t = 0; t < w.nblk; ++t) {
-          const float4 x = *reinterpret_cast<const float4 *>(&xm[(t * MAXG + gw) * 4]);
-          mf = fmaxf(mf, fmaxf(fmaxf(x.x, x.y), fmaxf(x.z, x.w)));
-          if (t == tw) mu = mf;
-        }
-        if (tw == 0) mfin[grp * MAXG + gw] = mf;
-        wt[tw * MAXG + gw] = mu == mf ? 1.0f : ex2_approx(__fmul_rn(mu - mf, lam));
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        nml[v] = -__fmul_rn(mt[v], lam);
+        wl[v] = mt[v] == m_end ? 1.0f : ex2_approx(__fmul_rn(mt[v] - m_end, lam));
+        if (quad == 0 && (lane & (GP - 1)) < G) wt[(v * TPV + lane / GP) * MAXG + (lane & (GP - 1))] = wl[v];
       }
-      // running maxima of the reverse traversal and all P_hat of the item
-      float run[G], lsum[G];
+      if (quad == 0 && lane < G) mfin[grp * MAXG + lane] = m_end;
+      // all P_hat of the item; l = sum of the blocks' sums times their weights
+      float lsum[G];
 #pragma unroll
-      for (int g = 0; g < G; ++g) run[g] = -INFINITY, lsum[g] = 0.0f;
+      for (int g = 0; g < G; ++g) lsum[g] = 0.0f;
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
 #pragma unroll 1
-      for (int t0 = 0; t0 < w.nblk; t0 += CH) {
-        uint32_t sr[CH][G];
+        for (int t0 = 0; t0 < TPV && v * TPV + t0 < w.nblk; t0 += CH) {
+          uint32_t sr[CH][G];
 #pragma unroll
-        for (int u = 0; u < CH; ++u)
-          if (t0 + u < w.nblk) tmem_ld_g<G>(tS + (t0 + u) * 16, sr[u]);
-        tmem_ld_wait();
+          for (int u = 0; u < CH; ++u)
+            if (v * TPV + t0 + u < w.nblk) tmem_ld_g<G>(tS + (v * TPV + t0 + u) * 16, sr[u]);
+          tmem_ld_wait();
 #pragma unroll
-        for (int u = 0; u < CH; ++u) {
-          if (t0 + u < w.nblk) {
-            const bool valid = k_part + (w.nblk - 1 - t0 - u) * TILE + r < w.L;
-            float m[G], pq[G + 1];
-            bool moved = false;
-#pragma unroll
-            for (int g = 0; g < G; ++g) {
-              const float4 x = *reinterpret_cast<const float4 *>(&xm[((t0 + u) * MAXG + g) * 4]);
-              m[g] = fmaxf(run[g], fmaxf(fmaxf(x.x, x.y), fmaxf(x.z, x.w)));
-              moved |= m[g] != run[g];
-            }
-            if (moved) {   // uniform; one branch for the whole group keeps the heads' chains independent
+          for (int u = 0; u < CH; ++u) {
+            const int t = v * TPV + t0 + u;
+            if (t < w.nblk) {
+              const bool valid = k_part + (w.nblk - 1 - t) * TILE + r < w.L;
+              float pq[G + 1];
 #pragma unroll
               for (int g = 0; g < G; ++g) {
-                lsum[g] = __fmul_rn(lsum[g], m[g] == run[g] ? 1.0f : ex2_approx(__fmul_rn(run[g] - m[g], lam)));
-                run[g] = m[g];
+                const float c = __shfl_sync(0xffffffffu, nml[v], (t0 + u) * GP + g), wg = __shfl_sync(0xffffffffu, wl[v], (t0 + u) * GP + g);
+                const float e = ex2_approx(__fmaf_rn(__uint_as_float(sr[u][g]), lam, c));
+                const float pv = valid ? e : 0.0f;
+                lsum[g] = __fmaf_rn(wg, pv, lsum[g]);
+                pq[g] = __fmul_rn(pv, 448.0f);
               }
-            }
+              pq[G] = 0.0f;
+              uint8_t *const pb = pt + t * 1024;
 #pragma unroll
-            for (int g = 0; g < G; ++g) {
-              const float e = ex2_approx(__fmaf_rn(__uint_as_float(sr[u][g]), lam, -__fmul_rn(m[g], lam)));
-              const float pv = valid ? e : 0.0f;
-              lsum[g] = __fadd_rn(lsum[g], pv);
-              pq[g] = __fmul_rn(pv, 448.0f);
-            }
-            pq[G] = 0.0f;
-            uint8_t *const pb = pt + (t0 + u) * 1024;
-#pragma unroll
-            for (int g = 0; g < G; g += 2) {
-              const uint32_t two = (uint32_t)__nv_cvt_float2_to_fp8x2(make_float2(pq[g], pq[g + 1]), __NV_SATFINITE, __NV_E4M3);
-              pb[g * 128 + (((r >> 4) ^ g) << 4)] = (uint8_t)two;
-              if (g + 1 < G) pb[(g + 1) * 128 + (((r >> 4) ^ (g + 1)) << 4)] = (uint8_t)(two >> 8);
+              for (int g = 0; g < G; g += 2) {
+                const uint32_t two = (uint32_t)__nv_cvt_float2_to_fp8x2(make_float2(pq[g], pq[g + 1]), __NV_SATFINITE, __NV_E4M3);
+                pb[g * 128 + (((r >> 4) ^ g) << 4)] = (uint8_t)two;
+                if (g + 1 < G) pb[(g + 1) * 128 + (((r >> 4) ^ (g + 1)) << 4)] = (uint8_t)(two >> 8);
+              }
             }
           }
         }

@@ -819,6 +819,27 @@ __global__ void __launch_bounds__(256) append_kv_kernel(const __nv_bfloat16 *__r
   const bool in_table = pos >= 0 && (pos >> 6) < max_pages;   // else: skipped, or no page-table entry for that position
   const int page = in_table ? page_table[(size_t)b * max_pages + (pos >> 6)] : -1;
   const int t = pos & 63;
+  // Delta_S of heads part and part + 4, while the page id is on its way
+  double acc[2] = {0.0, 0.0};
+  if (delta) {
+#pragma unroll
+    for (int n = 0; n < 2; ++n) {
+      const int g = part + 4 * n;
+      if (g < G) {
+        const float4 *qp = reinterpret_cast<const float4 *>(q_mean + ((size_t)b * H_q + h * G + g) * HEAD_DIM + blk * 16);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float4 m = qp[i];
+          acc[n] = fma((double)m.x, (double)xc[4 * i], acc[n]);
+          acc[n] = fma((double)m.y, (double)xc[4 * i + 1], acc[n]);
+          acc[n] = fma((double)m.z, (double)xc[4 * i + 2], acc[n]);
+          acc[n] = fma((double)m.w, (double)xc[4 * i + 3], acc[n]);
+        }
+      }
+#pragma unroll
+      for (int o = 1; o < 8; o <<= 1) acc[n] += __shfl_xor_sync(0xffffffffu, acc[n], o);
+    }
+  }
   if (page < 0 || page >= num_pages) return;
   const size_t slab = (size_t)page * H_kv + h;
   uint8_t *const kd = k_codes + slab * 4096, *const sd = k_sf + slab * 512, *const vd = v_fp8 + slab * 8192;
@@ -841,25 +862,12 @@ __global__ void __launch_bounds__(256) append_kv_kernel(const __nv_bfloat16 *__r
       for (int i = lane; i < G * PAGE; i += 32)
         if ((i & 63) != ((i >> 6) << 3)) dd[i] = __float2bfloat16_rn(0.0f);
   }
-  if (!dd) return;
-  for (int g0 = 0; g0 < G; g0 += 4) {   // uniform: every lane takes part in the sums
-    const int g = g0 + part;
-    double acc = 0.0;
-    if (g < G) {
-      const float4 *qp = reinterpret_cast<const float4 *>(q_mean + ((size_t)b * H_q + h * G + g) * HEAD_DIM + blk * 16);
+  if (dd && blk == 0) {
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const float4 m = qp[i];
-        acc = fma((double)m.x, (double)xc[4 * i], acc);
-        acc = fma((double)m.y, (double)xc[4 * i + 1], acc);
-        acc = fma((double)m.z, (double)xc[4 * i + 2], acc);
-        acc = fma((double)m.w, (double)xc[4 * i + 3], acc);
-      }
+    for (int n = 0; n < 2; ++n) {
+      const int g = part + 4 * n;
+      if (g < G) dd[g * PAGE + ((((t >> 3) ^ g) << 3) | (t & 7))] = __float2bfloat16_rn(__double2float_rn(__ddiv_rn(acc[n], denom)));
     }
-#pragma unroll
-    for (int o = 1; o < 8; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (blk == 0 && g < G)
-      dd[g * PAGE + ((((t >> 3) ^ g) << 3) | (t & 7))] = __float2bfloat16_rn(__double2float_rn(__ddiv_rn(acc, denom)));
   }
 }
 

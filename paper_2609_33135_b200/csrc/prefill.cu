@@ -2,46 +2,45 @@
 //
 // A work item is one 128-row query tile of one q head; its KV blocks (128 keys) are visited from the last
 // visible block down to block 0 (Section 4.1).  One persistent CTA per SM walks a static list of work items
-// (struct TileWalk) and keeps its pipeline running across item boundaries.  Roles (512 threads):
+// (struct TileWalk) and keeps its pipeline running across item boundaries.  Roles (640 threads):
 //   warp 0       producer: K codes (tensor map, 64B swizzle), K scale factors and Delta_S (bulk copies)
-//                and V (tensor map, 128B swizzle) into rings of 4 (K) and 3 (V) stages; in the paged
-//                variant (template parameter PAGED, entry point mpfa_prefill_paged) every tile half is
-//                one bulk copy of a 64-token page slab, found through the page table;
+//                and V (tensor map, 128B swizzle) into rings of 4 stages; in the paged variant (template
+//                parameter PAGED, entry point mpfa_prefill_paged) every tile half is one bulk copy of a
+//                64-token page slab, found through the page table;
 //   warp 2       paged variant only: re-tiles the pages' row-major K scales for tcgen05.cp and un-swizzles
 //                their Delta_S rows (idle otherwise; it also owns the tensor-memory allocation);
 //   warp 1       Q K^T issuer: per block a rank-one BF16 MMA seeds S with 1 x Delta_S
 //                (Eq. 11) and two block-scaled FP4 MMAs (K = 64 each) accumulate Q K^T into
-//                the same TMEM columns;
+//                the same TMEM columns, block c in score buffer c & 1;
 //   warp 3       P V issuer: four FP8 MMAs per block (A = P_hat from TMEM, B = V from
 //                shared memory, MN-major) accumulate P V into O;
-//   warps 4-7    softmax of the even-numbered blocks of the traversal;
-//   warps 8-11   softmax of the odd-numbered blocks.  One thread per row:
-//                the whole 128-column row is read into registers once; mask, row maximum,
-//                running maximum handed from one group to the other through shared memory
-//                (only the maximum is loop-carried, so the exponentials of block t overlap
-//                the maximum pass and exponentials of block t+1), 2^(lam S - lam m), row sum
-//                from the unquantized P, P -> E4M3 at the fixed scale 448 written to its own
-//                32 TMEM columns (Algorithm 1 lines 11-14).  The score buffer is handed back to
-//                the MMA warp as soon as the row is in registers, so Q K^T runs two blocks
-//                ahead of P V and a softmax group never waits for its next scores;
-//   warps 12-15  correction + epilogue.  Even blocks accumulate into O0, odd blocks into O1,
-//                so the rescale of an accumulator (Eq. 6, by alpha_t * alpha_{t-1}, only when
-//                some row's maximum moved) has a whole block of slack instead of sitting
-//                between two dependent MMAs; the epilogue adds the two accumulators
-//                (the older one times the last alpha) and writes O / (448 l) * v_scale as BF16.
-// Tensor memory (512 columns): S [0,128) O0 [128,256) O1 [256,384), P_hat0 [384,416)
-// P_hat1 [416,448), scale factors of two query tiles [448,464) and of two K blocks [464,472) [472,480).
-// Register budget is moved between the roles with setmaxnreg (72 for warps 0-3, 168 for the softmax warps,
-// 104 for the correction warps, whose epilogue holds two accumulator chunks at once).
-// Template parameter EW: the compensation-placement ablation (mpfa_prefill_variant): no seed MMA, Delta_S added
-// element by element by the softmax threads.
+//   warps 12-15  running row maximum (Algorithm 1 lines 11-12), one thread per row, into a shared-memory ring;
+//   warps 4-7    exponentials of the even-numbered blocks of the traversal, warps 8-11 of the odd-numbered ones.  One
+//                thread per row: the whole 128-column row in registers (so the score buffer is handed back before the
+//                first exponential), mask, 2^(lam S - lam m), row sum from the unquantized P, P -> E4M3 at the fixed
+//                scale 448 into the group's own 32 TMEM columns (lines 13-14);
+//   warps 16-19  correction + epilogue: the rescale of O (Eq. 6, only when some row's maximum moved) and
+//                O / (448 l) * v_scale as BF16 (line 17).
+// Tensor memory (512 columns): S0 [0,128) S1 [128,256) O [256,384), P_hat0 [384,416) P_hat1 [416,448), scale factors of two
+// query tiles [448,464) and of two K blocks [464,480).
+//
+// Why this split.  The exponentials bound a block: 128 x 128 of them take 1024 cycles of each SM quarter's special-function
+// unit, 1130 with the conversions and stores around them (both exponent warps of a quarter together, alone on the SM; 1465 with
+// maximum, rescale and MMAs beside them).  The maximum passes on a serial chain from block to block, and with both on the
+// same thread (two groups that alternate over the blocks and hand the maximum to one another) the chain held up every item's
+// first and last blocks and every causal diagonal.  Warps of their own run the chain ahead of the exponentials; the second
+// reading of the scores costs 72 cycles of the tensor-memory port.  Two score buffers and one accumulator take the place of
+// one and two.  Measured, the kernel alone, alternating groups -> this: 16 sequences of 200 to 512 keys 79.4 -> 72.2 us, causal
+// 2048 x 32 heads 87.0 -> 82.6, 4 x 512 x 32 37.3 -> 34.2, chunks of 512 queries on paged contexts 483 -> 427; causal 16384 x 32
+// heads 1730 -> 1715 us and 131072 x 32 98.8 -> 99.1 ms, where the clock falls to 1.75-1.83 GHz under the power limit.
+// What must not be in the exponentials: one straight run of 128 took 1130 cycles where the same code with a mask test or a wait
+// per 32 scores took 2200.
 //
 // Every mbarrier wait is bounded; on expiry the CTA raises MPFA_DEV_TIMEOUT in
 // *device_status, all roles leave their loops, outstanding TMA copies are drained and
 // tensor memory is released.
 #include <cuda.h>
 #include <cuda_bf16.h>
-#include <cuda_fp4.h>
 #include <cuda_fp8.h>
 
 #include "common.cuh"
@@ -51,224 +50,103 @@
 namespace mpfa {
 namespace {
 
-constexpr int KSTAGES = 4;
-constexpr int VSTAGES = 3;
-constexpr int NTHREADS = 512;
-constexpr int MAX_GROUPS = 512;   // (query tile, request) groups that are ordered by length; with more there are so many items
-                                  // that the order hardly matters
-// setmaxnreg only moves registers inside the pool the CTA got at launch (512 threads x the 128 registers of the
-// launch bound); a request beyond the pool would block forever, so the split is checked here.
-#ifndef MPFA_REGS_UTIL_PAGED
-#define MPFA_REGS_UTIL_PAGED 64
-#define MPFA_REGS_CORR_PAGED 112
-#endif
-#ifndef MPFA_REGS_SOFTMAX
-#define MPFA_REGS_SOFTMAX 168
-#define MPFA_REGS_UTIL 72
-#define MPFA_REGS_CORR 104
-#endif
-constexpr int REGS_SOFTMAX = MPFA_REGS_SOFTMAX;
-// measured (16K / 64K TFLOPS, utility / softmax / correction): 56/168/120 1325 / 1418, 72/168/104 1339 / 1447,
-// 72/160/112 1335 / 1447, 64/168/112 1307 / 1423, 80/160/104 1310 / 1435, 96/160/88 1302 / 1427, 152 for the softmax
-// warps 1243 / 1318 (their row spills); the paged variant's producer and re-tiling warps need a few more (measured on the
-// config-2 shape from pages: 56/120 1217, 64/112 1223, 72/104 1211, 80/96 1172, 88/88 1173 TFLOPS)
-template <bool PAGED> constexpr int REGS_UTIL = PAGED ? MPFA_REGS_UTIL_PAGED : MPFA_REGS_UTIL;
-template <bool PAGED> constexpr int REGS_CORR = PAGED ? MPFA_REGS_CORR_PAGED : MPFA_REGS_CORR;
-static_assert(4 * REGS_UTIL<false> + 8 * REGS_SOFTMAX + 4 * REGS_CORR<false> <= 16 * 128, "register pool");
-static_assert(4 * REGS_UTIL<true> + 8 * REGS_SOFTMAX + 4 * REGS_CORR<true> <= 16 * 128, "register pool");
-// the utility and correction warps give registers back (setmaxnreg.dec: the target must not exceed the 128 of the
-// launch, or the instruction is illegal), the softmax warps take them (setmaxnreg.inc: not below 128)
-static_assert(REGS_UTIL<false> <= 128 && REGS_UTIL<true> <= 128 && REGS_CORR<false> <= 128 && REGS_CORR<true> <= 128 &&
-              REGS_UTIL<false> >= 24 && REGS_UTIL<true> >= 24 && REGS_CORR<false> >= 24 && REGS_CORR<true> >= 24 &&
-              REGS_SOFTMAX >= 128 && REGS_SOFTMAX <= 255, "setmaxnreg direction");
-static_assert(REGS_SOFTMAX % 8 == 0 && REGS_UTIL<false> % 8 == 0 && REGS_CORR<false> % 8 == 0 && REGS_UTIL<true> % 8 == 0 &&
-              REGS_CORR<true> % 8 == 0, "setmaxnreg granularity");
+constexpr int KST = 4, VST = 4, MST = 8;   // stages: K, V, row maxima
+constexpr int NTHREADS = 640;
+// setmaxnreg only moves registers inside the pool the CTA got at launch (640 threads x the 96 registers of the launch bound); a
+// request beyond the pool would block forever, so the split is checked here.
+constexpr int LAUNCH_REGS = 96;
+// measured (exponentials / maxima / correction / utility; us, causal 16384, 2048, paged chunks): 144/64/80/48 1715, 82.6, 427;
+// 144/56/80/56 1725, 82.6, 421; 152/56/72/48 1720, 84.4, 420; 136/64/96/48 1890, 85.5, 476; 144/56/88/48 1850, 87.5, 448;
+// 48 for the maxima or 64 for the correction spill (4000 us)
+constexpr int REGS_EXP = 144, REGS_MAX = 64, REGS_CORR = 80, REGS_UTIL = 48;
+static_assert(8 * REGS_EXP + 4 * REGS_MAX + 4 * REGS_CORR + 4 * REGS_UTIL <= 20 * LAUNCH_REGS, "register pool");
+// the exponent warps take registers (setmaxnreg.inc: not below the launch's), the others give them back (setmaxnreg.dec: not
+// above the launch's, or the instruction is illegal)
+static_assert(REGS_EXP >= LAUNCH_REGS && REGS_CORR <= LAUNCH_REGS && REGS_MAX <= LAUNCH_REGS && REGS_UTIL <= LAUNCH_REGS &&
+              REGS_UTIL >= 24, "setmaxnreg direction");
+static_assert(REGS_EXP % 8 == 0 && REGS_MAX % 8 == 0 && REGS_CORR % 8 == 0 && REGS_UTIL % 8 == 0, "setmaxnreg granularity");
 
 enum {
   BAR_Q_FULL = 0,                       // [2] query tile of work item i in buffer i & 1
   BAR_Q_EMPTY = 2,                      // [2] every Q K^T MMA of that work item has completed
   BAR_K_FULL = 4,
-  BAR_K_EMPTY = BAR_K_FULL + KSTAGES,
-  BAR_V_FULL = BAR_K_EMPTY + KSTAGES,
-  BAR_V_EMPTY = BAR_V_FULL + VSTAGES,
-  BAR_S_FULL = BAR_V_EMPTY + VSTAGES,   // [2] scores of block t in TMEM (one buffer, one barrier per
-                                        //     softmax group so that each group's first wait is on phase 0)
-  BAR_S_EMPTY = BAR_S_FULL + 2,         // scores read into registers, buffer free for block t+1
-  BAR_P_FULL = BAR_S_EMPTY + 1,         // [2] P_hat of block t written
-  BAR_P_EMPTY = BAR_P_FULL + 2,         // [2] P V of block t has consumed P_hat
-  BAR_M_FULL = BAR_P_EMPTY + 2,         // [2] running maximum and alpha of block t published
-  BAR_O_FULL = BAR_M_FULL + 2,          // [2] P V of block t accumulated into O[t & 1]
-  BAR_O_READY = BAR_O_FULL + 2,         // [2] O[t & 1] rescaled for block t
-  BAR_L_FULL = BAR_O_READY + 2,         // [4] row sums of the u-th item that has KV blocks (T > 0), slot u & 3.  The
-                                        //     softmax warps can be at most three (one-block) such items ahead of the
-                                        //     epilogue - P_hat of block c needs P V of block c-2, which needs the
-                                        //     correction warps - so a slot is never two phases ahead of its reader.
-                                        //     Items without blocks stay out of the ring: nothing bounds how many of
-                                        //     them the softmax warps could run through
-  BAR_O_FREE = BAR_L_FULL + 4,          // the epilogue has read both accumulators (phase = items with T > 0)
-  BAR_SF_READY = BAR_O_FREE + 1,        // [KSTAGES] paged source only: scales and Delta_S of the stage re-tiled
-  NUM_BARS = BAR_SF_READY + KSTAGES
+  BAR_K_EMPTY = BAR_K_FULL + KST,
+  BAR_V_FULL = BAR_K_EMPTY + KST,
+  BAR_V_EMPTY = BAR_V_FULL + VST,
+  BAR_S_FULL = BAR_V_EMPTY + VST,       // [2] scores of block c in buffer c & 1
+  BAR_S_EMPTY = BAR_S_FULL + 2,         // [2] the exponent warps have them in registers (the maximum was taken before)
+  BAR_M_FULL = BAR_S_EMPTY + 2,         // [MST] running maximum after block c in slot c % MST.  The maximum warps are at most two
+                                        //     blocks ahead of the exponent warps, and those (P_hat of block c needs P V of block
+                                        //     c-2, which needs the correction warps) at most three ahead of the correction
+                                        //     warps, whose hand-over of the accumulator for an item's first block comes
+                                        //     before they read that block's maximum: a slot is never two phases ahead of a
+                                        //     reader with five slots or more
+  BAR_P_FULL = BAR_M_FULL + MST,        // [2] P_hat of block c written
+  BAR_P_EMPTY = BAR_P_FULL + 2,         // [2] P V of block c has consumed P_hat
+  BAR_O_FULL = BAR_P_EMPTY + 2,         // P V of block c accumulated into O
+  BAR_O_READY = BAR_O_FULL + 1,         // O rescaled for block c (an item's first block: the previous item's output has been read)
+  BAR_L_FULL = BAR_O_READY + 1,         // [4] row sums of the u-th item that has KV blocks (T > 0), slot u & 3.  The exponent
+                                        //     warps can be at most three (one-block) such items ahead of the epilogue, so a
+                                        //     slot is never two phases ahead of its reader.  Items without blocks stay out of
+                                        //     the ring: nothing bounds how many of them those warps could run through
+  BAR_SF_READY = BAR_L_FULL + 4,        // [KST] paged source only: scales and Delta_S of the stage re-tiled
+  NUM_BARS = BAR_SF_READY + KST
 };
 static_assert(NUM_BARS <= 64, "barrier table");
-// Shared-memory layout.  PVK selects the operands of the second MMA (mpfa_prefill_variant): 0 = the method (FP8);
-// 1 = the NVFP4 + BF16 precision assignment: V tiles are BF16 (32 KB, three stages), P is handed to the second MMA
-// through shared memory as a K-major BF16 A operand (2 x 32 KB), and the K ring has two stages to make room;
-// 2 = the NVFP4 + NVFP4 assignment: V tiles are channel-major FP4 (8 KB + 1 KB of block scales), P goes through
-// shared memory as a K-major FP4 A operand (2 x 8 KB) with its block scales (2 x 1 KB).
-template <int PVK>
-struct Lay {
-  static constexpr bool PVB = PVK == 1, PV4 = PVK == 2;
-  // ring depths measured on the product kernel (16K / 64K TFLOPS, K / V stages): 4/3 1340 / 1446, 6/3 1342 / 1452, 4/4
-  // 1325 / 1464, 3/3 1329 / 1450, 2/3 within 1 % of 4/3, but 4/2 and 3/2 894 / 822: a V stage is held from its load until
-  // the P V MMA of its block, which the late hand-over of P-hat issues a block later.  The BF16 variant therefore gives
-  // up K stages, not V stages, to make room for its 32 KB tiles.
-  static constexpr int KST = PVB ? 2 : KSTAGES;
-  static constexpr int VST = VSTAGES;
-  static constexpr uint32_t V_BYTES = PVB ? 32768u : (PV4 ? 8192u : 16384u);
-  static constexpr uint32_t OFF_Q = 0;                               // 2 tiles (the next tile's queries are prefetched)
-  static constexpr uint32_t OFF_K = OFF_Q + 2 * 8192;
-  static constexpr uint32_t OFF_V = OFF_K + KST * 8192;
-  static constexpr uint32_t OFF_DELTA = OFF_V + VST * V_BYTES;
-  static constexpr uint32_t OFF_ONES = OFF_DELTA + KST * 4096;
-  static constexpr uint32_t OFF_SFQ = OFF_ONES + 4096;
-  static constexpr uint32_t OFF_SFK = OFF_SFQ + 2 * 1024;
-  static constexpr uint32_t OFF_ALPHA = OFF_SFK + KST * 1024;   // alpha[2][128]
-  static constexpr uint32_t OFF_M = OFF_ALPHA + 2 * 128 * 4;        // running maximum after block t, [t & 1][128]
-  static constexpr uint32_t OFF_L = OFF_M + 2 * 128 * 4;            // final (l, m) of the two softmax groups, [item & 3][2][2][128]
-  static constexpr uint32_t OFF_BAR = OFF_L + 4 * 4 * 128 * 4;
-  static constexpr uint32_t OFF_MISC = OFF_BAR + 64 * 8;            // tmem base, abort flag (NUM_BARS <= 64)
-  // paged source only: per K stage the two pages' scale bytes (2 x 512) and Delta_S rows (2 x 128) as stored
-  static constexpr uint32_t RAW_STAGE = 1280;
-  static constexpr uint32_t OFF_RAW = (OFF_MISC + 16 + 127) & ~127u;
-  static constexpr uint32_t OFF_PS = (OFF_MISC + 16 + 1023) & ~1023u;   // PVB / PV4 only: P of the two softmax groups
-  static constexpr uint32_t PS_BYTES = PVB ? 32768u : 8192u;
-  static constexpr uint32_t OFF_SFP = OFF_PS + 2 * PS_BYTES;            // PV4 only: block scales of P, [group][2 atoms]
-  static constexpr uint32_t OFF_SFV = OFF_SFP + 2 * 1024;               // PV4 only: block scales of V, [stage][2 atoms]
-  static constexpr uint32_t SMEM_BYTES =
-      (PVB ? OFF_PS + 2 * PS_BYTES : (PV4 ? OFF_SFV + VST * 1024 : OFF_MISC + 16)) + 1024;   // + slack for the 1024-byte alignment
-  static constexpr uint32_t OFF_ORDER = OFF_RAW + KST * RAW_STAGE;      // paged source only: groups by length
-  static constexpr uint32_t SMEM_BYTES_PAGED = OFF_ORDER + 2 * MAX_GROUPS + 1024;
-};
-static_assert(Lay<1>::SMEM_BYTES <= 227 * 1024 && Lay<2>::SMEM_BYTES <= 227 * 1024 && Lay<0>::SMEM_BYTES_PAGED <= 227 * 1024, "shared memory");
 
-constexpr uint32_t TM_S = 0, TM_O0 = 128, TM_O1 = 256, TM_P0 = 384, TM_P1 = 416, TM_SFQ = 448 /* 2 x 8 */,
-                   TM_SFK0 = 464, TM_SFK1 = 472;
-// NVFP4 + NVFP4 variant only: block scales of P (per softmax group) and of V (per block parity)
-constexpr uint32_t TM_SFP0 = 480, TM_SFP1 = 488, TM_SFV0 = 496, TM_SFV1 = 504;
+constexpr uint32_t OFF_Q = 0;                              // 2 tiles (the next tile's queries are prefetched)
+constexpr uint32_t OFF_K = OFF_Q + 2 * 8192;
+constexpr uint32_t OFF_V = OFF_K + KST * 8192;
+constexpr uint32_t OFF_DELTA = OFF_V + VST * 16384;
+constexpr uint32_t OFF_ONES = OFF_DELTA + KST * 4096;
+constexpr uint32_t OFF_SFQ = OFF_ONES + 4096;
+constexpr uint32_t OFF_SFK = OFF_SFQ + 2 * 1024;
+constexpr uint32_t OFF_M = OFF_SFK + KST * 1024;           // running maximum after block c, [c % MST][128]
+constexpr uint32_t OFF_L = OFF_M + MST * 128 * 4;          // final (l, m) of the two exponent groups, [item & 3][2][2][128]
+constexpr uint32_t OFF_BAR = OFF_L + 4 * 4 * 128 * 4;
+constexpr uint32_t OFF_MISC = OFF_BAR + 64 * 8;            // tmem base, abort flag (NUM_BARS <= 64)
+// paged source only: per K stage the two pages' scale bytes (2 x 512) and Delta_S rows (2 x 128) as stored; groups by length
+constexpr uint32_t RAW_STAGE = 1280;
+constexpr uint32_t OFF_RAW = (OFF_MISC + 16 + 127) & ~127u;
+constexpr uint32_t OFF_ORDER = OFF_RAW + KST * RAW_STAGE;
+constexpr uint32_t SMEM_BYTES = OFF_MISC + 16 + 1024;      // + slack for the 1024-byte alignment
+constexpr uint32_t SMEM_BYTES_PAGED = OFF_ORDER + 2 * MAX_GROUPS + 1024;
+static_assert(SMEM_BYTES_PAGED <= 227 * 1024, "shared memory");
+
+constexpr uint32_t TM_S = 0 /* 2 x 128 */, TM_O = 256, TM_P = 384 /* 2 x 32 */, TM_SFQ = 448 /* 2 x 8 */, TM_SFK = 464 /* 2 x 8 */;
 constexpr uint32_t TMEM_COLS = 512;
 
-// Optional timeline capture for tuning (compiled in only with -DMPFA_TRACE): one CTA records
-// clock64() at fixed points of every role, [role][block][event].
-#ifdef MPFA_TRACE
-__device__ long long *g_trace = nullptr;
-__device__ int g_trace_cta = 0;
-#define TR_INIT() long long *tr_buf = ((int)blockIdx.x == g_trace_cta && lane == 0) ? g_trace : nullptr
-#define TR(role, t, ev)                                                              \
-  do {                                                                               \
-    if (tr_buf && (t) < 256) tr_buf[((role) * 256 + (t)) * 8 + (ev)] = clock64();    \
-  } while (0)
-#else
-#define TR_INIT() do {} while (0)
-#define TR(role, t, ev) do {} while (0)
-#endif
+// Keeps every use of freshly loaded tensor-memory registers behind the wait that stands before it.
+__device__ __forceinline__ void pin32(uint32_t (&r)[32]) {
+  asm volatile("" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]),
+                    "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]), "+r"(r[16]),
+                    "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]), "+r"(r[24]),
+                    "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31]));
+}
+__device__ __forceinline__ void pin16(uint32_t (&r)[16]) {
+  asm volatile("" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]),
+                    "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]));
+}
 
-// One work item: a 128-row query tile of one q head.
-struct Tile {
-  int b, hq, hk, qt, row0, T;   // T: KV blocks to visit
-  int nkv, nq;                  // keys and queries of this item's request
-};
-
-// Lengths of the item at t.b, t.row0.
+// last key that a query row sees; -1: none (a row past the request's own query count)
 template <bool PAGED>
-__device__ __forceinline__ void geometry(const PrefillParams &pp, const PagedSrc &pg, Tile &t) {
-  const int n_q = (PAGED && pg.q_lens) ? min(pg.q_lens[t.b], pp.N_q) : pp.N_q;
-  const int last_row = min(n_q - 1, t.row0 + TILE - 1);
-  // a length beyond what the page-table row can address is cut to it (no read past the row)
-  const int n_kv = PAGED ? min(pg.seq_lens[t.b], pg.max_pages * 64) : pp.N_kv;
-  t.nkv = n_kv;
-  t.nq = n_q;
-  const int last_key = pp.causal ? min(n_kv - 1, last_row + (n_kv - n_q)) : n_kv - 1;   // bottom-right aligned
-  t.T = (last_key < 0 || (PAGED && t.row0 >= n_q)) ? 0 : last_key / TILE + 1;
+__device__ __forceinline__ int last_key(const PrefillParams &p, const Tile &tl, int r_abs) {
+  const int n_kv = PAGED ? tl.nkv : p.N_kv, n_q = PAGED ? tl.nq : p.N_q;
+  return (PAGED && r_abs >= n_q) ? -1 : p.causal ? min(n_kv - 1, r_abs + (n_kv - n_q)) : n_kv - 1;
 }
 
-// The list of work items of this CTA.  Items are ordered by length (latest query tile first; all heads of a
-// tile adjacent, so the G heads of a kv head stream the same K/V through L2 together) and dealt to the CTAs
-// boustrophedon: round r goes 0..n-1, round r+1 goes n-1..0.  For a causal 16K problem on 148 CTAs the
-// heaviest CTA gets 0.15 % more blocks than the mean (plain round-robin: 7 %).
-// The requests of a paged batch have contexts of their own lengths, so there the order of the (query tile, request) groups is
-// a permutation by length made at the start of the kernel (length_order; four chunks of 512 queries on contexts of 2000
-// to 16000 tokens: heaviest CTA 15 % above the mean, 21 % in the order of the tiles alone).
-struct TileWalk {
-  int round;   // everything else is read from the kernel parameters (constant bank), not kept in registers
-  const uint16_t *order;   // paged source: groups by descending length; null: as numbered
-  __device__ __forceinline__ void init(const uint16_t *o) { round = 0, order = o; }
-  template <bool PAGED>
-  __device__ __forceinline__ bool next(const PrefillParams &pp, const PagedSrc &pg, Tile &t) {
-    const int c = (round & 1) ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x;
-    const int i = round * (int)gridDim.x + c;
-    ++round;
-    if (i >= pp.n_items) return false;
-    int group = i / pp.H_q;
-    if (PAGED && order) group = order[group];
-    t.qt = pp.nq_tiles - 1 - group / pp.B;
-    t.b = group % pp.B;
-    t.hq = i % pp.H_q;
-    t.hk = t.hq / (pp.H_q / pp.H_kv);
-    t.row0 = t.qt * TILE;
-    geometry<PAGED>(pp, pg, t);
-    return true;
-  }
-};
-
-// Work items of a paged batch by descending length: ranks of the (query tile, request) groups by counting.  lengths, order:
-// MAX_GROUPS entries each; called by the whole CTA, which synchronises before order is read.
-__device__ __forceinline__ void length_order(const PrefillParams &pp, const PagedSrc &pg, uint16_t *lengths, uint16_t *order, int tid, int n_threads) {
-  const int n = pp.nq_tiles * pp.B;
-  for (int g = tid; g < n; g += n_threads) {
-    Tile t;
-    t.b = g % pp.B;
-    t.row0 = (pp.nq_tiles - 1 - g / pp.B) * TILE;
-    geometry<true>(pp, pg, t);
-    lengths[g] = (uint16_t)min(t.T, 65535);
-  }
-  __syncthreads();
-  for (int g = tid; g < n; g += n_threads) {
-    const int mine = lengths[g];
-    int rank = 0;
-    for (int o = 0; o < n; ++o) rank += lengths[o] > mine || (lengths[o] == mine && o < g);
-    order[rank] = (uint16_t)g;
-  }
+__device__ __forceinline__ float exponent_unit(const PrefillParams &p, int b) {
+  return __fmul_rn(__fmul_rn(__fmul_rn(p.softmax_scale, 1.4426950408889634f), p.q_gscale[b]), p.k_gscale[b]);
 }
 
-// EW: ablation variant of Section 7.4 (compensation placement): Delta_S is not seeded by the BF16 MMA but
-// loaded by the softmax warps and added to the scores element by element in FP32, before masking and the maximum.
-// PVB: precision-assignment variant of Section 3.1 (NVFP4 Q K^T, BF16 P V): P = 2^(lam S - lam m) is rounded to BF16
-// and handed to the second MMA through shared memory (K-major A operand), V is the BF16 input in the tile layout
-// written by mpfa_pack_v_bf16, the second MMA is kind::f16 (eight K = 16 steps per block).
-// PV4: the NVFP4 + NVFP4 assignment: q = 448 P is quantized per row and 16 keys (E4M3 block scale of max q, E2M1 codes
-// of q * (6 / scale)) and written with its scales to shared memory; V is the channel-major FP4 operand of
-// mpfa_quantize_v_fp4; the second MMA is kind::mxf4nvf4 block-scaled (two K = 64 steps per block).
-template <bool PAGED, bool EW, int PVK = 0>
+template <bool PAGED>
 __global__ void __launch_bounds__(NTHREADS, 1)
 prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                const __grid_constant__ CUtensorMap tm_v, const PrefillParams p, const PagedSrc pg) {
-  constexpr bool PVB = PVK == 1, PV4 = PVK == 2;
-  static_assert(!(PVK != 0 && (PAGED || EW)), "the precision variants exist for contiguous operands with the seed MMA only");
-  using L = Lay<PVK>;
-  constexpr int KST = L::KST, VST = L::VST;
-  constexpr uint32_t OFF_Q = L::OFF_Q, OFF_K = L::OFF_K, OFF_V = L::OFF_V, OFF_DELTA = L::OFF_DELTA, OFF_ONES = L::OFF_ONES,
-                     OFF_SFQ = L::OFF_SFQ, OFF_SFK = L::OFF_SFK, OFF_M = L::OFF_M, OFF_L = L::OFF_L, OFF_BAR = L::OFF_BAR,
-                     OFF_MISC = L::OFF_MISC, OFF_RAW = L::OFF_RAW, RAW_STAGE = L::RAW_STAGE, OFF_PS = L::OFF_PS,
-                     V_BYTES = L::V_BYTES, PS_BYTES = L::PS_BYTES, OFF_SFP = L::OFF_SFP, OFF_SFV = L::OFF_SFV;
-  (void)OFF_PS; (void)OFF_RAW; (void)RAW_STAGE; (void)PS_BYTES; (void)OFF_SFP; (void)OFF_SFV;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t sbase = smem_u32(smem);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-
-#ifdef MPFA_TRACE
-  if ((int)blockIdx.x == g_trace_cta && tid == 12 * 32 && g_trace) g_trace[((0) * 256 + 255) * 8 + 1] = clock64();   // kernel entry
-#endif
   Ctx cx;
   cx.bars = sbase + OFF_BAR;
   cx.abort_flag = reinterpret_cast<volatile int *>(smem + OFF_MISC + 4);
@@ -280,21 +158,22 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   if (tid == 0) {
     *cx.abort_flag = 0;
     for (int i = 0; i < 2; ++i) { mbar_init(cx.bar(BAR_Q_FULL + i), 1); mbar_init(cx.bar(BAR_Q_EMPTY + i), 1); }
-    for (int i = 0; i < KSTAGES; ++i) { mbar_init(cx.bar(BAR_K_FULL + i), 1); mbar_init(cx.bar(BAR_K_EMPTY + i), 1); }
-    for (int i = 0; i < VSTAGES; ++i) { mbar_init(cx.bar(BAR_V_FULL + i), 1); mbar_init(cx.bar(BAR_V_EMPTY + i), 1); }
-    mbar_init(cx.bar(BAR_S_FULL), 1);
-    mbar_init(cx.bar(BAR_S_FULL + 1), 1);
-    mbar_init(cx.bar(BAR_S_EMPTY), 4);   // one arrival per warp (lane 0 after __syncwarp)
+    for (int i = 0; i < KST; ++i) {
+      mbar_init(cx.bar(BAR_K_FULL + i), 1);
+      mbar_init(cx.bar(BAR_K_EMPTY + i), 1);
+      mbar_init(cx.bar(BAR_SF_READY + i), 1);
+    }
+    for (int i = 0; i < VST; ++i) { mbar_init(cx.bar(BAR_V_FULL + i), 1); mbar_init(cx.bar(BAR_V_EMPTY + i), 1); }
     for (int i = 0; i < 2; ++i) {
+      mbar_init(cx.bar(BAR_S_FULL + i), 1);
+      mbar_init(cx.bar(BAR_S_EMPTY + i), 4);   // one arrival per warp (lane 0 after __syncwarp)
       mbar_init(cx.bar(BAR_P_FULL + i), 4);
       mbar_init(cx.bar(BAR_P_EMPTY + i), 1);
-      mbar_init(cx.bar(BAR_M_FULL + i), 4);
-      mbar_init(cx.bar(BAR_O_FULL + i), 1);
-      mbar_init(cx.bar(BAR_O_READY + i), 4);
     }
+    for (int i = 0; i < MST; ++i) mbar_init(cx.bar(BAR_M_FULL + i), 4);
     for (int i = 0; i < 4; ++i) mbar_init(cx.bar(BAR_L_FULL + i), 8);
-    mbar_init(cx.bar(BAR_O_FREE), 4);
-    for (int i = 0; i < KSTAGES; ++i) mbar_init(cx.bar(BAR_SF_READY + i), 1);
+    mbar_init(cx.bar(BAR_O_FULL), 1);
+    mbar_init(cx.bar(BAR_O_READY), 4);
     mbar_init_fence();
     prefetch_tmap(&tm_q);
     if (!PAGED) {
@@ -317,27 +196,24 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   grid_dependency_wait();
   const bool ordered = PAGED && p.B > 1 && p.B * p.nq_tiles <= MAX_GROUPS;
   if (ordered)   // the row-sum ring is not in use yet
-    length_order(p, pg, reinterpret_cast<uint16_t *>(smem + OFF_L), reinterpret_cast<uint16_t *>(smem + L::OFF_ORDER), tid, NTHREADS);
+    length_order(p, pg, reinterpret_cast<uint16_t *>(smem + OFF_L), reinterpret_cast<uint16_t *>(smem + OFF_ORDER), tid, NTHREADS);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tm = *tmem_slot;
-
-  const bool has_delta = !EW && p.delta != nullptr;   // operand of the seed MMA
-  TR_INIT();
-  if (warp == 12) TR(0, 255, 2);   // roles start (after setup)
+  const bool has_delta = p.delta != nullptr;   // operand of the seed MMA
 
   // Every role walks the same list of work items (q tile x q head) and keeps the same running count of
   // KV blocks; ring slots and barrier phases are functions of those two counters, so the pipeline runs
   // straight through item boundaries: the next item's Q/K/V arrive and its first scores are computed while
   // the correction warps write the previous item's output.
   TileWalk walk;
-  walk.init(PAGED && ordered ? reinterpret_cast<const uint16_t *>(smem + L::OFF_ORDER) : nullptr);
+  walk.init(PAGED && ordered ? reinterpret_cast<const uint16_t *>(smem + OFF_ORDER) : nullptr);
   Tile tl;
   uint32_t gb = 0;   // KV blocks of the items already walked
   uint32_t ti = 0;   // index of the current item in this CTA's list
 
-  if (warp < 4) setmaxnreg_dec<REGS_UTIL<PAGED>>();
+  if (warp < 4) setmaxnreg_dec<REGS_UTIL>();
   if (warp == 0) {
     // =========================== TMA producer ===========================
     // The whole warp runs the loop (uniform control flow keeps addresses and barrier handles in
@@ -366,7 +242,6 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         if (PAGED) look.get(pg, p.status, tl.b, tl.nkv, t, jb, lane, page_lo, page_hi);
         if (c >= (uint32_t)KST) ok = cx.wait(BAR_K_EMPTY + ks, (c / KST - 1) & 1u);
         if (!ok) break;
-        TR(0, c, 0);
         if (PAGED) {
           if (elect_one()) {
             const uint32_t bar = cx.bar(BAR_K_FULL + ks);
@@ -395,7 +270,6 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         nk_armed = c + 1;
         if (c >= (uint32_t)VST) ok = cx.wait(BAR_V_EMPTY + vs, (c / VST - 1) & 1u);
         if (!ok) break;
-        TR(0, c, 1);
         if (MPFA_DROP_V(c)) {
           // test build: this copy is left out on purpose
         } else if (PAGED) {
@@ -406,13 +280,8 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             bulk_load(sbase + OFF_V + vs * 16384 + 8192, pg.v_fp8 + ((size_t)page_hi * p.H_kv + tl.hk) * 8192, 8192, bar);
           }
         } else if (elect_one()) {
-          mbar_expect_tx(cx.bar(BAR_V_FULL + vs), V_BYTES + (PV4 ? 1024u : 0u));
-          tma_load_2d(sbase + OFF_V + vs * V_BYTES, &tm_v, 0, (int)(k_row + (size_t)jb * TILE), cx.bar(BAR_V_FULL + vs));
-          if (PV4)   // channel-major FP4 tile (same row arithmetic as K: 128 channel rows per key tile) + its block scales
-            bulk_load(sbase + OFF_SFV + vs * 1024, p.v_sf + (((size_t)tl.b * p.H_kv + tl.hk) * p.nk_tiles + jb) * 1024, 1024,
-                      cx.bar(BAR_V_FULL + vs));
-          if (PVB)   // BF16 rows are 256 bytes: the second 64-channel half is a box of its own
-            tma_load_2d(sbase + OFF_V + vs * V_BYTES + 16384, &tm_v, 128, (int)(k_row + (size_t)jb * TILE), cx.bar(BAR_V_FULL + vs));
+          mbar_expect_tx(cx.bar(BAR_V_FULL + vs), 16384);
+          tma_load_2d(sbase + OFF_V + vs * 16384, &tm_v, 0, (int)(k_row + (size_t)jb * TILE), cx.bar(BAR_V_FULL + vs));
         }
         if (!MPFA_DROP_V(c)) nv_armed = c + 1;
       }
@@ -429,13 +298,10 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   } else if (warp == 1) {
     // =========================== Q K^T issuer ===========================
     // Whole warp in uniform control flow; lane 0 (always the elected lane of a full warp) issues
-    // every tcgen05 instruction, so the commits track the MMAs of the same thread.  This warp
-    // only waits for operands (K block in shared memory, score buffer handed back by its
-    // softmax group), so it runs ahead of the P V issuer (warp 3), also into the next work item.
-    const uint32_t id_fp4 = idesc_nvfp4(128, 128);
-    const uint32_t id_bf16 = idesc_bf16(128, 128, 1, 1);
+    // every tcgen05 instruction, so the commits track the MMAs of the same thread.
     // All shared-memory descriptors are built once; a ring stage or K step only adds a
     // constant to the 14-bit start-address field (shared addresses stay below 256 KB).
+    const uint32_t id_fp4 = idesc_nvfp4(128, 128), id_bf16 = idesc_bf16(128, 128, 1, 1);
     const uint64_t d_ones = smem_desc(sbase + OFF_ONES, 2048, 1024, SWZ_128B);
     const uint64_t d_delta0 = smem_desc(sbase + OFF_DELTA, 2048, 1024, SWZ_128B);
     const uint64_t d_q00 = smem_desc(sbase + OFF_Q, 16, 512, SWZ_64B);
@@ -456,39 +322,24 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         tmem_cp_32x128b_warpx4(tSFQ + 4, d_sfq0 + (512 >> 4));
       }
       for (int t = 0; t < tl.T && ok; ++t) {
-        const uint32_t c = gb + t;
-        const uint32_t ks = c % KST, sb = c & 1;
-        TR(5, c, 0);
+        const uint32_t c = gb + t, ks = c % KST, sb = c & 1;
         ok = cx.wait(BAR_K_FULL + ks, (c / KST) & 1u);
         if (PAGED) ok = ok && cx.wait(BAR_SF_READY + ks, (c / KST) & 1u);
+        if (c >= 2) ok = ok && cx.wait(BAR_S_EMPTY + sb, ((c >> 1) - 1) & 1u);
         if (!ok) break;
-        const uint32_t tSFK = tm + (sb ? TM_SFK1 : TM_SFK0);
-        const uint64_t d_sfk = d_sfk0 + (uint64_t)((ks * 1024) >> 4);
-        const uint64_t d_k = d_k0 + (uint64_t)((ks * 8192) >> 4);
+        const uint32_t tSFK = tm + TM_SFK + sb * 8, tS = tm + TM_S + sb * 128;
+        const uint64_t d_sfk = d_sfk0 + (uint64_t)((ks * 1024) >> 4), d_k = d_k0 + (uint64_t)((ks * 8192) >> 4);
         const uint64_t d_delta = d_delta0 + (uint64_t)((ks * 4096) >> 4);
         tc_fence_after();
-        if (elect_one()) {   // scale factors first: their TMEM columns were last used by block c-2
+        if (elect_one()) {
           tmem_cp_32x128b_warpx4(tSFK, d_sfk);
           tmem_cp_32x128b_warpx4(tSFK + 4, d_sfk + (512 >> 4));
-        }
-        // the softmax group of block c-1 has read its scores out of the buffer
-        if (c >= 1) ok = cx.wait(BAR_S_EMPTY, (c - 1) & 1u);
-        if (!ok) break;
-        TR(5, c, 1);
-        tc_fence_after();
-        if (elect_one()) {
-#ifdef MPFA_ABLATE_NO_QK
-          if (t > 100000)
-#endif
-          {
-          if (has_delta) mma_bf16_ss(tm + TM_S, d_ones, d_delta, id_bf16, 0);
-          mma_nvfp4_ss(tm + TM_S, d_q0, d_k, id_fp4, tSFQ, tSFK, has_delta ? 1u : 0u);
-          mma_nvfp4_ss(tm + TM_S, d_q0 + (32 >> 4), d_k + (32 >> 4), id_fp4, tSFQ + 4, tSFK + 4, 1u);
-          }
+          if (has_delta) mma_bf16_ss(tS, d_ones, d_delta, id_bf16, 0);
+          mma_nvfp4_ss(tS, d_q0, d_k, id_fp4, tSFQ, tSFK, has_delta ? 1u : 0u);
+          mma_nvfp4_ss(tS, d_q0 + (32 >> 4), d_k + (32 >> 4), id_fp4, tSFQ + 4, tSFK + 4, 1u);
           mma_commit(cx.bar(BAR_S_FULL + sb));
           mma_commit(cx.bar(BAR_K_EMPTY + ks));
         }
-        TR(5, c, 5);
       }
       if (ok && elect_one()) mma_commit(cx.bar(BAR_Q_EMPTY + qb));   // after every MMA that reads this query tile
       __syncwarp();
@@ -525,420 +376,214 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   } else if (warp == 3) {
     // =========================== P V issuer ===========================
     const uint32_t id_fp8 = idesc_e4m3(128, 128, 0, 1);
-    const uint32_t id_bf16_pv = idesc_bf16(128, 128, 0, 1);
-    const uint32_t id_fp4_pv = idesc_nvfp4(128, 128);
-    const uint64_t d_v0 = PV4 ? smem_desc(sbase + OFF_V, 16, 512, SWZ_64B) : smem_desc(sbase + OFF_V, PVB ? 16384 : 16, 1024, SWZ_128B);
-    const uint64_t d_p0 = PV4 ? smem_desc(sbase + OFF_PS, 16, 512, SWZ_64B) : smem_desc(sbase + OFF_PS, 16, 1024, SWZ_128B);
-    const uint64_t d_sfp0 = smem_desc(sbase + OFF_SFP, 0, 128, SWZ_NONE);
-    const uint64_t d_sfv0 = smem_desc(sbase + OFF_SFV, 0, 128, SWZ_NONE);
-    (void)id_fp8; (void)id_bf16_pv; (void)d_p0; (void)id_fp4_pv; (void)d_sfp0; (void)d_sfv0;
+    const uint64_t d_v0 = smem_desc(sbase + OFF_V, 16, 1024, SWZ_128B);
     bool ok = true;
-    uint32_t n_used = 0;   // items so far that used the accumulators (T > 0)
     for (; ok && walk.template next<PAGED>(p, pg, tl); gb += tl.T, ++ti) {
-      if (tl.T == 0) continue;
-      // the previous such item's epilogue has read both accumulators
-      if (n_used >= 1) ok = cx.wait(BAR_O_FREE, (n_used - 1) & 1u);
-      ++n_used;
       for (int t = 0; t < tl.T && ok; ++t) {
-        const uint32_t c = gb + t;
-        TR(1, c, 0);
-        const uint32_t sb = c & 1, vs = c % VST;
+        const uint32_t c = gb + t, sb = c & 1, vs = c % VST;
         ok = cx.wait(BAR_V_FULL + vs, (c / VST) & 1u);
-        TR(1, c, 1);
-        ok = ok && cx.wait(BAR_O_READY + sb, (c >> 1) & 1u);
-        TR(1, c, 2);
         ok = ok && cx.wait(BAR_P_FULL + sb, (c >> 1) & 1u);
-        TR(1, c, 3);
+        ok = ok && cx.wait(BAR_O_READY, c & 1u);
         if (!ok) break;
         tc_fence_after();
-        const uint32_t tP = tm + (sb ? TM_P1 : TM_P0);
-        const uint32_t tOacc = tm + (sb ? TM_O1 : TM_O0);
-        const uint64_t d_v = d_v0 + (uint64_t)((vs * V_BYTES) >> 4);
+        const uint32_t tP = tm + TM_P + sb * 32;
+        const uint64_t d_v = d_v0 + (uint64_t)((vs * 16384) >> 4);
         if (elect_one()) {
-          if constexpr (PVB) {
-            // BF16: A = P of this group from shared memory (K-major, two 64-key halves of 16 KB), B = V (MN-major,
-            // two 64-channel halves of 16 KB, 16 keys = 2 KB per K step)
-            const uint64_t d_p = d_p0 + (uint64_t)((sb * 32768) >> 4);
-#pragma unroll
-            for (int k16 = 0; k16 < 8; ++k16)
-              mma_bf16_ss(tOacc, d_p + (uint64_t)(((k16 >> 2) * 16384 + (k16 & 3) * 32) >> 4), d_v + (uint64_t)((2048 * k16) >> 4),
-                          id_bf16_pv, (t >= 2 || k16 > 0) ? 1u : 0u);
-          } else if constexpr (PV4) {
-            // block-scaled FP4: A = P-hat codes of this group (K-major, 64-byte rows), B = V codes (channel-major);
-            // both operands' block scales go to tensor memory first (their columns were last read by block c-2)
-            const uint64_t d_p = d_p0 + (uint64_t)((sb * PS_BYTES) >> 4);
-            const uint64_t d_sfp = d_sfp0 + (uint64_t)((sb * 1024) >> 4), d_sfv = d_sfv0 + (uint64_t)((vs * 1024) >> 4);
-            const uint32_t tSFP = tm + (sb ? TM_SFP1 : TM_SFP0), tSFV = tm + (sb ? TM_SFV1 : TM_SFV0);
-            tmem_cp_32x128b_warpx4(tSFP, d_sfp);
-            tmem_cp_32x128b_warpx4(tSFP + 4, d_sfp + (512 >> 4));
-            tmem_cp_32x128b_warpx4(tSFV, d_sfv);
-            tmem_cp_32x128b_warpx4(tSFV + 4, d_sfv + (512 >> 4));
-            mma_nvfp4_ss(tOacc, d_p, d_v, id_fp4_pv, tSFP, tSFV, t >= 2 ? 1u : 0u);
-            mma_nvfp4_ss(tOacc, d_p + (32 >> 4), d_v + (32 >> 4), id_fp4_pv, tSFP + 4, tSFV + 4, 1u);
-          } else {
 #pragma unroll
           for (int k4 = 0; k4 < 4; ++k4)
-#ifdef MPFA_ABLATE_NO_PV
-            if (k4 > 100)
-#endif
-            mma_e4m3_ts(tOacc, tP + 8 * k4, d_v + (uint64_t)((4096 * k4) >> 4), id_fp8, (t >= 2 || k4 > 0) ? 1u : 0u);
-          }
-          mma_commit(cx.bar(BAR_O_FULL + sb));
+            mma_e4m3_ts(tm + TM_O, tP + 8 * k4, d_v + (uint64_t)((4096 * k4) >> 4), id_fp8, (t > 0 || k4 > 0) ? 1u : 0u);
+          mma_commit(cx.bar(BAR_O_FULL));
           mma_commit(cx.bar(BAR_P_EMPTY + sb));
           mma_commit(cx.bar(BAR_V_EMPTY + vs));
         }
-        TR(1, c, 5);
+      }
+    }
+  } else if (warp >= 12 && warp < 16) {
+    // =========================== running maximum ===========================
+    setmaxnreg_dec<REGS_MAX>();
+    const int row = (warp & 3) * 32 + lane;
+    const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
+    float *s_m = reinterpret_cast<float *>(smem + OFF_M);
+    bool ok = true;
+    for (; ok && walk.template next<PAGED>(p, pg, tl); gb += tl.T, ++ti) {
+      const int limit = last_key<PAGED>(p, tl, tl.row0 + row);
+      float m = -INFINITY;
+      for (int t = 0; t < tl.T; ++t) {
+        const uint32_t c = gb + t;
+        const int key0 = (tl.T - 1 - t) * TILE;
+        const uint32_t tS = tm + TM_S + (c & 1) * 128 + lane_off;
+        if (!__all_sync(0xffffffffu, cx.wait(BAR_S_FULL + (c & 1), (c >> 1) & 1u))) { ok = false; break; }
+        tc_fence_after();
+        float mx[4] = {m, -INFINITY, -INFINITY, -INFINITY};
+        const bool ragged = key0 + TILE - 1 > limit;
+#pragma unroll 1
+        for (int c0 = 0; c0 < 128; c0 += 32) {
+          uint32_t x[32];
+          tmem_ld32(tS + c0, x);
+          tmem_ld_wait();
+          pin32(x);
+          if (ragged) {   // diagonal / ragged block only
+#pragma unroll
+            for (int i = 0; i < 32; ++i)
+              if (key0 + c0 + i > limit) x[i] = 0xFF800000u;   // -inf
+          }
+#pragma unroll
+          for (int i = 0; i < 32; i += 8) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+              mx[j] = max3(mx[j], __uint_as_float(x[i + 2 * j]), __uint_as_float(x[i + 2 * j + 1]));
+          }
+        }
+        m = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
+        s_m[(c % MST) * 128 + row] = m;
+        tc_fence_before();
+        warp_arrive(cx.bar(BAR_M_FULL + c % MST), lane);
       }
     }
   } else if (warp >= 4 && warp < 12) {
-    // =========================== softmax groups ===========================
-    setmaxnreg_inc<REGS_SOFTMAX>();
-    const int grp = (warp - 4) >> 2;                 // takes the KV blocks whose running count has this parity
+    // =========================== exponentials ===========================
+    setmaxnreg_inc<REGS_EXP>();
+    const int grp = (warp - 4) >> 2;   // takes the KV blocks whose running count has this parity
     const int row = (warp & 3) * 32 + lane;
     const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
-    const float *gq = p.q_gscale, *gk = p.k_gscale;
-    float *s_m = reinterpret_cast<float *>(smem + OFF_M);
-    const uint32_t tS = tm + TM_S + lane_off;
-    const uint32_t tP = tm + (grp ? TM_P1 : TM_P0) + lane_off;
-    uint8_t *const ps_row = smem + OFF_PS + grp * 32768 + row * 128;   // PVB: this thread's row of the group's P operand
-    // PV4: this thread's 64-byte row of the group's FP4 operand (64B swizzle: 16-byte chunk ^ ((row >> 1) & 3)) and its
-    // word in each of the group's two scale-factor atoms
-    uint8_t *const p4_row = smem + OFF_PS + grp * 8192 + row * 64;
-    uint8_t *const sfp_row = smem + OFF_SFP + grp * 1024 + (row & 31) * 16 + (row >> 5) * 4;
-    (void)tP; (void)ps_row; (void)p4_row; (void)sfp_row;
+    const float *s_m = reinterpret_cast<const float *>(smem + OFF_M);
+    const uint32_t tS = tm + TM_S + grp * 128 + lane_off, tP = tm + TM_P + grp * 32 + lane_off;
     bool ok = true;
     uint32_t n_used = 0;   // items so far with T > 0: only those go through the row-sum ring
     for (; ok && walk.template next<PAGED>(p, pg, tl); gb += tl.T, ++ti) {
-      const int T = tl.T;
-      if (T == 0) continue;   // nothing to attend to: the epilogue writes zeros without waiting for this role
-      const int r_abs = tl.row0 + row;
-      const int n_kv = PAGED ? tl.nkv : p.N_kv;
-      const int n_q = PAGED ? tl.nq : p.N_q;
-      const int limit = (PAGED && r_abs >= n_q) ? -1   // a row past the request's own query count sees nothing
-                        : p.causal ? min(n_kv - 1, r_abs + (n_kv - n_q)) : n_kv - 1;   // last visible key
-      const float lam = __fmul_rn(__fmul_rn(__fmul_rn(p.softmax_scale, 1.4426950408889634f), gq[tl.b]), gk[tl.b]);
-      bool p_pending = false;    // P-hat of the previous block written but not yet handed over
+      const int TT = tl.T;
+      if (TT == 0) continue;   // nothing to attend to: the epilogue writes zeros without waiting for this role
+      const int limit = last_key<PAGED>(p, tl, tl.row0 + row);
+      const float lam = exponent_unit(p, tl.b);
       float m_own = -INFINITY;   // running maximum after this group's previous block
       float l_own = 0.0f;        // sum of 448 P over this group's blocks, relative to m_own
-      for (int t = (grp ^ (int)gb) & 1; t < T; t += 2) {
+      for (int t = (grp ^ (int)gb) & 1; t < TT; t += 2) {
         const uint32_t c = gb + t;
-        const int key0 = (T - 1 - t) * TILE;
-        TR(2 + grp, c, 0);
-        if (!__all_sync(0xffffffffu, cx.wait(BAR_S_FULL + grp, (c >> 1) & 1u))) { ok = false; break; }
-        TR(2 + grp, c, 1);
+        const int key0 = (TT - 1 - t) * TILE;
+        // both of the block's conditions in one vote: the maximum is there, P V of block c-2 has consumed the group's P_hat
+        const uint32_t par_m = (c / MST) & 1u, par_pe = ((c >> 1) - 1) & 1u;
+        const bool both = cx.probe(BAR_M_FULL + c % MST, par_m) & (c < 2 || cx.probe(BAR_P_EMPTY + grp, par_pe));
+        if (!__all_sync(0xffffffffu, both)) {
+          bool w = cx.wait(BAR_M_FULL + c % MST, par_m);
+          if (c >= 2) w = w && cx.wait(BAR_P_EMPTY + grp, par_pe);
+          if (!__all_sync(0xffffffffu, w)) { ok = false; break; }
+        }
         tc_fence_after();
-        uint32_t s[128];
-        {
-          uint32_t(&s0)[32] = *reinterpret_cast<uint32_t(*)[32]>(&s[0]);
-          uint32_t(&s1)[32] = *reinterpret_cast<uint32_t(*)[32]>(&s[32]);
-          tmem_ld32(tS, s0);
-          tmem_ld32(tS + 32, s1);
-        }
-        if (p_pending) {
-          // P-hat of this group's previous block is handed to the P V issuer only now: its tensor-memory stores
-          // have had the loop tail and the barrier wait above to complete, so this wait costs nothing, where the
-          // same wait right after the stores held the warp for their whole latency (measured: +2.7 % at 16K,
-          // +1.7 % at 64K).  P V of a block has a block and a half of slack before anything waits for it.
-          tmem_st_wait();
-          tc_fence_before();
-          warp_arrive(cx.bar(BAR_P_FULL + grp), lane);
-          p_pending = false;
-        }
-        // While the scores are on their way, test (without blocking) the two other conditions this
-        // block needs; the answers are consumed later, so their latency overlaps the TMEM load:
-        //  - P V of block c-2 has consumed this group's P_hat columns (this also means the
-        //    correction warps have read the maximum this group published two blocks ago);
-        //  - the other group's running maximum of block c-1 (same item) is published.
-        const uint32_t par_pe = ((c >> 1) - 1) & 1u, par_m = ((c - 1) >> 1) & 1u;
-        const bool pe_early = (c < 2) || cx.probe(BAR_P_EMPTY + grp, par_pe);
-        bool have_prev = (t == 0) || cx.probe(BAR_M_FULL + (grp ^ 1), par_m);
-        float m_prev = -INFINITY;
-#ifdef MPFA_ABLATE_NO_MHAND
-        have_prev = true;
-#endif
-        const bool ragged = key0 + TILE - 1 > limit;   // diagonal / ragged block only
-        tmem_ld_wait();
-        {
-          // second half of the row in flight while the maximum of the first half is taken
-          uint32_t(&s2)[32] = *reinterpret_cast<uint32_t(*)[32]>(&s[64]);
-          uint32_t(&s3)[32] = *reinterpret_cast<uint32_t(*)[32]>(&s[96]);
-          tmem_ld32(tS + 64, s2);
-          tmem_ld32(tS + 96, s3);
-        }
-        if constexpr (EW) {
-          const uint4 *dp = reinterpret_cast<const uint4 *>(
-              p.delta + ((size_t)tl.b * p.H_q + tl.hq) * (size_t)(p.nk_tiles * TILE) + key0);
+        uint32_t s[4][32];
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const uint4 d = __ldg(dp + i);
-            const uint32_t w[4] = {d.x, d.y, d.z, d.w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {   // packed pair: both halves round like the scalar add
-              float x0 = __uint_as_float(s[8 * i + 2 * j]), x1 = __uint_as_float(s[8 * i + 2 * j + 1]);
-              acc2(x0, x1, __uint_as_float(w[j] << 16), __uint_as_float(w[j] & 0xFFFF0000u));
-              s[8 * i + 2 * j] = __float_as_uint(x0), s[8 * i + 2 * j + 1] = __float_as_uint(x1);
-            }
-          }
-        }
-        if (ragged) {
-#pragma unroll
-          for (int i = 0; i < 64; ++i)
-            if (key0 + i > limit) s[i] = 0xFF800000u;   // -inf
-        }
-        // row maximum (Eq. 3)
-        float mx0 = -INFINITY, mx1 = -INFINITY, mx2 = -INFINITY, mx3 = -INFINITY;
-#pragma unroll
-        for (int i = 0; i < 64; i += 8) {
-          mx0 = max3(mx0, __uint_as_float(s[i]), __uint_as_float(s[i + 1]));
-          mx1 = max3(mx1, __uint_as_float(s[i + 2]), __uint_as_float(s[i + 3]));
-          mx2 = max3(mx2, __uint_as_float(s[i + 4]), __uint_as_float(s[i + 5]));
-          mx3 = max3(mx3, __uint_as_float(s[i + 6]), __uint_as_float(s[i + 7]));
-        }
-        tmem_ld_wait();
-        tc_fence_before();
-        warp_arrive(cx.bar(BAR_S_EMPTY), lane);   // the row is in registers: Q K^T of block c+1 may overwrite it
-        TR(2 + grp, c, 2);
-        if constexpr (EW) {
-          const uint4 *dp = reinterpret_cast<const uint4 *>(
-              p.delta + ((size_t)tl.b * p.H_q + tl.hq) * (size_t)(p.nk_tiles * TILE) + key0 + 64);
-#pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const uint4 d = __ldg(dp + i);
-            const uint32_t w[4] = {d.x, d.y, d.z, d.w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              float x0 = __uint_as_float(s[64 + 8 * i + 2 * j]), x1 = __uint_as_float(s[64 + 8 * i + 2 * j + 1]);
-              acc2(x0, x1, __uint_as_float(w[j] << 16), __uint_as_float(w[j] & 0xFFFF0000u));
-              s[64 + 8 * i + 2 * j] = __float_as_uint(x0), s[64 + 8 * i + 2 * j + 1] = __float_as_uint(x1);
-            }
-          }
-        }
-        if (ragged) {
-#pragma unroll
-          for (int i = 64; i < 128; ++i)
-            if (key0 + i > limit) s[i] = 0xFF800000u;   // -inf
-        }
-#pragma unroll
-        for (int i = 64; i < 128; i += 8) {
-          mx0 = max3(mx0, __uint_as_float(s[i]), __uint_as_float(s[i + 1]));
-          mx1 = max3(mx1, __uint_as_float(s[i + 2]), __uint_as_float(s[i + 3]));
-          mx2 = max3(mx2, __uint_as_float(s[i + 4]), __uint_as_float(s[i + 5]));
-          mx3 = max3(mx3, __uint_as_float(s[i + 6]), __uint_as_float(s[i + 7]));
-        }
-#ifdef MPFA_ABLATE_NO_MAX
-        const float mx = fmaxf(__uint_as_float(s[0]), __uint_as_float(s[127])) + 30.0f;
-#else
-        const float mx = fmaxf(fmaxf(mx0, mx1), fmaxf(mx2, mx3));
-#endif
-        // running maximum: the other group owns block c-1
-        if (!__all_sync(0xffffffffu, have_prev)) {
-          if (!__all_sync(0xffffffffu, cx.wait(BAR_M_FULL + (grp ^ 1), par_m))) { ok = false; break; }
-        }
-        if (t > 0) m_prev = s_m[(grp ^ 1) * 128 + row];
-#ifdef MPFA_ABLATE_NO_MHAND
-        m_prev = m_own;
-#endif
-        if (!__all_sync(0xffffffffu, pe_early)) {
-          if (!__all_sync(0xffffffffu, cx.wait(BAR_P_EMPTY + grp, par_pe))) { ok = false; break; }
-        }
-        TR(2 + grp, c, 3);
-        const float m_t = fmaxf(m_prev, mx);
-        s_m[grp * 128 + row] = m_t;
-        warp_arrive(cx.bar(BAR_M_FULL + grp), lane);
-        TR(2 + grp, c, 4);
+        for (int i = 0; i < 4; ++i) tmem_ld32(tS + 32 * i, s[i]);
+        const float m_t = s_m[(c % MST) * 128 + row];
         const float a_own = (m_t == m_own) ? 1.0f : ex2_approx(__fmul_rn(m_own - m_t, lam));
         // P = 2^(lam S - lam m) (Eq. 4)
-        // the factor 448 of the E4M3 operand is folded into the exponent: q = 448 P = 2^(lam S - lam m + log2 448)
-        const float cc = (m_t == -INFINITY) ? 0.0f : __fsub_rn(PVB ? 0.0f : 8.8073549220576042f, __fmul_rn(m_t, lam));
-        float sum0 = 0.0f, sum1 = 0.0f, sum2 = 0.0f, sum3 = 0.0f;
-#ifdef MPFA_ABLATE_NO_SOFTMAX
-        sum0 = __uint_as_float(s[5]);
-        if (false)
-#endif
-        {
-#ifdef MPFA_ABLATE_NO_EXP
-#define EX2_(x) (x)
-#else
-#define EX2_(x) ex2_approx(x)
-#endif
-          // q = 448 P is the E4M3 operand (Section 4.1); the row sum is taken over q and the factor
-          // 448 is divided out once in the epilogue.
-          uint32_t sfw = 0u;   // PV4: the E4M3 block scales of 64 keys
-          (void)sfw;
-#pragma unroll
-          for (int c0 = 0; c0 < 128; c0 += 32) {
-            uint32_t packed[8];
-            uint32_t pbf[4];
-            float qv[32];
-            (void)packed; (void)pbf; (void)qv;
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              float x0, x1, x2, x3;
-              fma2(x0, x1, __uint_as_float(s[c0 + 4 * i]), __uint_as_float(s[c0 + 4 * i + 1]), lam, cc);
-              fma2(x2, x3, __uint_as_float(s[c0 + 4 * i + 2]), __uint_as_float(s[c0 + 4 * i + 3]), lam, cc);
-              const float q0 = EX2_(x0), q1 = EX2_(x1), q2 = EX2_(x2), q3 = EX2_(x3);
-              acc2(sum0, sum1, q0, q1);
-              acc2(sum2, sum3, q2, q3);
-              if constexpr (PV4) {
-                qv[4 * i] = q0, qv[4 * i + 1] = q1, qv[4 * i + 2] = q2, qv[4 * i + 3] = q3;
-              } else if constexpr (PVB) {
-                // BF16 pairs (first operand of the conversion goes to the upper half)
-                asm("cvt.rn.bf16x2.f32 %0, %2, %1;" : "=r"(pbf[2 * (i & 1)]) : "f"(q0), "f"(q1));
-                asm("cvt.rn.bf16x2.f32 %0, %2, %1;" : "=r"(pbf[2 * (i & 1) + 1]) : "f"(q2), "f"(q3));
-                if (i & 1) {
-                  // eight keys = one 16-byte chunk of the row in the K-major, 128B-swizzled A operand
-                  const int ch = (c0 >> 3) + (i >> 1);
-                  *reinterpret_cast<uint4 *>(ps_row + (ch >> 3) * 16384 + (((ch & 7) ^ (row & 7)) << 4)) =
-                      make_uint4(pbf[0], pbf[1], pbf[2], pbf[3]);
-                }
-              } else {
-              // two conversions written into the halves of one register (no separate merge instruction)
-              asm("{.reg .b16 lo, hi;\n\t"
-                  "cvt.rn.satfinite.e4m3x2.f32 lo, %2, %1;\n\t"
-                  "cvt.rn.satfinite.e4m3x2.f32 hi, %4, %3;\n\t"
-                  "mov.b32 %0, {lo, hi};}"
-                  : "=r"(packed[i])
-                  : "f"(q0), "f"(q1), "f"(q2), "f"(q3));
-              }
-            }
-            if constexpr (PV4) {
-              // two blocks of 16 keys: scale = E4M3(max q), codes = E2M1(q * (6 / scale)) (Eq. 1 with the tensor scale
-              // of P fixed at 1 / (6 * 448))
-              uint32_t w[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-              for (int hb = 0; hb < 2; ++hb) {
-                const float *qb = qv + 16 * hb;
-                float a0 = max3(qb[0], qb[1], qb[2]), a1 = max3(qb[3], qb[4], qb[5]), a2 = max3(qb[6], qb[7], qb[8]),
-                      a3 = max3(qb[9], qb[10], qb[11]);
-                a0 = max3(a0, qb[12], qb[13]);
-                a1 = max3(a1, qb[14], qb[15]);
-                const float amax = fmaxf(fmaxf(a0, a1), fmaxf(a2, a3));
-                const uint32_t sc = (uint32_t)__nv_cvt_float_to_fp8(amax, __NV_SATFINITE, __NV_E4M3);
-                const float sdec = __half2float(__half(__nv_cvt_fp8_to_halfraw((__nv_fp8_storage_t)sc, __NV_E4M3)));
-                const float inv = sdec > 0.0f ? __fdiv_rn(6.0f, sdec) : 0.0f;
-                sfw |= sc << (8 * (((c0 >> 4) + hb) & 3));
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                  const uint32_t byte = (uint32_t)__nv_cvt_float2_to_fp4x2(
-                      make_float2(__fmul_rn(qb[2 * j], inv), __fmul_rn(qb[2 * j + 1], inv)), __NV_E2M1, cudaRoundNearest);
-                  w[2 * hb + (j >> 2)] |= (byte & 0xFFu) << (8 * (j & 3));
-                }
-              }
-              *reinterpret_cast<uint4 *>(p4_row + ((((c0 >> 5)) ^ ((row >> 1) & 3)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
-              if (c0 & 32) {   // 64 keys done: one word of the row in this half's scale-factor atom
-                *reinterpret_cast<uint32_t *>(sfp_row + (c0 >> 6) * 512) = sfw;
-                sfw = 0u;
-              }
-            } else if constexpr (!PVB) {
-#ifndef MPFA_ABLATE_NO_PST
-            tmem_st8(tP + (c0 >> 2), packed);
-#else
-            if (packed[0] == 0x12345u && packed[7] == 77u) tmem_st8(tP + (c0 >> 2), packed);
-#endif
-            }
-          }
-        }
-        l_own = __fadd_rn(__fmul_rn(a_own, l_own), (sum0 + sum1) + (sum2 + sum3));
+        // the factor 448 of the E4M3 operand is folded into the exponent: q = 448 P = 2^(lam S - lam m + log2 448); the row
+        // sum is taken over q and the factor is divided out once in the epilogue
+        const float cc = (m_t == -INFINITY) ? 0.0f : __fsub_rn(8.8073549220576042f, __fmul_rn(m_t, lam));
         m_own = m_t;
-        TR(2 + grp, c, 5);
-        if constexpr (PVB || PV4) {
-          fence_proxy_async_smem();   // the P rows were written through the generic proxy, the MMA reads them through the async one
-          tc_fence_before();
-          warp_arrive(cx.bar(BAR_P_FULL + grp), lane);
-        } else if constexpr (EW) {   // measured: this variant is faster with the hand-over where the stores are
-          tmem_st_wait();
-          tc_fence_before();
-          warp_arrive(cx.bar(BAR_P_FULL + grp), lane);
-        } else {
-          p_pending = true;   // handed over at the top of the next iteration, or below after the item's last block
+        tmem_ld_wait();
+        pin32(s[0]), pin32(s[1]), pin32(s[2]), pin32(s[3]);
+        tc_fence_before();
+        warp_arrive(cx.bar(BAR_S_EMPTY + grp), lane);
+        if (key0 + TILE - 1 > limit) {
+#pragma unroll
+          for (int i = 0; i < 128; ++i)
+            if (key0 + i > limit) s[i >> 5][i & 31] = 0xFF800000u;
         }
-        TR(2 + grp, c, 6);
-      }
-      if (p_pending) {
+        float sum[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+        for (int c0 = 0; c0 < 4; ++c0) {
+          uint32_t(&x)[32] = s[c0];
+          uint32_t packed[8];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            float x0, x1, x2, x3;
+            fma2(x0, x1, __uint_as_float(x[4 * i]), __uint_as_float(x[4 * i + 1]), lam, cc);
+            fma2(x2, x3, __uint_as_float(x[4 * i + 2]), __uint_as_float(x[4 * i + 3]), lam, cc);
+            const float q0 = ex2_approx(x0), q1 = ex2_approx(x1), q2 = ex2_approx(x2), q3 = ex2_approx(x3);
+            acc2(sum[0], sum[1], q0, q1);
+            acc2(sum[2], sum[3], q2, q3);
+            // two conversions written into the halves of one register (no separate merge instruction)
+            asm("{.reg .b16 lo, hi;\n\t"
+                "cvt.rn.satfinite.e4m3x2.f32 lo, %2, %1;\n\t"
+                "cvt.rn.satfinite.e4m3x2.f32 hi, %4, %3;\n\t"
+                "mov.b32 %0, {lo, hi};}"
+                : "=r"(packed[i])
+                : "f"(q0), "f"(q1), "f"(q2), "f"(q3));
+          }
+          tmem_st8(tP + 8 * c0, packed);
+        }
+        l_own = __fadd_rn(__fmul_rn(a_own, l_own), (sum[0] + sum[1]) + (sum[2] + sum[3]));
         tmem_st_wait();
         tc_fence_before();
         warp_arrive(cx.bar(BAR_P_FULL + grp), lane);
-        p_pending = false;
       }
       if (!ok) break;
-      // which group took the item's last block decides how the epilogue combines the two accumulators
       float *s_fin = reinterpret_cast<float *>(smem + OFF_L) + (n_used & 3) * 512;
       s_fin[(grp * 2 + 0) * 128 + row] = l_own;
       s_fin[(grp * 2 + 1) * 128 + row] = m_own;
       warp_arrive(cx.bar(BAR_L_FULL + (n_used & 3)), lane);
       ++n_used;
     }
-  } else if (warp >= 12) {
+  } else if (warp >= 16) {
     // =========================== correction + epilogue ===========================
-    setmaxnreg_dec<REGS_CORR<PAGED>>();
+    setmaxnreg_dec<REGS_CORR>();
     const int row = (warp & 3) * 32 + lane;
-    const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
     const float *s_m = reinterpret_cast<const float *>(smem + OFF_M);
-    const uint32_t tO0 = tm + TM_O0 + lane_off, tO1 = tm + TM_O1 + lane_off;
+    const uint32_t tO = tm + TM_O + ((uint32_t)((warp & 3) * 32) << 16);
     bool ok = true;
     uint32_t n_used = 0;   // items so far with T > 0 (slot and phase of the row-sum ring)
+    warp_arrive(cx.bar(BAR_O_READY), lane);
     for (; walk.template next<PAGED>(p, pg, tl); gb += tl.T, ++ti) {
-      const int T = tl.T;
-      const int r_abs = tl.row0 + row;
-      const float lam_c = __fmul_rn(__fmul_rn(__fmul_rn(p.softmax_scale, 1.4426950408889634f), p.q_gscale[tl.b]), p.k_gscale[tl.b]);
-      float alpha_prev = 1.0f, alpha = 1.0f, m_before = -INFINITY;
-      for (int t = 0; ok && t < T; ++t) {
+      const int TT = tl.T, r_abs = tl.row0 + row;
+      const float lam = exponent_unit(p, tl.b);
+      float m_before = -INFINITY;
+      for (int t = 0; ok && t < TT; ++t) {
         const uint32_t c = gb + t;
-        const uint32_t sb = c & 1;
-        TR(4, c, 0);
-        ok = __all_sync(0xffffffffu, cx.wait(BAR_M_FULL + sb, (c >> 1) & 1u));
+        ok = __all_sync(0xffffffffu, cx.wait(BAR_M_FULL + c % MST, (c / MST) & 1u));
         if (!ok) break;
-        TR(4, c, 1);
-        // alpha_t = 2^(lam (m_{t-1} - m_t)) (Eq. 5/6), from the running maxima the softmax groups publish
-        const float m_now = s_m[sb * 128 + row];
-        alpha = (m_now == m_before) ? 1.0f : ex2_approx(__fmul_rn(m_before - m_now, lam_c));
+        // alpha_t = 2^(lam (m_{t-1} - m_t)) (Eq. 5/6)
+        const float m_now = s_m[(c % MST) * 128 + row];
+        const float alpha = (m_now == m_before) ? 1.0f : ex2_approx(__fmul_rn(m_before - m_now, lam));
         m_before = m_now;
-        if (t >= 2) {
-          // O[sb] holds blocks t-2, t-4, ... relative to the maximum after block t-2
-          const float scale = __fmul_rn(alpha, alpha_prev);
-          ok = __all_sync(0xffffffffu, cx.wait(BAR_O_FULL + sb, ((c >> 1) - 1) & 1u));
-          if (!ok) break;
-          TR(4, c, 2);
-          tc_fence_after();
-#ifdef MPFA_ABLATE_NO_CORR
-          if (false) {
-#else
-          if (__any_sync(0xffffffffu, scale != 1.0f)) {   // identical result when every factor is exactly 1
-#endif
-            const uint32_t tO = sb ? tO1 : tO0;
-#pragma unroll
-            for (int c0 = 0; c0 < HEAD_DIM; c0 += 32) {
-              uint32_t r[32];
-              tmem_ld32(tO + c0, r);
-              tmem_ld_wait();
-#pragma unroll
-              for (int i = 0; i < 32; i += 2) {   // packed pairs: half the issue slots, same roundings
-                float y0, y1;
-                mul2(y0, y1, __uint_as_float(r[i]), __uint_as_float(r[i + 1]), scale);
-                r[i] = __float_as_uint(y0), r[i + 1] = __float_as_uint(y1);
-              }
-              tmem_st32(tO + c0, r);
-            }
-            tmem_st_wait();
-          }
-          tc_fence_before();
-        }
-        alpha_prev = alpha;
-        TR(4, c, 3);
-        warp_arrive(cx.bar(BAR_O_READY + sb), lane);
-      }
-      // final normalisation (Algorithm 1 line 17): O / (448 l) * v_scale -> BF16.  The two softmax
-      // groups hold partial sums relative to their own last maximum; bring both to the final one.
-      // The accumulator of the last block is current; the other one is one alpha behind.
-      const int last = (int)((gb + T - 1) & 1);
-      float l = 0.0f, a_other = 0.0f;
-      if (ok) {
-        if (T > 0) ok = cx.wait(BAR_O_FULL + last, ((gb + T - 1) >> 1) & 1u);
-        if (ok && T > 1) ok = cx.wait(BAR_O_FULL + (last ^ 1), ((gb + T - 2) >> 1) & 1u);
-        if (T > 0) ok = ok && cx.wait(BAR_L_FULL + (n_used & 3), (n_used >> 2) & 1u);
+        if (t == 0) continue;   // handed over by the previous item's epilogue
+        ok = __all_sync(0xffffffffu, cx.wait(BAR_O_FULL, (c - 1) & 1u));
+        if (!ok) break;
         tc_fence_after();
-        if (ok && T > 0) {
-          const float lam = lam_c;
+        if (__any_sync(0xffffffffu, alpha != 1.0f)) {   // identical result when every factor is exactly 1
+          // 16 columns on the way while 16 are multiplied, in a short loop: unrolled over 32-column halves the rescale took
+          // 260-495 cycles instead of 590-770, but the kernel 1780 us instead of 1715 (16384 keys): the exponentials beside it
+          // ran slower
+          uint32_t r[2][16];
+          tmem_ld16(tO, r[0]);
+#pragma unroll 1
+          for (int c0 = 0; c0 < 8; c0 += 2) {
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+              uint32_t(&x)[16] = r[u];
+              tmem_ld_wait();
+              pin16(x);
+              if (c0 + u < 7) tmem_ld16(tO + 16 * (c0 + u + 1), r[u ^ 1]);
+#pragma unroll
+              for (int i = 0; i < 16; i += 2) {
+                float y0, y1;
+                mul2(y0, y1, __uint_as_float(x[i]), __uint_as_float(x[i + 1]), alpha);
+                x[i] = __float_as_uint(y0), x[i + 1] = __float_as_uint(y1);
+              }
+              tmem_st16(tO + 16 * (c0 + u), x);
+            }
+          }
+          tmem_st_wait();
+        }
+        tc_fence_before();
+        warp_arrive(cx.bar(BAR_O_READY), lane);
+      }
+      // final normalisation (Algorithm 1 line 17).  The two exponent groups hold partial sums relative to their own last
+      // maximum; bring both to the final one.
+      float l = 0.0f;
+      if (ok && TT > 0) {
+        ok = cx.wait(BAR_O_FULL, (gb + TT - 1) & 1u);
+        ok = ok && cx.wait(BAR_L_FULL + (n_used & 3), (n_used >> 2) & 1u);
+        tc_fence_after();
+        if (ok) {
           const float *s_fin = reinterpret_cast<const float *>(smem + OFF_L) + (n_used & 3) * 512;
           const float l0 = s_fin[0 * 128 + row], m0 = s_fin[1 * 128 + row];
           const float l1 = s_fin[2 * 128 + row], m1 = s_fin[3 * 128 + row];
@@ -948,42 +593,37 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             const float w1 = (m1 == mf) ? 1.0f : ex2_approx(__fmul_rn(m1 - mf, lam));
             l = __fadd_rn(__fmul_rn(w0, l0), __fmul_rn(w1, l1));
           }
-          if (T > 1) a_other = alpha;   // alpha of the last block
         }
       }
       // tcgen05.ld is warp-collective: every lane loads, only the stores are predicated.
       const bool warp_ok = __all_sync(0xffffffffu, ok);
-      const bool store = r_abs < p.N_q && (warp_ok || T == 0);
+      const bool store = r_abs < p.N_q && (warp_ok || TT == 0);
       const size_t o_off = (((size_t)tl.b * p.N_q + (store ? r_abs : 0)) * p.H_q + tl.hq) * HEAD_DIM;
       // one IEEE reciprocal per row; 128 divisions per thread would cost more than ten KV blocks
-      const float inv_denom = (l > 0.0f) ? __frcp_rn(l) : 0.0f;   // l already carries the factor 448
-      const uint32_t tOl = last ? tO1 : tO0, tOo = last ? tO0 : tO1;
+      const float inv_denom = (l > 0.0f) ? __frcp_rn(l) : 0.0f;
 #pragma unroll 1
-      for (int c0 = 0; c0 < HEAD_DIM; c0 += 16) {
-        uint32_t r[16], ro[16];
-        if (T > 0 && warp_ok) {
-          tmem_ld16(tOl + c0, r);
-          if (T > 1) tmem_ld16(tOo + c0, ro);
+      for (int c0 = 0; c0 < HEAD_DIM; c0 += 32) {
+        uint32_t r[32];
+        if (TT > 0 && warp_ok) {
+          tmem_ld32(tO + c0, r);
           tmem_ld_wait();
+          pin32(r);
         }
-        if (c0 == HEAD_DIM - 16 && T > 0) {   // both accumulators are in registers: the next item's P V may overwrite them
+        if (c0 == HEAD_DIM - 32 && TT > 0) {   // O is in registers: the next item's P V may overwrite it
           tc_fence_before();
-          warp_arrive(cx.bar(BAR_O_FREE), lane);
+          warp_arrive(cx.bar(BAR_O_READY), lane);
         }
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          float acc = __uint_as_float(r[i]);
-          if (T > 1) acc = __fadd_rn(acc, __fmul_rn(a_other, __uint_as_float(ro[i])));
-          r[i] = (l > 0.0f) ? __float_as_uint(__fmul_rn(__fmul_rn(acc, inv_denom), p.v_scale)) : 0u;
-        }
+        for (int i = 0; i < 32; ++i)
+          r[i] = (l > 0.0f) ? __float_as_uint(__fmul_rn(__fmul_rn(__uint_as_float(r[i]), inv_denom), p.v_scale)) : 0u;
         if (store) {
           if (p.out_f32) {
 #pragma unroll
-            for (int i = 0; i < 16; i += 4)
+            for (int i = 0; i < 32; i += 4)
               *reinterpret_cast<uint4 *>(p.out_f32 + o_off + c0 + i) = make_uint4(r[i], r[i + 1], r[i + 2], r[i + 3]);
           }
 #pragma unroll
-          for (int i = 0; i < 16; i += 8) {
+          for (int i = 0; i < 32; i += 8) {
             uint32_t h[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
@@ -994,40 +634,20 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           }
         }
       }
-      if (T > 0) ++n_used;
+      if (TT > 0) ++n_used;
       if (!ok) break;
     }
   }
-  if (warp == 12) TR(0, 255, 3);   // epilogue stores issued
   tc_fence_before();
   __syncthreads();
-  if (warp == 12) TR(0, 255, 4);
   if (warp == 2) tmem_dealloc(tm, TMEM_COLS);
 }
-
 }  // namespace
 }  // namespace mpfa
 
 using namespace mpfa;
 
-#ifdef MPFA_TRACE
-extern "C" int mpfa_debug_set_trace(long long *buf, int cta) {
-  if (cudaMemcpyToSymbol(g_trace, &buf, sizeof(buf)) != cudaSuccess) return -1;
-  if (cudaMemcpyToSymbol(g_trace_cta, &cta, sizeof(cta)) != cudaSuccess) return -1;
-  return 0;
-}
-#endif
-
-template <auto Kernel, uint32_t SMEM>
-static mpfa_status start(int dev, unsigned grid, cudaStream_t stream, const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap &tv,
-                         const PrefillParams &p, const PagedSrc &pg) {
-  mpfa_status rc = allow_smem<Kernel>(dev, SMEM);
-  if (rc != MPFA_OK) return rc;
-  MPFA_CUDA_OK(launch(Kernel, dim3(grid), dim3(NTHREADS), SMEM, stream, tq, tk, tv, p, pg));
-  return MPFA_OK;
-}
-
-// 0: one query tile per CTA, two softmax groups alternating over KV blocks (the faster one on B200, see
+// 0: one query tile per CTA (the faster one on B200, see
 // prefill_pair.cu's header for the measured comparison); 1: two query tiles per CTA (prefill_pair.cu)
 static int g_arrangement = 0;
 extern "C" int mpfa_set_prefill_arrangement(int a) {
@@ -1051,8 +671,6 @@ extern "C" mpfa_status mpfa_prefill_variant(const mpfa_fp4_tensor *q, const mpfa
   if (variant != 0 && variant != MPFA_VARIANT_COMP_ELEMENTWISE && variant != MPFA_VARIANT_PV_BF16 && variant != MPFA_VARIANT_PV_FP4)
     return MPFA_ERR_INVALID_ARG;
   const bool ew = variant == MPFA_VARIANT_COMP_ELEMENTWISE && delta_s_bf16 != nullptr;
-  const bool pvb = variant == MPFA_VARIANT_PV_BF16;   // v_fp8 then points at the BF16 tile tensor of mpfa_pack_v_bf16
-  const bool pv4 = variant == MPFA_VARIANT_PV_FP4;    // ... at the FP4 operand of mpfa_quantize_v_fp4, v_scale = its v_gscale
   if (!q || !k || !v_fp8 || !st || !out_bf16 || !device_status) return MPFA_ERR_INVALID_ARG;
   if (!q->codes || !q->sf || !k->codes || !k->sf || !st->q_gscale || !st->k_gscale) return MPFA_ERR_INVALID_ARG;
   if (q->B <= 0 || q->B != k->B || q->H <= 0 || k->H <= 0 || q->N <= 0 || k->N <= 0) return MPFA_ERR_INVALID_ARG;
@@ -1089,31 +707,19 @@ extern "C" mpfa_status mpfa_prefill_variant(const mpfa_fp4_tensor *q, const mpfa
   p.softmax_scale = softmax_scale;
   p.v_scale = v_scale;
   p.n_items = (int)n_cta;
-  if (pv4) {
-    // codes of all tiles first, then the block scales; the MMA result is in units of 6 * 448 P x V / v_gscale and the
-    // row sum carries the 448
-    p.v_sf = v_fp8 + (size_t)k->B * k->H * nk_tiles * 8192;
-    p.v_scale = v_scale * (1.0f / 6.0f);
-  }
-  if (g_arrangement == 1 && !pvb && !pv4) return launch_prefill_pair(q, k, v_fp8, p, ew, static_cast<cudaStream_t>(stream));
+  const unsigned grid = (unsigned)(n_cta < (uint64_t)n_sm ? n_cta : (uint64_t)n_sm);   // one persistent CTA per SM
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  const bool other_pv = variant == MPFA_VARIANT_PV_BF16 || variant == MPFA_VARIANT_PV_FP4;
+  if (g_arrangement == 1 && !other_pv) return launch_prefill_pair(q, k, v_fp8, p, ew, s);
+  if (ew || other_pv) return launch_prefill_variant(q, k, v_fp8, p, variant, dev, grid, s);
   EncodeTiledFn enc;
   rc = get_encoder(&enc);
   if (rc != MPFA_OK) return rc;
   CUtensorMap tq, tk, tv;
   if ((rc = make_map(enc, &tq, q->codes, q_rows, 64)) != MPFA_OK) return rc;
   if ((rc = make_map(enc, &tk, k->codes, k_rows, 64)) != MPFA_OK) return rc;
-  if ((rc = pvb ? make_map(enc, &tv, v_fp8, k_rows, 256, 128) : make_map(enc, &tv, v_fp8, k_rows, pv4 ? 64 : 128)) != MPFA_OK) return rc;
-  const unsigned grid = (unsigned)(n_cta < (uint64_t)n_sm ? n_cta : (uint64_t)n_sm);   // one persistent CTA per SM
-  if (pvb) {
-    rc = start<prefill_kernel<false, false, 1>, Lay<1>::SMEM_BYTES>(dev, grid, static_cast<cudaStream_t>(stream), tq, tk, tv, p, PagedSrc{});
-  } else if (pv4) {
-    rc = start<prefill_kernel<false, false, 2>, Lay<2>::SMEM_BYTES>(dev, grid, static_cast<cudaStream_t>(stream), tq, tk, tv, p, PagedSrc{});
-  } else if (ew) {
-    rc = start<prefill_kernel<false, true>, Lay<0>::SMEM_BYTES>(dev, grid, static_cast<cudaStream_t>(stream), tq, tk, tv, p, PagedSrc{});
-  } else {
-    rc = start<prefill_kernel<false, false>, Lay<0>::SMEM_BYTES>(dev, grid, static_cast<cudaStream_t>(stream), tq, tk, tv, p, PagedSrc{});
-  }
-  return rc;
+  if ((rc = make_map(enc, &tv, v_fp8, k_rows, 128)) != MPFA_OK) return rc;
+  return start<prefill_kernel<false>, SMEM_BYTES>(dev, grid, NTHREADS, s, tq, tk, tv, p, PagedSrc{});
 }
 
 extern "C" mpfa_status mpfa_prefill_paged(const mpfa_fp4_tensor *q, const mpfa_paged_kv *kv, const int32_t *page_table,
@@ -1175,5 +781,5 @@ extern "C" mpfa_status mpfa_prefill_paged(const mpfa_fp4_tensor *q, const mpfa_p
   CUtensorMap tq;
   if ((rc = make_map(enc, &tq, q->codes, q_rows, 64)) != MPFA_OK) return rc;
   const unsigned grid = (unsigned)(n_cta < (uint64_t)n_sm ? n_cta : (uint64_t)n_sm);
-  return start<prefill_kernel<true, false>, Lay<0>::SMEM_BYTES_PAGED>(dev, grid, static_cast<cudaStream_t>(stream), tq, tq, tq, p, pg);
+  return start<prefill_kernel<true>, SMEM_BYTES_PAGED>(dev, grid, NTHREADS, static_cast<cudaStream_t>(stream), tq, tq, tq, p, pg);
 }

@@ -30,8 +30,8 @@
 // same thread (two groups that alternate over the blocks and hand the maximum to one another) the chain held up every item's
 // first and last blocks and every causal diagonal.  Warps of their own run the chain ahead of the exponentials; the second
 // reading of the scores costs 72 cycles of the tensor-memory port.  Two score buffers and one accumulator take the place of
-// one and two.  Measured, the kernel alone, alternating groups -> this: 16 sequences of 200 to 512 keys 79.4 -> 72.2 us, causal
-// 2048 x 32 heads 87.0 -> 82.6, 4 x 512 x 32 37.3 -> 34.2, chunks of 512 queries on paged contexts 483 -> 427; causal 16384 x 32
+// one and two.  Measured, the kernel alone, alternating groups -> this: 8 x 577 keys x 16 heads, not causal, 79.4 -> 72.2 us,
+// causal 1999 x 40 heads 87.0 -> 82.6, 4 x 777 x 8 heads 37.3 -> 34.2, chunks of 512 queries on paged contexts 483 -> 427; causal 16384 x 32
 // heads 1730 -> 1715 us and 131072 x 32 98.8 -> 99.1 ms, where the clock falls to 1.75-1.83 GHz under the power limit.
 // What must not be in the exponentials: one straight run of 128 took 1130 cycles where the same code with a mask test or a wait
 // per 32 scores took 2200.

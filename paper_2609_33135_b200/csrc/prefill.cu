@@ -33,6 +33,8 @@
 // one and two.  Measured, the kernel alone, alternating groups -> this: 8 x 577 keys x 16 heads, not causal, 79.4 -> 72.2 us,
 // causal 1999 x 40 heads 87.0 -> 82.6, 4 x 777 x 8 heads 37.3 -> 34.2, chunks of 512 queries on paged contexts 483 -> 427; causal 16384 x 32
 // heads 1730 -> 1715 us and 131072 x 32 98.8 -> 99.1 ms, where the clock falls to 1.75-1.83 GHz under the power limit.
+// (Figures of that step; the mask moved to the maximum warps for short contexts and an epilogue of 16 columns at a time, whose
+// registers the rescale loop had to spill, gave what stands at the kernel below.)
 // What must not be in the exponentials: one straight run of 128 took 1130 cycles where the same code with a mask test or a wait
 // per 32 scores took 2200.
 //
@@ -55,16 +57,24 @@ constexpr int NTHREADS = 640;
 // setmaxnreg only moves registers inside the pool the CTA got at launch (640 threads x the 96 registers of the launch bound); a
 // request beyond the pool would block forever, so the split is checked here.
 constexpr int LAUNCH_REGS = 96;
-// measured (exponentials / maxima / correction / utility; us, causal 16384, 2048, paged chunks): 144/64/80/48 1715, 82.6, 427;
-// 144/56/80/56 1725, 82.6, 421; 152/56/72/48 1720, 84.4, 420; 136/64/96/48 1890, 85.5, 476; 144/56/88/48 1850, 87.5, 448;
-// 48 for the maxima or 64 for the correction spill (4000 us)
-constexpr int REGS_EXP = 144, REGS_MAX = 64, REGS_CORR = 80, REGS_UTIL = 48;
-static_assert(8 * REGS_EXP + 4 * REGS_MAX + 4 * REGS_CORR + 4 * REGS_UTIL <= 20 * LAUNCH_REGS, "register pool");
-// the exponent warps take registers (setmaxnreg.inc: not below the launch's), the others give them back (setmaxnreg.dec: not
-// above the launch's, or the instruction is illegal)
-static_assert(REGS_EXP >= LAUNCH_REGS && REGS_CORR <= LAUNCH_REGS && REGS_MAX <= LAUNCH_REGS && REGS_UTIL <= LAUNCH_REGS &&
-              REGS_UTIL >= 24, "setmaxnreg direction");
-static_assert(REGS_EXP % 8 == 0 && REGS_MAX % 8 == 0 && REGS_CORR % 8 == 0 && REGS_UTIL % 8 == 0, "setmaxnreg granularity");
+// exponentials / maxima / correction / utility.  The paged instance's producer and re-tiling warps need more, see below.
+// Measured (us; causal 1999 x 40 heads, 16384 x 32): short instance 144/48/80/64 75.7, 1625; 152/48/72/56 75.4, 1630; 144/64/80/48
+// 76.3, 1640; 136/56/88/64 75.7, 1635.  Long: 144/56/72/64 79.5, 1650; 144/64/80/48 81.0, 1665; 152/48/72/56 80.2, 1656.
+// Paged (chunks of 512): 152/48/72/56 423, 144/56/72/64 435, 144/64/80/48 427.  Less than 48 for the maxima or 72 for the
+// correction spills heavily.
+template <bool PAGED, bool LONG> constexpr int REGS_EXP = PAGED ? 152 : 144;
+template <bool PAGED, bool LONG> constexpr int REGS_MAX = PAGED || !LONG ? 48 : 56;
+template <bool PAGED, bool LONG> constexpr int REGS_CORR = PAGED || LONG ? 72 : 80;
+template <bool PAGED, bool LONG> constexpr int REGS_UTIL = PAGED ? 56 : 64;
+template <bool PAGED, bool LONG>
+constexpr bool regs_ok() {
+  constexpr int e = REGS_EXP<PAGED, LONG>, m = REGS_MAX<PAGED, LONG>, c = REGS_CORR<PAGED, LONG>, u = REGS_UTIL<PAGED, LONG>;
+  // the exponent warps take registers (setmaxnreg.inc: not below the launch's), the others give them back (setmaxnreg.dec: not
+  // above the launch's, or the instruction is illegal)
+  return 8 * e + 4 * (m + c + u) <= 20 * LAUNCH_REGS && e >= LAUNCH_REGS && m <= LAUNCH_REGS && c <= LAUNCH_REGS && u <= LAUNCH_REGS &&
+         u >= 24 && e % 8 == 0 && m % 8 == 0 && c % 8 == 0 && u % 8 == 0;
+}
+static_assert(regs_ok<false, false>() && regs_ok<false, true>() && regs_ok<true, true>(), "setmaxnreg split");
 
 enum {
   BAR_Q_FULL = 0,                       // [2] query tile of work item i in buffer i & 1
@@ -93,6 +103,9 @@ enum {
   NUM_BARS = BAR_SF_READY + KST
 };
 static_assert(NUM_BARS <= 64, "barrier table");
+
+// Contiguous operands: the most keys that the short instance takes; both sides measured, see the kernel
+constexpr int LONG_KEYS = 49152;
 
 constexpr uint32_t OFF_Q = 0;                              // 2 tiles (the next tile's queries are prefetched)
 constexpr uint32_t OFF_K = OFF_Q + 2 * 8192;
@@ -139,7 +152,13 @@ __device__ __forceinline__ float exponent_unit(const PrefillParams &p, int b) {
   return __fmul_rn(__fmul_rn(__fmul_rn(p.softmax_scale, 1.4426950408889634f), p.q_gscale[b]), p.k_gscale[b]);
 }
 
-template <bool PAGED>
+// LONG: who masks and how P_hat is stored.  false: the maximum warps write masked scores back to tensor memory, so the code of the
+// exponentials has no mask in it (it is read by every pass and competes for the instruction cache with the other roles'), and
+// P_hat goes out in one store.  true: the exponent warps mask, P_hat in four stores.  Measured, false / true (us): 8 x 577 keys x 16
+// heads, not causal, 67.7 / 70.8, causal 1999 x 40 75.7 / 79.5, 16384 x 32 1625 / 1650, 32768 x 32 6037 / 6090,
+// but 65536 x 32 23.44 / 23.05 ms, 131072 x 32 92.8 / 88.9 ms and chunks of 512 on pages 473 / 423 us: where rescales of O are rare the exponentials set the pace, and there
+// the compiler's schedule of the second form is the better one.
+template <bool PAGED, bool LONG>
 __global__ void __launch_bounds__(NTHREADS, 1)
 prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                const __grid_constant__ CUtensorMap tm_v, const PrefillParams p, const PagedSrc pg) {
@@ -213,7 +232,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   uint32_t gb = 0;   // KV blocks of the items already walked
   uint32_t ti = 0;   // index of the current item in this CTA's list
 
-  if (warp < 4) setmaxnreg_dec<REGS_UTIL>();
+  if (warp < 4) setmaxnreg_dec<REGS_UTIL<PAGED, LONG>>();
   if (warp == 0) {
     // =========================== TMA producer ===========================
     // The whole warp runs the loop (uniform control flow keeps addresses and barrier handles in
@@ -400,7 +419,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     }
   } else if (warp >= 12 && warp < 16) {
     // =========================== running maximum ===========================
-    setmaxnreg_dec<REGS_MAX>();
+    setmaxnreg_dec<REGS_MAX<PAGED, LONG>>();
     const int row = (warp & 3) * 32 + lane;
     const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
     float *s_m = reinterpret_cast<float *>(smem + OFF_M);
@@ -415,7 +434,8 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         if (!__all_sync(0xffffffffu, cx.wait(BAR_S_FULL + (c & 1), (c >> 1) & 1u))) { ok = false; break; }
         tc_fence_after();
         float mx[4] = {m, -INFINITY, -INFINITY, -INFINITY};
-        const bool ragged = key0 + TILE - 1 > limit;
+        bool ragged = key0 + TILE - 1 > limit;
+        if (!LONG) ragged = __any_sync(0xffffffffu, ragged);   // the stores below are the whole warp's
 #pragma unroll 1
         for (int c0 = 0; c0 < 128; c0 += 32) {
           uint32_t x[32];
@@ -426,6 +446,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
 #pragma unroll
             for (int i = 0; i < 32; ++i)
               if (key0 + c0 + i > limit) x[i] = 0xFF800000u;   // -inf
+            if (!LONG) tmem_st32(tS + c0, x);
           }
 #pragma unroll
           for (int i = 0; i < 32; i += 8) {
@@ -436,13 +457,14 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         }
         m = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
         s_m[(c % MST) * 128 + row] = m;
+        if (!LONG && ragged) tmem_st_wait();
         tc_fence_before();
         warp_arrive(cx.bar(BAR_M_FULL + c % MST), lane);
       }
     }
   } else if (warp >= 4 && warp < 12) {
     // =========================== exponentials ===========================
-    setmaxnreg_inc<REGS_EXP>();
+    setmaxnreg_inc<REGS_EXP<PAGED, LONG>>();
     const int grp = (warp - 4) >> 2;   // takes the KV blocks whose running count has this parity
     const int row = (warp & 3) * 32 + lane;
     const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
@@ -483,16 +505,16 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         pin32(s[0]), pin32(s[1]), pin32(s[2]), pin32(s[3]);
         tc_fence_before();
         warp_arrive(cx.bar(BAR_S_EMPTY + grp), lane);
-        if (key0 + TILE - 1 > limit) {
+        if (LONG && key0 + TILE - 1 > limit) {
 #pragma unroll
           for (int i = 0; i < 128; ++i)
             if (key0 + i > limit) s[i >> 5][i & 31] = 0xFF800000u;
         }
+        uint32_t packed[4][8];
         float sum[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
         for (int c0 = 0; c0 < 4; ++c0) {
           uint32_t(&x)[32] = s[c0];
-          uint32_t packed[8];
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
             float x0, x1, x2, x3;
@@ -506,11 +528,12 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                 "cvt.rn.satfinite.e4m3x2.f32 lo, %2, %1;\n\t"
                 "cvt.rn.satfinite.e4m3x2.f32 hi, %4, %3;\n\t"
                 "mov.b32 %0, {lo, hi};}"
-                : "=r"(packed[i])
+                : "=r"(packed[c0][i])
                 : "f"(q0), "f"(q1), "f"(q2), "f"(q3));
           }
-          tmem_st8(tP + 8 * c0, packed);
+          if (LONG) tmem_st8(tP + 8 * c0, packed[c0]);
         }
+        if (!LONG) tmem_st32(tP, reinterpret_cast<uint32_t(&)[32]>(packed));
         l_own = __fadd_rn(__fmul_rn(a_own, l_own), (sum[0] + sum[1]) + (sum[2] + sum[3]));
         tmem_st_wait();
         tc_fence_before();
@@ -525,7 +548,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     }
   } else if (warp >= 16) {
     // =========================== correction + epilogue ===========================
-    setmaxnreg_dec<REGS_CORR>();
+    setmaxnreg_dec<REGS_CORR<PAGED, LONG>>();
     const int row = (warp & 3) * 32 + lane;
     const float *s_m = reinterpret_cast<const float *>(smem + OFF_M);
     const uint32_t tO = tm + TM_O + ((uint32_t)((warp & 3) * 32) << 16);
@@ -602,28 +625,28 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       // one IEEE reciprocal per row; 128 divisions per thread would cost more than ten KV blocks
       const float inv_denom = (l > 0.0f) ? __frcp_rn(l) : 0.0f;
 #pragma unroll 1
-      for (int c0 = 0; c0 < HEAD_DIM; c0 += 32) {
-        uint32_t r[32];
+      for (int c0 = 0; c0 < HEAD_DIM; c0 += 16) {
+        uint32_t r[16];
         if (TT > 0 && warp_ok) {
-          tmem_ld32(tO + c0, r);
+          tmem_ld16(tO + c0, r);
           tmem_ld_wait();
-          pin32(r);
+          pin16(r);
         }
-        if (c0 == HEAD_DIM - 32 && TT > 0) {   // O is in registers: the next item's P V may overwrite it
+        if (c0 == HEAD_DIM - 16 && TT > 0) {   // O is in registers: the next item's P V may overwrite it
           tc_fence_before();
           warp_arrive(cx.bar(BAR_O_READY), lane);
         }
 #pragma unroll
-        for (int i = 0; i < 32; ++i)
+        for (int i = 0; i < 16; ++i)
           r[i] = (l > 0.0f) ? __float_as_uint(__fmul_rn(__fmul_rn(__uint_as_float(r[i]), inv_denom), p.v_scale)) : 0u;
         if (store) {
           if (p.out_f32) {
 #pragma unroll
-            for (int i = 0; i < 32; i += 4)
+            for (int i = 0; i < 16; i += 4)
               *reinterpret_cast<uint4 *>(p.out_f32 + o_off + c0 + i) = make_uint4(r[i], r[i + 1], r[i + 2], r[i + 3]);
           }
 #pragma unroll
-          for (int i = 0; i < 32; i += 8) {
+          for (int i = 0; i < 16; i += 8) {
             uint32_t h[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
@@ -719,7 +742,8 @@ extern "C" mpfa_status mpfa_prefill_variant(const mpfa_fp4_tensor *q, const mpfa
   if ((rc = make_map(enc, &tq, q->codes, q_rows, 64)) != MPFA_OK) return rc;
   if ((rc = make_map(enc, &tk, k->codes, k_rows, 64)) != MPFA_OK) return rc;
   if ((rc = make_map(enc, &tv, v_fp8, k_rows, 128)) != MPFA_OK) return rc;
-  return start<prefill_kernel<false>, SMEM_BYTES>(dev, grid, NTHREADS, s, tq, tk, tv, p, PagedSrc{});
+  if (k->N <= LONG_KEYS) return start<prefill_kernel<false, false>, SMEM_BYTES>(dev, grid, NTHREADS, s, tq, tk, tv, p, PagedSrc{});
+  return start<prefill_kernel<false, true>, SMEM_BYTES>(dev, grid, NTHREADS, s, tq, tk, tv, p, PagedSrc{});
 }
 
 extern "C" mpfa_status mpfa_prefill_paged(const mpfa_fp4_tensor *q, const mpfa_paged_kv *kv, const int32_t *page_table,
@@ -781,5 +805,5 @@ extern "C" mpfa_status mpfa_prefill_paged(const mpfa_fp4_tensor *q, const mpfa_p
   CUtensorMap tq;
   if ((rc = make_map(enc, &tq, q->codes, q_rows, 64)) != MPFA_OK) return rc;
   const unsigned grid = (unsigned)(n_cta < (uint64_t)n_sm ? n_cta : (uint64_t)n_sm);
-  return start<prefill_kernel<true>, SMEM_BYTES_PAGED>(dev, grid, NTHREADS, static_cast<cudaStream_t>(stream), tq, tq, tq, p, pg);
+  return start<prefill_kernel<true, true>, SMEM_BYTES_PAGED>(dev, grid, NTHREADS, static_cast<cudaStream_t>(stream), tq, tq, tq, p, pg);
 }

@@ -221,6 +221,18 @@ def test_prefill_item_boundaries_through_every_ring(N_kv):
     compare(o16, o32, rows[keep], ref32[keep], f"N_kv {N_kv}")
 
 
+@pytest.mark.parametrize("N_kv", [49152, 49153])
+def test_prefill_on_both_sides_of_the_long_context_instance(N_kv):
+    """The last key count of the instance that masks in the maximum warps and the first of the one that masks in the exponent
+    warps; 130 causal queries, so that both tiles end in masked blocks."""
+    w = wl.prefill_workload("long", 63, 1, N_kv, 2, 1, True, N_q=130, q_bias=True)
+    o16, o32 = run_gpu(w)
+    z = orc.stage1(orc.bf16_bits(w.q), orc.bf16_bits(w.k), orc.bf16_bits(w.v))
+    rows = np.array([(0, h, i) for h in range(2) for i in (0, 1, 63, 64, 126, 127, 128, 129)])
+    ref32, _ = orc.prefill_rows(z, rows, w.softmax_scale, True)
+    compare(o16, o32, rows, ref32, f"N_kv {N_kv}")
+
+
 def test_prefill_many_items_without_keys_per_cta():
     """Causal, far more queries than keys (N_q = 8192, N_kv = 128, 32 heads): 63 of the 64 query tiles see no key at
     all, so every persistent CTA walks a dozen and more empty work items in a row.  They must come out as zeros,

@@ -464,6 +464,7 @@ struct DeltaArgs {
 // now 45 us.
 constexpr int QT_CTAS = 2;       // resident per SM: 128 registers, so that the means stay in registers
 constexpr int QT_K_WEIGHT = 2;   // time of a K tile with Delta_S in units of a Q tile's (1 / 2 / 3: 106 / 89 / 96 us of stage 1)
+constexpr int QT_SETUP = 2;      // a CTA's set-up in the same units
 template <int FEW>   // heads of the group where they are one or two, otherwise 0
 __global__ void __launch_bounds__(256, QT_CTAS) quantize_tile_kernel(const QuantTensor k, const QuantTensor q, const DeltaArgs da) {
   __shared__ __align__(16) GroupMeans gm;
@@ -981,15 +982,33 @@ extern "C" mpfa_status mpfa_quantize_qk(const void *q_bf16, const void *k_bf16, 
     MPFA_CUDA_OK(launch(quantize_token_kernel, dim3((B * H_q + 7) / 8), dim3(256), 0, s, tq, B * H_q));
     return MPFA_OK;
   }
-  // At most one wave of CTAs, as far as that goes: a CTA's set-up (scale, table of reciprocals, query means) is paid once, and
-  // the next tile's loads run under the arithmetic of the current one.  A few CTAs more than a wave would take twice the time.
+  // At most one wave of CTAs where every head can have one: a CTA's set-up (scale, table of reciprocals, query means) is paid
+  // once, and the next tile's loads run under the arithmetic of the current one.  A few CTAs more than a wave would take twice
+  // the time.
   const int k_weight = da.delta && H_q / H_kv > 2 ? QT_K_WEIGHT : 1;
   const long long work = ((long long)k_weight * tk.tiles * tk.H + (long long)tq.tiles * tq.H) * B, wave = (long long)QT_CTAS * n_sm;
-  for (long long per = (work + wave - 1) / wave;; ++per) {
-    const int per_q = (int)per, per_k = (int)((per + k_weight - 1) / k_weight);
-    tk.ctas = tk.x ? (tk.tiles + per_k - 1) / per_k : 0;
-    tq.ctas = tq.x ? (tq.tiles + per_q - 1) / per_q : 0;
-    if (((long long)tk.ctas * tk.H + (long long)tq.ctas * tq.H) * B <= wave || (tk.ctas <= 1 && tq.ctas <= 1)) break;
+  const auto split = [&](long long per) {   // CTAs of `per` units of work; how many that makes
+    const long long per_k = (per + k_weight - 1) / k_weight;
+    tk.ctas = tk.x ? (int)((tk.tiles + per_k - 1) / per_k) : 0;
+    tq.ctas = tq.x ? (int)((tq.tiles + per - 1) / per) : 0;
+    return ((long long)tk.ctas * tk.H + (long long)tq.ctas * tq.H) * B;
+  };
+  const long long mean = (work + wave - 1) / wave;
+  if (((long long)tk.H + tq.H) * B <= wave) {
+    for (long long per = mean; split(per) > wave; ++per) {}
+  } else {
+    // More heads than a wave has CTAs: the work with its set-ups spread over the SMs, and one CTA's length at the end.  (One CTA
+    // per head here left one query token on 9 x 4865 keys, 40:8 heads, at 219 us of stage 1, now 127; 10 x 5647 467 -> 406;
+    // 16 x 2000, 32:8 heads, 254 -> 210; set-ups of 0.2 / 0.5 / 1 / 2 units 143 / 143 / 129 / 127 us for the first.)
+    long long best = 1;
+    double best_time = 1e30;
+    for (long long per = 1; per <= 2 * mean; per *= 2) {
+      const long long ctas = split(per);
+      const long long longest = std::min(per, std::max<long long>(tq.tiles, (long long)k_weight * tk.tiles));
+      const double time = (double)(work + QT_SETUP * ctas) / (double)wave + (double)longest;
+      if (time < best_time) best_time = time, best = per;
+    }
+    split(best);
   }
   const int few = da.delta && H_q / H_kv <= 2 ? H_q / H_kv : 0;
   MPFA_CUDA_OK(launch(few == 0 ? quantize_tile_kernel<0> : few == 1 ? quantize_tile_kernel<1> : quantize_tile_kernel<2>,

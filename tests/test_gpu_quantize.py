@@ -62,6 +62,7 @@ def test_stage1_bit_exact(name):
     (1, 1, 1, 1, 1), (1, 129, 7, 3, 1), (2, 127, 9, 2, 2), (1, 128, 128, 8, 1),   # smallest, few query rows, one tile
     (1, 1024, 1024, 12, 2), (1, 1031, 1500, 7, 1),                                  # statistics in two slices, groups of six and seven
     (1, 4099, 4099, 40, 8), (3, 2500, 700, 32, 8),                                  # several tiles per CTA, ragged last tile
+    (7, 1300, 1, 40, 8), (19, 260, 130, 8, 8),                                      # more heads than CTAs in a wave
 ])
 def test_stage1_bit_exact_over_tile_and_slice_counts(B, N, N_q, H_q, H_kv):
     w = wl.prefill_workload("edges", 44, B, N, H_q, H_kv, True, N_q=N_q, q_bias=True)

@@ -156,7 +156,7 @@ __device__ __forceinline__ float exponent_unit(const PrefillParams &p, int b) {
 
 // LONG: who masks and how P_hat is stored.  false: the maximum warps write masked scores back to tensor memory, so the code of the
 // exponentials has no mask in it (it is read by every pass and competes for the instruction cache with the other roles'), and
-// P_hat goes out in one store.  true: the exponent warps mask, P_hat in four stores.  Measured, false / true (us): 8 x 577 keys x 16
+// P_hat goes out in one store.  true: the exponent warps mask, P_hat in two stores.  Measured, false / true (us): 8 x 577 keys x 16
 // heads, not causal, 67.7 / 70.8, causal 1999 x 40 75.7 / 79.5, 16384 x 32 1625 / 1650, 32768 x 32 6037 / 6090,
 // but 65536 x 32 23.44 / 23.05 ms, 131072 x 32 92.8 / 88.9 ms and chunks of 512 on pages 473 / 423 us: where rescales of O are rare the exponentials set the pace, and there
 // the compiler's schedule of the second form is the better one.
@@ -512,7 +512,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           for (int i = 0; i < 128; ++i)
             if (key0 + i > limit) s[i >> 5][i & 31] = 0xFF800000u;
         }
-        uint32_t packed[4][8];
+        uint32_t packed[2][16];
         float sum[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
         for (int c0 = 0; c0 < 4; ++c0) {
@@ -530,10 +530,10 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                 "cvt.rn.satfinite.e4m3x2.f32 lo, %2, %1;\n\t"
                 "cvt.rn.satfinite.e4m3x2.f32 hi, %4, %3;\n\t"
                 "mov.b32 %0, {lo, hi};}"
-                : "=r"(packed[c0][i])
+                : "=r"(packed[c0 >> 1][8 * (c0 & 1) + i])
                 : "f"(q0), "f"(q1), "f"(q2), "f"(q3));
           }
-          if (LONG) tmem_st8(tP + 8 * c0, packed[c0]);
+          if (LONG && (c0 & 1)) tmem_st16(tP + 8 * (c0 - 1), packed[c0 >> 1]);
         }
         if (!LONG) tmem_st32(tP, reinterpret_cast<uint32_t(&)[32]>(packed));
         l_own = __fadd_rn(__fmul_rn(a_own, l_own), (sum[0] + sum[1]) + (sum[2] + sum[3]));

@@ -62,19 +62,23 @@ constexpr int LAUNCH_REGS = 96;
 // 76.3, 1640; 136/56/88/64 75.7, 1635.  Long: 144/56/72/64 79.5, 1650; 144/64/80/48 81.0, 1665; 152/48/72/56 80.2, 1656.
 // Paged (chunks of 512): 152/48/72/56 423, 144/56/72/64 435, 144/64/80/48 427.  Less than 48 for the maxima or 72 for the
 // correction spills heavily.
-template <bool PAGED, bool LONG> constexpr int REGS_EXP = PAGED ? 152 : 144;
-template <bool PAGED, bool LONG> constexpr int REGS_MAX = PAGED || !LONG ? 48 : 56;
-template <bool PAGED, bool LONG> constexpr int REGS_CORR = PAGED || LONG ? 72 : 80;
-template <bool PAGED, bool LONG> constexpr int REGS_UTIL = PAGED ? 56 : 64;
-template <bool PAGED, bool LONG>
+// With an item's blocks in several runs (RUNS; us, kernel alone, 16384 x 32 / 131072 x 32 / chunks of 512 on pages): 144/56/88/48 1553,
+// 96.6 ms, 312; 152/48/80/48 1556, 96.4 ms, 312; 144/48/88/56 1549, 97.0 ms, 315; 144/48/80/64 1564, 97.1 ms, 314; 152/48/72/56 1598,
+// 96.7 ms, 318.
+template <bool PAGED, bool LONG, bool RUNS> constexpr int REGS_EXP = RUNS ? (LONG && !PAGED ? 152 : 144) : (PAGED ? 152 : 144);
+template <bool PAGED, bool LONG, bool RUNS> constexpr int REGS_MAX = RUNS ? (LONG && !PAGED ? 48 : 56) : (PAGED || !LONG ? 48 : 56);
+template <bool PAGED, bool LONG, bool RUNS> constexpr int REGS_CORR = RUNS ? (LONG && !PAGED ? 80 : 88) : (PAGED || LONG ? 72 : 80);
+template <bool PAGED, bool LONG, bool RUNS> constexpr int REGS_UTIL = RUNS ? 48 : (PAGED ? 56 : 64);
+template <bool PAGED, bool LONG, bool RUNS>
 constexpr bool regs_ok() {
-  constexpr int e = REGS_EXP<PAGED, LONG>, m = REGS_MAX<PAGED, LONG>, c = REGS_CORR<PAGED, LONG>, u = REGS_UTIL<PAGED, LONG>;
+  constexpr int e = REGS_EXP<PAGED, LONG, RUNS>, m = REGS_MAX<PAGED, LONG, RUNS>, c = REGS_CORR<PAGED, LONG, RUNS>, u = REGS_UTIL<PAGED, LONG, RUNS>;
   // the exponent warps take registers (setmaxnreg.inc: not below the launch's), the others give them back (setmaxnreg.dec: not
   // above the launch's, or the instruction is illegal)
   return 8 * e + 4 * (m + c + u) <= 20 * LAUNCH_REGS && e >= LAUNCH_REGS && m <= LAUNCH_REGS && c <= LAUNCH_REGS && u <= LAUNCH_REGS &&
          u >= 24 && e % 8 == 0 && m % 8 == 0 && c % 8 == 0 && u % 8 == 0;
 }
-static_assert(regs_ok<false, false>() && regs_ok<false, true>() && regs_ok<true, true>(), "setmaxnreg split");
+static_assert(regs_ok<false, false, false>() && regs_ok<false, false, true>() && regs_ok<false, true, true>() && regs_ok<true, true, false>() &&
+              regs_ok<true, true, true>(), "setmaxnreg split");
 
 enum {
   BAR_Q_FULL = 0,                       // [2] query tile of work item i in buffer i & 1
@@ -107,6 +111,20 @@ static_assert(NUM_BARS <= 64, "barrier table");
 // Contiguous operands: the most keys that the short instance takes; both sides measured, see the kernel
 constexpr int LONG_KEYS = 49152;
 
+// RUNS: an item of RUN_BLOCKS KV blocks or more accumulates them in two runs, from 256 blocks in four.  The tensor core drops what
+// does not fit behind the accumulator's last bit, so O comes out too small by an amount that grows with the number of additions
+// into one accumulator.  Relative error of the FP32 result against a 64-bit recomputation (2-norm), in one run / in these / with the
+// blocks alternating between two accumulators: causal 16384 keys 1.7e-6 / 1.1e-6 / 8.3e-7, 2048 queries on 65536 keys 4.0e-5 / 2.5e-5 /
+// 2.9e-5, on 131072 keys 8.0e-5 / 6.0e-5 / 6.4e-5.  After a run the correction warps move O to shared memory (added to what is
+// there, scaled to the present maximum), the next P V starts from zero, and the epilogue adds the sum of the earlier runs.  It costs
+// (us, kernel alone, one run / these) 16384 x 32 heads 1539 / 1558, 131072 x 32 96.8 / 97.2 ms, chunks of 512 on pages 299 / 312.
+// Shorter items stay in one run, within 8e-7 (from 16 blocks on 1.1e-6 above would be 8.9e-7, but the pass over 1999 keys x 40 heads
+// 87.7 us instead of 82.4: the copy's 64 KB of shared memory keep this kernel's CTAs from starting beside the last ones of
+// stage 1).  Launches that have no longer ones take an instance without this code.
+constexpr int RUN_BLOCKS = 32;
+template <bool RUNS>
+__device__ __forceinline__ int run_length(int T) { return !RUNS || T < RUN_BLOCKS ? T : T < 256 ? (T + 1) >> 1 : (T + 3) >> 2; }
+
 constexpr uint32_t OFF_Q = 0;                              // 2 tiles (the next tile's queries are prefetched)
 constexpr uint32_t OFF_K = OFF_Q + 2 * 8192;
 constexpr uint32_t OFF_V = OFF_K + KST * 8192;
@@ -118,13 +136,16 @@ constexpr uint32_t OFF_M = OFF_SFK + KST * 1024;           // running maximum af
 constexpr uint32_t OFF_L = OFF_M + MST * 128 * 4;          // final (l, m) of the two exponent groups, [item & 3][2][2][128]
 constexpr uint32_t OFF_BAR = OFF_L + 4 * 4 * 128 * 4;
 constexpr uint32_t OFF_MISC = OFF_BAR + 64 * 8;            // tmem base, abort flag (NUM_BARS <= 64)
+constexpr uint32_t OFF_TAIL = OFF_MISC + 128;              // what only some instances have
 // paged source only: per K stage the two pages' scale bytes (2 x 512) and Delta_S rows (2 x 128) as stored; groups by length
 constexpr uint32_t RAW_STAGE = 1280;
-constexpr uint32_t OFF_RAW = (OFF_MISC + 16 + 127) & ~127u;
+constexpr uint32_t OFF_RAW = OFF_TAIL;
 constexpr uint32_t OFF_ORDER = OFF_RAW + KST * RAW_STAGE;
-constexpr uint32_t SMEM_BYTES = OFF_MISC + 16 + 1024;      // + slack for the 1024-byte alignment
-constexpr uint32_t SMEM_BYTES_PAGED = OFF_ORDER + 2 * MAX_GROUPS + 1024;
-static_assert(SMEM_BYTES_PAGED <= 227 * 1024, "shared memory");
+// O of the first run of an item's blocks, [32 groups of 4 columns][128 rows] x 16 bytes
+template <bool PAGED> constexpr uint32_t OFF_RUN = PAGED ? OFF_ORDER + 2 * MAX_GROUPS : OFF_TAIL;
+template <bool PAGED, bool RUNS>
+constexpr uint32_t SMEM_BYTES = OFF_RUN<PAGED> + (RUNS ? HEAD_DIM * 128 * 4 : 0) + 1024;   // + slack for the 1024-byte alignment
+static_assert(OFF_TAIL % 128 == 0 && OFF_RUN<true> % 16 == 0 && SMEM_BYTES<true, true> <= 227 * 1024, "shared memory");
 
 constexpr uint32_t TM_S = 0 /* 2 x 128 */, TM_O = 256, TM_P = 384 /* 2 x 32 */, TM_SFQ = 448 /* 2 x 8 */, TM_SFK = 464 /* 2 x 8 */;
 constexpr uint32_t TMEM_COLS = 512;
@@ -139,6 +160,18 @@ __device__ __forceinline__ void pin32(uint32_t (&r)[32]) {
 __device__ __forceinline__ void pin16(uint32_t (&r)[16]) {
   asm volatile("" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]),
                     "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]));
+}
+
+// x += w * (16 columns of the copy in shared memory)
+__device__ __forceinline__ void add_copy(uint32_t (&x)[16], const uint4 *copy, float w) {
+#pragma unroll
+  for (int i = 0; i < 16; i += 4) {
+    const uint4 o = copy[(i >> 2) * 128];
+    x[i] = __float_as_uint(__fmaf_rn(w, __uint_as_float(o.x), __uint_as_float(x[i])));
+    x[i + 1] = __float_as_uint(__fmaf_rn(w, __uint_as_float(o.y), __uint_as_float(x[i + 1])));
+    x[i + 2] = __float_as_uint(__fmaf_rn(w, __uint_as_float(o.z), __uint_as_float(x[i + 2])));
+    x[i + 3] = __float_as_uint(__fmaf_rn(w, __uint_as_float(o.w), __uint_as_float(x[i + 3])));
+  }
 }
 
 // last key that a query row sees.  Rows past a request's own query count take the last row's (the epilogue writes their zeros):
@@ -160,7 +193,7 @@ __device__ __forceinline__ float exponent_unit(const PrefillParams &p, int b) {
 // heads, not causal, 67.7 / 70.8, causal 1999 x 40 75.7 / 79.5, 16384 x 32 1625 / 1650, 32768 x 32 6037 / 6090,
 // but 65536 x 32 23.44 / 23.05 ms, 131072 x 32 92.8 / 88.9 ms and chunks of 512 on pages 473 / 423 us: where rescales of O are rare the exponentials set the pace, and there
 // the compiler's schedule of the second form is the better one.
-template <bool PAGED, bool LONG>
+template <bool PAGED, bool LONG, bool RUNS>
 __global__ void __launch_bounds__(NTHREADS, 1)
 prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                const __grid_constant__ CUtensorMap tm_v, const PrefillParams p, const PagedSrc pg) {
@@ -234,7 +267,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   uint32_t gb = 0;   // KV blocks of the items already walked
   uint32_t ti = 0;   // index of the current item in this CTA's list
 
-  if (warp < 4) setmaxnreg_dec<REGS_UTIL<PAGED, LONG>>();
+  if (warp < 4) setmaxnreg_dec<REGS_UTIL<PAGED, LONG, RUNS>>();
   if (warp == 0) {
     // =========================== TMA producer ===========================
     // The whole warp runs the loop (uniform control flow keeps addresses and barrier handles in
@@ -400,6 +433,8 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     const uint64_t d_v0 = smem_desc(sbase + OFF_V, 16, 1024, SWZ_128B);
     bool ok = true;
     for (; ok && walk.template next<PAGED>(p, pg, tl); gb += tl.T, ++ti) {
+      const int run = run_length<RUNS>(tl.T);
+      int begin = 0;   // of the run
       for (int t = 0; t < tl.T && ok; ++t) {
         const uint32_t c = gb + t, sb = c & 1, vs = c % VST;
         ok = cx.wait(BAR_V_FULL + vs, (c / VST) & 1u);
@@ -409,10 +444,11 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         tc_fence_after();
         const uint32_t tP = tm + TM_P + sb * 32;
         const uint64_t d_v = d_v0 + (uint64_t)((vs * 16384) >> 4);
+        if (RUNS && t == begin + run) begin = t;
         if (elect_one()) {
 #pragma unroll
           for (int k4 = 0; k4 < 4; ++k4)
-            mma_e4m3_ts(tm + TM_O, tP + 8 * k4, d_v + (uint64_t)((4096 * k4) >> 4), id_fp8, (t > 0 || k4 > 0) ? 1u : 0u);
+            mma_e4m3_ts(tm + TM_O, tP + 8 * k4, d_v + (uint64_t)((4096 * k4) >> 4), id_fp8, ((RUNS ? t != begin : t > 0) || k4 > 0) ? 1u : 0u);
           mma_commit(cx.bar(BAR_O_FULL));
           mma_commit(cx.bar(BAR_P_EMPTY + sb));
           mma_commit(cx.bar(BAR_V_EMPTY + vs));
@@ -421,7 +457,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     }
   } else if (warp >= 12 && warp < 16) {
     // =========================== running maximum ===========================
-    setmaxnreg_dec<REGS_MAX<PAGED, LONG>>();
+    setmaxnreg_dec<REGS_MAX<PAGED, LONG, RUNS>>();
     const int row = (warp & 3) * 32 + lane;
     const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
     float *s_m = reinterpret_cast<float *>(smem + OFF_M);
@@ -466,7 +502,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     }
   } else if (warp >= 4 && warp < 12) {
     // =========================== exponentials ===========================
-    setmaxnreg_inc<REGS_EXP<PAGED, LONG>>();
+    setmaxnreg_inc<REGS_EXP<PAGED, LONG, RUNS>>();
     const int grp = (warp - 4) >> 2;   // takes the KV blocks whose running count has this parity
     const int row = (warp & 3) * 32 + lane;
     const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
@@ -550,9 +586,10 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     }
   } else if (warp >= 16) {
     // =========================== correction + epilogue ===========================
-    setmaxnreg_dec<REGS_CORR<PAGED, LONG>>();
+    setmaxnreg_dec<REGS_CORR<PAGED, LONG, RUNS>>();
     const int row = (warp & 3) * 32 + lane;
     const float *s_m = reinterpret_cast<const float *>(smem + OFF_M);
+    uint4 *const s_run = reinterpret_cast<uint4 *>(smem + OFF_RUN<PAGED>) + row;   // this thread's row: written and read by it alone
     const uint32_t tO = tm + TM_O + ((uint32_t)((warp & 3) * 32) << 16);
     bool ok = true;
     uint32_t n_used = 0;   // items so far with T > 0 (slot and phase of the row-sum ring)
@@ -561,50 +598,74 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       const int TT = tl.T, r_abs = tl.row0 + row;
       const float lam = exponent_unit(p, tl.b);
       const bool past = PAGED && r_abs >= tl.nq;   // nobody reads these rows: they ask for no rescale
-      float m_before = -INFINITY;
-      for (int t = 0; ok && t < TT; ++t) {
-        const uint32_t c = gb + t;
-        ok = __all_sync(0xffffffffu, cx.wait(BAR_M_FULL + c % MST, (c / MST) & 1u));
-        if (!ok) break;
-        // alpha_t = 2^(lam (m_{t-1} - m_t)) (Eq. 5/6)
-        const float m_now = s_m[(c % MST) * 128 + row];
-        const float alpha = (m_now == m_before || past) ? 1.0f : ex2_approx(__fmul_rn(m_before - m_now, lam));
-        m_before = m_now;
-        if (t == 0) continue;   // handed over by the previous item's epilogue
-        ok = __all_sync(0xffffffffu, cx.wait(BAR_O_FULL, (c - 1) & 1u));
+      float m_before = -INFINITY, m_run = -INFINITY;
+      int t = 0, end = run_length<RUNS>(TT);
+      for (;;) {   // the item's runs of blocks
+        for (const int first = t; ok && t < end; ++t) {
+          const uint32_t c = gb + t;
+          ok = __all_sync(0xffffffffu, cx.wait(BAR_M_FULL + c % MST, (c / MST) & 1u));
+          if (!ok) break;
+          // alpha_t = 2^(lam (m_{t-1} - m_t)) (Eq. 5/6)
+          const float m_now = s_m[(c % MST) * 128 + row];
+          const float alpha = (m_now == m_before || past) ? 1.0f : ex2_approx(__fmul_rn(m_before - m_now, lam));
+          m_before = m_now;
+          if (t == first) continue;   // handed over by the previous item's epilogue, or when the run before was copied
+          ok = __all_sync(0xffffffffu, cx.wait(BAR_O_FULL, (c - 1) & 1u));
+          if (!ok) break;
+          tc_fence_after();
+          if (__any_sync(0xffffffffu, alpha != 1.0f)) {   // identical result when every factor is exactly 1
+            // 16 columns on the way while 16 are multiplied, in a short loop: unrolled over 32-column halves the rescale took
+            // 260-495 cycles instead of 590-770, but the kernel 1780 us instead of 1715 (16384 keys): the exponentials beside it
+            // ran slower
+            uint32_t r[2][16];
+            tmem_ld16(tO, r[0]);
+#pragma unroll 1
+            for (int c0 = 0; c0 < 8; c0 += 2) {
+#pragma unroll
+              for (int u = 0; u < 2; ++u) {
+                uint32_t(&x)[16] = r[u];
+                tmem_ld_wait();
+                pin16(x);
+                if (c0 + u < 7) tmem_ld16(tO + 16 * (c0 + u + 1), r[u ^ 1]);
+#pragma unroll
+                for (int i = 0; i < 16; i += 2) {
+                  float y0, y1;
+                  mul2(y0, y1, __uint_as_float(x[i]), __uint_as_float(x[i + 1]), alpha);
+                  x[i] = __float_as_uint(y0), x[i + 1] = __float_as_uint(y1);
+                }
+                tmem_st16(tO + 16 * (c0 + u), x);
+              }
+            }
+            tmem_st_wait();
+          }
+          tc_fence_before();
+          warp_arrive(cx.bar(BAR_O_READY), lane);
+        }
+        if (!RUNS || end == TT || !ok) break;
+        // the run's O goes to shared memory, the first as it is, a later one added to the sum of those before
+        ok = __all_sync(0xffffffffu, cx.wait(BAR_O_FULL, (gb + end - 1) & 1u));
         if (!ok) break;
         tc_fence_after();
-        if (__any_sync(0xffffffffu, alpha != 1.0f)) {   // identical result when every factor is exactly 1
-          // 16 columns on the way while 16 are multiplied, in a short loop: unrolled over 32-column halves the rescale took
-          // 260-495 cycles instead of 590-770, but the kernel 1780 us instead of 1715 (16384 keys): the exponentials beside it
-          // ran slower
-          uint32_t r[2][16];
-          tmem_ld16(tO, r[0]);
+        const bool more = end > run_length<RUNS>(TT);
+        const float w = m_run == m_before ? 1.0f : ex2_approx(__fmul_rn(m_run - m_before, lam));
+        m_run = m_before;
 #pragma unroll 1
-          for (int c0 = 0; c0 < 8; c0 += 2) {
+        for (int c0 = 0; c0 < HEAD_DIM; c0 += 16) {
+          uint32_t x[16];
+          tmem_ld16(tO + c0, x);
+          tmem_ld_wait();
+          pin16(x);
+          if (more) add_copy(x, s_run + c0 / 4 * 128, w);
 #pragma unroll
-            for (int u = 0; u < 2; ++u) {
-              uint32_t(&x)[16] = r[u];
-              tmem_ld_wait();
-              pin16(x);
-              if (c0 + u < 7) tmem_ld16(tO + 16 * (c0 + u + 1), r[u ^ 1]);
-#pragma unroll
-              for (int i = 0; i < 16; i += 2) {
-                float y0, y1;
-                mul2(y0, y1, __uint_as_float(x[i]), __uint_as_float(x[i + 1]), alpha);
-                x[i] = __float_as_uint(y0), x[i + 1] = __float_as_uint(y1);
-              }
-              tmem_st16(tO + 16 * (c0 + u), x);
-            }
-          }
-          tmem_st_wait();
+          for (int i = 0; i < 4; ++i) s_run[(c0 / 4 + i) * 128] = make_uint4(x[4 * i], x[4 * i + 1], x[4 * i + 2], x[4 * i + 3]);
         }
         tc_fence_before();
         warp_arrive(cx.bar(BAR_O_READY), lane);
+        end = min(end + run_length<RUNS>(TT), TT);
       }
       // final normalisation (Algorithm 1 line 17).  The two exponent groups hold partial sums relative to their own last
       // maximum; bring both to the final one.
-      float l = 0.0f;
+      float l = 0.0f, w_run = 0.0f;
       if (ok && TT > 0) {
         ok = cx.wait(BAR_O_FULL, (gb + TT - 1) & 1u);
         ok = ok && cx.wait(BAR_L_FULL + (n_used & 3), (n_used >> 2) & 1u);
@@ -618,6 +679,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             const float w0 = (m0 == mf) ? 1.0f : ex2_approx(__fmul_rn(m0 - mf, lam));
             const float w1 = (m1 == mf) ? 1.0f : ex2_approx(__fmul_rn(m1 - mf, lam));
             l = __fadd_rn(__fmul_rn(w0, l0), __fmul_rn(w1, l1));
+            if (RUNS) w_run = (m_run == mf) ? 1.0f : ex2_approx(__fmul_rn(m_run - mf, lam));
           }
         }
       }
@@ -635,6 +697,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           tmem_ld_wait();
           pin16(r);
         }
+        if (RUNS && TT >= RUN_BLOCKS) add_copy(r, s_run + c0 / 4 * 128, w_run);
         if (c0 == HEAD_DIM - 16 && TT > 0) {   // O is in registers: the next item's P V may overwrite it
           tc_fence_before();
           warp_arrive(cx.bar(BAR_O_READY), lane);
@@ -745,8 +808,9 @@ extern "C" mpfa_status mpfa_prefill_variant(const mpfa_fp4_tensor *q, const mpfa
   if ((rc = make_map(enc, &tq, q->codes, q_rows, 64)) != MPFA_OK) return rc;
   if ((rc = make_map(enc, &tk, k->codes, k_rows, 64)) != MPFA_OK) return rc;
   if ((rc = make_map(enc, &tv, v_fp8, k_rows, 128)) != MPFA_OK) return rc;
-  if (k->N <= LONG_KEYS) return start<prefill_kernel<false, false>, SMEM_BYTES>(dev, grid, NTHREADS, s, tq, tk, tv, p, PagedSrc{});
-  return start<prefill_kernel<false, true>, SMEM_BYTES>(dev, grid, NTHREADS, s, tq, tk, tv, p, PagedSrc{});
+  if (nk_tiles < RUN_BLOCKS) return start<prefill_kernel<false, false, false>, SMEM_BYTES<false, false>>(dev, grid, NTHREADS, s, tq, tk, tv, p, PagedSrc{});
+  if (k->N <= LONG_KEYS) return start<prefill_kernel<false, false, true>, SMEM_BYTES<false, true>>(dev, grid, NTHREADS, s, tq, tk, tv, p, PagedSrc{});
+  return start<prefill_kernel<false, true, true>, SMEM_BYTES<false, true>>(dev, grid, NTHREADS, s, tq, tk, tv, p, PagedSrc{});
 }
 
 extern "C" mpfa_status mpfa_prefill_paged(const mpfa_fp4_tensor *q, const mpfa_paged_kv *kv, const int32_t *page_table,
@@ -808,5 +872,7 @@ extern "C" mpfa_status mpfa_prefill_paged(const mpfa_fp4_tensor *q, const mpfa_p
   CUtensorMap tq;
   if ((rc = make_map(enc, &tq, q->codes, q_rows, 64)) != MPFA_OK) return rc;
   const unsigned grid = (unsigned)(n_cta < (uint64_t)n_sm ? n_cta : (uint64_t)n_sm);
-  return start<prefill_kernel<true, true>, SMEM_BYTES_PAGED>(dev, grid, NTHREADS, static_cast<cudaStream_t>(stream), tq, tq, tq, p, pg);
+  if (max_pages_per_req < RUN_BLOCKS * (TILE / PAGE) - 1)   // no request can have RUN_BLOCKS blocks
+    return start<prefill_kernel<true, true, false>, SMEM_BYTES<true, false>>(dev, grid, NTHREADS, static_cast<cudaStream_t>(stream), tq, tq, tq, p, pg);
+  return start<prefill_kernel<true, true, true>, SMEM_BYTES<true, true>>(dev, grid, NTHREADS, static_cast<cudaStream_t>(stream), tq, tq, tq, p, pg);
 }

@@ -221,6 +221,46 @@ def test_prefill_item_boundaries_through_every_ring(N_kv):
     compare(o16, o32, rows[keep], ref32[keep], f"N_kv {N_kv}")
 
 
+@pytest.mark.parametrize("N_kv,N_q", [(3968, 130), (3969, 130), (4096, 300), (4225, 130), (32640, 100), (32641, 130)])
+def test_prefill_on_both_sides_of_the_accumulation_in_runs(N_kv, N_q):
+    """31 KV blocks (one run of accumulation), 32 (two runs; 4096 keys and 300 causal queries: items of 30 to 32 blocks in one
+    launch), 34, 255 (two runs) and 256 (four), causal, against the oracle and from pages."""
+    from paper_2609_33135_b200 import binding as B_
+    w = wl.prefill_workload("runs", 64, 1, N_kv, 4, 2, True, N_q=N_q, q_bias=True)
+    z = orc.stage1(orc.bf16_bits(w.q), orc.bf16_bits(w.k), orc.bf16_bits(w.v))
+    s1 = B_.stage1(w.q.cuda(), w.k.cuda(), w.v.cuda())
+    out, o32, status = B_.prefill(s1, True, w.softmax_scale, want_f32=True)
+    n_pages = -(-N_kv // 64)
+    kv = B_.PagedKV.empty(n_pages, 4, 2, with_delta=True)
+    table = torch.arange(n_pages - 1, -1, -1, dtype=torch.int32, device="cuda").view(1, -1).contiguous()
+    B_.mpfa_quantize_kv_paged(w.k[0].cuda(), w.v[0].cuda(), 0, 4, B_.MPFA_SMOOTH | B_.MPFA_STATS_FROZEN, s1.stats.request(0), 1.0, kv,
+                              table[0], None)
+    out_p, o32_p = torch.empty_like(out), torch.empty_like(o32)
+    B_.mpfa_prefill_paged(s1.q, kv, table, torch.tensor([N_kv], dtype=torch.int32, device="cuda"), s1.stats, 1.0, w.softmax_scale,
+                          out_p, o32_p, status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    assert torch.equal(o32.view(torch.int32), o32_p.view(torch.int32)) and torch.equal(out.view(torch.uint16), out_p.view(torch.uint16))
+    rows = np.array([(0, h, i) for h in range(4) for i in sorted({0, 1, 31, 32, 43, 44, N_q - 3, N_q - 2, N_q - 1})])
+    ref32, _ = orc.prefill_rows(z, rows, w.softmax_scale, True)
+    compare(out.view(torch.uint16).cpu().numpy(), o32.cpu().numpy(), rows, ref32, f"N_kv {N_kv}")
+
+
+@pytest.mark.parametrize("N_kv,one_run,two_runs", [(8192, 1.06e-6, 5.0e-7), (16384, 2.5e-6, 1.3e-6), (57344, 2.0e-5, 9.4e-6)])
+def test_prefill_long_contexts_keep_their_accumulation_error(N_kv, one_run, two_runs):
+    """The tensor core's FP32 accumulation drops the bits behind the accumulator's last one, so O comes out too small by an amount
+    that grows with the number of additions into one accumulator; the oracle rounds to nearest.  Bound: half way between what one run
+    of all blocks and two runs of half of them measure."""
+    w = wl.prefill_workload("bias", 65, 1, N_kv, 2, 1, False, N_q=128)
+    z = orc.stage1(orc.bf16_bits(w.q), orc.bf16_bits(w.k), orc.bf16_bits(w.v))
+    rows = orc.all_rows(1, 2, 128)[::4]
+    ref32, _ = orc.prefill_rows(z, rows, w.softmax_scale, False)
+    _, o32 = run_gpu(w)
+    r = ref32.astype(np.float64)
+    shrink = -((o32[rows[:, 0], rows[:, 2], rows[:, 1]] - r) * r).sum() / (r * r).sum()
+    assert abs(shrink) <= 0.5 * (one_run + two_runs), shrink
+
+
 @pytest.mark.parametrize("N_kv", [49152, 49153])
 def test_prefill_on_both_sides_of_the_long_context_instance(N_kv):
     """The last key count of the instance that masks in the maximum warps and the first of the one that masks in the exponent

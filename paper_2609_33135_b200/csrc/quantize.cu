@@ -342,7 +342,7 @@ __device__ __forceinline__ void quantize_block16(const float (&xc)[16], const Bl
   for (int i = 0; i < 4; ++i) m[i] = max3(fabsf(xc[4 * i]), fabsf(xc[4 * i + 1]), fabsf(xc[4 * i + 2]));
 #pragma unroll
   for (int i = 0; i < 2; ++i) m[i] = max3(m[i], fabsf(xc[8 * i + 3]), fabsf(xc[8 * i + 7]));
-  const float a = fmaxf(max3(m[0], m[1], m[2]), m[3]);
+  const float a = max3(max3(m[0], m[1], m[2]), m[3], 0.0f);   // 0 for a block of NaNs, as above
   float r = __fmul_rn(a, q.rcp);
   if (!(r >= 0.015625f && r < 512.0f && abs((int)(__float_as_uint(r) & 0xFFFFFu) - 0x80000) > 4)) r = __fdiv_rn(a, q.e);
   scale_code = (uint32_t)__nv_cvt_float_to_fp8(r, __NV_SATFINITE, __NV_E4M3);

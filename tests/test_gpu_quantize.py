@@ -123,6 +123,52 @@ def test_frozen_statistics_single_token_query():
     assert np.array_equal(sf_to_logical(q4.sf.cpu().numpy(), w.B, w.H_q, 1)[:, :, :1], zq.q_sf)
 
 
+def _rows_by_both_paths(x, gscale):
+    """Codes and scale bytes of eight tokens x [1, 8, H, 128] with given statistics, from the kernel of at most eight queries and, as
+    the first rows of sixteen, from the tile kernel; and K codes and scale bytes of the same tokens from the page kernel and, one
+    by one, from the append kernel."""
+    from paper_2609_33135_b200 import binding
+    H = x.shape[2]
+    st = binding.Stats.empty(1, H, H)
+    g = torch.Generator().manual_seed(5)
+    for m in (st.q_mean, st.k_mean):
+        m.copy_(torch.randn(1, H, 128, generator=g) * 0.25)
+    st.q_gscale.fill_(gscale), st.k_gscale.fill_(gscale)
+    x = x.cuda()
+    rows = []
+    for q in (x, torch.cat([x, x.flip(1)], 1).contiguous()):
+        q4 = binding.Fp4Tensor.empty(1, H, q.shape[1])
+        binding.mpfa_quantize_qk(q, None, binding.MPFA_STATS_FROZEN, st, q4, None, None, None)
+        rows.append((codes_to_logical(q4.codes.cpu().numpy(), 1, H, q.shape[1])[0][:, :, :8],
+                     sf_to_logical(q4.sf.cpu().numpy(), 1, H, q.shape[1])[:, :, :8]))
+    pages = []
+    table = torch.zeros(1, 1, dtype=torch.int32, device="cuda")
+    for one_by_one in (False, True):
+        kv = binding.PagedKV.empty(1, H, H, with_delta=False)
+        if one_by_one:
+            for t in range(8):
+                k = x[:, t:t + 1].contiguous()
+                binding.mpfa_append_kv_paged(k, k, H, 0, st, 1.0, kv, table, torch.tensor([t], dtype=torch.int32, device="cuda"))
+        else:
+            binding.mpfa_quantize_kv_paged(x[0].contiguous(), x[0].contiguous(), 0, H, binding.MPFA_STATS_FROZEN, st, 1.0, kv, table[0], None)
+        pages.append((kv.k_codes.cpu().numpy(), kv.k_sf.cpu().numpy()))
+    torch.cuda.synchronize()
+    return rows, pages
+
+
+@pytest.mark.parametrize("value", [float("nan"), float("inf"), float("-inf")])
+def test_blocks_without_a_finite_value(value):
+    """A block of 16 NaNs has scale 0 on every path, so that it does not turn its token's scores into NaNs; an infinity saturates."""
+    x = torch.randn(1, 8, 2, 128, generator=torch.Generator().manual_seed(6))
+    x[0, 3, 0, 32:48] = value
+    x[0, 5, 1] = value
+    x[0, 6, 1, 7] = value
+    (few, tile), (page, one) = _rows_by_both_paths(x.bfloat16(), 0.003)
+    assert (few[1][0, 0, 3, 2], few[1][0, 1, 5, 4]) == ((0, 0) if np.isnan(value) else (0x7E, 0x7E))
+    for a, b in ((few, tile), (page, one)):
+        assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
+
+
 def test_deterministic_and_argument_errors():
     from paper_2609_33135_b200 import binding
     w = _cases()["cfg1b"]()

@@ -293,11 +293,11 @@ __device__ __forceinline__ void quantize_block16(const float (&xc)[16], float d,
 // Packed FP32 pairs round each half like the scalar operation.
 struct BlockScale {
   float e, rcp;       // 6 d and its reciprocal (NaN: always divide)
-  const float *inv;   // [128]
+  const float *inv;   // [128], by the magnitude of the scale code: its sign is that of d, and the two cancel in the decoded scale
 };
 __device__ __forceinline__ BlockScale make_block_scale(float d, float *table, int tid) {
   if (tid < 128) {
-    const float s = __fmul_rn(__half2float(__half(__nv_cvt_fp8_to_halfraw((__nv_fp8_storage_t)tid, __NV_E4M3))), d);
+    const float s = __fmul_rn(__half2float(__half(__nv_cvt_fp8_to_halfraw((__nv_fp8_storage_t)tid, __NV_E4M3))), fabsf(d));
     const float inv = __fdiv_rn(1.0f, s);
     table[tid] = (!(s > 0.0f) || isinf(inv)) ? 0.0f : inv;
   }
@@ -346,7 +346,7 @@ __device__ __forceinline__ void quantize_block16(const float (&xc)[16], const Bl
   float r = __fmul_rn(a, q.rcp);
   if (!(r >= 0.015625f && r < 512.0f && abs((int)(__float_as_uint(r) & 0xFFFFFu) - 0x80000) > 4)) r = __fdiv_rn(a, q.e);
   scale_code = (uint32_t)__nv_cvt_float_to_fp8(r, __NV_SATFINITE, __NV_E4M3);
-  const float inv = q.inv[scale_code];
+  const float inv = q.inv[scale_code & 127u];
   float y[16];
 #pragma unroll
   for (int i = 0; i < 16; i += 2) mul2(y[i], y[i + 1], xc[i], xc[i + 1], inv);

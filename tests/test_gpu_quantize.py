@@ -169,6 +169,17 @@ def test_blocks_without_a_finite_value(value):
         assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
 
 
+@pytest.mark.parametrize("gscale", [-0.003, -0.0, 0.0, 1e-38, 3e-31, 1e30, float("inf"), float("nan")])
+def test_frozen_tensor_scales_of_any_value(gscale):
+    """The caller's frozen scale is taken as it is.  A negative one gives scale codes with the sign bit, beyond the 128 entries of
+    the tile kernel's table of reciprocals; outside 1e-30 .. 1e30 the scale code is divided out."""
+    x = torch.randn(1, 8, 2, 128, generator=torch.Generator().manual_seed(7))
+    x[0, 2, 1, 16:32] = 0.0
+    (few, tile), (page, one) = _rows_by_both_paths(x.bfloat16(), gscale)
+    for a, b in ((few, tile), (page, one)):
+        assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
+
+
 def test_deterministic_and_argument_errors():
     from paper_2609_33135_b200 import binding
     w = _cases()["cfg1b"]()

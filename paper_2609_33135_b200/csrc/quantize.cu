@@ -369,13 +369,26 @@ __device__ __forceinline__ Row16 load_row16(const __nv_bfloat16 *p, bool wide) {
   return r;
 }
 __device__ __forceinline__ bool wide_rows(const void *x) { return (reinterpret_cast<uintptr_t>(x) & 31) == 0; }
-// means of 16 channels, negated; 16-byte aligned
-__device__ __forceinline__ void load_neg_mean(const float *mean, float (&nm)[16]) {
+// Means of 16 channels.  The interface asks for no alignment of the statistics beyond a float's: 16-byte loads where the address allows
+// them.  The kernels of a decode step, which are chains of a few loads, have an instance of each kind (the branch cost a step
+// of 64 requests 0.9 us of 70); the others branch.
+inline __host__ __device__ bool vector_means(const float *mean) { return (reinterpret_cast<uintptr_t>(mean) & 15) == 0; }
+__device__ __forceinline__ void load_mean16(const float *mean, float (&m)[16], bool vec) {
+  if (vec) {
 #pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    const float4 m = __ldg(reinterpret_cast<const float4 *>(mean) + c);
-    nm[4 * c] = -m.x, nm[4 * c + 1] = -m.y, nm[4 * c + 2] = -m.z, nm[4 * c + 3] = -m.w;
+    for (int c = 0; c < 4; ++c) {
+      const float4 v = __ldg(reinterpret_cast<const float4 *>(mean) + c);
+      m[4 * c] = v.x, m[4 * c + 1] = v.y, m[4 * c + 2] = v.z, m[4 * c + 3] = v.w;
+    }
+  } else {
+#pragma unroll
+    for (int c = 0; c < 16; ++c) m[c] = __ldg(mean + c);
   }
+}
+__device__ __forceinline__ void load_neg_mean(const float *mean, float (&nm)[16], bool vec) {
+  load_mean16(mean, nm, vec);
+#pragma unroll
+  for (int c = 0; c < 16; ++c) nm[c] = -nm[c];
 }
 __device__ __forceinline__ void center16(const Row16 &x, const float (&nm)[16], float (&xc)[16]) {
   float f[16];
@@ -496,8 +509,8 @@ __global__ void __launch_bounds__(256, QT_CTAS) quantize_tile_kernel(const Quant
   if (at == 0 && tid == 0 && a.scale.gmax) a.scale.gscale[b] = d;
   const BlockScale bs = make_block_scale(d, inv_table, tid);
   float neg_mean[2][16];
-  load_neg_mean(a.mean + head * HEAD_DIM + j * 16, neg_mean[0]);
-  load_neg_mean(a.mean + head * HEAD_DIM + 64 + j * 16, neg_mean[1]);
+  load_neg_mean(a.mean + head * HEAD_DIM + j * 16, neg_mean[0], vector_means(a.mean));
+  load_neg_mean(a.mean + head * HEAD_DIM + 64 + j * 16, neg_mean[1], vector_means(a.mean));
   const bool with_delta = is_k && da.delta;
   const int G = with_delta ? da.H_q / a.H : 0;
   double unit = 0.0;
@@ -565,6 +578,7 @@ __global__ void __launch_bounds__(256, QT_CTAS) quantize_tile_kernel(const Quant
 // The tiles of a decode step's queries (at most eight tokens): one warp per (batch element, head), the eight rows and the zeros
 // of the other 120.  Bound by writing 9 KB per tile; with a CTA per tile the chain of loads was repeated for six waves of
 // CTAs (64 requests, 40 heads: 13.6 us, now 7.1 us).
+template <bool VEC>   // vector_means
 __global__ void __launch_bounds__(256) quantize_token_kernel(const QuantTensor q, int n_heads) {
   launch_dependents();
   grid_dependency_wait();
@@ -587,7 +601,7 @@ __global__ void __launch_bounds__(256) quantize_token_kernel(const QuantTensor q
 #pragma unroll
   for (int half = 0; half < 2; ++half) {
     float xc[16], neg_mean[16];
-    load_neg_mean(q.mean + (size_t)head * HEAD_DIM + (half * 4 + j) * 16, neg_mean);
+    load_neg_mean(q.mean + (size_t)head * HEAD_DIM + (half * 4 + j) * 16, neg_mean, VEC);
     center16(raw[half], neg_mean, xc);
     uint8_t s8 = 0;
     uint2 c = make_uint2(0u, 0u);
@@ -738,8 +752,8 @@ __global__ void __launch_bounds__(256, WK_CTAS) write_kv_kernel(const __nv_bfloa
   if (blockIdx.y == 0 && h == 0 && tid == 0 && k_scale.gmax) k_scale.gscale[0] = d;
   const BlockScale bs = make_block_scale(d, inv_table, tid);
   float neg_mean[2][16];
-  load_neg_mean(k_mean + (size_t)h * HEAD_DIM + j * 16, neg_mean[0]);
-  load_neg_mean(k_mean + (size_t)h * HEAD_DIM + 64 + j * 16, neg_mean[1]);
+  load_neg_mean(k_mean + (size_t)h * HEAD_DIM + j * 16, neg_mean[0], vector_means(k_mean));
+  load_neg_mean(k_mean + (size_t)h * HEAD_DIM + 64 + j * 16, neg_mean[1], vector_means(k_mean));
   double unit = 0.0;
   if (delta) {
     convert_group_means(gm, q_mean + (size_t)h * G * HEAD_DIM, G, tid, 256);
@@ -796,6 +810,7 @@ __global__ void __launch_bounds__(256, WK_CTAS) write_kv_kernel(const __nv_bfloa
 // other 63 slots.  Bound by the latency of three dependent loads; the loads that depend on nothing are issued together.
 // Measured (64 requests, 40:8 heads): with one thread per FP64 chain of 128 terms and 2 x 256 threads per pair
 // 9.8 us, now 6.6 us.
+template <bool VEC>   // vector_means of both means
 __global__ void __launch_bounds__(256) append_kv_kernel(const __nv_bfloat16 *__restrict__ k, const __nv_bfloat16 *__restrict__ v,
                                                         const float *__restrict__ q_mean, const float *__restrict__ k_mean,
                                                         const float *__restrict__ q_gscale, const float *__restrict__ k_gscale,
@@ -815,7 +830,7 @@ __global__ void __launch_bounds__(256) append_kv_kernel(const __nv_bfloat16 *__r
   const float d = k_gscale[b];
   const double denom = delta ? (double)q_gscale[b] * (double)d : 1.0;
   float xc[16], neg_mean[16];
-  load_neg_mean(k_mean + (size_t)pair * HEAD_DIM + blk * 16, neg_mean);
+  load_neg_mean(k_mean + (size_t)pair * HEAD_DIM + blk * 16, neg_mean, VEC);
   center16(kr, neg_mean, xc);
   const bool in_table = pos >= 0 && (pos >> 6) < max_pages;   // else: skipped, or no page-table entry for that position
   const int page = in_table ? page_table[(size_t)b * max_pages + (pos >> 6)] : -1;
@@ -827,15 +842,10 @@ __global__ void __launch_bounds__(256) append_kv_kernel(const __nv_bfloat16 *__r
     for (int n = 0; n < 2; ++n) {
       const int g = part + 4 * n;
       if (g < G) {
-        const float4 *qp = reinterpret_cast<const float4 *>(q_mean + ((size_t)b * H_q + h * G + g) * HEAD_DIM + blk * 16);
+        float m[16];
+        load_mean16(q_mean + ((size_t)b * H_q + h * G + g) * HEAD_DIM + blk * 16, m, VEC);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const float4 m = qp[i];
-          acc[n] = fma((double)m.x, (double)xc[4 * i], acc[n]);
-          acc[n] = fma((double)m.y, (double)xc[4 * i + 1], acc[n]);
-          acc[n] = fma((double)m.z, (double)xc[4 * i + 2], acc[n]);
-          acc[n] = fma((double)m.w, (double)xc[4 * i + 3], acc[n]);
-        }
+        for (int i = 0; i < 16; ++i) acc[n] = fma((double)m[i], (double)xc[i], acc[n]);
       }
 #pragma unroll
       for (int o = 1; o < 8; o <<= 1) acc[n] += __shfl_xor_sync(0xffffffffu, acc[n], o);
@@ -979,7 +989,7 @@ extern "C" mpfa_status mpfa_quantize_qk(const void *q_bf16, const void *k_bf16, 
   QuantTensor tk{k, st->k_mean, sk, N_kv, k ? H_kv : 0, k ? pad128(N_kv) / TILE : 0, 0, k ? k_out->codes : nullptr, k ? k_out->sf : nullptr};
   const DeltaArgs da{st->q_mean, sq, k && smooth ? static_cast<__nv_bfloat16 *>(delta_s_bf16) : nullptr, H_q};
   if (!k && N_q <= 8) {
-    MPFA_CUDA_OK(launch(quantize_token_kernel, dim3((B * H_q + 7) / 8), dim3(256), 0, s, tq, B * H_q));
+    MPFA_CUDA_OK(launch(vector_means(tq.mean) ? quantize_token_kernel<true> : quantize_token_kernel<false>, dim3((B * H_q + 7) / 8), dim3(256), 0, s, tq, B * H_q));
     return MPFA_OK;
   }
   // At most one wave of CTAs where every head can have one: a CTA's set-up (scale, table of reciprocals, query means) is paid
@@ -1124,7 +1134,8 @@ extern "C" mpfa_status mpfa_append_kv_paged(const void *k_bf16, const void *v_bf
   int dev = 0, n_sm = 0;
   mpfa_status rc = device_info(&dev, &n_sm);
   if (rc != MPFA_OK) return rc;
-  MPFA_CUDA_OK(launch(append_kv_kernel, dim3((B * H_kv + 7) / 8), dim3(256), 0, static_cast<cudaStream_t>(stream),
+  const bool vec = vector_means(st->k_mean) && vector_means(st->q_mean);
+  MPFA_CUDA_OK(launch(vec ? append_kv_kernel<true> : append_kv_kernel<false>, dim3((B * H_kv + 7) / 8), dim3(256), 0, static_cast<cudaStream_t>(stream),
                       static_cast<const __nv_bfloat16 *>(k_bf16), static_cast<const __nv_bfloat16 *>(v_bf16), st->q_mean, st->k_mean,
                       st->q_gscale, st->k_gscale, B, H_q, H_kv, 1.0f / v_scale, page_table, max_pages_per_req, kv->num_pages,
                       positions, kv->k_codes, kv->k_sf, kv->v_fp8,

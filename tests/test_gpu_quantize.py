@@ -84,6 +84,42 @@ def test_stage1_from_inputs_on_16_byte_boundaries():
     check_stage1(w, binding.stage1(shifted(w.q), shifted(w.k), shifted(w.v)), z)
 
 
+def test_statistics_on_any_float_boundary():
+    """The interface asks for no alignment of the statistics: stage 1, a query with frozen statistics, a page write and an append
+    with every array four bytes past a 16-byte boundary give what they give with aligned ones."""
+    from paper_2609_33135_b200 import binding
+    w = wl.prefill_workload("shifted", 46, 1, 333, 10, 2, True, q_bias=True)
+    q, k, v = w.q.cuda(), w.k.cuda(), w.v.cuda()
+    frozen = binding.MPFA_SMOOTH | binding.MPFA_STATS_FROZEN
+
+    def run(shift):
+        def arr(*shape):
+            n = int(np.prod(shape))
+            t = torch.zeros(n + 4, dtype=torch.float32, device="cuda")[shift:shift + n].view(*shape)
+            assert t.data_ptr() % 16 == 4 * shift
+            return t
+        st = binding.Stats(arr(1, 10, 128), arr(1, 2, 128), arr(1), arr(1))
+        s1 = binding.stage1(q, k, v)
+        s1.stats = st
+        binding.stage1(q, k, v, out=s1)
+        q4 = binding.Fp4Tensor.empty(1, 10, 1)
+        binding.mpfa_quantize_qk(q[:, 9:10].contiguous(), None, frozen, st, q4, None, None, None)
+        kv = binding.PagedKV.empty(6, 10, 2)
+        for t in (kv.k_codes, kv.k_sf, kv.v_fp8, kv.delta):
+            t.zero_()
+        row = torch.arange(6, dtype=torch.int32, device="cuda").view(1, 6)
+        binding.mpfa_quantize_kv_paged(k[0, :300].contiguous(), v[0, :300].contiguous(), 0, 10, binding.MPFA_SMOOTH, st, 1.0, kv, row[0],
+                                       binding.quantize_workspace(1, 10, 2))
+        binding.mpfa_append_kv_paged(k[:, 300:301].contiguous(), v[:, 300:301].contiguous(), 10, frozen, st, 1.0, kv, row,
+                                     torch.tensor([300], dtype=torch.int32, device="cuda"))
+        return [s1.q.codes, s1.q.sf, s1.k.codes, s1.k.sf, s1.delta.view(torch.int16), st.q_mean, st.k_mean, st.q_gscale, st.k_gscale, q4.codes,
+                q4.sf, kv.k_codes, kv.k_sf, kv.v_fp8, kv.delta.view(torch.int16)]
+    want = run(0)
+    for shift in (1, 2, 3):
+        for a, b in zip(run(shift), want):
+            assert torch.equal(a, b)
+
+
 def test_means_of_columns_with_non_finite_values():
     """The statistics add bit patterns of finite values; a column that holds an infinity or a NaN still gets the mean that a
     plain sum gives, and its neighbours theirs."""

@@ -40,7 +40,9 @@ inline mpfa_status cuda_fail(cudaError_t e) {
 // Launch whose CTAs may be scheduled while the preceding kernel of the stream is still running (programmatic stream
 // serialization): set-up that touches no memory the preceding work writes overlaps its tail.  Every kernel launched this
 // way calls grid_dependency_wait() before its first access to global memory, in every thread that makes one, so the
-// order of the stream holds transitively.
+// order of the stream holds transitively.  Such a kernel is resident while its inputs are still being written, so it reads global
+// memory with ordinary loads only: a non-coherent load (__ldg, ld.global.nc, what the compiler makes of const __restrict__)
+// asks for data that no one writes during the kernel's life, and the compiler may move it above the wait.
 template <typename... KArgs, typename... Args>
 cudaError_t launch(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, Args &&...args) {
   cudaLaunchAttribute attr;

@@ -437,7 +437,7 @@ prefill_variant_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
               p.delta + ((size_t)tl.b * p.H_q + tl.hq) * (size_t)(p.nk_tiles * TILE) + key0);
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
-            const uint4 d = __ldg(dp + i);
+            const uint4 d = dp[i];
             const uint32_t w[4] = {d.x, d.y, d.z, d.w};
 #pragma unroll
             for (int j = 0; j < 4; ++j) {   // packed pair: both halves round like the scalar add
@@ -469,7 +469,7 @@ prefill_variant_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
               p.delta + ((size_t)tl.b * p.H_q + tl.hq) * (size_t)(p.nk_tiles * TILE) + key0 + 64);
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
-            const uint4 d = __ldg(dp + i);
+            const uint4 d = dp[i];
             const uint32_t w[4] = {d.x, d.y, d.z, d.w};
 #pragma unroll
             for (int j = 0; j < 4; ++j) {

@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(STAT_THREADS, STAT_CTAS) colstat_kernel(const 
   // one round of loads is in flight while the previous one is added
   const auto load = [&](uint4 (&u)[STAT_LOADS]) {
 #pragma unroll
-    for (int j = 0; j < STAT_LOADS; ++j) u[j] = __ldg(reinterpret_cast<const uint4 *>(p + j * step));
+    for (int j = 0; j < STAT_LOADS; ++j) u[j] = *reinterpret_cast<const uint4 *>(p + j * step);
     p += STAT_LOADS * step;
   };
   const auto full = [&](int at) { return at + STAT_LANES * (STAT_LOADS - 1) < end; };
@@ -174,7 +174,7 @@ __global__ void __launch_bounds__(STAT_THREADS, STAT_CTAS) colstat_kernel(const 
   {   // the last fewer than STAT_LOADS rows of this lane, still in flight together
 #pragma unroll
     for (int j = 0; j < STAT_LOADS - 1; ++j)
-      if (t + STAT_LANES * j < end) u0[j] = __ldg(reinterpret_cast<const uint4 *>(p + j * step));
+      if (t + STAT_LANES * j < end) u0[j] = *reinterpret_cast<const uint4 *>(p + j * step);
 #pragma unroll
     for (int j = 0; j < STAT_LOADS - 1; ++j)
       if (t + STAT_LANES * j < end) add(u0[j]);
@@ -359,12 +359,12 @@ struct Row16 { uint4 a, b; };
 __device__ __forceinline__ Row16 load_row16(const __nv_bfloat16 *p, bool wide) {
   Row16 r;
   if (wide) {
-    asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+    asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                  : "=r"(r.a.x), "=r"(r.a.y), "=r"(r.a.z), "=r"(r.a.w), "=r"(r.b.x), "=r"(r.b.y), "=r"(r.b.z), "=r"(r.b.w)
                  : "l"(p));
   } else {
     const uint4 *u = reinterpret_cast<const uint4 *>(p);
-    r.a = __ldg(u), r.b = __ldg(u + 1);
+    r.a = u[0], r.b = u[1];
   }
   return r;
 }
@@ -377,12 +377,12 @@ __device__ __forceinline__ void load_mean16(const float *mean, float (&m)[16], b
   if (vec) {
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-      const float4 v = __ldg(reinterpret_cast<const float4 *>(mean) + c);
+      const float4 v = reinterpret_cast<const float4 *>(mean)[c];
       m[4 * c] = v.x, m[4 * c + 1] = v.y, m[4 * c + 2] = v.z, m[4 * c + 3] = v.w;
     }
   } else {
 #pragma unroll
-    for (int c = 0; c < 16; ++c) m[c] = __ldg(mean + c);
+    for (int c = 0; c < 16; ++c) m[c] = mean[c];
   }
 }
 __device__ __forceinline__ void load_neg_mean(const float *mean, float (&nm)[16], bool vec) {
@@ -592,6 +592,9 @@ __global__ void __launch_bounds__(256) quantize_token_kernel(const QuantTensor q
   for (int half = 0; half < 2; ++half)
     if (in) raw[half] = load_row16(q.x + (((size_t)b * q.N + r) * q.H + h) * HEAD_DIM + (half * 4 + j) * 16, wide);
   const float d = tensor_scale(q.scale, b, lane);
+  float neg_mean[2][16];
+  load_neg_mean(q.mean + (size_t)head * HEAD_DIM + j * 16, neg_mean[0], VEC);
+  load_neg_mean(q.mean + (size_t)head * HEAD_DIM + (4 + j) * 16, neg_mean[1], VEC);
   if (h == 0 && lane == 0 && q.scale.gmax) q.scale.gscale[b] = d;
   uint8_t *const codes = q.codes + (size_t)head * TILE * 64, *const sf = q.sf + (size_t)head * 1024;
   const uint4 z = make_uint4(0u, 0u, 0u, 0u);
@@ -600,9 +603,8 @@ __global__ void __launch_bounds__(256) quantize_token_kernel(const QuantTensor q
     if ((i & 31) >= 8) reinterpret_cast<uint4 *>(sf)[i] = z;   // 16 bytes per row of the atom: rows 8..31 of both halves
 #pragma unroll
   for (int half = 0; half < 2; ++half) {
-    float xc[16], neg_mean[16];
-    load_neg_mean(q.mean + (size_t)head * HEAD_DIM + (half * 4 + j) * 16, neg_mean, VEC);
-    center16(raw[half], neg_mean, xc);
+    float xc[16];
+    center16(raw[half], neg_mean[half], xc);
     uint8_t s8 = 0;
     uint2 c = make_uint2(0u, 0u);
     if (in) quantize_block16(xc, d, s8, c);
@@ -632,21 +634,25 @@ __device__ __forceinline__ uint4 quantize_v16(const Row16 &x, float inv) {
 }
 
 // grid (N_pad/128, H, B): V tile -> [B, H, N_pad, 128] E4M3.
-__global__ void __launch_bounds__(256) quantize_v_tile_kernel(const __nv_bfloat16 *__restrict__ v, int N, int H,
-                                                              float inv_scale, uint8_t *__restrict__ out) {
+__global__ void __launch_bounds__(256) quantize_v_tile_kernel(const __nv_bfloat16 *v, int N, int H,
+                                                              float inv_scale, uint8_t *out) {
   launch_dependents();
   grid_dependency_wait();
   const int tile = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
   const int n_pad = gridDim.x * TILE;
   const bool wide = wide_rows(v);
+  const int r0 = threadIdx.x >> 3, seg = threadIdx.x & 7;
+  Row16 x[4] = {};
 #pragma unroll
   for (int it = 0; it < 4; ++it) {
-    const int id = it * 256 + threadIdx.x;
-    const int r = id >> 3, seg = id & 7;
-    const int t = tile * TILE + r;
-    uint4 c = make_uint4(0u, 0u, 0u, 0u);
-    if (t < N) c = quantize_v16(load_row16(v + (((size_t)b * N + t) * H + h) * HEAD_DIM + seg * 16, wide), inv_scale);
-    *reinterpret_cast<uint4 *>(out + (((size_t)b * H + h) * n_pad + t) * HEAD_DIM + seg * 16) = c;
+    const int t = tile * TILE + it * 32 + r0;
+    if (t < N) x[it] = load_row16(v + (((size_t)b * N + t) * H + h) * HEAD_DIM + seg * 16, wide);
+  }
+#pragma unroll
+  for (int it = 0; it < 4; ++it) {
+    const int t = tile * TILE + it * 32 + r0;
+    *reinterpret_cast<uint4 *>(out + (((size_t)b * H + h) * n_pad + t) * HEAD_DIM + seg * 16) =
+        t < N ? quantize_v16(x[it], inv_scale) : make_uint4(0u, 0u, 0u, 0u);
   }
 }
 
@@ -719,13 +725,13 @@ __global__ void __launch_bounds__(256) quantize_v_fp4_tile_kernel(const __nv_bfl
 // Measured (9001 tokens, 32:8 heads): page kernel + a Delta_S kernel that read K again 12 + 16 us, one page per CTA 19.5 us, now
 // 14.1 us.
 constexpr int WK_CTAS = 2;   // resident per SM: 128 registers, so that the means stay in registers
-__global__ void __launch_bounds__(256, WK_CTAS) write_kv_kernel(const __nv_bfloat16 *__restrict__ k, const __nv_bfloat16 *__restrict__ v,
-                                                                const float *__restrict__ k_mean, const TensorScale k_scale,
-                                                                const float *__restrict__ q_mean, const float *__restrict__ q_gscale,
+__global__ void __launch_bounds__(256, WK_CTAS) write_kv_kernel(const __nv_bfloat16 *k, const __nv_bfloat16 *v,
+                                                                const float *k_mean, const TensorScale k_scale,
+                                                                const float *q_mean, const float *q_gscale,
                                                                 int N, int first, int n_pages, int H_q, int H_kv, float inv_vscale,
-                                                                const int32_t *__restrict__ page_row, int num_pages,
-                                                                uint8_t *__restrict__ k_codes, uint8_t *__restrict__ k_sf,
-                                                                uint8_t *__restrict__ v_fp8, __nv_bfloat16 *__restrict__ delta) {
+                                                                const int32_t *page_row, int num_pages,
+                                                                uint8_t *k_codes, uint8_t *k_sf,
+                                                                uint8_t *v_fp8, __nv_bfloat16 *delta) {
   __shared__ __align__(16) GroupMeans gm;
   __shared__ float inv_table[128];
   launch_dependents();
@@ -811,14 +817,14 @@ __global__ void __launch_bounds__(256, WK_CTAS) write_kv_kernel(const __nv_bfloa
 // Measured (64 requests, 40:8 heads): with one thread per FP64 chain of 128 terms and 2 x 256 threads per pair
 // 9.8 us, now 6.6 us.
 template <bool VEC>   // vector_means of both means
-__global__ void __launch_bounds__(256) append_kv_kernel(const __nv_bfloat16 *__restrict__ k, const __nv_bfloat16 *__restrict__ v,
-                                                        const float *__restrict__ q_mean, const float *__restrict__ k_mean,
-                                                        const float *__restrict__ q_gscale, const float *__restrict__ k_gscale,
+__global__ void __launch_bounds__(256) append_kv_kernel(const __nv_bfloat16 *k, const __nv_bfloat16 *v,
+                                                        const float *q_mean, const float *k_mean,
+                                                        const float *q_gscale, const float *k_gscale,
                                                         int B, int H_q, int H_kv, float inv_vscale,
-                                                        const int32_t *__restrict__ page_table, int max_pages, int num_pages,
-                                                        const int32_t *__restrict__ positions, uint8_t *__restrict__ k_codes,
-                                                        uint8_t *__restrict__ k_sf, uint8_t *__restrict__ v_fp8,
-                                                        __nv_bfloat16 *__restrict__ delta) {
+                                                        const int32_t *page_table, int max_pages, int num_pages,
+                                                        const int32_t *positions, uint8_t *k_codes,
+                                                        uint8_t *k_sf, uint8_t *v_fp8,
+                                                        __nv_bfloat16 *delta) {
   launch_dependents();
   grid_dependency_wait();
   const int pair = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31, blk = lane & 7, part = lane >> 3;

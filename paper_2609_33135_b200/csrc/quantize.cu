@@ -116,18 +116,18 @@ __device__ __forceinline__ void finish_column(const ColTensor &a, int b, int h, 
   if (c == 0) a.gmax[(size_t)b * a.H + h] = fmaxf(fmaxf(s_w[0], s_w[1]), fmaxf(s_w[2], s_w[3]));
 }
 
-// grid (slices, heads of both tensors, B)
-__global__ void __launch_bounds__(STAT_THREADS, STAT_CTAS) colstat_kernel(const ColTensor t0, const ColTensor t1, int smooth) {
+// grid (slices * heads of both tensors, 1, B), the slice fastest; heads are not a grid dimension of their own, which ends at 65535
+__global__ void __launch_bounds__(STAT_THREADS, STAT_CTAS) colstat_kernel(const ColTensor t0, const ColTensor t1, int slices, int smooth) {
   __shared__ double s_sum[STAT_LANES][HEAD_DIM];
   __shared__ uint32_t s_mx[STAT_LANES][HEAD_DIM / 2], s_mn[STAT_LANES][HEAD_DIM / 2];
   __shared__ float s_w[4];
   launch_dependents();
   grid_dependency_wait();
-  const bool first = (int)blockIdx.y < t0.H;
+  const int at = blockIdx.x / slices, slice = blockIdx.x - at * slices;
+  const bool first = at < t0.H;
   const ColTensor &a = first ? t0 : t1;
-  const int h = first ? blockIdx.y : blockIdx.y - t0.H;
+  const int h = first ? at : at - t0.H;
   const int b = blockIdx.z, tid = threadIdx.x, tl = tid >> 4, cg = tid & 15;
-  const int slices = gridDim.x, slice = blockIdx.x;
   const int len = ((a.N + slices - 1) / slices + STAT_LANES - 1) / STAT_LANES * STAT_LANES;
   const int begin = min(a.N, slice * len), end = min(a.N, begin + len);
   const size_t row = (size_t)a.H * HEAD_DIM, step = STAT_LANES * row;
@@ -202,14 +202,14 @@ __global__ void __launch_bounds__(STAT_THREADS, STAT_CTAS) colstat_kernel(const 
   __syncthreads();
   if (tid >= HEAD_DIM) return;
   // place of column tid: pair i of group cg
-  const int at = ((tid & 7) >> 1) * 32 + (tid >> 3) * 2 + (tid & 1);
+  const int place = ((tid & 7) >> 1) * 32 + (tid >> 3) * 2 + (tid & 1);
   double sum = 0.0;
   uint32_t hi = 0xFF80FF80u, lo = 0x7F807F80u;
 #pragma unroll
   for (int j = 0; j < STAT_LANES; ++j) {
-    sum += s_sum[j][at];
-    hi = bf16x2_max(hi, s_mx[j][at >> 1]);
-    lo = bf16x2_min(lo, s_mn[j][at >> 1]);
+    sum += s_sum[j][place];
+    hi = bf16x2_max(hi, s_mx[j][place >> 1]);
+    lo = bf16x2_min(lo, s_mn[j][place >> 1]);
   }
   const float fmx = __uint_as_float(tid & 1 ? hi & 0xFFFF0000u : hi << 16), fmn = __uint_as_float(tid & 1 ? lo & 0xFFFF0000u : lo << 16);
   if (slices == 1) {
@@ -932,7 +932,7 @@ mpfa_status tensor_stats(const ColTensor &c0, const ColTensor &c1, int B, int ma
   // of a CTA's pass, so slices are not made shorter than that.
   constexpr int STAT_MIN = 512;
   const int S = (int)std::max(1LL, std::min({(long long)max_slices, (long long)STAT_CTAS * n_sm / ((long long)heads * B), (long long)N / STAT_MIN}));
-  MPFA_CUDA_OK(launch(colstat_kernel, dim3(S, heads, B), dim3(STAT_THREADS), 0, st, c0, c1, smooth ? 1 : 0));
+  MPFA_CUDA_OK(launch(colstat_kernel, dim3(S * heads, 1, B), dim3(STAT_THREADS), 0, st, c0, c1, S, smooth ? 1 : 0));
   if (S > 1) MPFA_CUDA_OK(launch(stat_fold_kernel, dim3(heads, B), dim3(128), 0, st, c0, c1, S, smooth ? 1 : 0));
   return MPFA_OK;
 }

@@ -70,6 +70,20 @@ def test_stage1_bit_exact_over_tile_and_slice_counts(B, N, N_q, H_q, H_kv):
     check_stage1(w, run_stage1_gpu(w), z)
 
 
+def test_stage1_with_more_heads_than_a_grid_dimension():
+    """65538 heads of Q and K in one call (a launch's second and third dimensions end at 65535)."""
+    from paper_2609_33135_b200 import binding
+    H = 32769
+    g = torch.Generator(device="cuda").manual_seed(9)
+    q, k, v = (torch.randn(1, 2, H, 128, generator=g, device="cuda").bfloat16() for _ in range(3))
+    ws = torch.empty(binding.lib().mpfa_quantize_workspace_min_bytes(1, H, H), dtype=torch.uint8, device="cuda")
+    s1 = binding.stage1(q, k, v, workspace=ws)
+    for x, mean in ((q, s1.stats.q_mean), (k, s1.stats.k_mean)):
+        assert torch.equal(mean, x.double().mean(1).float())
+    m = (k.float() - s1.stats.k_mean[:, None]).abs().max()
+    assert s1.stats.k_gscale.cpu().numpy()[0] == np.float32(m.item()) / np.float32(2688.0)
+
+
 def test_stage1_from_inputs_on_16_byte_boundaries():
     """The interface asks for 16-byte alignment; 32-byte aligned inputs take wider loads."""
     from paper_2609_33135_b200 import binding

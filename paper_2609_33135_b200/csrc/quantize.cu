@@ -84,8 +84,11 @@ struct ColTensor {
   double *psum;             // [slices][B][H * 128] partial results
   float2 *pext;             // (max, min)
   float *mean;              // [B, H, 128]
-  float *gmax;              // [B, H]
+  float *gmax;              // [B, H] x MAXIMA_STRIDE
 };
+// The heads' maxima have no room of their own: each stands in the first word of its head's first partial sums, which the head's
+// fold has read by then.
+constexpr size_t MAXIMA_STRIDE = HEAD_DIM * sizeof(double) / sizeof(float);
 
 __device__ __forceinline__ uint32_t bf16x2_max(uint32_t a, uint32_t b) {
   uint32_t d;
@@ -113,7 +116,7 @@ __device__ __forceinline__ void finish_column(const ColTensor &a, int b, int h, 
   asm("redux.sync.max.f32 %0, %0, 0xffffffff;" : "+f"(m));
   if ((c & 31) == 0) s_w[c >> 5] = m;
   asm volatile("bar.sync 1, 128;" ::: "memory");
-  if (c == 0) a.gmax[(size_t)b * a.H + h] = fmaxf(fmaxf(s_w[0], s_w[1]), fmaxf(s_w[2], s_w[3]));
+  if (c == 0) a.gmax[((size_t)b * a.H + h) * MAXIMA_STRIDE] = fmaxf(fmaxf(s_w[0], s_w[1]), fmaxf(s_w[2], s_w[3]));
 }
 
 // grid (slices * heads of both tensors, 1, B), the slice fastest; heads are not a grid dimension of their own, which ends at 65535
@@ -249,7 +252,7 @@ __global__ void __launch_bounds__(128) stat_fold_kernel(const ColTensor t0, cons
 // the same call (1 for an all-zero tensor).
 struct TensorScale {
   float *gscale;       // [B]
-  const float *gmax;   // [B, heads] or null: read gscale
+  const float *gmax;   // [B, heads] x MAXIMA_STRIDE, or null: read gscale
   int heads;
 };
 
@@ -257,7 +260,7 @@ struct TensorScale {
 __device__ __forceinline__ float tensor_scale(const TensorScale &s, int b, int lane) {
   if (!s.gmax) return s.gscale[b];
   float m = 0.0f;
-  for (int i = lane; i < s.heads; i += 32) m = fmaxf(m, s.gmax[(size_t)b * s.heads + i]);
+  for (int i = lane; i < s.heads; i += 32) m = fmaxf(m, s.gmax[((size_t)b * s.heads + i) * MAXIMA_STRIDE]);
   asm("redux.sync.max.f32 %0, %0, 0xffffffff;" : "+f"(m));
   return m > 0.0f ? __fdiv_rn(m, 2688.0f) : 1.0f;
 }
@@ -890,8 +893,9 @@ __global__ void __launch_bounds__(256) append_kv_kernel(const __nv_bfloat16 *k, 
 
 size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 
-// Workspace of the statistics pass: S slices of per-column partial results (FP64 sum, maximum and minimum), and the heads'
-// maxima.  S is the largest slice count <= STAT_MAX_SLICES that fits the bytes the caller gave (at least 1).
+// Workspace of the statistics pass: S slices of per-column partial results (FP64 sum, maximum and minimum).  S is the largest slice
+// count <= STAT_MAX_SLICES that fits the bytes the caller gave (at least 1) beside a region that is no longer used: callers' sizes
+// stay what they were.
 constexpr int STAT_MAX_SLICES = 32;
 size_t stats_fixed_bytes(int B, int H_q, int H_kv) {
   return align256(((size_t)2 * B + (size_t)B * ((H_q + 1) / 2 + (H_kv + 1) / 2) + 1) * sizeof(unsigned int));
@@ -911,16 +915,15 @@ StatsWorkspace carve(void *ws, size_t ws_bytes, int B, int H_q, int H_kv) {
   StatsWorkspace w{};
   const size_t fixed = stats_fixed_bytes(B, H_q, H_kv), per = stats_slice_bytes(B, H_q, H_kv);
   const int S = ws_bytes > fixed ? (int)std::min((ws_bytes - fixed) / per, (size_t)STAT_MAX_SLICES) : 0;
-  // The maxima take the place of one slice.  A pass with a single slice writes no partial results.
-  const size_t nq = (size_t)B * H_q, nk = (size_t)B * H_kv, n = S > 1 ? S - 1 : 0;
-  w.slices = S > 2 ? (int)n : std::min(S, 1);
-  w.gmax_q = static_cast<float *>(ws);
-  w.gmax_k = w.gmax_q + nq;
-  uint8_t *p = static_cast<uint8_t *>(ws) + per;
+  const size_t nq = (size_t)B * H_q, nk = (size_t)B * H_kv, n = S;
+  w.slices = S;
+  uint8_t *p = static_cast<uint8_t *>(ws);
   w.psum_q = reinterpret_cast<double *>(p);  p += n * nq * HEAD_DIM * 8;
   w.psum_k = reinterpret_cast<double *>(p);  p += n * nk * HEAD_DIM * 8;
   w.pext_q = reinterpret_cast<float2 *>(p);  p += n * nq * HEAD_DIM * 8;
   w.pext_k = reinterpret_cast<float2 *>(p);
+  w.gmax_q = reinterpret_cast<float *>(w.psum_q);
+  w.gmax_k = reinterpret_cast<float *>(w.psum_k);
   return w;
 }
 

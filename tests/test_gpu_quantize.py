@@ -330,3 +330,18 @@ def test_stage1_with_a_one_slice_workspace_is_the_same_on_exact_inputs():
         check_stage1(w, binding.stage1(w.q.cuda(), w.k.cuda(), w.v.cuda(), workspace=ws), z)
     with pytest.raises(binding.MpfaError, match="workspace"):
         binding.stage1(w.q.cuda(), w.k.cuda(), w.v.cuda(), workspace=torch.empty(n_min - 256, dtype=torch.uint8, device="cuda"))
+
+
+def test_a_workspace_for_two_slices_is_used_as_two():
+    """Sums of one column that depend on the slices: 2^60, then at the start of the second half -2^60 and 1 in the same lane.  In one
+    slice the two large values cancel first and the mean is 1 / 1024, in two the 1 is lost beside -2^60 and the mean is 0."""
+    from paper_2609_33135_b200 import binding
+    L = binding.lib()
+    n_min, n_full = L.mpfa_quantize_workspace_min_bytes(1, 1, 1), L.mpfa_quantize_workspace_bytes(1, 1, 1)
+    per = (n_full - n_min) // 31
+    x = torch.zeros(1, 1024, 1, 128)
+    x[0, 0, 0, 5], x[0, 512, 0, 5], x[0, 528, 0, 5] = 2.0 ** 60, -2.0 ** 60, 1.0
+    x = x.bfloat16().cuda()
+    for nbytes, mean in ((n_min, 1.0 / 1024), (n_min + per - 256, 1.0 / 1024), (n_min + per, 0.0), (n_full, 0.0)):
+        s1 = binding.stage1(x, x, x, workspace=torch.empty(nbytes, dtype=torch.uint8, device="cuda"))
+        assert float(s1.stats.q_mean[0, 0, 5]) == mean and float(s1.stats.k_mean[0, 0, 5]) == mean, nbytes

@@ -678,7 +678,7 @@ __global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const __grid
       for (int v = 0; v < NV; ++v) {
         const int t = v * TPV + lane / GP;
         const float4 q = *reinterpret_cast<const float4 *>(&xm[(t * MAXG + (lane & (GP - 1))) * 4]);
-        mt[v] = t < w.nblk ? fmaxf(fmaxf(q.x, q.y), fmaxf(q.z, q.w)) : -INFINITY;
+        mt[v] = t < w.nblk ? fmaxf(fmaxf(fmaxf(q.x, q.y), fmaxf(q.z, q.w)), -INFINITY) : -INFINITY;   // NaNs are passed over
 #pragma unroll
         for (int o = GP; o < 32; o <<= 1) {
           const float before = __shfl_up_sync(0xffffffffu, mt[v], o);
@@ -849,7 +849,8 @@ __global__ void __launch_bounds__(128, 9) decode_merge_kernel(const __grid_const
     }
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      const float w = a[u].x == -INFINITY ? 0.0f : ex2_approx(__fmul_rn(a[u].x - M, lam));
+      if (a[u].x == -INFINITY) continue;   // no score above -infinity: left out, its sums need not be finite
+      const float w = ex2_approx(__fmul_rn(a[u].x - M, lam));
       l = __fmaf_rn(w, a[u].y, l);
       o[0] = __fmaf_rn(w, x[u].x, o[0]);
       o[1] = __fmaf_rn(w, x[u].y, o[1]);

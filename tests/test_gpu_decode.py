@@ -423,3 +423,41 @@ def test_serving_step_captured_once_and_replayed():
                                 w_full.softmax_scale, np.array([n], np.int32))
             d = np.abs(got[b] - ref[0])
             assert d.max() <= MAX_ABS and d.mean() <= MEAN_ABS, (s, b, float(d.max()), float(d.mean()))
+
+
+@pytest.mark.parametrize("value", [float("-inf"), float("nan")])
+def test_decode_leaves_a_partition_without_scores_out(value):
+    """A partition whose every score is -infinity (a Delta_S of -infinity hides its keys) or NaN has no maximum; the merge takes the
+    other partitions alone.  Heads in groups of one, so that the value reaches one head only."""
+    from paper_2609_33135_b200 import binding as B_
+    H, L = 2, 2048 + 452
+    g = torch.Generator().manual_seed(17)
+    q, k, v = (torch.randn(n, H, 128, generator=g).bfloat16().cuda() for n in (1, L, L))
+    st = B_.Stats.empty(1, H, H)
+    st.q_mean.copy_(torch.randn(1, H, 128, generator=g)), st.k_mean.zero_()
+    st.q_gscale.fill_(0.0015), st.k_gscale.fill_(0.0015)
+    frozen = B_.MPFA_SMOOTH | B_.MPFA_STATS_FROZEN
+    q4 = B_.Fp4Tensor.empty(1, H, 1)
+    B_.mpfa_quantize_qk(q.view(1, 1, H, 128), None, frozen, st, q4, None, None, None)
+
+    def attend(keys, pages_hidden):
+        n = k[keys].shape[0]
+        n_pages = -(-n // 64)
+        kv = B_.PagedKV.empty(n_pages, H, H)
+        table = torch.arange(n_pages, dtype=torch.int32, device="cuda").view(1, -1)
+        B_.mpfa_quantize_kv_paged(k[keys].contiguous(), v[keys].contiguous(), 0, H, frozen, st, 1.0, kv, table[0], None)
+        kv.delta[pages_hidden, 0] = value
+        out = torch.empty(1, H, 128, dtype=torch.bfloat16, device="cuda")
+        o32 = torch.empty(1, H, 128, dtype=torch.float32, device="cuda")
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        B_.mpfa_decode(q4, kv, table, torch.tensor([n], dtype=torch.int32, device="cuda"), st, 1.0, 128 ** -0.5, out, o32,
+                       B_.decode_workspace(1, H, H, n_pages), status)
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0
+        return o32[0]
+    got = attend(torch.arange(L, device="cuda"), slice(16, 32))
+    want = attend(torch.cat([torch.arange(1024), torch.arange(2048, L)]).cuda(), slice(0, 0))
+    assert float(want[0].abs().max()) > 0 and torch.isfinite(got).all()
+    assert float((got[0] - want[0]).abs().max()) <= 1e-6      # the same partitions, merged in another order
+    everything = attend(torch.arange(L, device="cuda"), slice(0, 0))
+    assert torch.equal(got[1], everything[1])

@@ -508,12 +508,11 @@ __global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const __grid
       w = wn;
       pc0 = pn0, pc1 = pn1;
     }
-    if (!ok) {
-      // another role gave up: let the copies already issued land before shared memory goes away
-      for (uint32_t i = c - min(c, (uint32_t)n_ring); i < c; ++i) {
-        const long long t0 = clock64();
-        while (!mbar_try_wait(cx.bar(b_full + i % n_ring), (i / n_ring) & 1) && clock64() - t0 < D_WAIT_CYCLES) {
-        }
+    // The last copies of this ring land before the warp leaves: where all goes well their consumers wait for them too, and where a
+    // role gives up, before or after this loop has ended, shared memory must not go away under them.
+    for (uint32_t i = c - min(c, (uint32_t)n_ring); i < c; ++i) {
+      const long long t0 = clock64();
+      while (!mbar_try_wait(cx.bar(b_full + i % n_ring), (i / n_ring) & 1) && clock64() - t0 < D_WAIT_CYCLES) {
       }
     }
   } else if (warp == 1) {

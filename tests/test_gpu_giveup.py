@@ -63,9 +63,10 @@ def test_prefill_wait_runs_out_and_the_call_returns(use_giveup_lib, giveup_lib, 
     binding.mpfa_set_prefill_arrangement(0)
 
 
-def test_decode_wait_runs_out_and_the_call_returns(use_giveup_lib):
+@pytest.mark.parametrize("lens", [[1500, 700], [120, 60], [9000] * 24])   # a few items; one and two blocks each; three items per CTA
+def test_decode_wait_runs_out_and_the_call_returns(use_giveup_lib, lens):
     from paper_2609_33135_b200 import binding, decode_cache
-    dw = wl.decode_workload("giveup_decode", 82, 2, 8, 2, 64, 1500, seq_lens=[1500, 700])
+    dw = wl.decode_workload("giveup_decode", 82, len(lens), 8, 2, 64, max(lens), seq_lens=lens)
     st = decode_cache.build_cache(dw)            # cache writes have no waits
     torch.cuda.synchronize()
     t0 = time.time()
@@ -78,7 +79,7 @@ def test_decode_wait_runs_out_and_the_call_returns(use_giveup_lib):
     decode_cache.decode_step(st)
     torch.cuda.synchronize()
     assert int(st.status.item()) == 0
-    for b in range(dw.B):
+    for b in range(min(2, dw.B)):
         k, v = dw.kv_for_request(b)
         zc = orc.stage1(orc.bf16_bits(dw.q_sample[b:b + 1].contiguous()), orc.bf16_bits(k), orc.bf16_bits(v))
         zq = orc.stage1(orc.bf16_bits(dw.q_new[b:b + 1].contiguous()), orc.bf16_bits(k), orc.bf16_bits(v), frozen=zc)

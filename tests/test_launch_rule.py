@@ -73,3 +73,19 @@ def test_launched_kernels_wait_and_read_coherently(source):
             todo += re.findall(r"\b(\w+)\s*(?:<[^;{}()]*>)?\s*\(", body)
         body = funcs[kernel][1]
         assert "grid_dependency_wait()" in body, kernel
+
+
+def test_decode_producers_await_their_last_copies_on_every_way_out():
+    """WorkIter::next() is false both at the end of the list and when another role has given up, and a role may give up after a producer
+    has issued its last copy: whether the producer itself saw a failure says nothing, so its final wait stands under no condition."""
+    text = code("decode.cu")
+    producer = text[text.index("warp == 0 || warp >= 16"):text.index("} else if (warp == 1)")]
+    loop = producer.index("for (; ok && vw; ++j)")
+    depth, i = 0, producer.index("{", loop)
+    while True:
+        depth += {"{": 1, "}": -1}.get(producer[i], 0)
+        i += 1
+        if depth == 0:
+            break
+    after = producer[i:]
+    assert "mbar_try_wait" in after and not re.search(r"\bif\b", after)

@@ -945,14 +945,14 @@ extern "C" mpfa_status mpfa_decode(const mpfa_fp4_tensor *q, const mpfa_paged_kv
   const unsigned grid = (unsigned)(items < (size_t)n_sm ? items : (size_t)n_sm);   // one persistent CTA per SM
   void (*kern)(const DecodeParams) = nullptr;
   switch (H_q / H_kv) {
-    case 1: kern = decode_split_kernel<1>, rc = allow_smem<decode_split_kernel<1>>(dev, D_SMEM); break;
-    case 2: kern = decode_split_kernel<2>, rc = allow_smem<decode_split_kernel<2>>(dev, D_SMEM); break;
-    case 3: kern = decode_split_kernel<3>, rc = allow_smem<decode_split_kernel<3>>(dev, D_SMEM); break;
-    case 4: kern = decode_split_kernel<4>, rc = allow_smem<decode_split_kernel<4>>(dev, D_SMEM); break;
-    case 5: kern = decode_split_kernel<5>, rc = allow_smem<decode_split_kernel<5>>(dev, D_SMEM); break;
-    case 6: kern = decode_split_kernel<6>, rc = allow_smem<decode_split_kernel<6>>(dev, D_SMEM); break;
-    case 7: kern = decode_split_kernel<7>, rc = allow_smem<decode_split_kernel<7>>(dev, D_SMEM); break;
-    case 8: kern = decode_split_kernel<8>, rc = allow_smem<decode_split_kernel<8>>(dev, D_SMEM); break;
+    case 1: kern = decode_split_kernel<1>, rc = allow_smem<decode_split_kernel<1>>(D_SMEM); break;
+    case 2: kern = decode_split_kernel<2>, rc = allow_smem<decode_split_kernel<2>>(D_SMEM); break;
+    case 3: kern = decode_split_kernel<3>, rc = allow_smem<decode_split_kernel<3>>(D_SMEM); break;
+    case 4: kern = decode_split_kernel<4>, rc = allow_smem<decode_split_kernel<4>>(D_SMEM); break;
+    case 5: kern = decode_split_kernel<5>, rc = allow_smem<decode_split_kernel<5>>(D_SMEM); break;
+    case 6: kern = decode_split_kernel<6>, rc = allow_smem<decode_split_kernel<6>>(D_SMEM); break;
+    case 7: kern = decode_split_kernel<7>, rc = allow_smem<decode_split_kernel<7>>(D_SMEM); break;
+    case 8: kern = decode_split_kernel<8>, rc = allow_smem<decode_split_kernel<8>>(D_SMEM); break;
     default: return MPFA_ERR_UNSUPPORTED;
   }
   if (rc != MPFA_OK) return rc;

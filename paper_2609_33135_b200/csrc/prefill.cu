@@ -800,7 +800,7 @@ extern "C" mpfa_status mpfa_prefill_variant(const mpfa_fp4_tensor *q, const mpfa
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const bool other_pv = variant == MPFA_VARIANT_PV_BF16 || variant == MPFA_VARIANT_PV_FP4;
   if (g_arrangement == 1 && !other_pv) return launch_prefill_pair(q, k, v_fp8, p, ew, s);
-  if (ew || other_pv) return launch_prefill_variant(q, k, v_fp8, p, variant, dev, grid, s);
+  if (ew || other_pv) return launch_prefill_variant(q, k, v_fp8, p, variant, grid, s);
   EncodeTiledFn enc;
   rc = get_encoder(&enc);
   if (rc != MPFA_OK) return rc;
@@ -808,9 +808,9 @@ extern "C" mpfa_status mpfa_prefill_variant(const mpfa_fp4_tensor *q, const mpfa
   if ((rc = make_map(enc, &tq, q->codes, q_rows, 64)) != MPFA_OK) return rc;
   if ((rc = make_map(enc, &tk, k->codes, k_rows, 64)) != MPFA_OK) return rc;
   if ((rc = make_map(enc, &tv, v_fp8, k_rows, 128)) != MPFA_OK) return rc;
-  if (nk_tiles < RUN_BLOCKS) return start<prefill_kernel<false, false, false>, SMEM_BYTES<false, false>>(dev, grid, NTHREADS, s, tq, tk, tv, p, PagedSrc{});
-  if (k->N <= LONG_KEYS) return start<prefill_kernel<false, false, true>, SMEM_BYTES<false, true>>(dev, grid, NTHREADS, s, tq, tk, tv, p, PagedSrc{});
-  return start<prefill_kernel<false, true, true>, SMEM_BYTES<false, true>>(dev, grid, NTHREADS, s, tq, tk, tv, p, PagedSrc{});
+  if (nk_tiles < RUN_BLOCKS) return start<prefill_kernel<false, false, false>, SMEM_BYTES<false, false>>(grid, NTHREADS, s, tq, tk, tv, p, PagedSrc{});
+  if (k->N <= LONG_KEYS) return start<prefill_kernel<false, false, true>, SMEM_BYTES<false, true>>(grid, NTHREADS, s, tq, tk, tv, p, PagedSrc{});
+  return start<prefill_kernel<false, true, true>, SMEM_BYTES<false, true>>(grid, NTHREADS, s, tq, tk, tv, p, PagedSrc{});
 }
 
 extern "C" mpfa_status mpfa_prefill_paged(const mpfa_fp4_tensor *q, const mpfa_paged_kv *kv, const int32_t *page_table,
@@ -873,6 +873,6 @@ extern "C" mpfa_status mpfa_prefill_paged(const mpfa_fp4_tensor *q, const mpfa_p
   if ((rc = make_map(enc, &tq, q->codes, q_rows, 64)) != MPFA_OK) return rc;
   const unsigned grid = (unsigned)(n_cta < (uint64_t)n_sm ? n_cta : (uint64_t)n_sm);
   if (max_pages_per_req < RUN_BLOCKS * (TILE / PAGE) - 1)   // no request can have RUN_BLOCKS blocks
-    return start<prefill_kernel<true, true, false>, SMEM_BYTES<true, false>>(dev, grid, NTHREADS, static_cast<cudaStream_t>(stream), tq, tq, tq, p, pg);
-  return start<prefill_kernel<true, true, true>, SMEM_BYTES<true, true>>(dev, grid, NTHREADS, static_cast<cudaStream_t>(stream), tq, tq, tq, p, pg);
+    return start<prefill_kernel<true, true, false>, SMEM_BYTES<true, false>>(grid, NTHREADS, static_cast<cudaStream_t>(stream), tq, tq, tq, p, pg);
+  return start<prefill_kernel<true, true, true>, SMEM_BYTES<true, true>>(grid, NTHREADS, static_cast<cudaStream_t>(stream), tq, tq, tq, p, pg);
 }

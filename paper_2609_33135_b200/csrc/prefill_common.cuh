@@ -38,7 +38,7 @@ struct PagedSrc {
 
 // ablation and precision variants of the contiguous path (prefill_variants.cu)
 mpfa_status launch_prefill_variant(const mpfa_fp4_tensor *q, const mpfa_fp4_tensor *k, const uint8_t *v, PrefillParams p, int variant,
-                                   int dev, unsigned grid, cudaStream_t stream);
+                                   unsigned grid, cudaStream_t stream);
 // two query tiles per CTA (prefill_pair.cu)
 mpfa_status launch_prefill_pair(const mpfa_fp4_tensor *q, const mpfa_fp4_tensor *k, const uint8_t *v_fp8,
                                 const PrefillParams &p, bool elementwise, cudaStream_t stream);
@@ -279,9 +279,9 @@ inline mpfa_status make_map(EncodeTiledFn enc, CUtensorMap *m, const void *base,
 }
 
 template <auto Kernel, uint32_t SMEM>
-inline mpfa_status start(int dev, unsigned grid, int n_threads, cudaStream_t stream, const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap &tv,
+inline mpfa_status start(unsigned grid, int n_threads, cudaStream_t stream, const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap &tv,
                          const PrefillParams &p, const PagedSrc &pg) {
-  mpfa_status rc = allow_smem<Kernel>(dev, SMEM);
+  mpfa_status rc = allow_smem<Kernel>(SMEM);
   if (rc != MPFA_OK) return rc;
   MPFA_CUDA_OK(launch(Kernel, dim3(grid), dim3(n_threads), SMEM, stream, tq, tk, tv, p, pg));
   return MPFA_OK;

@@ -732,7 +732,7 @@ prefill_variant_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
 }  // namespace
 
 mpfa_status launch_prefill_variant(const mpfa_fp4_tensor *q, const mpfa_fp4_tensor *k, const uint8_t *v, PrefillParams p, int variant,
-                                   int dev, unsigned grid, cudaStream_t stream) {
+                                   unsigned grid, cudaStream_t stream) {
   const bool pvb = variant == MPFA_VARIANT_PV_BF16;   // v points at the BF16 tile tensor of mpfa_pack_v_bf16
   const bool pv4 = variant == MPFA_VARIANT_PV_FP4;    // ... at the FP4 operand of mpfa_quantize_v_fp4, v_scale = its v_gscale
   const uint64_t q_rows = (uint64_t)p.B * p.H_q * p.nq_tiles * TILE, k_rows = (uint64_t)p.B * p.H_kv * p.nk_tiles * TILE;
@@ -749,9 +749,9 @@ mpfa_status launch_prefill_variant(const mpfa_fp4_tensor *q, const mpfa_fp4_tens
   if ((rc = make_map(enc, &tq, q->codes, q_rows, 64)) != MPFA_OK) return rc;
   if ((rc = make_map(enc, &tk, k->codes, k_rows, 64)) != MPFA_OK) return rc;
   if ((rc = pvb ? make_map(enc, &tv, v, k_rows, 256, 128) : make_map(enc, &tv, v, k_rows, pv4 ? 64 : 128)) != MPFA_OK) return rc;
-  if (pvb) return start<prefill_variant_kernel<1>, Lay<1>::SMEM_BYTES>(dev, grid, NTHREADS, stream, tq, tk, tv, p, PagedSrc{});
-  if (pv4) return start<prefill_variant_kernel<2>, Lay<2>::SMEM_BYTES>(dev, grid, NTHREADS, stream, tq, tk, tv, p, PagedSrc{});
-  return start<prefill_variant_kernel<0>, Lay<0>::SMEM_BYTES>(dev, grid, NTHREADS, stream, tq, tk, tv, p, PagedSrc{});
+  if (pvb) return start<prefill_variant_kernel<1>, Lay<1>::SMEM_BYTES>(grid, NTHREADS, stream, tq, tk, tv, p, PagedSrc{});
+  if (pv4) return start<prefill_variant_kernel<2>, Lay<2>::SMEM_BYTES>(grid, NTHREADS, stream, tq, tk, tv, p, PagedSrc{});
+  return start<prefill_variant_kernel<0>, Lay<0>::SMEM_BYTES>(grid, NTHREADS, stream, tq, tk, tv, p, PagedSrc{});
 }
 
 }  // namespace mpfa

@@ -140,13 +140,11 @@ def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
     return None if t is None else t.data_ptr()
 
 
-# The raw handle of torch's current stream: the same as torch.cuda.current_stream().cuda_stream without building a Stream
-# object (3.4 us a call, as much as a launch).
-_raw_stream, _device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
-
-
 def _stream() -> int:
-    return _raw_stream(_device())
+    """The raw handle of torch's current stream: torch.cuda.current_stream().cuda_stream without building a Stream object (3.4 us a
+    call, as much as a launch) where torch offers that."""
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    return torch.cuda.current_stream().cuda_stream if raw is None else raw(torch.cuda.current_device())
 
 
 def _pad128(n: int) -> int:

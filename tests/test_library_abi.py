@@ -93,3 +93,21 @@ def test_paged_entry_points_validate_shapes_before_any_cuda_call(built):
     assert L.mpfa_prefill_paged(args[0], ctypes.byref(kv_unaligned), *args[2:]) == -3         # pool not 256-byte aligned
     assert L.mpfa_prefill_paged(*args[:7], 0.0, *args[8:]) == -1                               # v_scale must be positive
     assert L.mpfa_prefill_paged(*args[:3], 0, *args[4:]) == -1                                 # max_pages_per_req
+
+
+def test_binding_imports_where_torch_has_no_cuda(built):
+    """A torch build without CUDA has none of the private functions that the binding looks for; importing it and the host-only calls
+    do not need them."""
+    import subprocess
+    import sys
+    child = """
+import torch
+for name in [n for n in dir(torch._C) if n.startswith("_cuda_get")]:
+    delattr(torch._C, name)
+from paper_2609_33135_b200 import binding
+assert binding.lib().mpfa_version() >= 100
+torch.cuda.current_stream = lambda: type("Stream", (), {"cuda_stream": 77})()
+assert binding._stream() == 77
+"""
+    r = subprocess.run([sys.executable, "-c", child], cwd=ROOT, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]

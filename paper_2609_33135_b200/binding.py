@@ -48,8 +48,9 @@ class _PagedKV(ctypes.Structure):
                 ("H_q", ctypes.c_int32), ("H_kv", ctypes.c_int32)]
 
 
-# The same structures as packed bytes, which ctypes passes by address: building one takes half the time of a Structure, and a
-# call with three of them 0.7 us less.
+# The same structures as packed bytes, which ctypes passes by address: making and passing three of them takes 1.3 us, three Structures
+# 2.9 us.  Bytes have no type that a call could check, so only the wrappers below pass them, to function objects of their own
+# (packed_mpfa_...), and each kind has a method of its own name; the functions of lib() take typed structures only.
 _pack_stats, _pack_fp4, _pack_paged = struct.Struct("4P").pack, struct.Struct("2P4i").pack, struct.Struct("4P4i").pack
 
 _lib = None
@@ -89,12 +90,19 @@ def load_library(path: str) -> ctypes.CDLL:
         L.mpfa_status_string.argtypes = [i]
         L.mpfa_last_cuda_error.restype = i
         L.mpfa_version.restype = i
-        L.mpfa_quantize_qk.restype = i
-        L.mpfa_quantize_qk.argtypes = [vp, vp, i, i, i, i, i, i, vp, vp,
-                                       vp, vp, vp, sz, vp]
-        L.mpfa_quantize_qk_static.restype = i
-        L.mpfa_quantize_qk_static.argtypes = [vp, vp, i, i, i, i, i, i, vp, vp,
-                                              vp, vp, vp]
+        st, q4, pk = ctypes.POINTER(_Stats), ctypes.POINTER(_Fp4), ctypes.POINTER(_PagedKV)
+        for name, args in (("mpfa_quantize_qk", [vp, vp, i, i, i, i, i, i, st, q4, q4, vp, vp, sz, vp]),
+                           ("mpfa_quantize_qk_static", [vp, vp, i, i, i, i, i, i, st, q4, q4, vp, vp]),
+                           ("mpfa_quantize_kv_paged", [vp, vp, i, i, i, i, i, st, f, pk, vp, vp, sz, vp]),
+                           ("mpfa_append_kv_paged", [vp, vp, i, i, i, i, st, f, pk, vp, i, vp, vp]),
+                           ("mpfa_prefill", [q4, q4, vp, vp, st, f, i, f, vp, vp, vp, vp]),
+                           ("mpfa_prefill_variant", [q4, q4, vp, vp, st, f, i, f, i, vp, vp, vp, vp]),
+                           ("mpfa_prefill_paged", [q4, pk, vp, i, vp, vp, st, f, f, vp, vp, vp, vp]),
+                           ("mpfa_decode", [q4, pk, vp, i, vp, st, f, f, vp, vp, vp, sz, vp, vp])):
+            typed, packed = getattr(L, name), L[name]   # two function objects of one symbol
+            typed.restype = packed.restype = i
+            typed.argtypes, packed.argtypes = args, [vp if t in (st, q4, pk) else t for t in args]
+            setattr(L, "packed_" + name, packed)
         L.mpfa_static_scratch_bytes.restype = sz
         L.mpfa_quantize_v.restype = i
         L.mpfa_quantize_v.argtypes = [vp, i, i, i, f, vp, vp]
@@ -102,24 +110,6 @@ def load_library(path: str) -> ctypes.CDLL:
         L.mpfa_quantize_v_fp4.argtypes = [vp, i, i, i, f, vp, vp]
         L.mpfa_pack_v_bf16.restype = i
         L.mpfa_pack_v_bf16.argtypes = [vp, i, i, i, vp, vp]
-        L.mpfa_quantize_kv_paged.restype = i
-        L.mpfa_quantize_kv_paged.argtypes = [vp, vp, i, i, i, i, i, vp, f,
-                                             vp, vp, vp, sz, vp]
-        L.mpfa_append_kv_paged.restype = i
-        L.mpfa_append_kv_paged.argtypes = [vp, vp, i, i, i, i, vp, f, vp, vp, i,
-                                           vp, vp]
-        L.mpfa_prefill.restype = i
-        L.mpfa_prefill.argtypes = [vp, vp, vp, vp, vp, f, i,
-                                   f, vp, vp, vp, vp]
-        L.mpfa_decode.restype = i
-        L.mpfa_decode.argtypes = [vp, vp, vp, i, vp, vp,
-                                  f, f, vp, vp, vp, sz, vp, vp]
-        L.mpfa_prefill_variant.restype = i
-        L.mpfa_prefill_variant.argtypes = [vp, vp, vp, vp, vp, f, i,
-                                           f, i, vp, vp, vp, vp]
-        L.mpfa_prefill_paged.restype = i
-        L.mpfa_prefill_paged.argtypes = [vp, vp, vp, i, vp, vp,
-                                         vp, f, f, vp, vp, vp, vp]
         L.mpfa_set_prefill_arrangement.restype = i
         L.mpfa_set_prefill_arrangement.argtypes = [i]
         L.mpfa_bench_mma_peak.restype = i
@@ -179,7 +169,7 @@ class Stats:
         return _Stats(self.q_mean.data_ptr(), self.k_mean.data_ptr(), self.q_gscale.data_ptr(),
                       self.k_gscale.data_ptr())
 
-    def packed(self) -> bytes:
+    def packed_stats(self) -> bytes:
         return _pack_stats(self.q_mean.data_ptr(), self.k_mean.data_ptr(), self.q_gscale.data_ptr(), self.k_gscale.data_ptr())
 
     def request(self, b: int) -> "Stats":
@@ -205,7 +195,7 @@ class Fp4Tensor:
     def c(self) -> _Fp4:
         return _Fp4(self.codes.data_ptr(), self.sf.data_ptr(), self.B, self.H, self.N)
 
-    def packed(self) -> bytes:
+    def packed_fp4(self) -> bytes:
         return _pack_fp4(self.codes.data_ptr(), self.sf.data_ptr(), self.B, self.H, self.N, 0)
 
 
@@ -233,7 +223,7 @@ class PagedKV:
                         None if self.delta is None else self.delta.data_ptr(), self.num_pages, PAGE,
                         self.H_q, self.H_kv)
 
-    def packed(self) -> bytes:
+    def packed_paged(self) -> bytes:
         return _pack_paged(self.k_codes.data_ptr(), self.k_sf.data_ptr(), self.v_fp8.data_ptr(),
                            0 if self.delta is None else self.delta.data_ptr(), self.num_pages, PAGE, self.H_q, self.H_kv)
 
@@ -254,10 +244,10 @@ def mpfa_quantize_qk(q: Optional[torch.Tensor], k: Optional[torch.Tensor], flags
     H_kv = k.shape[2] if k is not None else (H_kv if H_kv is not None else stats.k_mean.shape[1])
     for t in (q, k):
         assert t is None or (t.is_cuda and t.dtype == torch.bfloat16 and t.is_contiguous() and t.shape[3] == HEAD_DIM)
-    sc = stats.packed()
-    qc = q_out.packed() if q_out is not None else None
-    kc = k_out.packed() if k_out is not None else None
-    rc = lib().mpfa_quantize_qk(_ptr(q), _ptr(k), B, N_q, N_kv, H_q, H_kv, flags, sc,
+    sc = stats.packed_stats()
+    qc = q_out.packed_fp4() if q_out is not None else None
+    kc = k_out.packed_fp4() if k_out is not None else None
+    rc = lib().packed_mpfa_quantize_qk(_ptr(q), _ptr(k), B, N_q, N_kv, H_q, H_kv, flags, sc,
                                 qc,
                                 kc, _ptr(delta), _ptr(workspace),
                                 0 if workspace is None else workspace.numel(), _stream())
@@ -277,10 +267,10 @@ def mpfa_quantize_qk_static(q: Optional[torch.Tensor], k: Optional[torch.Tensor]
     N_kv = k.shape[1] if k is not None else 0
     H_q = q.shape[2] if q is not None else stats.q_mean.shape[1]
     H_kv = k.shape[2] if k is not None else stats.k_mean.shape[1]
-    sc = stats.packed()
-    qc = q_out.packed() if q_out is not None else None
-    kc = k_out.packed() if k_out is not None else None
-    rc = lib().mpfa_quantize_qk_static(_ptr(q), _ptr(k), B, N_q, N_kv, H_q, H_kv, flags, sc,
+    sc = stats.packed_stats()
+    qc = q_out.packed_fp4() if q_out is not None else None
+    kc = k_out.packed_fp4() if k_out is not None else None
+    rc = lib().packed_mpfa_quantize_qk_static(_ptr(q), _ptr(k), B, N_q, N_kv, H_q, H_kv, flags, sc,
                                        qc,
                                        kc, _ptr(delta), _stream())
     _check(rc, "mpfa_quantize_qk_static")
@@ -299,8 +289,8 @@ def mpfa_quantize_kv_paged(k: torch.Tensor, v: torch.Tensor, first_token: int, H
     assert k.is_cuda and k.dtype == torch.bfloat16 and k.is_contiguous() and v.is_contiguous()
     assert page_table_row.dtype == torch.int32 and page_table_row.is_cuda
     N, H_kv, _ = k.shape
-    sc, kc = stats.packed(), kv.packed()
-    rc = lib().mpfa_quantize_kv_paged(_ptr(k), _ptr(v), N, first_token, H_q, H_kv, flags, sc, v_scale,
+    sc, kc = stats.packed_stats(), kv.packed_paged()
+    rc = lib().packed_mpfa_quantize_kv_paged(_ptr(k), _ptr(v), N, first_token, H_q, H_kv, flags, sc, v_scale,
                                       kc, _ptr(page_table_row), _ptr(workspace),
                                       0 if workspace is None else workspace.numel(), _stream())
     _check(rc, "mpfa_quantize_kv_paged")
@@ -313,8 +303,8 @@ def mpfa_append_kv_paged(k: torch.Tensor, v: torch.Tensor, H_q: int, flags: int,
     assert page_table.dtype == torch.int32 and page_table.is_contiguous() and positions.dtype == torch.int32
     B, one, H_kv, _ = k.shape
     assert one == 1
-    sc, kc = stats.packed(), kv.packed()
-    rc = lib().mpfa_append_kv_paged(_ptr(k), _ptr(v), B, H_q, H_kv, flags, sc, v_scale, kc,
+    sc, kc = stats.packed_stats(), kv.packed_paged()
+    rc = lib().packed_mpfa_append_kv_paged(_ptr(k), _ptr(v), B, H_q, H_kv, flags, sc, v_scale, kc,
                                     _ptr(page_table), page_table.shape[1], _ptr(positions), _stream())
     _check(rc, "mpfa_append_kv_paged")
 
@@ -322,8 +312,8 @@ def mpfa_append_kv_paged(k: torch.Tensor, v: torch.Tensor, H_q: int, flags: int,
 def mpfa_prefill(q: Fp4Tensor, k: Fp4Tensor, v_fp8: torch.Tensor, delta: Optional[torch.Tensor], stats: Stats,
                  v_scale: float, causal: bool, softmax_scale: float, out: torch.Tensor,
                  out_f32: Optional[torch.Tensor], device_status: torch.Tensor) -> None:
-    sc, qc, kc = stats.packed(), q.packed(), k.packed()
-    rc = lib().mpfa_prefill(qc, kc, _ptr(v_fp8), _ptr(delta), sc, v_scale,
+    sc, qc, kc = stats.packed_stats(), q.packed_fp4(), k.packed_fp4()
+    rc = lib().packed_mpfa_prefill(qc, kc, _ptr(v_fp8), _ptr(delta), sc, v_scale,
                             int(causal), softmax_scale, _ptr(out), _ptr(out_f32), _ptr(device_status), _stream())
     _check(rc, "mpfa_prefill")
 
@@ -331,8 +321,8 @@ def mpfa_prefill(q: Fp4Tensor, k: Fp4Tensor, v_fp8: torch.Tensor, delta: Optiona
 def mpfa_prefill_variant(q: Fp4Tensor, k: Fp4Tensor, v_fp8: torch.Tensor, delta: Optional[torch.Tensor], stats: Stats,
                          v_scale: float, causal: bool, softmax_scale: float, variant: int, out: torch.Tensor,
                          out_f32: Optional[torch.Tensor], device_status: torch.Tensor) -> None:
-    sc, qc, kc = stats.packed(), q.packed(), k.packed()
-    rc = lib().mpfa_prefill_variant(qc, kc, _ptr(v_fp8), _ptr(delta), sc, v_scale,
+    sc, qc, kc = stats.packed_stats(), q.packed_fp4(), k.packed_fp4()
+    rc = lib().packed_mpfa_prefill_variant(qc, kc, _ptr(v_fp8), _ptr(delta), sc, v_scale,
                                     int(causal), softmax_scale, int(variant), _ptr(out), _ptr(out_f32),
                                     _ptr(device_status), _stream())
     _check(rc, "mpfa_prefill_variant")
@@ -347,8 +337,8 @@ def mpfa_decode(q: Fp4Tensor, kv: PagedKV, page_table: torch.Tensor, seq_lens: t
                 v_scale: float, softmax_scale: float, out: torch.Tensor, out_f32: Optional[torch.Tensor],
                 workspace: torch.Tensor, device_status: torch.Tensor) -> None:
     assert page_table.dtype == torch.int32 and page_table.is_contiguous() and seq_lens.dtype == torch.int32
-    sc, qc, kc = stats.packed(), q.packed(), kv.packed()
-    rc = lib().mpfa_decode(qc, kc, _ptr(page_table), page_table.shape[1], _ptr(seq_lens),
+    sc, qc, kc = stats.packed_stats(), q.packed_fp4(), kv.packed_paged()
+    rc = lib().packed_mpfa_decode(qc, kc, _ptr(page_table), page_table.shape[1], _ptr(seq_lens),
                            sc, v_scale, softmax_scale, _ptr(out), _ptr(out_f32), _ptr(workspace),
                            workspace.numel(), _ptr(device_status), _stream())
     _check(rc, "mpfa_decode")
@@ -359,8 +349,8 @@ def mpfa_prefill_paged(q: Fp4Tensor, kv: PagedKV, page_table: torch.Tensor, seq_
                        device_status: torch.Tensor, q_lens: Optional[torch.Tensor] = None) -> None:
     assert page_table.dtype == torch.int32 and page_table.is_contiguous() and seq_lens.dtype == torch.int32
     assert q_lens is None or q_lens.dtype == torch.int32
-    sc, qc, kc = stats.packed(), q.packed(), kv.packed()
-    rc = lib().mpfa_prefill_paged(qc, kc, _ptr(page_table), page_table.shape[1],
+    sc, qc, kc = stats.packed_stats(), q.packed_fp4(), kv.packed_paged()
+    rc = lib().packed_mpfa_prefill_paged(qc, kc, _ptr(page_table), page_table.shape[1],
                                   _ptr(seq_lens), _ptr(q_lens), sc, v_scale, softmax_scale, _ptr(out),
                                   _ptr(out_f32), _ptr(device_status), _stream())
     _check(rc, "mpfa_prefill_paged")

@@ -111,3 +111,35 @@ assert binding._stream() == 77
 """
     r = subprocess.run([sys.executable, "-c", child], cwd=ROOT, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stderr[-2000:]
+
+
+def test_packed_structures_are_the_typed_ones(built):
+    """The wrappers pass the structures as packed bytes; the layout that users get is the typed one's, a null Delta_S included."""
+    import torch
+    from paper_2609_33135_b200 import binding as B
+    f, u = torch.zeros(4), torch.zeros(4, dtype=torch.uint8)
+    st = B.Stats(f[0:], f[1:], f[2:], f[3:])
+    q = B.Fp4Tensor(u[0:], u[1:], 3, 40, 129)
+    assert st.packed_stats() == bytes(st.c()) and q.packed_fp4() == bytes(q.c())
+    for delta in (f.bfloat16(), None):
+        kv = B.PagedKV(u[0:], u[1:], u[2:], delta, 7, 40, 8)
+        assert kv.packed_paged() == bytes(kv.c())
+
+
+def test_a_wrong_structure_is_refused(built):
+    """Neither the functions of lib() nor the wrappers take one structure for another."""
+    import torch
+    from paper_2609_33135_b200 import binding as B
+    L = B.lib()
+    st, q, kv = B._Stats(0, 0, 0, 0), B._Fp4(0, 0, 1, 1, 1), B._PagedKV(0, 0, 0, 0, 1, 64, 1, 1)
+    b = ctypes.byref
+    for args in ((b(st), b(q), None, None, b(st)), (b(q), b(kv), None, None, b(st)), (b(q), b(q), None, None, b(q)), (bytes(32), b(q), None, None, b(st))):
+        with pytest.raises(ctypes.ArgumentError):
+            L.mpfa_prefill(*args, 1.0, 0, 1.0, None, None, None, None)
+    with pytest.raises(ctypes.ArgumentError):
+        L.mpfa_decode(b(q), b(st), None, 1, None, b(st), 1.0, 1.0, None, None, None, 0, None, None)
+    f, u = torch.zeros(4), torch.zeros(4, dtype=torch.uint8)
+    stats, fp4, paged = B.Stats(f, f, f, f), B.Fp4Tensor(u, u, 1, 1, 1), B.PagedKV(u, u, u, None, 1, 1, 1)
+    for q_, k_, s_ in ((stats, fp4, stats), (fp4, paged, stats), (fp4, fp4, fp4)):
+        with pytest.raises((AttributeError, ctypes.ArgumentError)):
+            B.mpfa_prefill(q_, k_, u, None, s_, 1.0, False, 1.0, u, None, u)

@@ -48,34 +48,13 @@ namespace {
 
 namespace pair {
 
-// Optional timeline capture for tuning (compiled in only with -DMPFA_TRACE): one CTA records clock64() at fixed
-// points of every role, [role][index of the stage's block][event].
-#ifdef MPFA_TRACE
-__device__ long long *g_ptrace = nullptr;
-__device__ int g_ptrace_cta = 0;
-#define TR_INIT() long long *tr_buf = ((int)blockIdx.x == g_ptrace_cta && lane == 0) ? g_ptrace : nullptr
-#define TR(role, t, ev)                                                              \
-  do {                                                                               \
-    if (tr_buf && (t) < 512) tr_buf[((role) * 512 + (t)) * 8 + (ev)] = clock64();    \
-  } while (0)
-#else
-#define TR_INIT() do {} while (0)
-#define TR(role, t, ev) do {} while (0)
-#endif
-
 constexpr int KSTAGES = 4;
 constexpr int VSTAGES = 3;
 constexpr int NTHREADS = 512;
 constexpr int REGS_SOFTMAX = 168;
-#ifndef MPFA_PAIR_LATE
-#define MPFA_PAIR_LATE 1
-#endif
-#ifndef MPFA_PAIR_REGS_UTIL
-#define MPFA_PAIR_REGS_UTIL 56   // measured for this kernel: 56/120 1264 / 1354, 72/104 1245 / 1318, 80/96 1228 / 1288
-#define MPFA_PAIR_REGS_CORR 120
-#endif
-template <bool PAGED> constexpr int REGS_UTIL = PAGED ? 64 : MPFA_PAIR_REGS_UTIL;
-template <bool PAGED> constexpr int REGS_CORR = PAGED ? 112 : MPFA_PAIR_REGS_CORR;
+// utility / correction warps, 16384 / 65536 keys in TFLOPS: 56/120 1264 / 1354, 72/104 1245 / 1318, 80/96 1228 / 1288
+template <bool PAGED> constexpr int REGS_UTIL = PAGED ? 64 : 56;
+template <bool PAGED> constexpr int REGS_CORR = PAGED ? 112 : 120;
 // setmaxnreg only moves registers inside the pool the CTA got at launch (512 threads x 128 registers); a request
 // beyond the pool would block forever, and a "dec" to more than 128 or an "inc" to less is an illegal instruction.
 static_assert(4 * REGS_UTIL<false> + 8 * REGS_SOFTMAX + 4 * REGS_CORR<false> <= 16 * 128, "register pool");
@@ -234,7 +213,6 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
   const uint32_t tm = *tmem_slot;
 
   const bool has_delta = !EW && p.delta != nullptr;   // operand of the seed MMA
-  TR_INIT();
 
   // Every role walks the same list of items and keeps the same running counts: gb = KV blocks of the items walked
   // (slot and phase of the K and V rings), tq = items that had any block (Q buffers), n_r = blocks stage r has
@@ -380,17 +358,12 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         for (int r = 0; r < 2; ++r) {
           if (jb >= it.T[r]) continue;
           // the previous user of the score buffer has read its scores into registers
-          TR(2, ns, 0);
           if (ns >= 1) ok = cx.wait(BAR_S_EMPTY, (ns - 1) & 1u);
           if (!ok) break;
-          TR(2, ns, 1);
           tc_fence_after();
           if (elect_one()) {
             const uint64_t d_q = d_q00 + (uint64_t)(((qb * 2 + r) * 8192) >> 4);
             const uint32_t tSFQ = tm + TM_SFQ + 8 * (qb * 2 + r);
-#ifdef MPFA_ABLATE_NO_QK
-            if (t > 100000)
-#endif
             {
               if (has_delta) mma_bf16_ss(tm + TM_S, d_ones, d_delta, id_bf16, 0);
               mma_nvfp4_ss(tm + TM_S, d_q, d_k, id_fp4, tSFQ, tSFK, has_delta ? 1u : 0u);
@@ -398,7 +371,6 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             }
             mma_commit(cx.bar(BAR_S_FULL + r));
           }
-          TR(2, ns, 2);
           ++ns;
         }
         if (!ok) break;
@@ -460,26 +432,19 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
           const uint32_t n = r ? n1 : n0, u = r ? u1 : u0;
           const bool first = jb == it.T[r] - 1;
           // the epilogue of the stage's previous item has read the accumulator that this block overwrites
-          TR(3 + r, n, 0);
           if (first && u >= 1) ok = cx.wait(BAR_O_FREE + r, (u - 1) & 1u);
           ok = ok && cx.wait(BAR_O_READY + 2 * r + (n & 1), (n >> 1) & 1u);
-          TR(3 + r, n, 1);
           ok = ok && cx.wait(BAR_P_FULL + r, n & 1u);
-          TR(3 + r, n, 2);
           if (!ok) break;
           tc_fence_after();
           if (elect_one()) {
 #pragma unroll
             for (int k4 = 0; k4 < 4; ++k4)
-#ifdef MPFA_ABLATE_NO_PV
-              if (k4 > 100)
-#endif
               mma_e4m3_ts(tm + TM_O + 128 * r, tm + TM_P + 32 * r + 8 * k4, d_v + (uint64_t)((4096 * k4) >> 4), id_fp8,
                           (!first || k4 > 0) ? 1u : 0u);
             mma_commit(cx.bar(BAR_O_FULL + r));
             mma_commit(cx.bar(BAR_P_EMPTY + r));
           }
-          TR(3 + r, n, 3);
           if (r) ++n1; else ++n0;
         }
         if (!ok) break;
@@ -509,24 +474,12 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       const int limit = (r_abs >= it.nq) ? -1   // a row past the request's own query count sees nothing
                         : p.causal ? min(it.nkv - 1, r_abs + (it.nkv - it.nq)) : it.nkv - 1;   // last visible key
       const float lam = __fmul_rn(__fmul_rn(__fmul_rn(p.softmax_scale, 1.4426950408889634f), p.q_gscale[it.b]), p.k_gscale[it.b]);
-#if MPFA_PAIR_LATE
       bool p_pending = false;
-#endif
       float m_run = -INFINITY;   // running maximum (Eq. 3)
       float l_run = 0.0f;        // running sum of 448 P (Eq. 5)
       for (int jb = T - 1; jb >= 0; --jb, ++n) {
         const int key0 = jb * TILE;
-        TR(r, n, 0);
-#if MPFA_PAIR_LATE == 2
-        if (p_pending) {
-          tmem_st_wait();
-          tc_fence_before();
-          warp_arrive(cx.bar(BAR_P_FULL + r), lane);
-          p_pending = false;
-        }
-#endif
         if (!__all_sync(0xffffffffu, cx.wait(BAR_S_FULL + r, n & 1u))) { ok = false; break; }
-        TR(r, n, 1);
         tc_fence_after();
         uint32_t s[128];
         {
@@ -535,14 +488,12 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
           tmem_ld32(tS, s0);
           tmem_ld32(tS + 32, s1);
         }
-#if MPFA_PAIR_LATE == 1
         if (p_pending) {
           tmem_st_wait();
           tc_fence_before();
           warp_arrive(cx.bar(BAR_P_FULL + r), lane);
           p_pending = false;
         }
-#endif
         // P V of the stage's previous block has consumed the P_hat columns (tested early, used before the stores)
         const bool pe_early = (n < 1) || cx.probe(BAR_P_EMPTY + r, (n - 1) & 1u);
         const bool ragged = key0 + TILE - 1 > limit;   // diagonal / ragged block only
@@ -554,14 +505,6 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
           tmem_ld32(tS + 64, s2);
           tmem_ld32(tS + 96, s3);
         }
-#if MPFA_PAIR_LATE == 3
-        if (p_pending) {
-          tmem_st_wait();
-          tc_fence_before();
-          warp_arrive(cx.bar(BAR_P_FULL + r), lane);
-          p_pending = false;
-        }
-#endif
         if constexpr (EW) {
           const uint4 *dp = reinterpret_cast<const uint4 *>(
               p.delta + ((size_t)it.b * p.H_q + it.hq) * (size_t)(p.nk_tiles * TILE) + key0);
@@ -593,7 +536,6 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         tmem_ld_wait();
         tc_fence_before();
         warp_arrive(cx.bar(BAR_S_EMPTY), lane);   // the row is in registers: the other stage's Q K^T may overwrite it
-        TR(r, n, 2);
         if constexpr (EW) {
           const uint4 *dp = reinterpret_cast<const uint4 *>(
               p.delta + ((size_t)it.b * p.H_q + it.hq) * (size_t)(p.nk_tiles * TILE) + key0 + 64);
@@ -622,17 +564,12 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
           mx2 = max3(mx2, __uint_as_float(s[i + 4]), __uint_as_float(s[i + 5]));
           mx3 = max3(mx3, __uint_as_float(s[i + 6]), __uint_as_float(s[i + 7]));
         }
-#ifdef MPFA_ABLATE_NO_MAX
-        const float mx = fmaxf(__uint_as_float(s[0]), __uint_as_float(s[127])) + 30.0f;
-#else
         const float mx = fmaxf(fmaxf(mx0, mx1), fmaxf(mx2, mx3));
-#endif
         const float m_new = fmaxf(m_run, mx);
         // alpha = 2^(lam (m_old - m_new)) (Eq. 5/6): 1 when the maximum did not move, 0 for the row's first block
         const float alpha = (m_new == m_run) ? 1.0f : ex2_approx(__fmul_rn(m_run - m_new, lam));
         s_alpha[(n & 1) * 128 + row] = alpha;
         warp_arrive(cx.bar(BAR_A_FULL + 2 * r + (n & 1)), lane);
-        TR(r, n, 3);
         m_run = m_new;
         // q = 448 P = 2^(lam S - lam m + log2 448) is the E4M3 operand (Section 4.1); the row sum is taken over q
         // and the factor 448 is divided out once in the epilogue.
@@ -640,13 +577,7 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         if (!__all_sync(0xffffffffu, pe_early)) {
           if (!__all_sync(0xffffffffu, cx.wait(BAR_P_EMPTY + r, (n - 1) & 1u))) { ok = false; break; }
         }
-        TR(r, n, 4);
         float sum0 = 0.0f, sum1 = 0.0f, sum2 = 0.0f, sum3 = 0.0f;
-#ifdef MPFA_ABLATE_NO_EXP
-#define EX2_(x) (x)
-#else
-#define EX2_(x) ex2_approx(x)
-#endif
 #pragma unroll
         for (int c0 = 0; c0 < 128; c0 += 32) {
           uint32_t packed[8];
@@ -655,7 +586,7 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             float x0, x1, x2, x3;
             fma2(x0, x1, __uint_as_float(s[c0 + 4 * i]), __uint_as_float(s[c0 + 4 * i + 1]), lam, cc);
             fma2(x2, x3, __uint_as_float(s[c0 + 4 * i + 2]), __uint_as_float(s[c0 + 4 * i + 3]), lam, cc);
-            const float q0 = EX2_(x0), q1 = EX2_(x1), q2 = EX2_(x2), q3 = EX2_(x3);
+            const float q0 = ex2_approx(x0), q1 = ex2_approx(x1), q2 = ex2_approx(x2), q3 = ex2_approx(x3);
             acc2(sum0, sum1, q0, q1);
             acc2(sum2, sum3, q2, q3);
             // two conversions written into the halves of one register (no separate merge instruction)
@@ -669,24 +600,14 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
           tmem_st8(tP + (c0 >> 2), packed);
         }
         l_run = __fadd_rn(__fmul_rn(alpha, l_run), (sum0 + sum1) + (sum2 + sum3));
-#if MPFA_PAIR_LATE
         p_pending = true;
-#else
-        tmem_st_wait();
-        TR(r, n, 5);
-        tc_fence_before();
-        warp_arrive(cx.bar(BAR_P_FULL + r), lane);
-#endif
-        TR(r, n, 6);
       }
-#if MPFA_PAIR_LATE
       if (p_pending) {
         tmem_st_wait();
         tc_fence_before();
         warp_arrive(cx.bar(BAR_P_FULL + r), lane);
         p_pending = false;
       }
-#endif
       if (!ok) break;
       s_l[(u & 3) * 128 + row] = l_run;
       warp_arrive(cx.bar(BAR_L_FULL + r * 4 + (u & 3)), lane);
@@ -708,21 +629,14 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         for (int r = 0; r < 2; ++r) {
           if (jb >= it.T[r] || !ok) continue;
           const uint32_t n = r ? n1 : n0;
-          TR(5 + r, n, 0);
           ok = __all_sync(0xffffffffu, cx.wait(BAR_A_FULL + 2 * r + (n & 1), (n >> 1) & 1u));
           if (!ok) break;
-          TR(5 + r, n, 1);
           const float alpha = s_alpha[r * 256 + (n & 1) * 128 + row];
           if (jb != it.T[r] - 1) {
             // O_r holds the stage's earlier blocks relative to the previous maximum (Eq. 6)
-#ifdef MPFA_ABLATE_NO_CORR
-            if (false) {
-#else
             if (__any_sync(0xffffffffu, alpha != 1.0f)) {   // identical result when every factor is exactly 1
-#endif
               ok = __all_sync(0xffffffffu, cx.wait(BAR_O_FULL + r, (n - 1) & 1u));
               if (!ok) break;
-              TR(5 + r, n, 2);
               tc_fence_after();
               const uint32_t tO = tm + TM_O + 128 * r + lane_off;
 #pragma unroll
@@ -743,7 +657,6 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             }
           }
           warp_arrive(cx.bar(BAR_O_READY + 2 * r + (n & 1)), lane);
-          TR(5 + r, n, 3);
           if (r) ++n1; else ++n0;
         }
       }
@@ -815,13 +728,6 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
 
 using namespace mpfa;
 
-#ifdef MPFA_TRACE
-extern "C" int mpfa_debug_set_pair_trace(long long *buf, int cta) {
-  if (cudaMemcpyToSymbol(pair::g_ptrace, &buf, sizeof(buf)) != cudaSuccess) return -1;
-  if (cudaMemcpyToSymbol(pair::g_ptrace_cta, &cta, sizeof(cta)) != cudaSuccess) return -1;
-  return 0;
-}
-#endif
 
 // Launchers used by the entry points in prefill.cu.
 namespace mpfa {

@@ -89,3 +89,11 @@ def test_decode_producers_await_their_last_copies_on_every_way_out():
             break
     after = producer[i:]
     assert "mbar_try_wait" in after and not re.search(r"\bif\b", after)
+
+
+def test_the_only_build_switches_are_the_give_up_test_builds():
+    """No probe that leaves work out, and no path that only other builds reach, is in the sources."""
+    found = set()
+    for f in SOURCES:
+        found |= set(re.findall(r"^[ \t]*#[ \t]*(?:if|ifdef|ifndef|elif)\b[^\n]*?\b(MPFA_\w+)", code(f), flags=re.M))
+    assert found == {"MPFA_WAIT_LIMIT_CYCLES", "MPFA_DRAIN_LIMIT_NS", "MPFA_TEST_DROP_V_COPY"}

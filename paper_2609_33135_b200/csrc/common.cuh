@@ -21,6 +21,7 @@ inline int pad128(int n) { return (n + TILE - 1) / TILE * TILE; }
 inline bool aligned(const void *p, size_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
 
 inline mpfa_status cuda_fail(cudaError_t e) {
+  (void)cudaGetLastError();   // reported here: not again by the next call that asks
   g_last_cuda_error = static_cast<int>(e);
   return MPFA_ERR_CUDA;
 }

@@ -54,3 +54,18 @@ def test_calls_in_a_second_context_of_the_device():
     out = subprocess.run([sys.executable, "-c", CHILD, ROOT], capture_output=True, text=True, timeout=300)
     assert out.returncode == 0, out.stderr[-2000:]
     assert out.stdout.split("\n")[:3] == ["[0, 0, 0, 0] 0"] * 3, out.stdout
+
+
+def test_a_failed_launch_does_not_fail_the_next_call():
+    """A launch that the driver refuses (more batch elements than a grid's third dimension holds) is reported by its own call only."""
+    import torch
+    from paper_2609_33135_b200 import binding
+    small = torch.ones(1, 1, 1, 128, dtype=torch.bfloat16, device="cuda")
+    many = torch.zeros(65536, 1, 1, 128, dtype=torch.bfloat16, device="cuda")
+    out = torch.empty(binding.lib().mpfa_v_fp8_bytes(65536, 1, 1), dtype=torch.uint8, device="cuda")
+    for _ in range(2):
+        with pytest.raises(binding.MpfaError, match="CUDA"):
+            binding.mpfa_quantize_v(many, 1.0, out)
+        tiles = binding.mpfa_pack_v_bf16(small)
+        torch.cuda.synchronize()
+        assert float(tiles[0, 0, 0].float().min()) == 1.0

@@ -197,6 +197,32 @@ def test_prefill_on_degenerate_inputs(kind):
     compare(o16, o32, rows[keep], ref32[keep], kind)
 
 
+def explain(z, rows, o32, ref32, scale, causal, n_vis):
+    """The rows of a call whose every row sees the first n_vis keys that are within MAX_ABS of the oracle (mask).  The two sides' 2^x
+    differ by up to 2 ulp, so the E4M3 code of a key whose 448 P is within 2e-6 of a rounding boundary may come out one step (6 %)
+    apart.  A row beyond the bound must be such a row: the oracle with one or two of those keys' codes moved one step across
+    reproduces it."""
+    g32 = o32[rows[:, 0], rows[:, 2], rows[:, 1]]
+    assert np.isfinite(g32).all()
+    d = np.abs(g32 - ref32).max(axis=1)
+    grid = np.array([orc.e4m3_decode(c) for c in range(0x7F)], np.float64)
+    bounds = (grid[1:] + grid[:-1]) / 2
+    over = np.nonzero(d > MAX_ABS)[0]
+    assert len(over) <= max(1, len(rows) // 100), len(over)
+    for r in over:
+        row = rows[r:r + 1]
+        codes, _, q, base = orc.phat_rows(z, row, scale, causal, want_q=True)
+        qv = q[0, :n_vis].astype(np.float64)
+        nearest = np.abs(qv[:, None] - bounds[None, :])
+        j = nearest.argmin(axis=1)
+        cands = np.nonzero(nearest[np.arange(n_vis), j] <= 2e-6 * bounds[j])[0]
+        moved = [orc.phat_rows(z, row, scale, causal, want_q=True, flip_key=int(k), flip_dir=1 if codes[0, k] == j[k] else -1)[3][0] - base[0]
+                 for k in cands]
+        sums = moved + [x + y for i, x in enumerate(moved) for y in moved[:i]]   # the moves add: the row sum is not quantized
+        assert any(np.abs(g32[r] - (ref32[r] + m)).max() <= MAX_ABS for m in sums), (row, float(d[r]), len(cands))
+    return d <= MAX_ABS
+
+
 @pytest.mark.parametrize("N_kv", [128, 130, 300, 513])
 def test_prefill_item_boundaries_through_every_ring(N_kv):
     """1920 items of one, two, three and five blocks, thirteen on each persistent CTA: item boundaries at every slot and
@@ -207,17 +233,7 @@ def test_prefill_item_boundaries_through_every_ring(N_kv):
     z = orc.stage1(orc.bf16_bits(w.q), orc.bf16_bits(w.k), orc.bf16_bits(w.v))
     rows = np.array([(0, h, 128 * t + (37 * t + 11 * h) % 128) for t in range(60) for h in range(32)])   # (b, head, query)
     ref32, _ = orc.prefill_rows(z, rows, w.softmax_scale, False)
-    # the two sides' 2^x differ by up to 2 ulp, so the E4M3 code of a key whose 448 P is within 2e-6 of a rounding boundary may
-    # come out one step (6 %) apart: rows with such a key (a few per cent, known from the oracle alone) are left out
-    _, _, q, _ = orc.phat_rows(z, rows, w.softmax_scale, False, want_q=True)
-    grid = np.array([orc.e4m3_decode(c) for c in range(0x7F)], np.float64)
-    bounds = (grid[1:] + grid[:-1]) / 2
-    qv = q[:, :N_kv].astype(np.float64)
-    j = np.searchsorted(bounds, qv)
-    rel = np.minimum(np.abs(qv - bounds[np.minimum(j, 125)]) / bounds[np.minimum(j, 125)],
-                     np.abs(qv - bounds[np.maximum(j - 1, 0)]) / bounds[np.maximum(j - 1, 0)])
-    keep = rel.min(axis=1) > 2e-6
-    assert keep.mean() > 0.9
+    keep = explain(z, rows, o32, ref32, w.softmax_scale, False, N_kv)
     compare(o16, o32, rows[keep], ref32[keep], f"N_kv {N_kv}")
 
 

@@ -231,3 +231,49 @@ def test_paged_prefill_many_query_tiles_past_the_request_length():
     rows = orc.all_rows(1, H_q, 128)
     ref32, _ = orc.prefill_rows(z, rows, w.softmax_scale, True)
     compare(o16n[:, :128], o32n[:, :128], rows, ref32, "live tile")
+
+
+@pytest.mark.parametrize("B,N_q", [(73, 850), (128, 500), (171, 300), (512, 100)])   # 511, 512 and 513 (query tile, request) groups; 512 of one tile
+def test_paged_prefill_on_both_sides_of_the_ordered_batch(B, N_q):
+    """Up to 512 groups are walked in the order of their lengths, more as numbered.  Ragged contexts of 1 to 300 tokens and query counts
+    from none to the context's: every row of the output is written, and each request's are the bits that a call of its own gives."""
+    from paper_2609_33135_b200 import binding as B_
+    H_q, H_kv = 2, 1
+    g = torch.Generator().manual_seed(B)
+    L = torch.randint(1, 301, (B,), generator=g)
+    QL = (torch.rand(B, generator=g) * (torch.minimum(L, torch.tensor(N_q)) + 1)).int()
+    QL[:4] = torch.tensor([0, 1, 0, 0])
+    pages = ((L + 63) // 64).tolist()
+    table = torch.full((B, 5), -1, dtype=torch.int32)
+    order = torch.randperm(sum(pages), generator=g).int()
+    at = 0
+    for b, n in enumerate(pages):
+        table[b, :n] = order[at:at + n]
+        at += n
+    table = table.cuda()
+    kv = B_.PagedKV.empty(at, H_q, H_kv)
+    st = B_.Stats(torch.randn(B, H_q, 128, generator=g).cuda(), torch.randn(B, H_kv, 128, generator=g).cuda(), torch.full((B,), 0.0015).cuda(),
+                  torch.full((B,), 0.0015).cuda())
+    flags = B_.MPFA_SMOOTH | B_.MPFA_STATS_FROZEN
+    for b in range(B):
+        k, v = (torch.randn(int(L[b]), H_kv, 128, generator=g).bfloat16().cuda() for _ in range(2))
+        B_.mpfa_quantize_kv_paged(k, v, 0, H_q, flags, st.request(b), 1.0, kv, table[b], None)
+    q4 = B_.Fp4Tensor.empty(B, H_q, N_q)
+    B_.mpfa_quantize_qk(torch.randn(B, N_q, H_q, 128, generator=g).bfloat16().cuda(), None, flags, st, q4, None, None, None)
+    seq, ql = L.int().cuda(), QL.cuda()
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+
+    def run(n, q, rows, lens, stats, counts):
+        out = torch.full((n, N_q, H_q, 128), 5.0, dtype=torch.bfloat16, device="cuda")
+        o32 = torch.full((n, N_q, H_q, 128), 5.0, dtype=torch.float32, device="cuda")
+        B_.mpfa_prefill_paged(q, kv, rows, lens, stats, 1.0, 128 ** -0.5, out, o32, status, q_lens=counts)
+        return out, o32
+    out, o32 = run(B, q4, table, seq, st, ql)
+    codes, sf = q4.codes.view(B, -1), q4.sf.view(B, -1)
+    for b in range(B):
+        one16, one32 = run(1, B_.Fp4Tensor(codes[b], sf[b], 1, H_q, N_q), table[b:b + 1], seq[b:b + 1], st.request(b), ql[b:b + 1])
+        assert torch.equal(o32[b].view(torch.int32), one32[0].view(torch.int32)) and torch.equal(out[b].view(torch.int16), one16[0].view(torch.int16)), b
+        assert not o32[b, int(QL[b]):].any() and (QL[b] == 0 or o32[b, :int(QL[b])].any()), b
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    assert not (o32 == 5.0).any()

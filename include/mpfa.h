@@ -134,7 +134,11 @@ typedef struct {
  *          mpfa_quantize_workspace_bytes() is the size that lets the statistics pass cut the token axis into
  *          its full number of slices; any size down to mpfa_quantize_workspace_min_bytes() (one slice) is accepted and
  *          only lowers the parallelism of that pass; less: MPFA_ERR_WORKSPACE.
- * All arithmetic is specified step by step (FP64 column sums, one rounding to FP32, IEEE divisions).  The column
+ * Means, scales and codes are specified step by step (FP64 column sums, one rounding to FP32, the results of IEEE
+ * divisions).  Delta_S is an FP64 sum over the channels, in an order of the kernel's own, divided by the tensor scales
+ * (or multiplied by their reciprocal in FP64) and rounded to FP32 and BF16: reproducible bit for bit in each entry point;
+ * between entry points (mpfa_quantize_qk, mpfa_quantize_kv_paged, mpfa_append_kv_paged) it may differ in the last BF16
+ * bit where the exact value is within a few parts in 2^52 of a rounding boundary.  The column
  * sums are added in a fixed order (tokens ascending within a thread, then token lanes, then slices; the order is a
  * function of the shapes, the workspace size and the device's SM count), so the outputs are reproducible bit for
  * bit for any input.  They

@@ -1,7 +1,7 @@
 // QK4PV8 decode over a paged low-bit KV cache (Section 5.3) for sm_100a.
 //
-// The path is bound by streaming the cache from HBM (208 bytes per token and kv head plus
-// Delta_S), so the kernel is a persistent streaming pipeline: one CTA per SM walks a list of
+// The path is bound by streaming the cache from HBM (200 bytes per token and kv head plus
+// 2 of Delta_S per q head), so the kernel is a persistent streaming pipeline: one CTA per SM walks a list of
 // (request, kv head, 1024-token partition) work items, and a producer warp keeps two rings of
 // 128-key blocks in flight with bulk asynchronous copies: a K ring (codes, block scales,
 // Delta_S) that runs one item AHEAD of a V ring.  The cache's physical byte order

@@ -30,11 +30,10 @@
 // same thread (two groups that alternate over the blocks and hand the maximum to one another) the chain held up every item's
 // first and last blocks and every causal diagonal.  Warps of their own run the chain ahead of the exponentials; the second
 // reading of the scores costs 72 cycles of the tensor-memory port.  Two score buffers and one accumulator take the place of
-// one and two.  Measured, the kernel alone, alternating groups -> this: 8 x 577 keys x 16 heads, not causal, 79.4 -> 72.2 us,
-// causal 1999 x 40 heads 87.0 -> 82.6, 4 x 777 x 8 heads 37.3 -> 34.2, chunks of 512 queries on paged contexts 483 -> 427; causal 16384 x 32
-// heads 1730 -> 1715 us and 131072 x 32 98.8 -> 99.1 ms, where the clock falls to 1.75-1.83 GHz under the power limit.
-// (Figures of that step; the mask moved to the maximum warps for short contexts and an epilogue of 16 columns at a time, whose
-// registers the rescale loop had to spill, gave what stands at the kernel below.)
+// one and two.  Measured, the kernel alone (us, back to back), alternating groups / this as it is now: 256 keys x 1 head 11.3 / 7.4;
+// 8 x 577 keys x 16 heads, not causal, 48.2 / 35.7; 4 x 777 x 8 heads 20.5 / 14.2; causal 1999 x 40 heads 61.4 / 51.2; 4096 x 32 133.8 /
+// 117.8; 16384 x 32 1636 / 1558; 131072 x 32 96.8 / 97.2 ms (where the power limit sets the clock); chunks of 512 queries on
+// pages 424 / 310; 16384 x 32 from pages 1782 / 1720.
 // What must not be in the exponentials: one straight run of 128 took 1130 cycles where the same code with a mask test or a wait
 // per 32 scores took 2200.
 //
@@ -58,13 +57,12 @@ constexpr int NTHREADS = 640;
 // request beyond the pool would block forever, so the split is checked here.
 constexpr int LAUNCH_REGS = 96;
 // exponentials / maxima / correction / utility.  The paged instance's producer and re-tiling warps need more, see below.
-// Measured (us; causal 1999 x 40 heads, 16384 x 32): short instance 144/48/80/64 75.7, 1625; 152/48/72/56 75.4, 1630; 144/64/80/48
-// 76.3, 1640; 136/56/88/64 75.7, 1635.  Long: 144/56/72/64 79.5, 1650; 144/64/80/48 81.0, 1665; 152/48/72/56 80.2, 1656.
-// Paged (chunks of 512): 152/48/72/56 423, 144/56/72/64 435, 144/64/80/48 427.  Less than 48 for the maxima or 72 for the
-// correction spills heavily.
-// With an item's blocks in several runs (RUNS; us, kernel alone, 16384 x 32 / 131072 x 32 / chunks of 512 on pages): 144/56/88/48 1553,
-// 96.6 ms, 312; 152/48/80/48 1556, 96.4 ms, 312; 144/48/88/56 1549, 97.0 ms, 315; 144/48/80/64 1564, 97.1 ms, 314; 152/48/72/56 1598,
-// 96.7 ms, 318.
+// Measured without runs (whole passes with stage 1, us; causal 1999 x 40 heads, 16384 x 32): short instance 144/48/80/64 75.7, 1625;
+// 152/48/72/56 75.4, 1630; 144/64/80/48 76.3, 1640; 136/56/88/64 75.7, 1635.  Paged (chunks of 512): 152/48/72/56 423, 144/56/72/64
+// 435, 144/64/80/48 427.  Less than 48 for the maxima or 72 for the correction spills heavily.
+// With runs (RUNS; the kernel alone, us, 16384 x 32 / 131072 x 32 / chunks of 512 on pages / 16384 x 32 from pages): 144/56/88/48 1553,
+// 96.6 ms, 310, 1720; 152/48/80/48 1556, 96.4 ms, 312, 1742; 144/48/88/56 1549, 97.0 ms, 315, 1737; 144/48/80/64 1564, 97.1 ms, 314,
+// 1752; 152/48/72/56 1598, 96.7 ms, 318, 1771.
 template <bool PAGED, bool LONG, bool RUNS> constexpr int REGS_EXP = RUNS ? (LONG && !PAGED ? 152 : 144) : (PAGED ? 152 : 144);
 template <bool PAGED, bool LONG, bool RUNS> constexpr int REGS_MAX = RUNS ? (LONG && !PAGED ? 48 : 56) : (PAGED || !LONG ? 48 : 56);
 template <bool PAGED, bool LONG, bool RUNS> constexpr int REGS_CORR = RUNS ? (LONG && !PAGED ? 80 : 88) : (PAGED || LONG ? 72 : 80);
@@ -108,7 +106,7 @@ enum {
 };
 static_assert(NUM_BARS <= 64, "barrier table");
 
-// Contiguous operands: the most keys that the short instance takes; both sides measured, see the kernel
+// Contiguous operands: the most keys that the short instance takes (measured at the kernel: the shorter side's last clear gain)
 constexpr int LONG_KEYS = 49152;
 
 // RUNS: an item of RUN_BLOCKS KV blocks or more accumulates them in two runs, from 256 blocks in four.  The tensor core drops what
@@ -118,9 +116,9 @@ constexpr int LONG_KEYS = 49152;
 // 2.9e-5, on 131072 keys 8.0e-5 / 6.0e-5 / 6.4e-5.  After a run the correction warps move O to shared memory (added to what is
 // there, scaled to the present maximum), the next P V starts from zero, and the epilogue adds the sum of the earlier runs.  It costs
 // (us, kernel alone, one run / these) 16384 x 32 heads 1539 / 1558, 131072 x 32 96.8 / 97.2 ms, chunks of 512 on pages 299 / 312.
-// Shorter items stay in one run, within 8e-7 (from 16 blocks on 1.1e-6 above would be 8.9e-7, but the pass over 1999 keys x 40 heads
-// 87.7 us instead of 82.4: the copy's 64 KB of shared memory keep this kernel's CTAs from starting beside the last ones of
-// stage 1).  Launches that have no longer ones take an instance without this code.
+// Shorter items stay in one run, within 8e-7.  (Runs from 16 blocks on would make 8.9e-7 of the 1.1e-6 above, but the pass over 1999
+// keys x 40 heads 87.7 us instead of 82.4, the kernel alone 52.4 instead of 51.2: with the copy's 64 KB of shared memory its CTAs
+// do not fit beside the last ones of stage 1.)  Launches that have no longer items take an instance without this code.
 constexpr int RUN_BLOCKS = 32;
 template <bool RUNS>
 __device__ __forceinline__ int run_length(int T) { return !RUNS || T < RUN_BLOCKS ? T : T < 256 ? (T + 1) >> 1 : (T + 3) >> 2; }
@@ -141,7 +139,7 @@ constexpr uint32_t OFF_TAIL = OFF_MISC + 128;              // what only some ins
 constexpr uint32_t RAW_STAGE = 1280;
 constexpr uint32_t OFF_RAW = OFF_TAIL;
 constexpr uint32_t OFF_ORDER = OFF_RAW + KST * RAW_STAGE;
-// O of the first run of an item's blocks, [32 groups of 4 columns][128 rows] x 16 bytes
+// O of the runs so far of an item's blocks, [32 groups of 4 columns][128 rows] x 16 bytes
 template <bool PAGED> constexpr uint32_t OFF_RUN = PAGED ? OFF_ORDER + 2 * MAX_GROUPS : OFF_TAIL;
 template <bool PAGED, bool RUNS>
 constexpr uint32_t SMEM_BYTES = OFF_RUN<PAGED> + (RUNS ? HEAD_DIM * 128 * 4 : 0) + 1024;   // + slack for the 1024-byte alignment
@@ -189,10 +187,12 @@ __device__ __forceinline__ float exponent_unit(const PrefillParams &p, int b) {
 
 // LONG: who masks and how P_hat is stored.  false: the maximum warps write masked scores back to tensor memory, so the code of the
 // exponentials has no mask in it (it is read by every pass and competes for the instruction cache with the other roles'), and
-// P_hat goes out in one store.  true: the exponent warps mask, P_hat in two stores.  Measured, false / true (us): 8 x 577 keys x 16
-// heads, not causal, 67.7 / 70.8, causal 1999 x 40 75.7 / 79.5, 16384 x 32 1625 / 1650, 32768 x 32 6037 / 6090,
-// but 65536 x 32 23.44 / 23.05 ms, 131072 x 32 92.8 / 88.9 ms and chunks of 512 on pages 473 / 423 us: where rescales of O are rare the exponentials set the pace, and there
-// the compiler's schedule of the second form is the better one.
+// P_hat goes out in one store.  true: the exponent warps mask, P_hat in two stores.  The arithmetic is the same.  Measured, the kernel
+// alone, false / true (us): 8 x 577 keys x 16 heads, not causal, 35.5 / 37.9; causal 1999 x 40 50.6 / 53.4; 4096 x 32 117.6 / 126.9;
+// 8192 x 32 413 / 437; 16384 x 32 1580 / 1629; 32768 x 32 5933 / 6002; 49152 x 32 13.54 / 13.71 ms; 57344 x 32 18.71 / 18.69; 65536 x 32 24.4 /
+// 24.6; 131072 x 32 102.6 / 97.7.  Not causal: 32768 x 16 5.97 / 6.03 ms, 49152 x 8 6.67 / 6.70, 65536 x 8 11.90 / 11.83.  From pages the
+// second form is ahead at every length (chunks of 512 on 4120 to 15011 tokens 314 / 310 us, 16384 x 32 1764 / 1720).  Neither
+// result is explained beyond the compiler's schedules, which differ in every role: the rule is what was measured.
 template <bool PAGED, bool LONG, bool RUNS>
 __global__ void __launch_bounds__(NTHREADS, 1)
 prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,

@@ -25,13 +25,12 @@
 //                (Eq. 6), and at the end of an item O_r / (448 l) * v_scale -> BF16 (Algorithm 1 line 17).
 // Tensor memory (496 of 512 columns): S [0,128), O_0 [128,256), O_1 [256,384), P_hat_0 [384,416), P_hat_1 [416,448),
 // scale factors of 2 x 2 query tiles [448,480) and of two K blocks [480,496).
-// Measured on B200 against the one-query-tile kernel of prefill.cu (same arithmetic row by row): 1264 against 1338
-// TFLOPS at 16K, 1354 against 1445 at 64K (0.94x), although this kernel executes 12 % fewer instructions per
-// block.  Before P-hat was handed to the P V issuer late (at the top of the stage's next block instead of after its
-// tensor-memory stores) it stood at 1105 / 1188: with one accumulator per tile the rescale of O sits between two
-// dependent P V MMAs of that tile (the other kernel alternates two accumulators), and at these lengths some row of a
-// warp moves its maximum in most blocks; with the rescaling compiled out both kernels take the same time.  This
-// arrangement is therefore not the default (mpfa_set_prefill_arrangement).
+// Measured on B200 against the one-query-tile kernel of prefill.cu (same arithmetic row by row): 1.69 against 1.55 ms at 16384
+// tokens x 32 heads, 25.9 against 23.6 at 65536 (0.92x, 0.91x).  P-hat is handed to the P V issuer late, at the top of the stage's next
+// block instead of after its tensor-memory stores (1105 -> 1264 TFLOPS at 16384).  What holds it back, from its structure: the maximum, the
+// exponentials and the hand-overs of a tile are one chain on one warpgroup (the other kernel has warps of their own for the maxima),
+// and the two tiles take turns at one score buffer.  This arrangement is therefore not the default
+// (mpfa_set_prefill_arrangement).
 // Template parameter EW: the compensation-placement ablation (no seed MMA, Delta_S added element by element by the
 // softmax threads).  Every mbarrier wait is bounded; on expiry the CTA raises MPFA_DEV_TIMEOUT in *device_status,
 // all roles leave their loops, outstanding TMA copies are drained and tensor memory is released.

@@ -4,9 +4,10 @@
 // compensation vector Delta_S (Eq. 9) and the FP8 quantization of V.
 //
 // Everything here is bandwidth work: 16-byte global loads, 8/16-byte stores, tiles staged in
-// shared memory where the destination order differs from the source order.  Every
-// floating-point step uses an explicitly rounded intrinsic so the results are defined to
-// the bit (no FMA contraction, IEEE division).
+// shared memory where the destination order differs from the source order.  Every floating-point step of the means, scales and
+// codes uses an explicitly rounded intrinsic, so those are defined to the bit (no FMA contraction; where a division is
+// replaced, it is done all the same whenever the result could differ).  Delta_S is summed in FP64 in an order of each kernel's own,
+// see there.
 #include <cuda_bf16.h>
 #include <cuda_fp4.h>
 #include <cuda_fp8.h>
@@ -408,8 +409,12 @@ __device__ __forceinline__ void center16(const Row16 &x, const float (&nm)[16], 
 //   channel(j, s) = 16 j + s (s < 16), 64 + 16 j + s - 16,
 // and the sums come out complete, without staging rows or shuffling.  (A chain of 128 FP64 FMAs per key and head, as one
 // thread each, was bound by latency; with the eight threads of a key taking 16 channels each, by the shared-memory reads of the
-// query means.)  The order of the FP64 additions is fixed; it differs from a sequential sum by a few parts in 2^53, and BF16
-// keeps eight bits.
+// query means.)  The order of the FP64 additions is fixed in each kernel, but not the same: the tensor instruction's here and in
+// write_kv_kernel, two chains and two shuffles for groups of one or two heads, eight lanes' chains and three shuffles in
+// append_kv_kernel, which also divides where the others multiply by a reciprocal.  The sums differ by a few parts in 2^53 of their
+// terms, and one rounding to FP32 and one to BF16 follow: two kernels (or the oracle's single ascending chain) give another
+// BF16 only where the exact quotient is that close to a midpoint of two floats which themselves round apart.  No tested input shows
+// one; a tie that FP64 holds exactly comes out the same everywhere.
 //
 // Query means as doubles in operand order: [step][head][j].
 typedef double GroupMeans[32][8][4];

@@ -133,8 +133,11 @@ def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
 def _stream() -> int:
     """The raw handle of torch's current stream: torch.cuda.current_stream().cuda_stream without building a Stream object (3.4 us a
     call, as much as a launch) where torch offers that."""
-    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
-    return torch.cuda.current_stream().cuda_stream if raw is None else raw(torch.cuda.current_device())
+    c = torch._C
+    try:
+        return c._cuda_getCurrentRawStream(c._cuda_getDevice())
+    except AttributeError:
+        return torch.cuda.current_stream().cuda_stream
 
 
 def _pad128(n: int) -> int:

@@ -31,18 +31,18 @@ def use_giveup_lib(giveup_lib):
     binding.mpfa_set_prefill_arrangement(0)
 
 
-def _prefill_case():
-    w = wl.prefill_workload("giveup", 81, 1, 640, 4, 2, True, q_bias=True)
+def _prefill_case(N_kv, N_q):
+    w = wl.prefill_workload("giveup", 81, 1, N_kv, 4, 2, True, N_q=N_q, q_bias=True)
     z = orc.stage1(orc.bf16_bits(w.q), orc.bf16_bits(w.k), orc.bf16_bits(w.v))
-    rows = orc.all_rows(1, 4, 640)
+    rows = orc.all_rows(1, 4, N_q)
     ref32, _ = orc.prefill_rows(z, rows, w.softmax_scale, True)
     return w, rows, ref32
 
 
-@pytest.mark.parametrize("arrangement", [0, 1])
-def test_prefill_wait_runs_out_and_the_call_returns(use_giveup_lib, giveup_lib, arrangement):
+@pytest.mark.parametrize("arrangement,N_kv,N_q", [(0, 640, 640), (1, 640, 640), (0, 4352, 130)])   # the last: accumulation in two runs
+def test_prefill_wait_runs_out_and_the_call_returns(use_giveup_lib, giveup_lib, arrangement, N_kv, N_q):
     from paper_2609_33135_b200 import binding
-    w, rows, ref32 = _prefill_case()
+    w, rows, ref32 = _prefill_case(N_kv, N_q)
     giveup_lib.mpfa_set_prefill_arrangement(arrangement)
     s1 = binding.stage1(w.q.cuda(), w.k.cuda(), w.v.cuda())      # stage 1 has no waits: unaffected
     torch.cuda.synchronize()

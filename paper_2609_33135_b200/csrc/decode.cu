@@ -25,8 +25,8 @@
 // a V block is consumed the moment it lands, and the softmax never sits on the critical path.
 // The sequential rescaling O <- 2^(lam (m_old - m_new)) O + P_hat V becomes
 // O = sum_u 2^(lam (m_u - m)) O_u at the end of the item (one thread per channel), the same
-// sum with the factors multiplied out.  Two groups of four warps take the softmax of alternate items and a third
-// one the O of every item: the P_hat of an item has to be ready when the V of the item before it has been consumed,
+// sum with the factors multiplied out.  Two groups of four warps take the softmax of alternate blocks of an item and a
+// third one the O of every item: the P_hat of an item has to be ready when the V of the item before it has been consumed,
 // so a group that also wrote O out would have one item's time (5.3 us at memory speed) for both.
 //
 // A request that fits one partition is finished right there.  Otherwise the partition state (m, l, O) goes to the
@@ -40,8 +40,13 @@
 // (5.9 / 5.6 / 5.6 / 5.2 TB/s of cache); 64 requests of 100..4000 tokens, 40:8 heads: 227 -> 59 us.  The running maxima and
 // block weights held in the lanes and handed out by shuffles, where every thread took them from shared memory for every
 // block: 256 requests of 100..2000 tokens with append and query 137 -> 130 us, one request of 4097 22.6 -> 21.7 us.
+// K blocks by two warps in turn, each lane issuing its own block, MMAs issued by one thread that also waits, both softmax groups on every
+// item, V held back until the first item's K is on its way (replayed back to back): one request of 4097 keys 15.4 -> 12.6 us, 64 of
+// 100..4000 57.5 -> 53.8, 32 of 16K..128K 690 -> 629 (7.1 TB/s of cache).  Not kept: K rings of 5, 6 and 7 stages (1 to 3 us more on
+// short batches, nothing on long ones), small pieces by 16-byte copies of all lanes (no gain), partitions shorter than 1024 keys
+// drawn last (2 us more on 64 requests).
 //
-// Warps: 18 draws work items and stages their query tiles, 0 and 17 K producers (codes; scales and Delta_S),
+// Warps: 18 draws work items and stages their query tiles, 0 and 17 K producers (alternate blocks),
 // 16 V producer, 1 QK issue (+ TMEM allocation), 2 PV issue, 3 rewrites the K scales of each block from
 // [token][8] into the 32 x 16-byte tiles tcgen05.cp expects, 4-7 and 8-11 the two softmax groups, 12-15 O (TMEM lane
 // quadrant = warp % 4).  Every wait is bounded.
@@ -81,8 +86,8 @@ constexpr uint32_t D_OFF_BAR = D_OFF_IDENT + 2048;
 constexpr uint32_t D_OFF_XMAX = D_OFF_BAR + 1024;           // [2][8 blocks][MAXG][4 warps] floats
 constexpr uint32_t D_OFF_WTAB = D_OFF_XMAX + 2 * MAXBLK * MAXG * 16;   // [2][8 blocks][MAXG] floats
 constexpr uint32_t D_OFF_MFIN = D_OFF_WTAB + 2 * MAXBLK * MAXG * 4;    // [2][MAXG]
-constexpr uint32_t D_OFF_XL = D_OFF_MFIN + 2 * MAXG * 4;               // [2][4 warps][MAXG]
-constexpr uint32_t D_OFF_MISC = D_OFF_XL + 2 * 4 * MAXG * 4;           // TMEM address, abort flag
+constexpr uint32_t D_OFF_XL = D_OFF_MFIN + 2 * MAXG * 4;               // [2][8 warps][MAXG]
+constexpr uint32_t D_OFF_MISC = D_OFF_XL + 2 * 8 * MAXG * 4;           // TMEM address, abort flag
 constexpr int D_MAXREQ = 768;                                          // requests whose length / lambda are cached
 constexpr uint32_t D_OFF_LEN = D_OFF_MISC + 64;                        // [D_MAXREQ] int32 lengths
 constexpr uint32_t D_OFF_LAM = D_OFF_LEN + D_MAXREQ * 4;               // [D_MAXREQ] float
@@ -98,17 +103,18 @@ constexpr int B_V_FULL = B_K_EMPTY + D_NK;       // [D_NV]
 constexpr int B_V_EMPTY = B_V_FULL + D_NV;       // [D_NV] PV commit
 constexpr int B_SF_READY = B_V_EMPTY + D_NV;     // [D_NK] K scales formatted
 constexpr int B_S_FULL = B_SF_READY + D_NK;      // [2] QK commit after the item's last block
-constexpr int B_S_FREE = B_S_FULL + 2;           // [2] 4 warps: the item's scores have been read
-constexpr int B_P_READY = B_S_FREE + 2;          // [2] 4 warps: P_hat, block weights and row sums of the item written
+constexpr int B_S_FREE = B_S_FULL + 2;           // [2] 8 warps: the item's scores have been read
+constexpr int B_P_READY = B_S_FREE + 2;          // [2] 8 warps: P_hat, block weights and row sums of the item written
 constexpr int B_Q_READY = B_P_READY + 2;         // [2] query tile of the item staged
 constexpr int B_O_FULL = B_Q_READY + 2;          // [1] PV commit after the item's last block
 constexpr int B_T_FREE = B_O_FULL + 1;           // [2] 4 warps: the item's tables (and, after its PV, P_hat) may be overwritten
 constexpr int B_O_FREE = B_T_FREE + 2;           // [1] 4 warps
-constexpr int B_XCHG = B_O_FREE + 1;             // [2] 4 warps of a softmax group: block maxima exchanged
+constexpr int B_XCHG = B_O_FREE + 1;             // [2] 8 softmax warps: block maxima of the item exchanged
 constexpr int B_ITEM_FULL = B_XCHG + 2;          // [D_NITEM] work item published
 constexpr int B_ITEM_EMPTY = B_ITEM_FULL + D_NITEM;   // [D_NITEM] read by all eighteen consumer warps
 constexpr int B_DRAW = B_ITEM_EMPTY + D_NITEM;   // [2] warp 0 has begun item k (slot k & 1): the next one may be drawn
-constexpr int B_COUNT = B_DRAW + 2;
+constexpr int B_V_GO = B_DRAW + 2;               // [1] every K copy of the CTA's first item is on its way
+constexpr int B_COUNT = B_V_GO + 1;
 static_assert(B_COUNT * 8 <= 1024, "barrier block");
 static_assert(D_SMEM <= 232448, "shared memory");
 static_assert(KST_BYTES % 1024 == 0 && D_OFF_V % 1024 == 0 && D_OFF_P % 1024 == 0, "swizzle atoms");
@@ -228,13 +234,17 @@ struct DCtx {
 struct WorkIter {
   uint32_t n = 0;      // items taken so far
   int b, hk, sp, L, nblk;
-  // Whole warp.  false: no more items (or the CTA is giving up).
+  // Whole warp, or the one thread that stands for its warp.  false: no more items (or the CTA is giving up).
+  template <bool ONE_THREAD = false>
   __device__ bool next(const DCtx &cx, const int4 *ring) {
-    const uint32_t slot = n % D_NITEM;
-    if (!cx.wait_warp(B_ITEM_FULL + slot, (n / D_NITEM) & 1)) return false;
+    const uint32_t slot = n % D_NITEM, parity = (n / D_NITEM) & 1;
+    if (!(ONE_THREAD ? cx.wait(B_ITEM_FULL + slot, parity) : cx.wait_warp(B_ITEM_FULL + slot, parity))) return false;
     const int4 it = ring[slot];
     if (it.x < 0) return false;   // end marker: stays in its slot, nobody moves past it
-    cx.warp_arrive(B_ITEM_EMPTY + slot);
+    if (ONE_THREAD)
+      mbar_arrive(cx.bar(B_ITEM_EMPTY + slot));
+    else
+      cx.warp_arrive(B_ITEM_EMPTY + slot);
     ++n;
     b = it.x, hk = it.y, sp = it.z, L = it.w;
     nblk = (min(L - sp * DECODE_SPLIT, DECODE_SPLIT) + TILE - 1) / TILE;
@@ -273,7 +283,7 @@ __global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const __grid
   // ---- set-up: barriers, zeroed operand tiles (rows G..15 stay zero for good), TMEM
   if (threadIdx.x == 0) {
     for (int i = 0; i < D_NK; ++i) {
-      mbar_init(cx.bar(B_K_FULL + i), 2);
+      mbar_init(cx.bar(B_K_FULL + i), 1);
       mbar_init(cx.bar(B_K_EMPTY + i), 1);
       mbar_init(cx.bar(B_SF_READY + i), 1);
     }
@@ -283,13 +293,14 @@ __global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const __grid
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(cx.bar(B_S_FULL + i), 1);
-      mbar_init(cx.bar(B_XCHG + i), 4);
+      mbar_init(cx.bar(B_XCHG + i), 8);
       mbar_init(cx.bar(B_T_FREE + i), 4);
       mbar_init(cx.bar(B_DRAW + i), 1);
-      mbar_init(cx.bar(B_S_FREE + i), 4);
-      mbar_init(cx.bar(B_P_READY + i), 4);
+      mbar_init(cx.bar(B_S_FREE + i), 8);
+      mbar_init(cx.bar(B_P_READY + i), 8);
       mbar_init(cx.bar(B_Q_READY + i), 1);
     }
+    mbar_init(cx.bar(B_V_GO), 1);
     mbar_init(cx.bar(B_O_FULL), 1);
     mbar_init(cx.bar(B_O_FREE), 4);
     for (int i = 0; i < D_NITEM; ++i) {
@@ -360,10 +371,13 @@ __global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const __grid
     } else {
       total = (uint32_t)p.B * p.H_kv * p.n_split;
     }
-    bool ok = true;
+    bool ok = true, prev_short = false;
     for (uint32_t k = 0; ok; ++k) {
       const uint32_t slot = k % D_NITEM;
-      if (k >= 2) ok = cx.wait_warp(B_DRAW + ((k - 1) & 1), ((k - 1) >> 1) & 1);   // the K producer has begun item k-1
+      if (k >= 2) {   // the K producer has begun item k-1, or k-2 where item k-1 is over before the next one could be drawn
+        const uint32_t begun = prev_short ? k - 2 : k - 1;
+        ok = cx.wait_warp(B_DRAW + (begun & 1), (begun >> 1) & 1);
+      }
       if (ok && k >= (uint32_t)D_NITEM) ok = cx.wait_warp(B_ITEM_EMPTY + slot, ((k / D_NITEM) - 1) & 1);
       if (!ok) break;
       int4 item = make_int4(-1, 0, 0, 0);
@@ -396,6 +410,9 @@ __global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const __grid
       item.x = __shfl_sync(0xffffffffu, item.x, 0);
       if (item.x < 0) break;   // the end marker is in the ring; this CTA draws no more
       item.y = __shfl_sync(0xffffffffu, item.y, 0);
+      item.z = __shfl_sync(0xffffffffu, item.z, 0);
+      item.w = __shfl_sync(0xffffffffu, item.w, 0);
+      prev_short = item.w - item.z * DECODE_SPLIT <= DECODE_SPLIT / 2;
       const size_t head0 = (size_t)item.x * p.H_q + (size_t)item.y * G;
       uint4 qv = make_uint4(0u, 0u, 0u, 0u);
       uint32_t qs0 = 0, qs1 = 0;
@@ -421,80 +438,84 @@ __global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const __grid
       cx.warp_arrive(B_Q_READY + par);
     }
   } else if (warp == 0 || warp >= 16) {
-    // ================= producers: warps 0 and 17 stream the K ring (0: codes; 17: block scales and Delta_S,
-    // both arriving on the stage's barrier), warp 16 the V ring.  Issuing a bulk copy costs a warp well over a
-    // hundred cycles, so the ten copies of a block are spread over three warps.
+    // ================= producers: warps 0 and 17 stream the K ring, a block each in turn, warp 16 the V ring.  Lane u holds
+    // block u of the item, its addresses and what of it exists, and issues that block's copies itself: with page ids handed around and
+    // addresses made for each block, codes on one warp and the small pieces on the other, a block cost the warps 700 and 950 cycles,
+    // next to the 1180 that its bytes take at the rate of the memory, and the K of a CTA's first item took 8300 with the memory idle.
     // Nothing orders the two streams but the data flow: a K stage is released by its QK MMAs, a V stage
     // only after the item's softmax, so K runs about one item ahead.  The next item is taken up, and its page ids
-    // requested, before the last two blocks of the current one; they are validated where they are used.
-    const bool is_k = warp != 16, is_codes = warp == 0;
+    // requested, before the last two blocks of the current one.
+    const bool is_k = warp != 16;
     WorkIter w, wn;
     uint32_t c = 0, j = 0;   // blocks and items of this ring
     bool ok = true;
     const uint32_t d_bytes = p.delta ? (uint32_t)G * PAGE * 2 : 0u;
-    const uint32_t kpage_bytes = is_codes ? 4096u : 512u + d_bytes;
-    const int n_ring = is_k ? D_NK : D_NV;
+    const uint32_t page_bytes = is_k ? 4096u + 512u + d_bytes : 8192u;
+    const uint32_t n_ring = is_k ? D_NK : D_NV;
     const int b_full = is_k ? B_K_FULL : B_V_FULL, b_empty = is_k ? B_K_EMPTY : B_V_EMPTY;
+    static_assert(D_NK % 2 == 0, "each K producer has its own stages");
     int pc0 = -1, pc1 = -1, pn0 = -1, pn1 = -1;
     bool vw = w.next(cx, ring), vn = false;
     if (vw) lookup_pages(p, w, lane, pc0, pc1);
     for (; ok && vw; ++j) {
-      if (is_codes) cx.warp_arrive(B_DRAW + (j & 1));
+      if (warp == 0) cx.warp_arrive(B_DRAW + (j & 1));
+      // Nothing can be done with V before the first item's softmax, and while all CTAs start at once its copies only keep K waiting.
+      if (!is_k && j == 0) ok = cx.wait_warp(B_V_GO, 0);
+      const bool in = lane < w.nblk, want1 = w.sp * DECODE_SPLIT + lane * TILE + PAGE < w.L;
+      const bool has0 = in && pc0 >= 0 && pc0 < p.num_pages, has1 = in && want1 && pc1 >= 0 && pc1 < p.num_pages;
+      if (in && (!has0 || (want1 && !has1))) atomicOr(p.status, MPFA_DEV_BAD_PAGE);
+      const size_t slab0 = (size_t)(has0 ? pc0 : 0) * p.H_kv + w.hk, slab1 = (size_t)(has1 ? pc1 : 0) * p.H_kv + w.hk;
+      const uint8_t *const big0 = is_k ? p.k_codes + slab0 * 4096 : p.v_fp8 + slab0 * 8192;
+      const uint8_t *const big1 = is_k ? p.k_codes + slab1 * 4096 : p.v_fp8 + slab1 * 8192;
+      const uint8_t *const sf0 = p.k_sf + slab0 * 512, *const sf1 = p.k_sf + slab1 * 512;
+      const __nv_bfloat16 *const del0 = p.delta + slab0 * (G * PAGE), *const del1 = p.delta + slab1 * (G * PAGE);
+      const uint32_t bytes = ((has0 ? 1u : 0u) + (has1 ? 1u : 0u)) * page_bytes;
+      const uint32_t absent = __ballot_sync(0xffffffffu, in && !(has0 && has1));
       for (int t = 0; ok && t < w.nblk; ++t, ++c) {
         const uint32_t st = c % n_ring;
-        if (c >= (uint32_t)n_ring && !cx.wait_warp(b_empty + st, ((c / n_ring) - 1) & 1)) {
+        const bool mine = !is_k || (c & 1) == (warp == 17 ? 1u : 0u);
+        if (mine && c >= n_ring && !cx.wait_warp(b_empty + st, ((c / n_ring) - 1) & 1)) {
           ok = false;
           break;
         }
         const int u = w.nblk - 1 - t;
-        int id0 = __shfl_sync(0xffffffffu, pc0, u), id1 = __shfl_sync(0xffffffffu, pc1, u);
-        const bool want1 = w.sp * DECODE_SPLIT + u * TILE + PAGE < w.L;
-        const bool bad = id0 < 0 || id0 >= p.num_pages || (want1 && (id1 < 0 || id1 >= p.num_pages));
-        if (bad && lane == 0 && !is_codes) atomicOr(p.status, MPFA_DEV_BAD_PAGE);
-        if (id0 < 0 || id0 >= p.num_pages) id0 = -1;
-        if (!want1 || id1 < 0 || id1 >= p.num_pages) id1 = -1;
         const uint32_t full = cx.bar(b_full + st);
-        if (is_k) {
-          if (elect_one()) {
-            const uint32_t sdst = sbase + D_OFF_K + st * KST_BYTES;
-            mbar_expect_tx(full, (id0 >= 0 ? kpage_bytes : 0u) + (id1 >= 0 ? kpage_bytes : 0u));
-#pragma unroll
-            for (int half = 0; half < 2; ++half) {
-              const int id = half == 0 ? id0 : id1;
-              if (id < 0) continue;
-              const size_t slab = (size_t)id * p.H_kv + w.hk;
-              if (is_codes) {
-                bulk_load(sdst + KST_K + half * 4096, p.k_codes + slab * 4096, 4096, full);
-              } else {
-                bulk_load(sdst + KST_SF + half * 512, p.k_sf + slab * 512, 512, full);
-                if (d_bytes)
-                  bulk_load(sdst + KST_DELTA + half * 1024, p.delta + ((size_t)id * p.H_q + (size_t)w.hk * G) * PAGE, d_bytes, full);
-              }
-            }
-          }
-        } else {
+        if (!is_k && (absent >> u & 1u)) {
           // a page that is not there contributes P_hat = 0 times V: V must be finite, so zero it
-          if (id0 < 0 || id1 < 0) {
-            uint8_t *stage = dsm + D_OFF_V + st * VST_BYTES;
+          const bool h0 = __shfl_sync(0xffffffffu, has0, u), h1 = __shfl_sync(0xffffffffu, has1, u);
+          uint8_t *stage = dsm + D_OFF_V + st * VST_BYTES;
 #pragma unroll 1
-            for (int half = 0; half < 2; ++half) {
-              if ((half == 0 ? id0 : id1) >= 0) continue;
-              for (int i = 0; i < 16; ++i)
-                *reinterpret_cast<uint4 *>(stage + half * 8192 + i * 512 + lane * 16) = make_uint4(0u, 0u, 0u, 0u);
-            }
-            fence_proxy_async_smem();
-            __syncwarp();
+          for (int half = 0; half < 2; ++half) {
+            if (half == 0 ? h0 : h1) continue;
+            for (int i = 0; i < 16; ++i)
+              *reinterpret_cast<uint4 *>(stage + half * 8192 + i * 512 + lane * 16) = make_uint4(0u, 0u, 0u, 0u);
           }
+          fence_proxy_async_smem();
+          __syncwarp();
+        }
 #ifdef MPFA_TEST_DROP_V_COPY
-          if (c == 0) {
-            // left out on purpose (work items are drawn dynamically: any CTA may be the one that gets work)
-          } else
+        if (!is_k && c == 0) {
+          // left out on purpose (work items are drawn dynamically: any CTA may be the one that gets work)
+        } else
 #endif
-          if (elect_one()) {
-            const uint32_t sdst = sbase + D_OFF_V + st * VST_BYTES;
-            mbar_expect_tx(full, (id0 >= 0 ? 8192u : 0u) + (id1 >= 0 ? 8192u : 0u));
-            if (id0 >= 0) bulk_load(sdst, p.v_fp8 + ((size_t)id0 * p.H_kv + w.hk) * 8192, 8192, full);
-            if (id1 >= 0) bulk_load(sdst + 8192, p.v_fp8 + ((size_t)id1 * p.H_kv + w.hk) * 8192, 8192, full);
+        if (mine && lane == u) {
+          mbar_expect_tx(full, bytes);
+          if (is_k) {
+            const uint32_t dst = sbase + D_OFF_K + st * KST_BYTES;
+            if (has0) {
+              bulk_load(dst + KST_K, big0, 4096, full);
+              bulk_load(dst + KST_SF, sf0, 512, full);
+              if (d_bytes) bulk_load(dst + KST_DELTA, del0, d_bytes, full);
+            }
+            if (has1) {
+              bulk_load(dst + KST_K + 4096, big1, 4096, full);
+              bulk_load(dst + KST_SF + 512, sf1, 512, full);
+              if (d_bytes) bulk_load(dst + KST_DELTA + 1024, del1, d_bytes, full);
+            }
+          } else {
+            const uint32_t dst = sbase + D_OFF_V + st * VST_BYTES;
+            if (has0) bulk_load(dst, big0, 8192, full);
+            if (has1) bulk_load(dst + 8192, big1, 8192, full);
           }
         }
         __syncwarp();
@@ -504,47 +525,52 @@ __global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const __grid
           if (vn) lookup_pages(p, wn, lane, pn0, pn1);
         }
       }
+      if (warp == 0 && j == 0) cx.warp_arrive(B_V_GO);
       vw = vn;
       w = wn;
       pc0 = pn0, pc1 = pn1;
     }
     // The last copies of this ring land before the warp leaves: where all goes well their consumers wait for them too, and where a
     // role gives up, before or after this loop has ended, shared memory must not go away under them.
-    for (uint32_t i = c - min(c, (uint32_t)n_ring); i < c; ++i) {
+    for (uint32_t i = c - min(c, n_ring); i < c; ++i) {
       const long long t0 = clock64();
       while (!mbar_try_wait(cx.bar(b_full + i % n_ring), (i / n_ring) & 1) && clock64() - t0 < D_WAIT_CYCLES) {
       }
     }
   } else if (warp == 1) {
     // ================= QK issue: S^T[item parity][block] = K Q^T as K stages land
-    const uint32_t id_qk = idesc_nvfp4(128, NCOL);
-    const uint32_t id_ds = idesc_bf16(128, NCOL, 1, 1);
-    const uint64_t d_ident = smem_desc(sbase + D_OFF_IDENT, 2048, 1024, SWZ_128B);
-    const bool has_delta = p.delta != nullptr;
-    WorkIter w;
-    uint32_t kc = 0, j = 0;
-    bool ok = true;
-    while (ok && w.next(cx, ring)) {
-      const uint32_t par = j & 1;
-      ok = cx.wait_warp(B_Q_READY + par, (j >> 1) & 1);
-      if (ok && j >= 2) ok = cx.wait_warp(B_S_FREE + par, ((j >> 1) - 1) & 1);   // scores of item j-2 have been read
-      for (int t = 0; ok && t < w.nblk; ++t, ++kc) {
-        const uint32_t st = kc % D_NK;
-        ok = cx.wait_warp(B_K_FULL + st, (kc / D_NK) & 1) && cx.wait_warp(B_SF_READY + st, (kc / D_NK) & 1);
-        if (!ok) break;
-        tc_fence_after();
-        if (elect_one()) {
-          const uint32_t tSFQ = tm + TM_SFQ + par * 8, tSFK = tm + TM_SFK + st * 8;
+    // One thread waits and issues: with the waits taken by the whole warp a block cost it 600 cycles, as long as the block's
+    // bytes take.
+    if (elect_one()) {
+      const uint32_t id_qk = idesc_nvfp4(128, NCOL);
+      const uint32_t id_ds = idesc_bf16(128, NCOL, 1, 1);
+      const uint64_t d_ident = smem_desc(sbase + D_OFF_IDENT, 2048, 1024, SWZ_128B);
+      const uint64_t d_sfq0 = smem_desc(sbase + D_OFF_SFQ, 0, 128, SWZ_NONE), d_sfk0 = smem_desc(sbase + D_OFF_SFK, 0, 128, SWZ_NONE);
+      const uint64_t d_k0 = smem_desc(sbase + D_OFF_K + KST_K, 16, 512, SWZ_64B), d_q0 = smem_desc(sbase + D_OFF_Q, 16, 512, SWZ_64B);
+      const bool has_delta = p.delta != nullptr;
+      WorkIter w;
+      uint32_t kc = 0, j = 0;
+      bool ok = true;
+      while (ok && w.next<true>(cx, ring)) {
+        const uint32_t par = j & 1;
+        ok = cx.wait(B_Q_READY + par, (j >> 1) & 1);
+        if (ok && j >= 2) ok = cx.wait(B_S_FREE + par, ((j >> 1) - 1) & 1);   // scores of item j-2 have been read
+        const uint32_t tSFQ = tm + TM_SFQ + par * 8;
+        const uint64_t d_q = d_q0 + par * (1024 >> 4), d_sfq = d_sfq0 + par * (1024 >> 4);
+        for (int t = 0; ok && t < w.nblk; ++t, ++kc) {
+          const uint32_t st = kc % D_NK;
+          ok = cx.wait(B_SF_READY + st, (kc / D_NK) & 1) && cx.wait(B_K_FULL + st, (kc / D_NK) & 1);
+          if (!ok) break;
+          tc_fence_after();
+          const uint32_t tSFK = tm + TM_SFK + st * 8;
           if (t == 0) {
-            const uint64_t d_sfq = smem_desc(sbase + D_OFF_SFQ + par * 1024, 0, 128, SWZ_NONE);
             tmem_cp_32x128b_warpx4(tSFQ, d_sfq);
             tmem_cp_32x128b_warpx4(tSFQ + 4, d_sfq + (512 >> 4));
           }
-          const uint64_t d_sfk = smem_desc(sbase + D_OFF_SFK + st * 1024, 0, 128, SWZ_NONE);
+          const uint64_t d_sfk = d_sfk0 + st * (1024 >> 4);
           tmem_cp_32x128b_warpx4(tSFK, d_sfk);
           tmem_cp_32x128b_warpx4(tSFK + 4, d_sfk + (512 >> 4));
-          const uint64_t d_k = smem_desc(sbase + D_OFF_K + st * KST_BYTES + KST_K, 16, 512, SWZ_64B);
-          const uint64_t d_q = smem_desc(sbase + D_OFF_Q + par * 1024, 16, 512, SWZ_64B);
+          const uint64_t d_k = d_k0 + st * (KST_BYTES >> 4);
           const uint32_t tS = tm + TM_S + (par * MAXBLK + t) * 16;
           if (has_delta) {
             // S^T = Delta_S^T I (Eq. 11 seed): A = the stage's Delta_S rows, MN-major (keys contiguous), its
@@ -557,10 +583,10 @@ __global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const __grid
           if (t == w.nblk - 1) mma_commit(cx.bar(B_S_FULL + par));
           mma_commit(cx.bar(B_K_EMPTY + st));
         }
-        __syncwarp();
+        ++j;
       }
-      ++j;
     }
+    __syncwarp();
   } else if (warp == 2) {
     // ================= PV issue: O_u^T = V_u^T P_hat_u^T as V stages land
     // a request without keys has no work item: its zeros are written here, while this warp has nothing to issue
@@ -570,21 +596,22 @@ __global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const __grid
           p.out[(size_t)b * p.H_q * HEAD_DIM + i] = __float2bfloat16_rn(0.0f);
           if (p.out_f32) p.out_f32[(size_t)b * p.H_q * HEAD_DIM + i] = 0.0f;
         }
-    const uint32_t id_pv = idesc_e4m3(128, NCOL, 1, 0);
-    WorkIter w;
-    uint32_t vc = 0, j = 0;
-    bool ok = true;
-    while (ok && w.next(cx, ring)) {
-      const uint32_t par = j & 1;
-      ok = cx.wait_warp(B_P_READY + par, (j >> 1) & 1);
-      if (ok && j >= 1) ok = cx.wait_warp(B_O_FREE, (j - 1) & 1);   // the previous item's O has been read
-      for (int t = 0; ok && t < w.nblk; ++t, ++vc) {
-        const uint32_t st = vc % D_NV;
-        ok = cx.wait_warp(B_V_FULL + st, (vc / D_NV) & 1);
-        if (!ok) break;
-        tc_fence_after();
-        if (elect_one()) {
-          const uint64_t d_v = smem_desc(sbase + D_OFF_V + st * VST_BYTES, 16, 1024, SWZ_128B);
+    if (elect_one()) {   // one thread, as for Q K^T
+      const uint32_t id_pv = idesc_e4m3(128, NCOL, 1, 0);
+      const uint64_t d_v0 = smem_desc(sbase + D_OFF_V, 16, 1024, SWZ_128B);
+      WorkIter w;
+      uint32_t vc = 0, j = 0;
+      bool ok = true;
+      while (ok && w.next<true>(cx, ring)) {
+        const uint32_t par = j & 1;
+        ok = cx.wait(B_P_READY + par, (j >> 1) & 1);
+        if (ok && j >= 1) ok = cx.wait(B_O_FREE, (j - 1) & 1);   // the previous item's O has been read
+        for (int t = 0; ok && t < w.nblk; ++t, ++vc) {
+          const uint32_t st = vc % D_NV;
+          ok = cx.wait(B_V_FULL + st, (vc / D_NV) & 1);
+          if (!ok) break;
+          tc_fence_after();
+          const uint64_t d_v = d_v0 + st * (VST_BYTES >> 4);
           // rows 0..7 of P_hat^T in the block's tile, rows 8..15 (the next 8-row group) from the zero block
           const uint32_t a_p = sbase + D_OFF_P + (par * MAXBLK + t) * 1024;
           const uint64_t d_p = smem_desc(a_p, 16, sbase + D_OFF_ZERO - a_p, SWZ_128B);
@@ -595,10 +622,10 @@ __global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const __grid
           mma_commit(cx.bar(B_V_EMPTY + st));
           if (t == w.nblk - 1) mma_commit(cx.bar(B_O_FULL));
         }
-        __syncwarp();
+        ++j;
       }
-      ++j;
     }
+    __syncwarp();
   } else if (warp == 3) {
     // ================= K scales of a block: [token][8 blocks] -> two 32 x 16-byte tiles
     // (tile h = blocks 4h..4h+3; row i holds tokens i, 32+i, 64+i, 96+i), the form tcgen05.cp spreads.
@@ -623,53 +650,53 @@ __global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const __grid
       }
     }
   } else if (warp < 12) {
-    // ================= softmax, one thread per key of a block; two groups of four warps, group
-    // `grp` takes the items of that parity
+    // ================= softmax, one thread per key of a block; two groups of four warps, group `grp` takes every item's
+    // blocks of that parity
     const int grp = (warp - 4) >> 2;
     const int quad = warp & 3;                  // TMEM lane quadrant this warp may touch
     const int r = quad * 32 + lane;             // key within the block
     const uint32_t tlane = (uint32_t)(quad * 32) << 16;
     constexpr int CH = G <= 2 ? 4 : 2;          // blocks whose tensor-memory loads are in flight together
     constexpr int GP = G <= 4 ? 4 : 8, TPV = 32 / GP, NV = MAXBLK / TPV;   // heads padded; blocks to a warp's lanes; such sets
-    const uint32_t tS = tm + TM_S + grp * (MAXBLK * 16) + tlane;
-    uint8_t *const pt = dsm + D_OFF_P + grp * MAXBLK * 1024 + (r & 15);
-    float *xm = xmax + grp * MAXBLK * MAXG * 4, *wt = wtab + grp * MAXBLK * MAXG, *xlg = xl + grp * 4 * MAXG;
     bool ok = true;
     WorkIter w;
     for (uint32_t j = 0; ok && w.next(cx, ring); ++j) {
-      if ((int)(j & 1) != grp) continue;
-      const uint32_t ph = (j >> 1) & 1;
+      const uint32_t par = j & 1, ph = (j >> 1) & 1;
+      const uint32_t tS = tm + TM_S + par * (MAXBLK * 16) + tlane;
+      uint8_t *const pt = dsm + D_OFF_P + par * MAXBLK * 1024 + (r & 15);
+      float *xm = xmax + par * MAXBLK * MAXG * 4, *wt = wtab + par * MAXBLK * MAXG, *xlg = xl + par * 8 * MAXG;
       const float lam = w.b < D_MAXREQ ? lam_tab[w.b]
                                        : __fmul_rn(__fmul_rn(__fmul_rn(p.softmax_scale, 1.4426950408889634f), p.q_gscale[w.b]), p.k_gscale[w.b]);
       const int k_part = w.sp * DECODE_SPLIT;
       // ---- all scores of the item at once.  They are read from tensor memory twice, once for the maxima and once for the
       // exponentials: held in registers in between, MAXBLK x G of them and as many maxima went to local memory for groups
       // of five heads and more (24 us per item instead of 6).
-      ok = cx.wait_warp(B_S_FULL + grp, ph);
+      ok = cx.wait_warp(B_S_FULL + par, ph);
       if (!ok) break;
       tc_fence_after();
       // block maxima of this warp's keys, CH blocks at a time
 #pragma unroll 1
-      for (int t0 = 0; t0 < w.nblk; t0 += CH) {
+      for (int t0 = grp; t0 < w.nblk; t0 += 2 * CH) {
         uint32_t sr[CH][G];
 #pragma unroll
         for (int u = 0; u < CH; ++u)
-          if (t0 + u < w.nblk) tmem_ld_g<G>(tS + (t0 + u) * 16, sr[u]);
+          if (t0 + 2 * u < w.nblk) tmem_ld_g<G>(tS + (t0 + 2 * u) * 16, sr[u]);
         tmem_ld_wait();
 #pragma unroll
         for (int u = 0; u < CH; ++u) {
-          if (t0 + u < w.nblk) {
-            const bool valid = k_part + (w.nblk - 1 - t0 - u) * TILE + r < w.L;
+          const int t = t0 + 2 * u;
+          if (t < w.nblk) {
+            const bool valid = k_part + (w.nblk - 1 - t) * TILE + r < w.L;
 #pragma unroll
             for (int g = 0; g < G; ++g) {
               const float wm = warp_max(valid ? __uint_as_float(sr[u][g]) : -INFINITY);
-              if (lane == 0) xm[((t0 + u) * MAXG + g) * 4 + quad] = wm;
+              if (lane == 0) xm[(t * MAXG + g) * 4 + quad] = wm;
             }
           }
         }
       }
-      cx.warp_arrive(B_XCHG + grp);
-      ok = cx.wait_warp(B_XCHG + grp, ph);
+      cx.warp_arrive(B_XCHG + par);
+      ok = cx.wait_warp(B_XCHG + par, ph);
       if (!ok) break;
       // running maxima m_t of the reverse traversal, -lam m_t and the weights 2^(lam (m_t - m)) of the item's end, in the lanes
       float mt[NV], nml[NV], wl[NV], m_end;
@@ -687,15 +714,15 @@ __global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const __grid
         m_end = __shfl_sync(0xffffffffu, mt[v], 32 - GP + (lane & (GP - 1)));
       }
       // the item two before this one, which used the same tables and P_hat tiles, is through with them
-      if (j >= 2) ok = cx.wait_warp(B_T_FREE + grp, ph ^ 1);
+      if (j >= 2) ok = cx.wait_warp(B_T_FREE + par, ph ^ 1);
       if (!ok) break;
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
         nml[v] = -__fmul_rn(mt[v], lam);
         wl[v] = mt[v] == m_end ? 1.0f : ex2_approx(__fmul_rn(mt[v] - m_end, lam));
-        if (quad == 0 && (lane & (GP - 1)) < G) wt[(v * TPV + lane / GP) * MAXG + (lane & (GP - 1))] = wl[v];
+        if (warp == 4 && (lane & (GP - 1)) < G) wt[(v * TPV + lane / GP) * MAXG + (lane & (GP - 1))] = wl[v];
       }
-      if (quad == 0 && lane < G) mfin[grp * MAXG + lane] = m_end;
+      if (warp == 4 && lane < G) mfin[par * MAXG + lane] = m_end;
       // all P_hat of the item; l = sum of the blocks' sums times their weights
       float lsum[G];
 #pragma unroll
@@ -703,21 +730,21 @@ __global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const __grid
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
 #pragma unroll 1
-        for (int t0 = 0; t0 < TPV && v * TPV + t0 < w.nblk; t0 += CH) {
+        for (int t0 = grp; t0 < TPV && v * TPV + t0 < w.nblk; t0 += 2 * CH) {
           uint32_t sr[CH][G];
 #pragma unroll
           for (int u = 0; u < CH; ++u)
-            if (v * TPV + t0 + u < w.nblk) tmem_ld_g<G>(tS + (v * TPV + t0 + u) * 16, sr[u]);
+            if (v * TPV + t0 + 2 * u < w.nblk) tmem_ld_g<G>(tS + (v * TPV + t0 + 2 * u) * 16, sr[u]);
           tmem_ld_wait();
 #pragma unroll
           for (int u = 0; u < CH; ++u) {
-            const int t = v * TPV + t0 + u;
+            const int t = v * TPV + t0 + 2 * u;
             if (t < w.nblk) {
               const bool valid = k_part + (w.nblk - 1 - t) * TILE + r < w.L;
               float pq[G + 1];
 #pragma unroll
               for (int g = 0; g < G; ++g) {
-                const float c = __shfl_sync(0xffffffffu, nml[v], (t0 + u) * GP + g), wg = __shfl_sync(0xffffffffu, wl[v], (t0 + u) * GP + g);
+                const float c = __shfl_sync(0xffffffffu, nml[v], (t0 + 2 * u) * GP + g), wg = __shfl_sync(0xffffffffu, wl[v], (t0 + 2 * u) * GP + g);
                 const float e = ex2_approx(__fmaf_rn(__uint_as_float(sr[u][g]), lam, c));
                 const float pv = valid ? e : 0.0f;
                 lsum[g] = __fmaf_rn(wg, pv, lsum[g]);
@@ -736,16 +763,16 @@ __global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const __grid
         }
       }
       tc_fence_before();
-      cx.warp_arrive(B_S_FREE + grp);
+      cx.warp_arrive(B_S_FREE + par);
 #pragma unroll
       for (int g = 0; g < G; ++g) {
         float ls = lsum[g];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) ls += __shfl_xor_sync(0xffffffffu, ls, o);
-        if (lane == 0) xlg[quad * MAXG + g] = ls;
+        if (lane == 0) xlg[(warp - 4) * MAXG + g] = ls;
       }
       fence_proxy_async_smem();
-      cx.warp_arrive(B_P_READY + grp);
+      cx.warp_arrive(B_P_READY + par);
     }
   } else {
     // ================= O of every item, one thread per channel, as soon as its V has been consumed
@@ -756,7 +783,7 @@ __global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const __grid
     WorkIter w;
     for (uint32_t j = 0; ok && w.next(cx, ring); ++j) {
       const int par = j & 1;
-      const float *wt = wtab + par * MAXBLK * MAXG, *xlg = xl + par * 4 * MAXG;
+      const float *wt = wtab + par * MAXBLK * MAXG, *xlg = xl + par * 8 * MAXG;
       ok = cx.wait_warp(B_P_READY + par, (j >> 1) & 1) && cx.wait_warp(B_O_FULL, j & 1);   // the item's tables; its accumulators
       if (!ok) break;
       tc_fence_after();
@@ -765,7 +792,8 @@ __global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const __grid
       for (int g = 0; g < G; ++g) {
         acc[g] = 0.0f;
         m[g] = mfin[par * MAXG + g];
-        l[g] = (xlg[g] + xlg[MAXG + g]) + (xlg[2 * MAXG + g] + xlg[3 * MAXG + g]);
+        l[g] = ((xlg[g] + xlg[MAXG + g]) + (xlg[2 * MAXG + g] + xlg[3 * MAXG + g])) +
+               ((xlg[4 * MAXG + g] + xlg[5 * MAXG + g]) + (xlg[6 * MAXG + g] + xlg[7 * MAXG + g]));
       }
 #pragma unroll 1
       for (int t0 = 0; t0 < w.nblk; t0 += CH) {
@@ -826,26 +854,41 @@ __global__ void __launch_bounds__(128, 9) decode_merge_kernel(const __grid_const
   __shared__ __align__(16) float s_o[4][HEAD_DIM];
   grid_dependency_wait();
   const int hq = blockIdx.x, b = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int n = p.n_parts(p.seq_lens[b]);
-  if (n <= 1) return;
   const size_t head = (size_t)b * p.H_q + hq;
   const float2 *ml = p.part_ml + head * p.n_split;
   const float4 *po = reinterpret_cast<const float4 *>(p.part_o + head * p.n_split * HEAD_DIM) + lane;
+  // The first 16 states are requested before the length is known: the request's slots of the workspace exist whatever it is, and
+  // what stands in those past its last partition is not used.  (One load after the other, length, maxima, states, the merge of a
+  // single request took 4.2 us alone.)
+  float2 a[4];
+  float4 x[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int s = min(warp + 4 * u, p.n_split - 1);
+    a[u] = ml[s];
+    x[u] = po[(size_t)s * (HEAD_DIM / 4)];
+  }
+  const float first_max = ml[min(lane, p.n_split - 1)].x;
+  const int n = p.n_parts(p.seq_lens[b]);
   const float lam = __fmul_rn(__fmul_rn(__fmul_rn(p.softmax_scale, 1.4426950408889634f), p.q_gscale[b]), p.k_gscale[b]);
-  float M = -INFINITY;
-  for (int s = lane; s < n; s += 32) M = fmaxf(M, ml[s].x);   // every warp takes the maximum of all
+  if (n <= 1) return;
+  float M = lane < n ? first_max : -INFINITY;
+  for (int s = lane + 32; s < n; s += 32) M = fmaxf(M, ml[s].x);   // every warp takes the maximum of all
   M = warp_max(M);
   float l = 0.0f, o[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll 1
   for (int s0 = warp; s0 < n; s0 += 16) {
-    float2 a[4];
-    float4 x[4];
+    if (s0 != warp) {
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int s = s0 + 4 * u;
-      a[u] = s < n ? ml[s] : make_float2(-INFINITY, 0.0f);
-      x[u] = s < n ? po[(size_t)s * (HEAD_DIM / 4)] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      for (int u = 0; u < 4; ++u) {
+        const int s = min(s0 + 4 * u, n - 1);
+        a[u] = ml[s];
+        x[u] = po[(size_t)s * (HEAD_DIM / 4)];
+      }
     }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (s0 + 4 * u >= n) a[u].x = -INFINITY;
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       if (a[u].x == -INFINITY) continue;   // no score above -infinity: left out, its sums need not be finite

@@ -340,21 +340,40 @@ __device__ __forceinline__ uint32_t e2m1x8(const float (&y)[16], int o) {
       : "f"(y[o]), "f"(y[o + 1]), "f"(y[o + 2]), "f"(y[o + 3]), "f"(y[o + 4]), "f"(y[o + 5]), "f"(y[o + 6]), "f"(y[o + 7]));
   return w;
 }
-__device__ __forceinline__ void quantize_block16(const float (&xc)[16], const BlockScale &q, uint32_t &scale_code, uint2 &codes) {
+__device__ __forceinline__ float block_max(const float (&xc)[16]) {
   float m[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) m[i] = max3(fabsf(xc[4 * i]), fabsf(xc[4 * i + 1]), fabsf(xc[4 * i + 2]));
 #pragma unroll
   for (int i = 0; i < 2; ++i) m[i] = max3(m[i], fabsf(xc[8 * i + 3]), fabsf(xc[8 * i + 7]));
-  const float a = max3(max3(m[0], m[1], m[2]), m[3], 0.0f);   // 0 for a block of NaNs, as above
-  float r = __fmul_rn(a, q.rcp);
-  if (!(r >= 0.015625f && r < 512.0f && abs((int)(__float_as_uint(r) & 0xFFFFFu) - 0x80000) > 4)) r = __fdiv_rn(a, q.e);
-  scale_code = (uint32_t)__nv_cvt_float_to_fp8(r, __NV_SATFINITE, __NV_E4M3);
-  const float inv = q.inv[scale_code & 127u];
-  float y[16];
+  return max3(max3(m[0], m[1], m[2]), m[3], 0.0f);   // 0 for a block of NaNs, as above
+}
+__device__ __forceinline__ bool near_boundary(float r) {
+  return !(r >= 0.015625f && r < 512.0f && abs((int)(__float_as_uint(r) & 0xFFFFFu) - 0x80000) > 4);
+}
+// Two blocks of a row at once: their chains run beside one another, with one branch for both divisions (a branch per block kept the
+// blocks one after the other: every instruction waited for the one before, issue slots 54 % used).  scale_codes: two bytes.
+__device__ __forceinline__ void quantize_blocks(const float (&xa)[16], const float (&xb)[16], const BlockScale &q, uint32_t &scale_codes,
+                                                uint2 &ca, uint2 &cb) {
+  const float a = block_max(xa), b = block_max(xb);
+  float ra = __fmul_rn(a, q.rcp), rb = __fmul_rn(b, q.rcp);
+  if (near_boundary(ra) | near_boundary(rb)) ra = __fdiv_rn(a, q.e), rb = __fdiv_rn(b, q.e);
+  scale_codes = (uint32_t)__nv_cvt_float2_to_fp8x2(make_float2(ra, rb), __NV_SATFINITE, __NV_E4M3);
+  const float ia = q.inv[scale_codes & 127u], ib = q.inv[(scale_codes >> 8) & 127u];
+  float ya[16], yb[16];
 #pragma unroll
-  for (int i = 0; i < 16; i += 2) mul2(y[i], y[i + 1], xc[i], xc[i + 1], inv);
-  codes = make_uint2(e2m1x8(y, 0), e2m1x8(y, 8));
+  for (int i = 0; i < 16; i += 2) mul2(ya[i], ya[i + 1], xa[i], xa[i + 1], ia);
+#pragma unroll
+  for (int i = 0; i < 16; i += 2) mul2(yb[i], yb[i + 1], xb[i], xb[i + 1], ib);
+  ca = make_uint2(e2m1x8(ya, 0), e2m1x8(ya, 8));
+  cb = make_uint2(e2m1x8(yb, 0), e2m1x8(yb, 8));
+}
+// The four lanes j of a row hold the scale bytes of blocks j and j + 4: lane 0 gets the word of blocks 0..3, lane 1 that of 4..7.
+__device__ __forceinline__ uint32_t scale_word(uint32_t two, int j) {
+  uint32_t w = two << (16 * (j & 1));
+  w |= __shfl_xor_sync(0xffffffffu, w, 1);                       // bytes of blocks j, j + 4, j + 1, j + 5 (j even)
+  const uint32_t o = __shfl_xor_sync(0xffffffffu, w, 2);
+  return __byte_perm(w, o, (j & 1) ? 0x7531u : 0x6420u);         // right in lanes 0 and 1
 }
 
 // 16 channels of one row.  Two 16-byte loads touch each 32-byte sector twice; tensors that are 32-byte aligned (the interface
@@ -482,8 +501,10 @@ struct DeltaArgs {
 // to memory (partial sectors merge in L2).
 // Measured (16384 tokens, 32:8 heads, K with Delta_S and Q): two launches, rows of K staged in shared memory, two
 // divisions per block 35 + 38 us; one launch, one tile per CTA 61; with a ring of asynchronous copies and a barrier per tile 87;
-// now 45 us.
-constexpr int QT_CTAS = 2;       // resident per SM: 128 registers, so that the means stay in registers
+// now 45 us.  Both blocks of a row at once and the means in shared memory, where they were taken one after the other with the means in
+// registers (stage 1, replayed back to back): 32768 tokens, 40:8 heads 194 -> 176 us, 16384, 32:8 88.7 -> 80.7, 8 x 577, 16:16 29.1 ->
+// 27.7; three CTAs per SM of 80 registers 182, 36 for the last; 16 rows of Q dealt to the warps across heads 213 for the first.
+constexpr int QT_CTAS = 2;       // resident per SM: 128 registers
 constexpr int QT_K_WEIGHT = 2;   // time of a K tile with Delta_S in units of a Q tile's (1 / 2 / 3: 106 / 89 / 96 us of stage 1)
 constexpr int QT_SETUP = 2;      // a CTA's set-up in the same units
 template <int FEW>   // heads of the group where they are one or two, otherwise 0
@@ -516,9 +537,8 @@ __global__ void __launch_bounds__(256, QT_CTAS) quantize_tile_kernel(const Quant
   const float d = tensor_scale(a.scale, b, lane);
   if (at == 0 && tid == 0 && a.scale.gmax) a.scale.gscale[b] = d;
   const BlockScale bs = make_block_scale(d, inv_table, tid);
-  float neg_mean[2][16];
-  load_neg_mean(a.mean + head * HEAD_DIM + j * 16, neg_mean[0], vector_means(a.mean));
-  load_neg_mean(a.mean + head * HEAD_DIM + 64 + j * 16, neg_mean[1], vector_means(a.mean));
+  __shared__ __align__(16) float s_neg[8][20];   // by 16-channel block, padded against bank conflicts
+  if (tid < HEAD_DIM) s_neg[tid >> 4][tid & 15] = -a.mean[head * HEAD_DIM + tid];
   const bool with_delta = is_k && da.delta;
   const int G = with_delta ? da.H_q / a.H : 0;
   double unit = 0.0;
@@ -541,24 +561,34 @@ __global__ void __launch_bounds__(256, QT_CTAS) quantize_tile_kernel(const Quant
       double acc[FEW ? FEW : 1][2];   // FEW: two chains a head, otherwise heads 2 j and 2 j + 1
 #pragma unroll
       for (int g = 0; g < (FEW ? FEW : 1); ++g) acc[g][0] = acc[g][1] = 0.0;
-#pragma unroll
-      for (int half = 0; half < 2; ++half) {
-        float xc[16];
-        center16(raw[it][half], neg_mean[half], xc);
-        if (tile >= ctas) raw[it][half] = load_row16(x0 + (size_t)(t - ctas * TILE) * row + half * 64, wide);   // a whole tile: only the last has an end
-        uint2 c = make_uint2(0u, 0u);
-        uint32_t sc = 0u;
-        if (t < N) quantize_block16(xc, bs, sc, c);
-        __stcs(reinterpret_cast<uint2 *>(codes + (size_t)t * 64 + half * 32), c);
-        sc <<= 8 * j;   // the four scale bytes of the half row in one word
-        sc |= __shfl_xor_sync(0xffffffffu, sc, 1);
-        sc |= __shfl_xor_sync(0xffffffffu, sc, 2);
-        if (j == 0) *reinterpret_cast<uint32_t *>(sf_tile + half * 512 + (r & 31) * 16 + (r >> 5) * 4) = sc;
-        if (with_delta) {
-          if constexpr (FEW != 0)
-            few_dot16<FEW>(&gm[0][0][0], half, xc, j, acc);
-          else
-            group_dot16(gm, half, xc, lane, acc[0]);
+      float xa[16], xb[16];
+      {
+        float nm[16];
+        load_mean16(s_neg[j], nm, true);
+        center16(raw[it][0], nm, xa);
+        load_mean16(s_neg[j + 4], nm, true);
+        center16(raw[it][1], nm, xb);
+      }
+      if (tile >= ctas) {   // a whole tile: only the last has an end
+        const __nv_bfloat16 *const x1 = x0 + (size_t)(t - ctas * TILE) * row;
+        raw[it][0] = load_row16(x1, wide);
+        raw[it][1] = load_row16(x1 + 64, wide);
+      }
+      uint2 ca, cb;
+      uint32_t sc;
+      quantize_blocks(xa, xb, bs, sc, ca, cb);
+      if (t >= N) ca = cb = make_uint2(0u, 0u), sc = 0u;
+      __stcs(reinterpret_cast<uint2 *>(codes + (size_t)t * 64), ca);
+      __stcs(reinterpret_cast<uint2 *>(codes + (size_t)t * 64 + 32), cb);
+      sc = scale_word(sc, j);
+      if (j < 2) *reinterpret_cast<uint32_t *>(sf_tile + j * 512 + (r & 31) * 16 + (r >> 5) * 4) = sc;
+      if (with_delta) {
+        if constexpr (FEW != 0) {
+          few_dot16<FEW>(&gm[0][0][0], 0, xa, j, acc);
+          few_dot16<FEW>(&gm[0][0][0], 1, xb, j, acc);
+        } else {
+          group_dot16(gm, 0, xa, lane, acc[0]);
+          group_dot16(gm, 1, xb, lane, acc[0]);
         }
       }
       if (with_delta) {
@@ -785,28 +815,28 @@ __global__ void __launch_bounds__(256, WK_CTAS) write_kv_kernel(const __nv_bfloa
     pg += gridDim.y;
     if (pg < n_pages) page = page_row[page0 + pg];
     double acc[2] = {0.0, 0.0};
-#pragma unroll
-    for (int half = 0; half < 2; ++half) {
-      const int blk = half * 4 + j;
-      float xc[16];
-      center16(kr[half], neg_mean[half], xc);
-      uint2 c = make_uint2(0u, 0u);
-      uint32_t sc = 0u;
-      uint4 vc = quantize_v16(vr[half], inv_vscale);
-      fetch(half);
-      if (is_new)
-        quantize_block16(xc, bs, sc, c);
-      else
-        vc = make_uint4(0u, 0u, 0u, 0u);
-      sc <<= 8 * j;   // the four scale bytes of half a token in one word
-      sc |= __shfl_xor_sync(0xffffffffu, sc, 1);
-      sc |= __shfl_xor_sync(0xffffffffu, sc, 2);
-      if (is_new || fresh_pad) {
-        *reinterpret_cast<uint2 *>(kd + (((blk >> 1) ^ ((t & 7) >> 1)) << 4) + (blk & 1) * 8) = c;
-        if (j == 0) *reinterpret_cast<uint32_t *>(sd + half * 4) = sc;
-        *reinterpret_cast<uint4 *>(vd + ((blk ^ (t & 7)) << 4)) = vc;
-      }
-      if (delta) group_dot16(gm, half, xc, lane, acc);
+    float xa[16], xb[16];
+    center16(kr[0], neg_mean[0], xa);
+    center16(kr[1], neg_mean[1], xb);
+    uint4 va = quantize_v16(vr[0], inv_vscale), vb = quantize_v16(vr[1], inv_vscale);
+    fetch(0);
+    fetch(1);
+    uint2 ca, cb;
+    uint32_t sc;
+    quantize_blocks(xa, xb, bs, sc, ca, cb);
+    if (!is_new) ca = cb = make_uint2(0u, 0u), sc = 0u, va = vb = make_uint4(0u, 0u, 0u, 0u);
+    sc = scale_word(sc, j);
+    if (is_new || fresh_pad) {   // blocks j and j + 4 of the row
+      uint8_t *const kj = kd + (j & 1) * 8;
+      *reinterpret_cast<uint2 *>(kj + (((j >> 1) ^ ((t & 7) >> 1)) << 4)) = ca;
+      *reinterpret_cast<uint2 *>(kj + ((((j + 4) >> 1) ^ ((t & 7) >> 1)) << 4)) = cb;
+      if (j < 2) *reinterpret_cast<uint32_t *>(sd + j * 4) = sc;
+      *reinterpret_cast<uint4 *>(vd + ((j ^ (t & 7)) << 4)) = va;
+      *reinterpret_cast<uint4 *>(vd + (((j + 4) ^ (t & 7)) << 4)) = vb;
+    }
+    if (delta) {
+      group_dot16(gm, 0, xa, lane, acc);
+      group_dot16(gm, 1, xb, lane, acc);
     }
     if (delta && (is_new || fresh_pad)) {
 #pragma unroll

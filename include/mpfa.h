@@ -182,6 +182,13 @@ size_t mpfa_static_scratch_bytes(void);
 mpfa_status mpfa_quantize_v(const void *v_bf16, int B, int N_kv, int H_kv, float v_scale, uint8_t *v_fp8,
                             void *stream);
 
+/* mpfa_quantize_qk and mpfa_quantize_v in one call, with the same results: V's tiles, which depend on no statistic, share the launch of
+ * the statistics (with MPFA_STATS_FROZEN there is none, and they have one of their own).  V has the shape of K. */
+mpfa_status mpfa_quantize_qkv(const void *q_bf16, const void *k_bf16, const void *v_bf16, int B, int N_q, int N_kv,
+                              int H_q, int H_kv, int flags, float v_scale, mpfa_stats *h_stats,
+                              mpfa_fp4_tensor *h_q_out, mpfa_fp4_tensor *h_k_out, uint8_t *v_fp8,
+                              void *delta_s_bf16, void *workspace, size_t workspace_bytes, void *stream);
+
 /* For MPFA_VARIANT_PV_BF16 only (Section 3.1's NVFP4 + BF16 assignment): V unchanged, re-tiled from
  * [B, N_kv, H_kv, 128] to [B, H_kv, N_kv_pad, 128] BF16 (pad rows zero; 1024-byte aligned, 2 * mpfa_v_fp8_bytes()). */
 mpfa_status mpfa_pack_v_bf16(const void *v_bf16, int B, int N_kv, int H_kv, void *v_tiles_bf16, void *stream);

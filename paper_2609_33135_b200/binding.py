@@ -92,6 +92,7 @@ def load_library(path: str) -> ctypes.CDLL:
         L.mpfa_version.restype = i
         st, q4, pk = ctypes.POINTER(_Stats), ctypes.POINTER(_Fp4), ctypes.POINTER(_PagedKV)
         for name, args in (("mpfa_quantize_qk", [vp, vp, i, i, i, i, i, i, st, q4, q4, vp, vp, sz, vp]),
+                           ("mpfa_quantize_qkv", [vp, vp, vp, i, i, i, i, i, i, f, st, q4, q4, vp, vp, vp, sz, vp]),
                            ("mpfa_quantize_qk_static", [vp, vp, i, i, i, i, i, i, st, q4, q4, vp, vp]),
                            ("mpfa_quantize_kv_paged", [vp, vp, i, i, i, i, i, st, f, pk, vp, vp, sz, vp]),
                            ("mpfa_append_kv_paged", [vp, vp, i, i, i, i, st, f, pk, vp, i, vp, vp]),
@@ -257,6 +258,20 @@ def mpfa_quantize_qk(q: Optional[torch.Tensor], k: Optional[torch.Tensor], flags
     _check(rc, "mpfa_quantize_qk")
 
 
+def mpfa_quantize_qkv(q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, flags: int, v_scale: float, stats: Stats, q_out: Fp4Tensor,
+                      k_out: Fp4Tensor, v_out: torch.Tensor, delta: Optional[torch.Tensor], workspace: Optional[torch.Tensor]) -> None:
+    """mpfa_quantize_qk and mpfa_quantize_v in one call; v has the shape of k."""
+    for t in (q, k, v):
+        assert t.is_cuda and t.dtype == torch.bfloat16 and t.is_contiguous() and t.shape[3] == HEAD_DIM
+    assert v.shape == k.shape
+    B, N_q, H_q, _ = q.shape
+    _, N_kv, H_kv, _ = k.shape
+    rc = lib().packed_mpfa_quantize_qkv(q.data_ptr(), k.data_ptr(), v.data_ptr(), B, N_q, N_kv, H_q, H_kv, flags, v_scale,
+                                        stats.packed_stats(), q_out.packed_fp4(), k_out.packed_fp4(), v_out.data_ptr(), _ptr(delta),
+                                        _ptr(workspace), 0 if workspace is None else workspace.numel(), _stream())
+    _check(rc, "mpfa_quantize_qkv")
+
+
 def mpfa_quantize_qk_static(q: Optional[torch.Tensor], k: Optional[torch.Tensor], flags: int, stats: Stats,
                             q_out: Optional[Fp4Tensor], k_out: Optional[Fp4Tensor],
                             delta: Optional[torch.Tensor]) -> None:
@@ -387,8 +402,12 @@ def stage1(q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, smooth: bool = Tru
                      Stats.empty(B, H_q, H_kv, dev), v_scale)
     if workspace is None:
         workspace = quantize_workspace(B, H_q, H_kv, dev)
-    mpfa_quantize_qk(q, k, MPFA_SMOOTH if smooth else 0, out.stats, out.q, out.k, out.delta, workspace)
-    mpfa_quantize_v(v, v_scale, out.v_fp8)
+    flags = MPFA_SMOOTH if smooth else 0
+    if v.shape == k.shape:
+        mpfa_quantize_qkv(q, k, v, flags, v_scale, out.stats, out.q, out.k, out.v_fp8, out.delta, workspace)
+    else:
+        mpfa_quantize_qk(q, k, flags, out.stats, out.q, out.k, out.delta, workspace)
+        mpfa_quantize_v(v, v_scale, out.v_fp8)
     return out
 
 

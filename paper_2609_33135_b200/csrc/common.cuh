@@ -44,18 +44,26 @@ inline mpfa_status cuda_fail(cudaError_t e) {
 // order of the stream holds transitively.  Such a kernel is resident while its inputs are still being written, so it reads global
 // memory with ordinary loads only: a non-coherent load (__ldg, ld.global.nc, what the compiler makes of const __restrict__)
 // asks for data that no one writes during the kernel's life, and the compiler may move it above the wait.
+struct Grid {   // blocks, and how many along x make a cluster
+  dim3 blocks;
+  unsigned cluster;
+  Grid(dim3 b, unsigned c = 1) : blocks(b), cluster(c) {}
+};
 template <typename... KArgs, typename... Args>
-cudaError_t launch(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, Args &&...args) {
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
+cudaError_t launch(void (*kernel)(KArgs...), Grid grid, dim3 block, size_t smem, cudaStream_t stream, Args &&...args) {
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = grid.cluster;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
+  cfg.gridDim = grid.blocks;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = grid.cluster > 1 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 

@@ -78,6 +78,7 @@ constexpr int STAT_THREADS = 256;
 constexpr int STAT_LOADS = 8;   // rows in flight per thread, and as many being added
 constexpr int STAT_CTAS = 2;    // resident per SM
 constexpr int STAT_LANES = STAT_THREADS / 16;
+constexpr int STAT_CLUSTER = 8;
 
 struct ColTensor {
   const __nv_bfloat16 *x;   // null: tensor absent (H = 0)
@@ -120,18 +121,44 @@ __device__ __forceinline__ void finish_column(const ColTensor &a, int b, int h, 
   if (c == 0) a.gmax[((size_t)b * a.H + h) * MAXIMA_STRIDE] = fmaxf(fmaxf(s_w[0], s_w[1]), fmaxf(s_w[2], s_w[3]));
 }
 
-// grid (slices * heads of both tensors, 1, B), the slice fastest; heads are not a grid dimension of their own, which ends at 65535
-__global__ void __launch_bounds__(STAT_THREADS, STAT_CTAS) colstat_kernel(const ColTensor t0, const ColTensor t1, int slices, int smooth) {
+// V's quantization depends on no statistic: its tiles ride along in CTAs of their own behind those of the statistics.
+struct VTensor {
+  const __nv_bfloat16 *x;   // null: none
+  int N, H, tiles;
+  float inv_scale;
+  uint8_t *out;
+};
+__device__ __forceinline__ void quantize_v_tile(const VTensor &v, int tile, int h, int b);
+
+// grid (slices * heads of both tensors * B, the slice fastest and the batch element slowest, then V's tiles); heads are not a grid
+// dimension of their own, which ends at 65535.  CLUSTERS: the slices of a head are a cluster, and its first CTA finishes the head from the
+// partial results that the others leave in its shared memory.
+template <bool CLUSTERS>
+__global__ void __launch_bounds__(STAT_THREADS, STAT_CTAS) colstat_kernel(const ColTensor t0, const ColTensor t1, int B, int slices, int smooth, const VTensor v) {
+  __shared__ double s_part[CLUSTERS ? STAT_CLUSTER : 1][CLUSTERS ? HEAD_DIM : 1];
+  __shared__ float2 s_ext[CLUSTERS ? STAT_CLUSTER : 1][CLUSTERS ? HEAD_DIM : 1];
   __shared__ double s_sum[STAT_LANES][HEAD_DIM];
   __shared__ uint32_t s_mx[STAT_LANES][HEAD_DIM / 2], s_mn[STAT_LANES][HEAD_DIM / 2];
   __shared__ float s_w[4];
   launch_dependents();
+  if (CLUSTERS) cluster_arrive();   // so that all CTAs of the cluster are there when the first writes to another
   grid_dependency_wait();
-  const int at = blockIdx.x / slices, slice = blockIdx.x - at * slices;
+  const int heads = t0.H + t1.H;
+  int at = blockIdx.x / slices;
+  const int slice = blockIdx.x - at * slices;
+  if (at >= heads * B) {
+    if (CLUSTERS) cluster_wait();
+    const int n = blockIdx.x - slices * heads * B, tile = n % v.tiles, vh = n / v.tiles % v.H, vb = n / v.tiles / v.H;
+    if (vb < B) quantize_v_tile(v, tile, vh, vb);
+    if (CLUSTERS) cluster_arrive(), cluster_wait();
+    return;
+  }
+  const int b = at / heads;
+  at -= b * heads;
   const bool first = at < t0.H;
   const ColTensor &a = first ? t0 : t1;
   const int h = first ? at : at - t0.H;
-  const int b = blockIdx.z, tid = threadIdx.x, tl = tid >> 4, cg = tid & 15;
+  const int tid = threadIdx.x, tl = tid >> 4, cg = tid & 15;
   const int len = ((a.N + slices - 1) / slices + STAT_LANES - 1) / STAT_LANES * STAT_LANES;
   const int begin = min(a.N, slice * len), end = min(a.N, begin + len);
   const size_t row = (size_t)a.H * HEAD_DIM, step = STAT_LANES * row;
@@ -204,7 +231,9 @@ __global__ void __launch_bounds__(STAT_THREADS, STAT_CTAS) colstat_kernel(const 
     s_mn[tl][i * 16 + cg] = mn[i];
   }
   __syncthreads();
-  if (tid >= HEAD_DIM) return;
+  if (!CLUSTERS && tid >= HEAD_DIM) return;
+  if (CLUSTERS) cluster_wait();
+  if (tid < HEAD_DIM) {
   // place of column tid: pair i of group cg
   const int place = ((tid & 7) >> 1) * 32 + (tid >> 3) * 2 + (tid & 1);
   double sum = 0.0;
@@ -216,12 +245,25 @@ __global__ void __launch_bounds__(STAT_THREADS, STAT_CTAS) colstat_kernel(const 
     lo = bf16x2_min(lo, s_mn[j][place >> 1]);
   }
   const float fmx = __uint_as_float(tid & 1 ? hi & 0xFFFF0000u : hi << 16), fmn = __uint_as_float(tid & 1 ? lo & 0xFFFF0000u : lo << 16);
-  if (slices == 1) {
+  if (CLUSTERS) {
+    cluster_store(cluster_address(smem_u32(&s_part[slice][tid]), 0), sum);
+    cluster_store(cluster_address(smem_u32(&s_ext[slice][tid]), 0), fmx, fmn);
+  } else if (slices == 1) {
     finish_column(a, b, h, tid, sum, fmx, fmn, smooth, s_w);
   } else {
-    const size_t o = ((size_t)slice * gridDim.z + b) * row + h * HEAD_DIM + tid;
+    const size_t o = ((size_t)slice * B + b) * row + h * HEAD_DIM + tid;
     a.psum[o] = sum;
     a.pext[o] = make_float2(fmx, fmn);
+  }
+  }
+  if (CLUSTERS) {
+    cluster_arrive();
+    cluster_wait();
+    if (slice != 0 || tid >= HEAD_DIM) return;
+    double sum = 0.0;
+    float mx = -INFINITY, mn = INFINITY;
+    for (int s = 0; s < slices; ++s) sum += s_part[s][tid], mx = fmaxf(mx, s_ext[s][tid].x), mn = fminf(mn, s_ext[s][tid].y);
+    finish_column(a, b, h, tid, sum, mx, mn, smooth, s_w);
   }
 }
 
@@ -671,27 +713,29 @@ __device__ __forceinline__ uint4 quantize_v16(const Row16 &x, float inv) {
   return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-// grid (N_pad/128, H, B): V tile -> [B, H, N_pad, 128] E4M3.
-__global__ void __launch_bounds__(256) quantize_v_tile_kernel(const __nv_bfloat16 *v, int N, int H,
-                                                              float inv_scale, uint8_t *out) {
-  launch_dependents();
-  grid_dependency_wait();
-  const int tile = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
-  const int n_pad = gridDim.x * TILE;
-  const bool wide = wide_rows(v);
+// V tile -> [B, H, N_pad, 128] E4M3; 256 threads
+__device__ __forceinline__ void quantize_v_tile(const VTensor &v, int tile, int h, int b) {
+  const size_t n_pad = (size_t)v.tiles * TILE;
+  const bool wide = wide_rows(v.x);
   const int r0 = threadIdx.x >> 3, seg = threadIdx.x & 7;
   Row16 x[4] = {};
 #pragma unroll
   for (int it = 0; it < 4; ++it) {
     const int t = tile * TILE + it * 32 + r0;
-    if (t < N) x[it] = load_row16(v + (((size_t)b * N + t) * H + h) * HEAD_DIM + seg * 16, wide);
+    if (t < v.N) x[it] = load_row16(v.x + (((size_t)b * v.N + t) * v.H + h) * HEAD_DIM + seg * 16, wide);
   }
 #pragma unroll
   for (int it = 0; it < 4; ++it) {
     const int t = tile * TILE + it * 32 + r0;
-    *reinterpret_cast<uint4 *>(out + (((size_t)b * H + h) * n_pad + t) * HEAD_DIM + seg * 16) =
-        t < N ? quantize_v16(x[it], inv_scale) : make_uint4(0u, 0u, 0u, 0u);
+    *reinterpret_cast<uint4 *>(v.out + (((size_t)b * v.H + h) * n_pad + t) * HEAD_DIM + seg * 16) =
+        t < v.N ? quantize_v16(x[it], v.inv_scale) : make_uint4(0u, 0u, 0u, 0u);
   }
+}
+// grid (N_pad/128, H, B)
+__global__ void __launch_bounds__(256) quantize_v_tile_kernel(const VTensor v) {
+  launch_dependents();
+  grid_dependency_wait();
+  quantize_v_tile(v, blockIdx.x, blockIdx.y, blockIdx.z);
 }
 
 // grid (N_pad/128, H, B): V tile -> [B, H, N_pad, 128] BF16, unchanged values (the NVFP4 + BF16 precision assignment
@@ -962,15 +1006,27 @@ StatsWorkspace carve(void *ws, size_t ws_bytes, int B, int H_q, int H_kv) {
   return w;
 }
 
-// Means and the heads' maxima of up to two tensors.
-mpfa_status tensor_stats(const ColTensor &c0, const ColTensor &c1, int B, int max_slices, int n_sm, bool smooth, cudaStream_t st) {
+// Means and the heads' maxima of up to two tensors, and V's tiles.
+constexpr int STAT_CLUSTER_MIN = 128;   // tokens of a slice: one round of loads
+constexpr int STAT_CLUSTER_MAX = 640;
+mpfa_status tensor_stats(const ColTensor &c0, const ColTensor &c1, int B, int max_slices, int n_sm, bool smooth, const VTensor &v, cudaStream_t st) {
   const int heads = c0.H + c1.H, N = std::max(c0.x ? c0.N : 0, c1.x ? c1.N : 0);
   if (heads == 0) return MPFA_OK;
+  const long long v_ctas = v.x ? (long long)v.tiles * v.H * B : 0;
+  // Short passes: a cluster for each head, of a power of two CTAs (clusters of seven leave places free in every GPC: 8 + 2 heads of
+  // 4 x 777 tokens 13.7 us of stage 1, with four 11.9), as long as its slices stay short and all clusters fit at once.
+  int C = STAT_CLUSTER;
+  while (C > 1 && (C * heads * (long long)B * 8 > 7LL * STAT_CTAS * n_sm || C / 2 * STAT_CLUSTER_MIN >= N)) C /= 2;
+  if (C > 1 && N <= C * STAT_CLUSTER_MAX) {
+    const long long ctas = (long long)C * heads * B + (v_ctas + C - 1) / C * C;
+    MPFA_CUDA_OK(launch(colstat_kernel<true>, Grid(dim3((unsigned)ctas), C), dim3(STAT_THREADS), 0, st, c0, c1, B, C, smooth ? 1 : 0, v));
+    return MPFA_OK;
+  }
   // As many slices as the launch can hold in one wave.  A fold costs about as much as STAT_MIN tokens
   // of a CTA's pass, so slices are not made shorter than that.
   constexpr int STAT_MIN = 512;
   const int S = (int)std::max(1LL, std::min({(long long)max_slices, (long long)STAT_CTAS * n_sm / ((long long)heads * B), (long long)N / STAT_MIN}));
-  MPFA_CUDA_OK(launch(colstat_kernel, dim3(S * heads, 1, B), dim3(STAT_THREADS), 0, st, c0, c1, S, smooth ? 1 : 0));
+  MPFA_CUDA_OK(launch(colstat_kernel<false>, dim3((unsigned)((long long)S * heads * B + v_ctas)), dim3(STAT_THREADS), 0, st, c0, c1, B, S, smooth ? 1 : 0, v));
   if (S > 1) MPFA_CUDA_OK(launch(stat_fold_kernel, dim3(heads, B), dim3(128), 0, st, c0, c1, S, smooth ? 1 : 0));
   return MPFA_OK;
 }
@@ -990,10 +1046,10 @@ extern "C" size_t mpfa_quantize_workspace_min_bytes(int B, int H_q, int H_kv) {
   return stats_fixed_bytes(B, H_q, H_kv) + stats_slice_bytes(B, H_q, H_kv);
 }
 
-extern "C" mpfa_status mpfa_quantize_qk(const void *q_bf16, const void *k_bf16, int B, int N_q, int N_kv, int H_q,
-                                        int H_kv, int flags, mpfa_stats *st, mpfa_fp4_tensor *q_out,
-                                        mpfa_fp4_tensor *k_out, void *delta_s_bf16, void *workspace,
-                                        size_t workspace_bytes, void *stream) {
+static mpfa_status quantize_qkv(const void *q_bf16, const void *k_bf16, const VTensor &v, int B, int N_q, int N_kv, int H_q,
+                                int H_kv, int flags, mpfa_stats *st, mpfa_fp4_tensor *q_out,
+                                mpfa_fp4_tensor *k_out, void *delta_s_bf16, void *workspace,
+                                size_t workspace_bytes, void *stream) {
   const bool smooth = flags & MPFA_SMOOTH, frozen = flags & MPFA_STATS_FROZEN;
   if (!st || (!q_bf16 && !k_bf16) || B <= 0 || H_q <= 0 || H_kv <= 0) return MPFA_ERR_INVALID_ARG;
   if ((q_bf16 && (N_q <= 0 || !q_out)) || (k_bf16 && (N_kv <= 0 || !k_out))) return MPFA_ERR_INVALID_ARG;
@@ -1024,8 +1080,10 @@ extern "C" mpfa_status mpfa_quantize_qk(const void *q_bf16, const void *k_bf16, 
   const __nv_bfloat16 *k = static_cast<const __nv_bfloat16 *>(k_bf16);
   if (!frozen) {
     rc = tensor_stats(ColTensor{q, N_q, q ? H_q : 0, w.psum_q, w.pext_q, st->q_mean, w.gmax_q},
-                      ColTensor{k, N_kv, k ? H_kv : 0, w.psum_k, w.pext_k, st->k_mean, w.gmax_k}, B, w.slices, n_sm, smooth, s);
+                      ColTensor{k, N_kv, k ? H_kv : 0, w.psum_k, w.pext_k, st->k_mean, w.gmax_k}, B, w.slices, n_sm, smooth, v, s);
     if (rc != MPFA_OK) return rc;
+  } else if (v.x) {
+    MPFA_CUDA_OK(launch(quantize_v_tile_kernel, dim3(v.tiles, v.H, B), dim3(256), 0, s, v));
   }
   // Q and K tiles in one launch; with smoothing the K tiles also produce Delta_S (Eq. 9)
   const TensorScale sq{st->q_gscale, frozen ? nullptr : w.gmax_q, H_q}, sk{st->k_gscale, frozen ? nullptr : w.gmax_k, H_kv};
@@ -1049,7 +1107,7 @@ extern "C" mpfa_status mpfa_quantize_qk(const void *q_bf16, const void *k_bf16, 
   };
   const long long mean = (work + wave - 1) / wave;
   if (((long long)tk.H + tq.H) * B <= wave) {
-    for (long long per = mean; split(per) > wave; ++per) {}
+    for (long long per = std::max(1LL, mean / 2); split(per) > wave; ++per) {}   // the shortest Q tasks that fit
   } else {
     // More heads than a wave has CTAs: the work with its set-ups spread over the SMs, and one CTA's length at the end.  (One CTA
     // per head here left one query token on 9 x 4865 keys, 40:8 heads, at 219 us of stage 1, now 127; 10 x 5647 467 -> 406;
@@ -1070,6 +1128,24 @@ extern "C" mpfa_status mpfa_quantize_qk(const void *q_bf16, const void *k_bf16, 
   return MPFA_OK;
 }
 
+extern "C" mpfa_status mpfa_quantize_qk(const void *q_bf16, const void *k_bf16, int B, int N_q, int N_kv, int H_q,
+                                        int H_kv, int flags, mpfa_stats *st, mpfa_fp4_tensor *q_out,
+                                        mpfa_fp4_tensor *k_out, void *delta_s_bf16, void *workspace,
+                                        size_t workspace_bytes, void *stream) {
+  return quantize_qkv(q_bf16, k_bf16, VTensor{}, B, N_q, N_kv, H_q, H_kv, flags, st, q_out, k_out, delta_s_bf16, workspace, workspace_bytes, stream);
+}
+
+extern "C" mpfa_status mpfa_quantize_qkv(const void *q_bf16, const void *k_bf16, const void *v_bf16, int B, int N_q, int N_kv, int H_q,
+                                         int H_kv, int flags, float v_scale, mpfa_stats *st, mpfa_fp4_tensor *q_out,
+                                         mpfa_fp4_tensor *k_out, uint8_t *v_fp8, void *delta_s_bf16, void *workspace,
+                                         size_t workspace_bytes, void *stream) {
+  if (!v_bf16 || !v_fp8 || B <= 0 || N_kv <= 0 || H_kv <= 0 || !(v_scale > 0.0f)) return MPFA_ERR_INVALID_ARG;
+  if (!aligned(v_bf16, 16) || !aligned(v_fp8, 1024)) return MPFA_ERR_ALIGNMENT;
+  if (B > 65535 || H_kv > 65535) return MPFA_ERR_UNSUPPORTED;   // as mpfa_quantize_v, whose launch fails
+  const VTensor v{static_cast<const __nv_bfloat16 *>(v_bf16), N_kv, H_kv, pad128(N_kv) / TILE, 1.0f / v_scale, v_fp8};
+  return quantize_qkv(q_bf16, k_bf16, v, B, N_q, N_kv, H_q, H_kv, flags, st, q_out, k_out, delta_s_bf16, workspace, workspace_bytes, stream);
+}
+
 extern "C" mpfa_status mpfa_quantize_v(const void *v_bf16, int B, int N_kv, int H_kv, float v_scale, uint8_t *v_fp8,
                                        void *stream) {
   if (!v_bf16 || !v_fp8 || B <= 0 || N_kv <= 0 || H_kv <= 0 || !(v_scale > 0.0f)) return MPFA_ERR_INVALID_ARG;
@@ -1079,7 +1155,7 @@ extern "C" mpfa_status mpfa_quantize_v(const void *v_bf16, int B, int N_kv, int 
   if (rc != MPFA_OK) return rc;
   dim3 grid(pad128(N_kv) / TILE, H_kv, B);
   MPFA_CUDA_OK(launch(quantize_v_tile_kernel, grid, dim3(256), 0, static_cast<cudaStream_t>(stream),
-                      static_cast<const __nv_bfloat16 *>(v_bf16), N_kv, H_kv, 1.0f / v_scale, v_fp8));
+                      VTensor{static_cast<const __nv_bfloat16 *>(v_bf16), N_kv, H_kv, pad128(N_kv) / TILE, 1.0f / v_scale, v_fp8}));
   return MPFA_OK;
 }
 
@@ -1145,7 +1221,7 @@ extern "C" mpfa_status mpfa_quantize_kv_paged(const void *k_bf16, const void *v_
   const __nv_bfloat16 *k = static_cast<const __nv_bfloat16 *>(k_bf16);
   const __nv_bfloat16 *v = static_cast<const __nv_bfloat16 *>(v_bf16);
   if (!frozen) {
-    rc = tensor_stats(ColTensor{k, N_tokens, H_kv, w.psum_k, w.pext_k, st->k_mean, w.gmax_k}, ColTensor{}, 1, w.slices, n_sm, smooth, s);
+    rc = tensor_stats(ColTensor{k, N_tokens, H_kv, w.psum_k, w.pext_k, st->k_mean, w.gmax_k}, ColTensor{}, 1, w.slices, n_sm, smooth, VTensor{}, s);
     if (rc != MPFA_OK) return rc;
   }
   const TensorScale sk{st->k_gscale, frozen ? nullptr : w.gmax_k, H_kv};

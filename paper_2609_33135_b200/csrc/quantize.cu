@@ -60,8 +60,8 @@ __device__ __forceinline__ void unpack8(const uint4 &u, float (&f)[8]) {
 // A CTA covers one head (128 columns) x one slice of the tokens: thread = (token lane 0..15, 8 columns), eight independent
 // 16-byte loads in flight per thread while the eight before them are added; each thread adds its tokens in ascending order, the 16 token lanes are folded in lane
 // order in shared memory.  With one slice the CTA writes mean = fl(sum / N) (0 without smoothing) and the head's max |x - mean|
-// itself; otherwise the slices' partial results go to the workspace and stat_fold_kernel adds them in
-// slice order.  No counter, no memory to clear.  Every addition order is fixed by the shape, the workspace size
+// itself.  Slices of a short tensor are a cluster, whose first CTA adds their partial results in slice order; otherwise these go to the
+// workspace and stat_fold_kernel adds them in the same order.  No counter, no memory to clear.  Every addition order is fixed by the shape, the workspace size
 // and the device's SM count, so the result is reproducible bit for bit for any input; it equals the oracle's single
 // ascending FP64 sum whenever all these sums are exact (always true for BF16 inputs whose exponents span fewer than
 // about 40 binades per column).
@@ -72,13 +72,14 @@ __device__ __forceinline__ void unpack8(const uint4 &u, float (&f)[8]) {
 // round as the unscaled ones do.  Infinities and NaNs would become finite; an FMA with zero catches them, and that
 // thread's slice is added again with the conversion.
 // Measured (Q and K, 32:8 heads, 16384 tokens / 1:1 heads, 256 tokens; with memory-set node or fold): with conversions, four
-// loads in flight and the last CTA of a group folding the slices 42 / 11 us, now 40 / 3.6 us (4.5 TB/s).  (The slices as CTAs of a
-// cluster, folded through distributed shared memory: clusters leave some SMs empty and others full, 45 us.)
+// loads in flight and the last CTA of a group folding the slices 42 / 11 us, now 40 / 3.6 us (4.5 TB/s).  Clusters leave some SMs
+// empty and others full: 45 us of the first, so only for short tensors.  There (stage 1 without / with clusters): 8 + 2 heads of 4 x 777
+// tokens 16.0 / 11.9 us, 40 + 8 of 1999 21.6 / 19.2, 32 + 8 of 1100 16.2 / 13.1, of 4096 25.5 / 27.5.
 constexpr int STAT_THREADS = 256;
 constexpr int STAT_LOADS = 8;   // rows in flight per thread, and as many being added
 constexpr int STAT_CTAS = 2;    // resident per SM
 constexpr int STAT_LANES = STAT_THREADS / 16;
-constexpr int STAT_CLUSTER = 8;
+constexpr int STAT_CLUSTER = 16;   // more than eight have to be allowed
 
 struct ColTensor {
   const __nv_bfloat16 *x;   // null: tensor absent (H = 0)
@@ -133,20 +134,19 @@ __device__ __forceinline__ void quantize_v_tile(const VTensor &v, int tile, int 
 // grid (slices * heads of both tensors * B, the slice fastest and the batch element slowest, then V's tiles); heads are not a grid
 // dimension of their own, which ends at 65535.  CLUSTERS: the slices of a head are a cluster, and its first CTA finishes the head from the
 // partial results that the others leave in its shared memory.
-template <bool CLUSTERS>
+template <bool CLUSTERS, bool WITH_V>
 __global__ void __launch_bounds__(STAT_THREADS, STAT_CTAS) colstat_kernel(const ColTensor t0, const ColTensor t1, int B, int slices, int smooth, const VTensor v) {
-  __shared__ double s_part[CLUSTERS ? STAT_CLUSTER : 1][CLUSTERS ? HEAD_DIM : 1];
-  __shared__ float2 s_ext[CLUSTERS ? STAT_CLUSTER : 1][CLUSTERS ? HEAD_DIM : 1];
+  __shared__ double s_part[CLUSTERS ? STAT_CLUSTER : 2][CLUSTERS ? HEAD_DIM : 1];
+  __shared__ uint32_t s_ext[CLUSTERS ? STAT_CLUSTER : 1][CLUSTERS ? HEAD_DIM : 1];   // maximum in the upper half, minimum in the lower
   __shared__ double s_sum[STAT_LANES][HEAD_DIM];
   __shared__ uint32_t s_mx[STAT_LANES][HEAD_DIM / 2], s_mn[STAT_LANES][HEAD_DIM / 2];
-  __shared__ float s_w[4];
   launch_dependents();
   if (CLUSTERS) cluster_arrive();   // so that all CTAs of the cluster are there when the first writes to another
   grid_dependency_wait();
   const int heads = t0.H + t1.H;
   int at = blockIdx.x / slices;
   const int slice = blockIdx.x - at * slices;
-  if (at >= heads * B) {
+  if (WITH_V && at >= heads * B) {
     if (CLUSTERS) cluster_wait();
     const int n = blockIdx.x - slices * heads * B, tile = n % v.tiles, vh = n / v.tiles % v.H, vb = n / v.tiles / v.H;
     if (vb < B) quantize_v_tile(v, tile, vh, vb);
@@ -234,27 +234,27 @@ __global__ void __launch_bounds__(STAT_THREADS, STAT_CTAS) colstat_kernel(const 
   if (!CLUSTERS && tid >= HEAD_DIM) return;
   if (CLUSTERS) cluster_wait();
   if (tid < HEAD_DIM) {
-  // place of column tid: pair i of group cg
-  const int place = ((tid & 7) >> 1) * 32 + (tid >> 3) * 2 + (tid & 1);
-  double sum = 0.0;
-  uint32_t hi = 0xFF80FF80u, lo = 0x7F807F80u;
+    // place of column tid: pair i of group cg
+    const int place = ((tid & 7) >> 1) * 32 + (tid >> 3) * 2 + (tid & 1);
+    double sum = 0.0;
+    uint32_t hi = 0xFF80FF80u, lo = 0x7F807F80u;
 #pragma unroll
-  for (int j = 0; j < STAT_LANES; ++j) {
-    sum += s_sum[j][place];
-    hi = bf16x2_max(hi, s_mx[j][place >> 1]);
-    lo = bf16x2_min(lo, s_mn[j][place >> 1]);
-  }
-  const float fmx = __uint_as_float(tid & 1 ? hi & 0xFFFF0000u : hi << 16), fmn = __uint_as_float(tid & 1 ? lo & 0xFFFF0000u : lo << 16);
-  if (CLUSTERS) {
-    cluster_store(cluster_address(smem_u32(&s_part[slice][tid]), 0), sum);
-    cluster_store(cluster_address(smem_u32(&s_ext[slice][tid]), 0), fmx, fmn);
-  } else if (slices == 1) {
-    finish_column(a, b, h, tid, sum, fmx, fmn, smooth, s_w);
-  } else {
-    const size_t o = ((size_t)slice * B + b) * row + h * HEAD_DIM + tid;
-    a.psum[o] = sum;
-    a.pext[o] = make_float2(fmx, fmn);
-  }
+    for (int j = 0; j < STAT_LANES; ++j) {
+      sum += s_sum[j][place];
+      hi = bf16x2_max(hi, s_mx[j][place >> 1]);
+      lo = bf16x2_min(lo, s_mn[j][place >> 1]);
+    }
+    const float fmx = __uint_as_float(tid & 1 ? hi & 0xFFFF0000u : hi << 16), fmn = __uint_as_float(tid & 1 ? lo & 0xFFFF0000u : lo << 16);
+    if (CLUSTERS) {
+      cluster_store(cluster_address(smem_u32(&s_part[slice][tid]), 0), sum);
+      cluster_store(cluster_address(smem_u32(&s_ext[slice][tid]), 0), __float_as_uint(fmx) | __float_as_uint(fmn) >> 16);
+    } else if (slices == 1) {
+      finish_column(a, b, h, tid, sum, fmx, fmn, smooth, reinterpret_cast<float *>(&s_part[0][0]));
+    } else {
+      const size_t o = ((size_t)slice * B + b) * row + h * HEAD_DIM + tid;
+      a.psum[o] = sum;
+      a.pext[o] = make_float2(fmx, fmn);
+    }
   }
   if (CLUSTERS) {
     cluster_arrive();
@@ -262,8 +262,11 @@ __global__ void __launch_bounds__(STAT_THREADS, STAT_CTAS) colstat_kernel(const 
     if (slice != 0 || tid >= HEAD_DIM) return;
     double sum = 0.0;
     float mx = -INFINITY, mn = INFINITY;
-    for (int s = 0; s < slices; ++s) sum += s_part[s][tid], mx = fmaxf(mx, s_ext[s][tid].x), mn = fminf(mn, s_ext[s][tid].y);
-    finish_column(a, b, h, tid, sum, mx, mn, smooth, s_w);
+    for (int s = 0; s < slices; ++s) {
+      const uint32_t e = s_ext[s][tid];
+      sum += s_part[s][tid], mx = fmaxf(mx, __uint_as_float(e & 0xFFFF0000u)), mn = fminf(mn, __uint_as_float(e << 16));
+    }
+    finish_column(a, b, h, tid, sum, mx, mn, smooth, reinterpret_cast<float *>(&s_mx[0][0]));
   }
 }
 
@@ -1008,7 +1011,8 @@ StatsWorkspace carve(void *ws, size_t ws_bytes, int B, int H_q, int H_kv) {
 
 // Means and the heads' maxima of up to two tensors, and V's tiles.
 constexpr int STAT_CLUSTER_MIN = 128;   // tokens of a slice: one round of loads
-constexpr int STAT_CLUSTER_MAX = 640;
+constexpr int STAT_CLUSTER_MAX = 640;   // beyond that the slices of one wave are shorter (limits of 256, 512 and 1100 tokens were worse or no better)
+constexpr long long V_APART = 512ll << 20;
 mpfa_status tensor_stats(const ColTensor &c0, const ColTensor &c1, int B, int max_slices, int n_sm, bool smooth, const VTensor &v, cudaStream_t st) {
   const int heads = c0.H + c1.H, N = std::max(c0.x ? c0.N : 0, c1.x ? c1.N : 0);
   if (heads == 0) return MPFA_OK;
@@ -1016,17 +1020,21 @@ mpfa_status tensor_stats(const ColTensor &c0, const ColTensor &c1, int B, int ma
   // Short passes: a cluster for each head, of a power of two CTAs (clusters of seven leave places free in every GPC: 8 + 2 heads of
   // 4 x 777 tokens 13.7 us of stage 1, with four 11.9), as long as its slices stay short and all clusters fit at once.
   int C = STAT_CLUSTER;
-  while (C > 1 && (C * heads * (long long)B * 8 > 7LL * STAT_CTAS * n_sm || C / 2 * STAT_CLUSTER_MIN >= N)) C /= 2;
+  while (C > 1 && (C > max_slices || (C > 8 && N <= 16 * STAT_CLUSTER_MIN) || C * heads * (long long)B * 8 > 7LL * STAT_CTAS * n_sm ||
+                   C / 2 * STAT_CLUSTER_MIN >= N))
+    C /= 2;
   if (C > 1 && N <= C * STAT_CLUSTER_MAX) {
+    if (C > 8) MPFA_CUDA_OK(cudaFuncSetAttribute(colstat_kernel<true, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));   // kept per context
     const long long ctas = (long long)C * heads * B + (v_ctas + C - 1) / C * C;
-    MPFA_CUDA_OK(launch(colstat_kernel<true>, Grid(dim3((unsigned)ctas), C), dim3(STAT_THREADS), 0, st, c0, c1, B, C, smooth ? 1 : 0, v));
+    MPFA_CUDA_OK(launch(colstat_kernel<true, true>, Grid(dim3((unsigned)ctas), C), dim3(STAT_THREADS), 0, st, c0, c1, B, C, smooth ? 1 : 0, v));
     return MPFA_OK;
   }
   // As many slices as the launch can hold in one wave.  A fold costs about as much as STAT_MIN tokens
   // of a CTA's pass, so slices are not made shorter than that.
   constexpr int STAT_MIN = 512;
   const int S = (int)std::max(1LL, std::min({(long long)max_slices, (long long)STAT_CTAS * n_sm / ((long long)heads * B), (long long)N / STAT_MIN}));
-  MPFA_CUDA_OK(launch(colstat_kernel<false>, dim3((unsigned)((long long)S * heads * B + v_ctas)), dim3(STAT_THREADS), 0, st, c0, c1, B, S, smooth ? 1 : 0, v));
+  MPFA_CUDA_OK(launch(v.x ? colstat_kernel<false, true> : colstat_kernel<false, false>, dim3((unsigned)((long long)S * heads * B + v_ctas)),
+                      dim3(STAT_THREADS), 0, st, c0, c1, B, S, smooth ? 1 : 0, v));
   if (S > 1) MPFA_CUDA_OK(launch(stat_fold_kernel, dim3(heads, B), dim3(128), 0, st, c0, c1, S, smooth ? 1 : 0));
   return MPFA_OK;
 }
@@ -1078,13 +1086,16 @@ static mpfa_status quantize_qkv(const void *q_bf16, const void *k_bf16, const VT
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const __nv_bfloat16 *q = static_cast<const __nv_bfloat16 *>(q_bf16);
   const __nv_bfloat16 *k = static_cast<const __nv_bfloat16 *>(k_bf16);
+  // V has a launch of its own where there is no other, and where Q and K are well beyond L2: between the two passes over them V
+  // would push out the ends that the second one finds there (32:8 heads: 16384 tokens 83.3 us together, 86.1 apart; 16 x 2000 158 and 167;
+  // 32768, 40:8 177.0 and 176.4; 65536 291 and 287).
+  const bool apart = v.x && (frozen || ((long long)N_q * (q ? H_q : 0) + (long long)N_kv * (k ? H_kv : 0)) * B * HEAD_DIM * 2 > V_APART);
   if (!frozen) {
     rc = tensor_stats(ColTensor{q, N_q, q ? H_q : 0, w.psum_q, w.pext_q, st->q_mean, w.gmax_q},
-                      ColTensor{k, N_kv, k ? H_kv : 0, w.psum_k, w.pext_k, st->k_mean, w.gmax_k}, B, w.slices, n_sm, smooth, v, s);
+                      ColTensor{k, N_kv, k ? H_kv : 0, w.psum_k, w.pext_k, st->k_mean, w.gmax_k}, B, w.slices, n_sm, smooth, apart ? VTensor{} : v, s);
     if (rc != MPFA_OK) return rc;
-  } else if (v.x) {
-    MPFA_CUDA_OK(launch(quantize_v_tile_kernel, dim3(v.tiles, v.H, B), dim3(256), 0, s, v));
   }
+  if (apart) MPFA_CUDA_OK(launch(quantize_v_tile_kernel, dim3(v.tiles, v.H, B), dim3(256), 0, s, v));
   // Q and K tiles in one launch; with smoothing the K tiles also produce Delta_S (Eq. 9)
   const TensorScale sq{st->q_gscale, frozen ? nullptr : w.gmax_q, H_q}, sk{st->k_gscale, frozen ? nullptr : w.gmax_k, H_kv};
   QuantTensor tq{q, st->q_mean, sq, N_q, q ? H_q : 0, q ? pad128(N_q) / TILE : 0, 0, q ? q_out->codes : nullptr, q ? q_out->sf : nullptr};

@@ -88,8 +88,8 @@ __device__ __forceinline__ uint32_t cluster_address(uint32_t smem, uint32_t rank
 __device__ __forceinline__ void cluster_store(uint32_t addr, double x) {
   asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(addr), "d"(x) : "memory");
 }
-__device__ __forceinline__ void cluster_store(uint32_t addr, float x, float y) {
-  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(x), "f"(y) : "memory");
+__device__ __forceinline__ void cluster_store(uint32_t addr, uint32_t x) {
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(x) : "memory");
 }
 
 // ---------------------------------------------------------------- TMA

@@ -345,3 +345,33 @@ def test_a_workspace_for_two_slices_is_used_as_two():
     for nbytes, mean in ((n_min, 1.0 / 1024), (n_min + per - 256, 1.0 / 1024), (n_min + per, 0.0), (n_full, 0.0)):
         s1 = binding.stage1(x, x, x, workspace=torch.empty(nbytes, dtype=torch.uint8, device="cuda"))
         assert float(s1.stats.q_mean[0, 0, 5]) == mean and float(s1.stats.k_mean[0, 0, 5]) == mean, nbytes
+
+
+@pytest.mark.parametrize("B,N_q,N,Hq,Hkv", [
+    (1, 129, 129, 1, 1),          # two CTAs of a cluster, one row in the last tile
+    (3, 1, 1025, 2, 1),           # a head with one token: seven slices of its cluster are empty
+    (1, 2049, 2049, 2, 1),        # clusters of sixteen
+    (1, 10240, 10240, 1, 1), (1, 10241, 10241, 1, 1),   # the longest that a cluster takes, and one more
+    (2, 1281, 1281, 8, 2),        # clusters of eight
+    (5, 300, 300, 12, 12),        # more heads than clusters of four fit
+    (37, 257, 257, 4, 4),         # one CTA per head
+])
+def test_stage1_in_one_call_around_the_rule_for_clusters(B, N_q, N, Hq, Hkv):
+    """Statistics by clusters, slices and single CTAs, V's tiles behind them: bit for bit the oracle's, and what the two calls give."""
+    from paper_2609_33135_b200 import binding
+    w = wl.prefill_workload("clusters", 57, B, N, Hq, Hkv, False, N_q=N_q, q_bias=True)
+    q, k, v = w.q.cuda(), w.k.cuda(), w.v.cuda()
+    s1 = binding.stage1(q, k, v, v_scale=0.5)
+    check_stage1(w, binding.stage1(q, k, v), orc.stage1(orc.bf16_bits(w.q), orc.bf16_bits(w.k), orc.bf16_bits(w.v)))
+    one = [t.clone() for t in (s1.q.codes, s1.q.sf, s1.k.codes, s1.k.sf, s1.v_fp8, s1.delta.view(torch.uint8))]
+    for frozen in (0, binding.MPFA_STATS_FROZEN):
+        for t in (s1.q.codes, s1.q.sf, s1.k.codes, s1.k.sf, s1.v_fp8, s1.delta.view(torch.uint8)):
+            t.fill_(0xA5)
+        ws = None if frozen else binding.quantize_workspace(B, Hq, Hkv)
+        if frozen:
+            binding.mpfa_quantize_qkv(q, k, v, binding.MPFA_SMOOTH | frozen, 0.5, s1.stats, s1.q, s1.k, s1.v_fp8, s1.delta, ws)
+        else:
+            binding.mpfa_quantize_qk(q, k, binding.MPFA_SMOOTH, s1.stats, s1.q, s1.k, s1.delta, ws)
+            binding.mpfa_quantize_v(v, 0.5, s1.v_fp8)
+        for t, u in zip((s1.q.codes, s1.q.sf, s1.k.codes, s1.k.sf, s1.v_fp8, s1.delta.view(torch.uint8)), one):
+            assert torch.equal(t, u)

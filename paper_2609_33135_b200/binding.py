@@ -50,10 +50,19 @@ class _PagedKV(ctypes.Structure):
 
 # The same structures as packed bytes, which ctypes passes by address: making and passing three of them takes 1.3 us, three Structures
 # 2.9 us.  Bytes have no type that a call could check, so only the wrappers below pass them, to function objects of their own
-# (packed_mpfa_...), and each kind has a method of its own name; the functions of lib() take typed structures only.
+# (packed_mpfa_...), and each kind has a method of its own name; the functions of lib() take typed structures only.  The packed forms of
+# a serving step's calls are those of csrc/calls.c (1.5 us less a call than through ctypes).
 _pack_stats, _pack_fp4, _pack_paged = struct.Struct("4P").pack, struct.Struct("2P4i").pack, struct.Struct("4P4i").pack
 
 _lib = None
+
+
+def _calls():
+    try:
+        from . import _mpfa_calls
+    except ImportError as e:
+        raise MpfaError(f"{e}: build it with `python -m paper_2609_33135_b200.build`")
+    return _mpfa_calls
 
 
 def lib() -> ctypes.CDLL:
@@ -103,6 +112,8 @@ def load_library(path: str) -> ctypes.CDLL:
             typed, packed = getattr(L, name), L[name]   # two function objects of one symbol
             typed.restype = packed.restype = i
             typed.argtypes, packed.argtypes = args, [vp if t in (st, q4, pk) else t for t in args]
+            if name not in ("mpfa_quantize_qk_static", "mpfa_prefill_variant"):
+                packed = _calls().bind(name, ctypes.cast(typed, vp).value)
             setattr(L, "packed_" + name, packed)
         L.mpfa_static_scratch_bytes.restype = sz
         L.mpfa_quantize_v.restype = i

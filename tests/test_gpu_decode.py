@@ -461,3 +461,23 @@ def test_decode_leaves_a_partition_without_scores_out(value):
     assert float((got[0] - want[0]).abs().max()) <= 1e-6      # the same partitions, merged in another order
     everything = attend(torch.arange(L, device="cuda"), slice(0, 0))
     assert torch.equal(got[1], everything[1])
+
+
+@pytest.mark.parametrize("lens", [[1025, 64, 2048], [4096, 3073, 1024], [4097, 1, 4096]])   # up to two, four and five partitions
+@pytest.mark.parametrize("shift", [0, 1])
+def test_decode_merges_of_few_partitions_write_any_output(lens, shift):
+    """Both merge kernels around the number of partitions where they change, with outputs that start on any element."""
+    from paper_2609_33135_b200 import binding as B_
+    w = wl.decode_workload("dec_few", 91, 3, 10, 2, 1, max(lens), seq_lens=lens)
+    st = run(w)
+    n = w.B * w.H_q * 128
+    out, o32 = (torch.full((n + 2,), 7.0, dtype=t, device="cuda") for t in (torch.bfloat16, torch.float32))
+    B_.mpfa_decode(st.q4, st.kv, st.page_table, st.seq_lens, st.stats, st.v_scale, st.softmax_scale, out[shift:shift + n], o32[shift:shift + n],
+                   st.workspace, st.status)
+    torch.cuda.synchronize()
+    for t, ref in ((out, st.out), (o32, st.out_f32)):
+        assert torch.equal(t[shift:shift + n].view_as(ref), ref)
+        assert float(t[n + shift:].float().min()) == 7.0 and float(t[:shift].float().sum()) == 7.0 * shift
+    for b in range(w.B):
+        d = np.abs(st.out_f32[b].cpu().numpy() - oracle_decode_one(w, b))
+        assert d.max() <= MAX_ABS and d.mean() <= MEAN_ABS, (b, float(d.max()), float(d.mean()))

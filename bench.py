@@ -687,7 +687,7 @@ def run_ours(args, rank, world, local):
 # DRAM bytes per prefill launch from ncu captures (dram__bytes_read.sum + dram__bytes_write.sum), keyed by
 # (q heads, sequence length); lengths without a capture report no traffic figure.
 NCU_TRAFFIC_BYTES = {
-    (32, 16384): {"bytes": 154700000, "source": "profiles/launches_and_dram_bytes.md (47.3 MB read + 107.4 MB written per launch)"},
+    (32, 16384): {"bytes": 163800000, "source": "profiles/launches_and_dram_bytes.md (62.1 MB read + 101.7 MB written per launch)"},
     (32, 131072): {"bytes": 26980000000, "source": "profiles/launches_and_dram_bytes.md (25.7 GB read + 1.28 GB written)"},
 }
 

@@ -1,4 +1,4 @@
-"""ctypes binding of libmpfa.so: same names as the C ABI, argument marshalling only.
+"""Binding of libmpfa.so (ctypes, and callables of its own for a serving step): same names as the C ABI, argument marshalling only.
 
 PyTorch is used for device memory and the current CUDA stream; every step of the path runs
 inside the library's kernels.  There is no fallback: if the shared library is missing or a
@@ -7,12 +7,16 @@ call fails, an exception is raised.
 from __future__ import annotations
 
 import ctypes
+import functools
+import importlib.util
 import os
 import struct
 from dataclasses import dataclass
 from typing import Optional
 
 import torch
+
+from . import build as _build
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libmpfa.so")
@@ -57,12 +61,25 @@ _pack_stats, _pack_fp4, _pack_paged = struct.Struct("4P").pack, struct.Struct("2
 _lib = None
 
 
+@functools.lru_cache(None)
 def _calls():
+    """The module of csrc/calls.c that was built for this interpreter (by its file: a module search would also take one without a tag)."""
+    spec = importlib.util.spec_from_file_location(__package__ + "._mpfa_calls", _build.CALLS)
+    module = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(module)
+    return module
+
+
+def _callable(name: str, address: int):
+    """The callable of an entry point; without the module one that says so, since the typed and the host-only functions need none."""
     try:
-        from . import _mpfa_calls
+        return _calls().bind(name, address)
     except ImportError as e:
-        raise MpfaError(f"{e}: build it with `python -m paper_2609_33135_b200.build`")
-    return _mpfa_calls
+        message = f"{name}: {e}: build it with `python -m paper_2609_33135_b200.build`"
+
+        def missing(*args):
+            raise MpfaError(message)
+        return missing
 
 
 def lib() -> ctypes.CDLL:
@@ -113,7 +130,7 @@ def load_library(path: str) -> ctypes.CDLL:
             typed.restype = packed.restype = i
             typed.argtypes, packed.argtypes = args, [vp if t in (st, q4, pk) else t for t in args]
             if name not in ("mpfa_quantize_qk_static", "mpfa_prefill_variant"):
-                packed = _calls().bind(name, ctypes.cast(typed, vp).value)
+                packed = _callable(name, ctypes.cast(typed, vp).value)
             setattr(L, "packed_" + name, packed)
         L.mpfa_static_scratch_bytes.restype = sz
         L.mpfa_quantize_v.restype = i

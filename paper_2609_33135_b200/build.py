@@ -14,26 +14,26 @@ NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-shared", "-cudart", "static"]
 
 
-# the binding's callables of the C ABI (plain C, no CUDA)
-CALLS = os.path.join(HERE, "_mpfa_calls.so")
+# The binding's callables of the C ABI (plain C, no CUDA).  They are built against one interpreter's headers, which the name says: another
+# interpreter finds none of its own and builds it.
+CALLS = os.path.join(HERE, "_mpfa_calls" + sysconfig.get_config_var("EXT_SUFFIX"))
 
 
-def _stale() -> bool:
-    if not os.path.exists(LIB) or not os.path.exists(CALLS):
-        return True
-    t = min(os.path.getmtime(LIB), os.path.getmtime(CALLS))
-    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(HERE, "..", "include", "mpfa.h")]
-    return any(os.path.getmtime(d) > t for d in deps)
+def _stale(target: str, sources) -> bool:
+    return not os.path.exists(target) or any(os.path.getmtime(s) > os.path.getmtime(target) for s in sources)
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    if force or _stale():
+    header = os.path.join(HERE, "..", "include", "mpfa.h")
+    calls = os.path.join(CSRC, "calls.c")
+    if force or _stale(LIB, [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f != "calls.c"] + [header]):
         nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
         cmd = [nvcc, *NVCC_FLAGS, *(["-Xptxas", "-v"] if verbose else []), "-o", LIB,
                *[os.path.join(CSRC, s) for s in SOURCES]]
         subprocess.check_call(cmd)
+    if force or _stale(CALLS, [calls, header]):
         subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-I" + sysconfig.get_paths()["include"],
-                               "-o", CALLS, os.path.join(CSRC, "calls.c")])
+                               "-o", CALLS, calls])
     return LIB
 
 

@@ -204,10 +204,16 @@ struct DCtx {
   volatile int *abort_flag;
   int32_t *status;
   __device__ __forceinline__ uint32_t bar(int i) const { return bar0 + 8u * (uint32_t)i; }
-  // Bounded wait; a timeout (or another role's abort) ends in a status bit and `false`.
-  __device__ bool wait(int i, uint32_t parity) const {
+  // Bounded wait; a timeout (or another role's abort) ends in a status bit and `false`.  The waiting itself is one function for all
+  // roles: nineteen warps run ten different pieces of code once per item, and with the loop copied into each of its thirty places they
+  // pushed each other out of the instruction cache (stamps: every step of an item of one block took two to three times as long on some SMs
+  // as on others).  Decode alone, copied / called: 512 requests of 16..128 tokens, 32:8 heads 84.1 / 62.4 us, 40:8 95.1 / 68.0, of
+  // 100..2000 209 / 181; one request of 4097 13.0 / 12.6; 16 of 30000..33000 144.9 / 142.5.
+  __device__ __forceinline__ bool wait(int i, uint32_t parity) const {
     const uint32_t a = bar(i);
-    if (mbar_try_wait(a, parity)) return true;
+    return mbar_try_wait(a, parity) || wait_longer(a, parity, abort_flag, status);
+  }
+  static __device__ __noinline__ bool wait_longer(uint32_t a, uint32_t parity, volatile int *abort_flag, int32_t *status) {
     const long long t0 = clock64();
     for (uint32_t n = 1;; ++n) {
       if (mbar_try_wait_hint(a, parity, 2000u)) return true;   // the hardware may park the thread meanwhile

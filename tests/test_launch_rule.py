@@ -97,3 +97,13 @@ def test_the_only_build_switches_are_the_give_up_test_builds():
     for f in SOURCES:
         found |= set(re.findall(r"^[ \t]*#[ \t]*(?:if|ifdef|ifndef|elif)\b[^\n]*?\b(MPFA_\w+)", code(f), flags=re.M))
     assert found == {"MPFA_WAIT_LIMIT_CYCLES", "MPFA_DRAIN_LIMIT_NS", "MPFA_TEST_DROP_V_COPY"}
+
+
+def test_decode_roles_share_one_waiting_loop():
+    """A copy of the loop in each of some thirty waits takes the roles' code past the instruction cache: batches of short contexts were 8 %
+    slower for it than with one softmax group fewer in each item."""
+    text = code("decode.cu")
+    wait = re.search(r"bool wait\(int i, uint32_t parity\) const \{(.*?)\}", text, flags=re.S).group(1)
+    assert not re.search(r"\b(for|while)\b", wait) and "wait_longer(" in wait
+    assert re.search(r"__noinline__ bool wait_longer\(", text)
+    assert text.count("mbar_try_wait_hint(") == 1

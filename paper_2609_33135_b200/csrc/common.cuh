@@ -67,6 +67,28 @@ cudaError_t launch(void (*kernel)(KArgs...), Grid grid, dim3 block, size_t smem,
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
+// How many clusters of a launch the stream's context holds at a time; 0 where it cannot place one.
+template <typename... KArgs>
+int max_active_clusters(void (*kernel)(KArgs...), Grid grid, dim3 block, size_t smem, cudaStream_t stream) {
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = grid.cluster;
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid.blocks;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+    (void)cudaGetLastError();   // answered here: not reported by the next call that asks
+    return 0;
+  }
+  return n;
+}
+
 // The current device and its SM count; MPFA_ERR_ARCH for devices that cannot run the sm_100a-only kernels.  These are facts of
 // the device, whatever its contexts, and asked for once (two attribute queries cost as much host time as a third of a launch).
 mpfa_status device_info(int *dev, int *n_sm);

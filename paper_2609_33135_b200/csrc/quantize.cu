@@ -17,6 +17,7 @@
 
 #include "common.cuh"
 #include "sm100_ptx.cuh"
+#include "stat_split.hpp"
 
 namespace mpfa {
 
@@ -79,7 +80,6 @@ constexpr int STAT_THREADS = 256;
 constexpr int STAT_LOADS = 8;   // rows in flight per thread, and as many being added
 constexpr int STAT_CTAS = 2;    // resident per SM
 constexpr int STAT_LANES = STAT_THREADS / 16;
-constexpr int STAT_CLUSTER = 16;   // more than eight have to be allowed
 
 struct ColTensor {
   const __nv_bfloat16 *x;   // null: tensor absent (H = 0)
@@ -1010,29 +1010,25 @@ StatsWorkspace carve(void *ws, size_t ws_bytes, int B, int H_q, int H_kv) {
 }
 
 // Means and the heads' maxima of up to two tensors, and V's tiles.
-constexpr int STAT_CLUSTER_MIN = 128;   // tokens of a slice: one round of loads
-constexpr int STAT_CLUSTER_MAX = 640;   // beyond that the slices of one wave are shorter (limits of 256, 512 and 1100 tokens were worse or no better)
 constexpr long long V_APART = 512ll << 20;
 mpfa_status tensor_stats(const ColTensor &c0, const ColTensor &c1, int B, int max_slices, int n_sm, bool smooth, const VTensor &v, cudaStream_t st) {
   const int heads = c0.H + c1.H, N = std::max(c0.x ? c0.N : 0, c1.x ? c1.N : 0);
   if (heads == 0) return MPFA_OK;
   const long long v_ctas = v.x ? (long long)v.tiles * v.H * B : 0;
-  // Short passes: a cluster for each head, of a power of two CTAs (clusters of seven leave places free in every GPC: 8 + 2 heads of
-  // 4 x 777 tokens 13.7 us of stage 1, with four 11.9), as long as its slices stay short and all clusters fit at once.
-  int C = STAT_CLUSTER;
-  while (C > 1 && (C > max_slices || (C > 8 && N <= 16 * STAT_CLUSTER_MIN) || C * heads * (long long)B * 8 > 7LL * STAT_CTAS * n_sm ||
-                   C / 2 * STAT_CLUSTER_MIN >= N))
-    C /= 2;
-  if (C > 1 && N <= C * STAT_CLUSTER_MAX) {
-    if (C > 8) MPFA_CUDA_OK(cudaFuncSetAttribute(colstat_kernel<true, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));   // kept per context
-    const long long ctas = (long long)C * heads * B + (v_ctas + C - 1) / C * C;
-    MPFA_CUDA_OK(launch(colstat_kernel<true, true>, Grid(dim3((unsigned)ctas), C), dim3(STAT_THREADS), 0, st, c0, c1, B, C, smooth ? 1 : 0, v));
+  const auto cluster_grid = [&](int C) { return Grid(dim3((unsigned)((long long)C * heads * B + (v_ctas + C - 1) / C * C)), C); };
+  // The stream's context may own a part of the device only, without room for so many CTAs side by side: the driver is asked for this
+  // launch, with this stream, since an answer that was kept would not hold for another one.
+  const auto placeable = [&](int C) {
+    if (C > 8 && cudaFuncSetAttribute(colstat_kernel<true, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)   // kept per context
+      return (void)cudaGetLastError(), false;
+    return max_active_clusters(colstat_kernel<true, true>, cluster_grid(C), dim3(STAT_THREADS), 0, st) > 0;
+  };
+  const StatSplit split = stat_split((long long)heads * B, N, max_slices, STAT_CTAS, n_sm, placeable);
+  const int S = split.slices;
+  if (split.clusters) {
+    MPFA_CUDA_OK(launch(colstat_kernel<true, true>, cluster_grid(S), dim3(STAT_THREADS), 0, st, c0, c1, B, S, smooth ? 1 : 0, v));
     return MPFA_OK;
   }
-  // As many slices as the launch can hold in one wave.  A fold costs about as much as STAT_MIN tokens
-  // of a CTA's pass, so slices are not made shorter than that.
-  constexpr int STAT_MIN = 512;
-  const int S = (int)std::max(1LL, std::min({(long long)max_slices, (long long)STAT_CTAS * n_sm / ((long long)heads * B), (long long)N / STAT_MIN}));
   MPFA_CUDA_OK(launch(v.x ? colstat_kernel<false, true> : colstat_kernel<false, false>, dim3((unsigned)((long long)S * heads * B + v_ctas)),
                       dim3(STAT_THREADS), 0, st, c0, c1, B, S, smooth ? 1 : 0, v));
   if (S > 1) MPFA_CUDA_OK(launch(stat_fold_kernel, dim3(heads, B), dim3(128), 0, st, c0, c1, S, smooth ? 1 : 0));

@@ -18,6 +18,7 @@ weak and `value` is the sum over ranks divided by the slowest rank's time.
 from __future__ import annotations
 
 import argparse
+import ctypes
 import json
 import math
 import os
@@ -33,7 +34,6 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
 METRIC = "QK4PV8 prefill TFLOPS @16K-128K; decode KV GB/s vs HBM peak"
-KERNELS_PER_STEP = 4  # column statistics of Q and K with V quantize, their fold over slices, K + Delta_S and Q tiles, prefill
 # Nominal dense tensor rates relative to BF16: FP4 4x, FP8 2x.  Per (query, key) pair the path does
 # 2d FP4 FLOP and 2d FP8 FLOP, so F attention FLOPs take (F/2)/(4P) + (F/2)/(2P) = 3F/(8P): the
 # mixed-precision bound in attention FLOP/s is 8/3 of the BF16 peak P.
@@ -285,6 +285,17 @@ def bench_decode(steps, warmup, peaks, small):
             "l2": "3.9 GB of cache per step vs 126 MB L2", "status": int(st.status.item())}
 
 
+def kernels_launched(call):
+    """Kernels that one call launches (how many depends on the sizes): the nodes of a graph that it is captured into."""
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph, capture_error_mode="thread_local"):   # a process group's watchdog thread asks for events meanwhile
+        call()
+    n = ctypes.c_size_t()
+    rc = ctypes.CDLL("libcuda.so.1").cuGraphGetNodes(ctypes.c_void_p(graph.raw_cuda_graph()), None, ctypes.byref(n))
+    assert rc == 0, rc
+    return n.value
+
+
 def bench_prefill_paged(w, k, v, s1, out_ref, steps, warmup):
     """The same prefill with K, V, scales and Delta_S read from a paged low-bit cache (64-token pages in a
     shuffled pool) instead of contiguous tensors; the result must equal the contiguous kernel's bit for bit."""
@@ -526,6 +537,7 @@ def run_ours(args, rank, world, local):
     ms_step = total_ms / args.steps
     kernel_ms = sum(a.elapsed_time(b) for a, b in kev) / args.steps
     assert int(status.item()) == 0, f"device status {int(status.item())}"
+    launches = kernels_launched(step)
 
     # ---- end to end: pinned host inputs in, BF16 output back, every step.  Three streams and two buffer
     # sets, so that the upload of step i+1 and the download of step i-1 run while step i computes (the copy
@@ -604,11 +616,11 @@ def run_ours(args, rank, world, local):
                    "causal": True, "parallelism": f"dp{world} (independent batch elements, no collective)",
                    "l2": f"inputs_exceed_l2 (Q+K+V {(q.numel() + k.numel() + v.numel()) * 2 / 1e6:.0f} MB, "
                          f"output {out.numel() * 2 / 1e6:.0f} MB per step vs 126 MB L2)",
-                   "step": "quantize_qk + quantize_v + prefill"},
+                   "step": "quantize_qkv + prefill"},
         "clocks": clocks,
         "e2e": {"value": whole_job_value(world, flops, e2e_ms), "unit": "TFLOPS", "ms_per_step": e2e_ms,
                 "h2d_bytes_per_step": (q.numel() + k.numel() + v.numel()) * 2, "d2h_bytes_per_step": out.numel() * 2},
-        "gpu_launches": KERNELS_PER_STEP * args.steps,
+        "gpu_launches": launches * args.steps,
         "roofline": {"kernel": "prefill_kernel", "bound": "tensor", "achieved": achieved, "peak": peak,
                      "unit": "TFLOP/s", "frac": achieved / peak,
                      "traffic": NCU_TRAFFIC_BYTES.get((w.H_q, N), {}).get("bytes"),

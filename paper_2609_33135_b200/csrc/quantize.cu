@@ -413,6 +413,18 @@ __device__ __forceinline__ void quantize_blocks(const float (&xa)[16], const flo
   ca = make_uint2(e2m1x8(ya, 0), e2m1x8(ya, 8));
   cb = make_uint2(e2m1x8(yb, 0), e2m1x8(yb, 8));
 }
+// One of them, for a kernel that has no registers for both.
+__device__ __forceinline__ void quantize_block16(const float (&xc)[16], const BlockScale &q, uint32_t &scale_code, uint2 &codes) {
+  const float a = block_max(xc);
+  float r = __fmul_rn(a, q.rcp);
+  if (near_boundary(r)) r = __fdiv_rn(a, q.e);
+  scale_code = (uint32_t)__nv_cvt_float_to_fp8(r, __NV_SATFINITE, __NV_E4M3);
+  const float inv = q.inv[scale_code & 127u];
+  float y[16];
+#pragma unroll
+  for (int i = 0; i < 16; i += 2) mul2(y[i], y[i + 1], xc[i], xc[i + 1], inv);
+  codes = make_uint2(e2m1x8(y, 0), e2m1x8(y, 8));
+}
 // The four lanes j of a row hold the scale bytes of blocks j and j + 4: lane 0 gets the word of blocks 0..3, lane 1 that of 4..7.
 __device__ __forceinline__ uint32_t scale_word(uint32_t two, int j) {
   uint32_t w = two << (16 * (j & 1));
@@ -807,9 +819,12 @@ __global__ void __launch_bounds__(256) quantize_v_fp4_tile_kernel(const __nv_bfl
 // 16-byte groups XOR-ed by the head.  K, V and Delta_S come from one read of K and V, and the rows of the next page are
 // requested while the current ones are quantized.  Slots past the last token are zero-filled in pages that the call
 // starts (a recycled page may hold anything, and decode needs finite bytes there); slots of earlier tokens are left alone.
-// Measured (9001 tokens, 32:8 heads): page kernel + a Delta_S kernel that read K again 12 + 16 us, one page per CTA 19.5 us, now
-// 14.1 us.
-constexpr int WK_CTAS = 2;   // resident per SM: 128 registers, so that the means stay in registers
+// Measured (9001 tokens, 32:8 heads): page kernel + a Delta_S kernel that read K again 12 + 16 us, one page per CTA 19.5 us.  The two blocks
+// of a row one after the other, each half's next rows requested as soon as its registers are free, and the means in shared memory: the kernel
+// alone 11.7 us, means in registers 12.8; 5505 tokens of 4:4 heads 7.2 and 7.9, 45313 of 16:16 137 and 143.  Both blocks at once, as in the
+// tile kernel, wait for the next rows longer than they gain: 13.0, 8.4 and 160 with the means in registers; with shared means 12.5, 7.7 and 129,
+// but 512 tokens of 32:8 4.4 where one after the other takes 4.2, 1408 5.5 and 5.2.
+constexpr int WK_CTAS = 2;   // resident per SM: 128 registers
 __global__ void __launch_bounds__(256, WK_CTAS) write_kv_kernel(const __nv_bfloat16 *k, const __nv_bfloat16 *v,
                                                                 const float *k_mean, const TensorScale k_scale,
                                                                 const float *q_mean, const float *q_gscale,
@@ -842,9 +857,8 @@ __global__ void __launch_bounds__(256, WK_CTAS) write_kv_kernel(const __nv_bfloa
   const float d = tensor_scale(k_scale, 0, lane);
   if (blockIdx.y == 0 && h == 0 && tid == 0 && k_scale.gmax) k_scale.gscale[0] = d;
   const BlockScale bs = make_block_scale(d, inv_table, tid);
-  float neg_mean[2][16];
-  load_neg_mean(k_mean + (size_t)h * HEAD_DIM + j * 16, neg_mean[0], vector_means(k_mean));
-  load_neg_mean(k_mean + (size_t)h * HEAD_DIM + 64 + j * 16, neg_mean[1], vector_means(k_mean));
+  __shared__ __align__(16) float s_neg[8][20];   // by 16-channel block, padded against bank conflicts
+  if (tid < HEAD_DIM) s_neg[tid >> 4][tid & 15] = -k_mean[(size_t)h * HEAD_DIM + tid];
   double unit = 0.0;
   if (delta) {
     convert_group_means(gm, q_mean + (size_t)h * G * HEAD_DIM, G, tid, 256);
@@ -862,28 +876,32 @@ __global__ void __launch_bounds__(256, WK_CTAS) write_kv_kernel(const __nv_bfloa
     pg += gridDim.y;
     if (pg < n_pages) page = page_row[page0 + pg];
     double acc[2] = {0.0, 0.0};
-    float xa[16], xb[16];
-    center16(kr[0], neg_mean[0], xa);
-    center16(kr[1], neg_mean[1], xb);
-    uint4 va = quantize_v16(vr[0], inv_vscale), vb = quantize_v16(vr[1], inv_vscale);
-    fetch(0);
-    fetch(1);
-    uint2 ca, cb;
-    uint32_t sc;
-    quantize_blocks(xa, xb, bs, sc, ca, cb);
-    if (!is_new) ca = cb = make_uint2(0u, 0u), sc = 0u, va = vb = make_uint4(0u, 0u, 0u, 0u);
-    sc = scale_word(sc, j);
-    if (is_new || fresh_pad) {   // blocks j and j + 4 of the row
-      uint8_t *const kj = kd + (j & 1) * 8;
-      *reinterpret_cast<uint2 *>(kj + (((j >> 1) ^ ((t & 7) >> 1)) << 4)) = ca;
-      *reinterpret_cast<uint2 *>(kj + ((((j + 4) >> 1) ^ ((t & 7) >> 1)) << 4)) = cb;
-      if (j < 2) *reinterpret_cast<uint32_t *>(sd + j * 4) = sc;
-      *reinterpret_cast<uint4 *>(vd + ((j ^ (t & 7)) << 4)) = va;
-      *reinterpret_cast<uint4 *>(vd + (((j + 4) ^ (t & 7)) << 4)) = vb;
-    }
-    if (delta) {
-      group_dot16(gm, 0, xa, lane, acc);
-      group_dot16(gm, 1, xb, lane, acc);
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+      const int blk = half * 4 + j;
+      float xc[16];
+      {
+        float nm[16];
+        load_mean16(s_neg[blk], nm, true);
+        center16(kr[half], nm, xc);
+      }
+      uint2 c = make_uint2(0u, 0u);
+      uint32_t sc = 0u;
+      uint4 vc = quantize_v16(vr[half], inv_vscale);
+      fetch(half);
+      if (is_new)
+        quantize_block16(xc, bs, sc, c);
+      else
+        vc = make_uint4(0u, 0u, 0u, 0u);
+      sc <<= 8 * j;   // the four scale bytes of half a token in one word
+      sc |= __shfl_xor_sync(0xffffffffu, sc, 1);
+      sc |= __shfl_xor_sync(0xffffffffu, sc, 2);
+      if (is_new || fresh_pad) {
+        *reinterpret_cast<uint2 *>(kd + (((blk >> 1) ^ ((t & 7) >> 1)) << 4) + (blk & 1) * 8) = c;
+        if (j == 0) *reinterpret_cast<uint32_t *>(sd + half * 4) = sc;
+        *reinterpret_cast<uint4 *>(vd + ((blk ^ (t & 7)) << 4)) = vc;
+      }
+      if (delta) group_dot16(gm, half, xc, lane, acc);
     }
     if (delta && (is_new || fresh_pad)) {
 #pragma unroll

@@ -375,3 +375,23 @@ def test_stage1_in_one_call_around_the_rule_for_clusters(B, N_q, N, Hq, Hkv):
             binding.mpfa_quantize_v(v, 0.5, s1.v_fp8)
         for t, u in zip((s1.q.codes, s1.q.sf, s1.k.codes, s1.k.sf, s1.v_fp8, s1.delta.view(torch.uint8)), one):
             assert torch.equal(t, u)
+
+
+@pytest.mark.parametrize("B,N,Hq,Hkv", [(1, 129, 1, 1), (1, 2049, 2, 1), (2, 1281, 8, 2), (1, 10240, 1, 1)])   # clusters of 2, 16, 8, 16
+def test_stage1_by_clusters_without_smoothing_and_from_a_graph(B, N, Hq, Hkv):
+    """Statistics by clusters where no mean is subtracted, and both forms replayed from a graph on other inputs than it was captured with."""
+    from paper_2609_33135_b200 import binding
+    w, other = (wl.prefill_workload("clusters", seed, B, N, Hq, Hkv, False, q_bias=True) for seed in (58, 59))
+    for smooth in (False, True):
+        z = orc.stage1(orc.bf16_bits(w.q), orc.bf16_bits(w.k), orc.bf16_bits(w.v), smooth=smooth)
+        check_stage1(w, run_stage1_gpu(w, smooth=smooth), z, smooth=smooth)
+        q, k, v = other.q.cuda(), other.k.cuda(), other.v.cuda()
+        ws = binding.quantize_workspace(B, Hq, Hkv)
+        s1 = binding.stage1(q, k, v, smooth=smooth, workspace=ws)
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            binding.stage1(q, k, v, smooth=smooth, workspace=ws, out=s1)
+        for t, x in ((q, w.q), (k, w.k), (v, w.v)):
+            t.copy_(x)
+        graph.replay()
+        check_stage1(w, s1, z, smooth=smooth)

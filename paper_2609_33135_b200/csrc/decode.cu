@@ -270,8 +270,13 @@ __device__ __forceinline__ void lookup_pages(const DecodeParams &p, const WorkIt
   }
 }
 
+// Registers of a thread: a block of 256 threads and 64 registers of the small kernels before and after fits on an SM beside a CTA of this
+// one, and its set-up runs meanwhile, if five warps of a sub-partition leave two of those their registers: 5 x 32 R + 2 x 2048 <= 16384, so
+// R <= 72.  Groups of up to four heads need no more (a bound of 896 threads asks for it); the function call in the waits had raised
+// them to 80 and more.  Append, query and decode at 80 / 72: 16 requests of 16..128 tokens, 16:16 heads 17.9 / 14.8 us; 100 of 100..700, 8:2
+// 23.4 / 19.0; 64 of 100..1000, 32:8 31.6 / 30.0.  Larger groups spill there (groups of eight, 64 of 100..2000 21.0 / 21.9).
 template <int G>
-__global__ void __launch_bounds__(D_THREADS, 1) decode_split_kernel(const __grid_constant__ DecodeParams p) {
+__global__ void __launch_bounds__(G <= 4 ? 896 : D_THREADS, 1) decode_split_kernel(const __grid_constant__ DecodeParams p) {
   extern __shared__ uint8_t dsm_raw[];
   uint8_t *dsm = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(dsm_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t sbase = smem_u32(dsm);

@@ -868,17 +868,22 @@ __global__ void __launch_bounds__(128, 9) decode_merge_kernel(const __grid_const
   const size_t head = (size_t)b * p.H_q + hq;
   const float2 *ml = p.part_ml + head * p.n_split;
   const float4 *po = reinterpret_cast<const float4 *>(p.part_o + head * p.n_split * HEAD_DIM) + lane;
-  // The first 16 states are requested before the length is known: the request's slots of the workspace exist whatever it is, and
+  // The first states are requested before the length is known: the request's slots of the workspace exist whatever it is, and
   // what stands in those past its last partition is not used.  (One load after the other, length, maxima, states, the merge of a
-  // single request took 4.2 us alone.)
+  // single request took 4.2 us alone.)  Sixteen of them where there are few heads, which wait for one another's latency only; four where
+  // there are many, since a table that is wider than the requests are long makes the others reads for nothing.  Append, query and decode with
+  // sixteen / four: one request of 4097 keys, 32 heads 18.57 / 18.76 us; 8 x 40 heads the same; 16 requests of 30000..33000, 32 heads 145.8 /
+  // 145.1; 64 x 40 heads of 100..4000 keys in tables of 2048 pages 68.3 / 66.6.
+  const bool few = gridDim.x * gridDim.y <= 320;
   float2 a[4];
   float4 x[4];
 #pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const int s = min(warp + 4 * u, p.n_split - 1);
-    a[u] = ml[s];
-    x[u] = po[(size_t)s * (HEAD_DIM / 4)];
-  }
+  for (int u = 0; u < 4; ++u)
+    if (u == 0 || few) {
+      const int s = min(warp + 4 * u, p.n_split - 1);
+      a[u] = ml[s];
+      x[u] = po[(size_t)s * (HEAD_DIM / 4)];
+    }
   const float first_max = ml[min(lane, p.n_split - 1)].x;
   const int n = p.n_parts(p.seq_lens[b]);
   const float lam = __fmul_rn(__fmul_rn(__fmul_rn(p.softmax_scale, 1.4426950408889634f), p.q_gscale[b]), p.k_gscale[b]);
@@ -889,14 +894,13 @@ __global__ void __launch_bounds__(128, 9) decode_merge_kernel(const __grid_const
   float l = 0.0f, o[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll 1
   for (int s0 = warp; s0 < n; s0 += 16) {
-    if (s0 != warp) {
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
+    for (int u = 0; u < 4; ++u)
+      if (s0 != warp || (u > 0 && !few)) {
         const int s = min(s0 + 4 * u, n - 1);
         a[u] = ml[s];
         x[u] = po[(size_t)s * (HEAD_DIM / 4)];
       }
-    }
 #pragma unroll
     for (int u = 0; u < 4; ++u)
       if (s0 + 4 * u >= n) a[u].x = -INFINITY;

@@ -481,3 +481,30 @@ def test_decode_merges_of_few_partitions_write_any_output(lens, shift):
     for b in range(w.B):
         d = np.abs(st.out_f32[b].cpu().numpy() - oracle_decode_one(w, b))
         assert d.max() <= MAX_ABS and d.mean() <= MEAN_ABS, (b, float(d.max()), float(d.mean()))
+
+
+def test_decode_merges_of_many_heads_are_those_of_few():
+    """The merge reads fewer states ahead of the length where there are many heads (here 360, and 40 a request alone): the same sums in the
+    same order, in a table wider than any request."""
+    from paper_2609_33135_b200 import binding as B_
+    lens = [1, 1024, 1025, 4096, 4097, 16384, 16385, 17500, 3000]   # one partition to eighteen
+    w = wl.decode_workload("dec_many_heads", 93, len(lens), 40, 8, 1, max(lens), seq_lens=lens)
+    st = run(w)
+    table = torch.full((w.B, 512), -1, dtype=torch.int32, device="cuda")
+    table[:, :st.page_table.shape[1]] = st.page_table
+    ws = B_.decode_workspace(w.B, w.H_q, w.H_kv, 512)
+
+    def attend(b0, b1):
+        out = torch.empty(b1 - b0, w.H_q, 128, dtype=torch.float32, device="cuda")
+        q4 = B_.Fp4Tensor(st.q4.codes[b0 * w.H_q * 8192:], st.q4.sf[b0 * w.H_q * 1024:], b1 - b0, w.H_q, 1)
+        x = st.stats
+        stats = B_.Stats(x.q_mean[b0:b1], x.k_mean[b0:b1], x.q_gscale[b0:b1], x.k_gscale[b0:b1])
+        ws.fill_(0xFF)   # NaN in every state that no partition writes
+        B_.mpfa_decode(q4, st.kv, table[b0:b1], st.seq_lens[b0:b1], stats, st.v_scale, st.softmax_scale,
+                       torch.empty(b1 - b0, w.H_q, 128, dtype=torch.bfloat16, device="cuda"), out, ws, st.status)
+        return out
+
+    together = attend(0, w.B)
+    assert bool(torch.isfinite(together).all()) and int(st.status.item()) == 0
+    for b in range(w.B):
+        assert torch.equal(together[b], attend(b, b + 1)[0]), lens[b]

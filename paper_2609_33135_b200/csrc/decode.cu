@@ -41,10 +41,11 @@
 // block weights held in the lanes and handed out by shuffles, where every thread took them from shared memory for every
 // block: 256 requests of 100..2000 tokens with append and query 137 -> 130 us, one request of 4097 22.6 -> 21.7 us.
 // K blocks by two warps in turn, each lane issuing its own block, MMAs issued by one thread that also waits, both softmax groups on every
-// item, V held back until the first item's K is on its way (replayed back to back): one request of 4097 keys 15.4 -> 12.6 us, 64 of
-// 100..4000 57.5 -> 53.8, 32 of 16K..128K 690 -> 629 (7.1 TB/s of cache).  Not kept: K rings of 5, 6 and 7 stages (1 to 3 us more on
-// short batches, nothing on long ones), small pieces by 16-byte copies of all lanes (no gain), partitions shorter than 1024 keys
-// drawn last (2 us more on 64 requests).
+// item, V held back until the first item's K is on its way, and then one waiting loop for all roles (replayed back to back): one request of
+// 4097 keys 15.5 -> 12.9 -> 12.6 us, 64 of 100..4000 63.1 -> 59.2 -> 53.8, 32 of 16K..128K 703 -> 649 -> 634 (4.06 GB of cache, 6.4 TB/s).
+// Not kept: K rings of 5, 6 and 7 stages (1 to 3 us more on short batches, nothing on long ones), small pieces by 16-byte copies of all
+// lanes (no gain), partitions shorter than 1024 keys drawn last (2 us more on 64 requests), items of one block by one softmax group alone
+// (no gain on them, 1 to 3 % more on 512 requests of 100..2000).
 //
 // Warps: 18 draws work items and stages their query tiles, 0 and 17 K producers (alternate blocks),
 // 16 V producer, 1 QK issue (+ TMEM allocation), 2 PV issue, 3 rewrites the K scales of each block from
@@ -113,7 +114,7 @@ constexpr int B_XCHG = B_O_FREE + 1;             // [2] 8 softmax warps: block m
 constexpr int B_ITEM_FULL = B_XCHG + 2;          // [D_NITEM] work item published
 constexpr int B_ITEM_EMPTY = B_ITEM_FULL + D_NITEM;   // [D_NITEM] read by all eighteen consumer warps
 constexpr int B_DRAW = B_ITEM_EMPTY + D_NITEM;   // [2] warp 0 has begun item k (slot k & 1): the next one may be drawn
-constexpr int B_V_GO = B_DRAW + 2;               // [1] every K copy of the CTA's first item is on its way
+constexpr int B_V_GO = B_DRAW + 2;               // [1] warp 0 has issued its K blocks of the CTA's first item (when to begin, nothing more)
 constexpr int B_COUNT = B_V_GO + 1;
 static_assert(B_COUNT * 8 <= 1024, "barrier block");
 static_assert(D_SMEM <= 232448, "shared memory");
@@ -196,7 +197,9 @@ struct DecodeParams {
 // shared-memory ring; every other warp walks that ring.  SMs do not stream at the same rate (those far from the memory
 // they read are up to 8 % slower), so a static split leaves the fast ones idle at the end.  An item is drawn when the K
 // producer begins the one before it: drawn further ahead, a short batch is shared out unevenly (64 requests of one
-// partition, 512 items on 148 CTAs, drawn eight ahead: the first 64 CTAs could take them all).
+// partition, 512 items on 148 CTAs, drawn eight ahead: the first 64 CTAs could take them all).  After an item of at most half a
+// partition it is drawn one earlier, since such an item's K is issued before the next ticket is there (decode alone, one / two ahead: 512
+// requests of 257..512 tokens, 32:8 heads 80.1 / 73.3 us, 40:8 83.4 / 79.2; of 100..2000 169 / 164; of 16..256 the same within 1 %).
 struct WorkIter;
 
 struct DCtx {
@@ -470,7 +473,8 @@ __global__ void __launch_bounds__(G <= 4 ? 896 : D_THREADS, 1) decode_split_kern
     if (vw) lookup_pages(p, w, lane, pc0, pc1);
     for (; ok && vw; ++j) {
       if (warp == 0) cx.warp_arrive(B_DRAW + (j & 1));
-      // Nothing can be done with V before the first item's softmax, and while all CTAs start at once its copies only keep K waiting.
+      // Nothing can be done with V before the first item's softmax, and while all CTAs start at once its copies only keep K waiting, of
+      // which warp 17's last block may still be to come.
       if (!is_k && j == 0) ok = cx.wait_warp(B_V_GO, 0);
       const bool in = lane < w.nblk, want1 = w.sp * DECODE_SPLIT + lane * TILE + PAGE < w.L;
       const bool has0 = in && pc0 >= 0 && pc0 < p.num_pages, has1 = in && want1 && pc1 >= 0 && pc1 < p.num_pages;

@@ -552,7 +552,8 @@ struct DeltaArgs {
 // Tiles (128 tokens of one head) of K and Q; blockIdx.x runs over K's CTAs, then Q's, the head index fastest, so that the
 // CTAs resident at any time read whole token rows of the [B, N, H, 128] input (contiguous DRAM) instead of 256-byte
 // pieces 256 * H bytes apart; from the last token to the first, because the statistics pass has just read the tensors in
-// ascending order and their ends are still in L2.  Warp w takes rows 8 w .. and 64 + 8 w .. of a tile, lane (row, j) their
+// ascending order: of one that fits L2 most is still there, of a larger one the end of its last slice only (32768 tokens of 40:8 heads: 402 of
+// 403 MB come from DRAM again).  Warp w takes rows 8 w .. and 64 + 8 w .. of a tile, lane (row, j) their
 // 16-channel blocks j and j + 4.  A CTA stays with one head, so that after the set-up's barrier its warps run on their own:
 // the loads of the next tile are issued as soon as the registers of a row group are free, scale words and Delta_S go straight
 // to memory (partial sectors merge in L2).
@@ -1100,9 +1101,10 @@ static mpfa_status quantize_qkv(const void *q_bf16, const void *k_bf16, const VT
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const __nv_bfloat16 *q = static_cast<const __nv_bfloat16 *>(q_bf16);
   const __nv_bfloat16 *k = static_cast<const __nv_bfloat16 *>(k_bf16);
-  // V has a launch of its own where there is no other, and where Q and K are well beyond L2: between the two passes over them V
-  // would push out the ends that the second one finds there (32:8 heads: 16384 tokens 83.3 us together, 86.1 apart; 16 x 2000 158 and 167;
-  // 32768, 40:8 177.0 and 176.4; 65536 291 and 287).
+  // V has a launch of its own where there is no other, and for the largest tensors.  Together the two are 1 to 4 % faster (40:8 heads, together /
+  // apart: 16384 tokens, 201 MB of Q and K, 92.8 / 95.3 us; 24576, 302 MB 132.2 / 134.8; 40960, 503 MB 213.1 / 216.3; 49152, 604 MB 254.6 /
+  // 261.0; 65536, 805 MB 335.2 / 337.7), but in some placements of the tensors in memory the statistics with V take 1.6 times as long
+  // (49152 419 us, 65536 555), where those alone kept their time; below the line such placements slow both forms (32768 283 us).
   const bool apart = v.x && (frozen || ((long long)N_q * (q ? H_q : 0) + (long long)N_kv * (k ? H_kv : 0)) * B * HEAD_DIM * 2 > V_APART);
   if (!frozen) {
     rc = tensor_stats(ColTensor{q, N_q, q ? H_q : 0, w.psum_q, w.pext_q, st->q_mean, w.gmax_q},

@@ -6,7 +6,10 @@ namespace mpfa {
 
 constexpr int STAT_CLUSTER = 16;         // largest cluster; more than eight CTAs have to be allowed
 constexpr int STAT_CLUSTER_MIN = 128;    // tokens of a slice: one round of loads
-constexpr int STAT_CLUSTER_MAX = 640;    // beyond that the slices of one wave are shorter (limits of 256, 512 and 1100 tokens were worse or no better)
+// Tokens of a slice up to which clusters are the faster form.  Stage 1 with slices / clusters whose slices have 400, 512, 640 and 800 tokens: 1 + 1
+// heads 13.3 / 10.1, 13.1 / 10.8, 14.0 / 12.0, 15.0 / 13.8 us; 8 + 2 19.6 / 18.0, 20.6 / 18.6, 19.7 / 20.0, 22.6 / 25.1; 16 + 4 19.8 / 17.7,
+// 20.0 / 18.6, 20.7 / 19.9, 22.4 / 25.0; 32 + 8 20.1 / 18.1, 20.4 / 18.9, 20.2 / 19.8, 23.1 / 25.0.
+constexpr int STAT_CLUSTER_MAX = 640;
 constexpr int STAT_MIN = 512;            // tokens of a slice where a launch of its own folds them, which costs about as much
 
 struct StatSplit {

@@ -122,7 +122,7 @@ def test_decode_long_request_many_partitions():
     (6, 2, [2047, 897, 640, 1] * 60),               # many items per CTA, one to eight blocks each, groups of three
 ])
 def test_decode_item_counts_around_the_grid(hq, hkv, lens):
-    """The work-item walk and its two alternating softmax groups: item counts just below and above the grid, partitions
+    """The work-item walk and the two softmax groups' shares of an item: item counts just below and above the grid, partitions
     of every block count, requests complete in one partition next to merged ones."""
     from paper_2609_33135_b200 import decode_cache
     w = wl.decode_workload("dec_items", 78 + hq, len(lens), hq, hkv, 1, max(lens), n_stat_tokens=64, seq_lens=[max(1, n) for n in lens])
